@@ -138,6 +138,8 @@ struct sbnn_packed {
     mutable std::map<long long, sbnn::Plan3x3> plans3x3;           // per (stream, row tiles of the launch, CTAs)
     mutable void* bf16_stream = nullptr;  // see conv1x1_bf16.cu
     mutable void* umma_weights = nullptr; // dense bf16 copy of the masked weights, see conv1x1_umma.cu
+    mutable std::map<int, void*> tc_weights;  // split bf16 images of the masked weights, see conv_tc.cu
+    bool finite = true;                   // every stored weight is finite
 };
 
 namespace sbnn {
@@ -163,10 +165,15 @@ sbnn_status async_status_word(int** out);
 // Fills a 128-byte tensor-map descriptor (CUtensorMap) for tiled copies out of an fp32 (elem_bytes 4) or bf16 (2)
 // tensor: `rank` dimensions, innermost first, `strides_bytes` for dimensions 1.. (multiples of 16), `box` = elements
 // copied per dimension.  Elements outside the tensor are delivered as zeros.
-// With swizzle128 the box's rows (at most 128 bytes) are written to shared memory with the 128-byte swizzle that the
-// tcgen05 operand descriptors expect.
+// swizzle: 0, or 64 or 128 = the box's rows (at most that many bytes) sit in shared memory with that swizzle (128 is what
+// the tcgen05 operand descriptors expect).
 sbnn_status encode_tiled_map(void* out, const void* base, int elem_bytes, int rank, const unsigned long long* dims,
-                             const unsigned long long* strides_bytes, const unsigned* box, bool swizzle128 = false);
+                             const unsigned long long* strides_bytes, const unsigned* box, int swizzle = 0);
+// im2col tensor map of NHWC fp32 activations for a 3x3 kernel with padding 1: boxes of `pixels` consecutive output positions
+// x `channels` channels (128-byte rows, 128-byte swizzle), zeros outside the image.
+sbnn_status encode_im2col_3x3_map(void* out, const float* x, int N, int H, int W, int C, int channels, int pixels);
+// SMs of the current device.
+int device_sms();
 // Per-device scratch buffer for channel-major copies made on behalf of NHWC callers.  Grows on demand with a
 // synchronous allocation (the outgrown buffer is kept until the process exits, so work already enqueued or recorded
 // on it stays valid); growth while `st` is being captured is refused with SBNN_ERR_UNSUPPORTED.
@@ -187,6 +194,15 @@ void free_stream_bf16(sbnn_packed* p);
 // conv1x1_umma.cu: bf16 mode as a dense contraction over the masked weights (tcgen05); *done = false if the shape is not taken
 sbnn_status conv1x1_umma(const sbnn_packed* w, const float* x, float* y, int M, int relu, cudaStream_t st, bool* done);
 void free_umma_weights(sbnn_packed* p);
+// conv_tc.cu: fp32 layers on the tensor cores by a three-way bf16 split; *done = false (and SBNN_OK) when the shape or the
+// density is better served by the FMA kernels (or outside what the kernel takes)
+sbnn_status conv1x1_tc(const sbnn_packed* p, const float* x, float* y, long long M, int relu, cudaStream_t st, bool* done);
+sbnn_status conv1x1_tc_cm(const sbnn_packed* p, const float* x, int ldx, float* y, int ldy, long long M, int relu, bool out_cm, cudaStream_t st,
+                          bool* done);
+sbnn_status conv3x3_tc(const sbnn_packed* p, const float* x, float* y, int N, int H, int W, int relu, cudaStream_t st, bool* done);
+// Builds the weight images for calls of up to M pixels.
+sbnn_status prepare_tc(const sbnn_packed* p, long long M);
+void free_tc_weights(sbnn_packed* p);
 // conv3x3_gs.cu
 sbnn_status prepare_default_3x3(const sbnn_packed* p);
 void free_streams_3x3(sbnn_packed* p);

@@ -811,7 +811,7 @@ sbnn_status get_encode(EncodeTiledFn* out) {
 // fp32 (elem_bytes 4) or bf16 (2) tensor of `rank` dimensions (innermost first), tiled copies of `box` elements,
 // zeros outside the tensor.
 sbnn_status encode_generic(void* out, const void* base, int elem_bytes, int rank, const unsigned long long* dims,
-                           const unsigned long long* strides_bytes, const unsigned* box, bool swizzle128 = false) {
+                           const unsigned long long* strides_bytes, const unsigned* box, int swizzle = 0) {
     EncodeTiledFn encode = nullptr;
     sbnn_status r = get_encode(&encode);
     if (r != SBNN_OK) return r;
@@ -830,9 +830,36 @@ sbnn_status encode_generic(void* out, const void* base, int elem_bytes, int rank
     const CUresult cr = encode(static_cast<CUtensorMap*>(out),
                                elem_bytes == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
                                (cuuint32_t)rank, const_cast<void*>(base), d, st, b, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                               swizzle128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                               swizzle == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : (swizzle == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE),
                                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (cr != CUDA_SUCCESS) return fail(SBNN_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d)", (int)cr);
+    return SBNN_OK;
+}
+
+typedef CUresult (*EncodeIm2colFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const int*,
+                                   const int*, cuuint32_t, cuuint32_t, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+sbnn_status encode_im2col(void* out, const float* x, int N, int H, int W, int C, int channels, int pixels) {
+    static std::mutex mu;
+    static EncodeIm2colFn encode = nullptr;
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        if (!encode) {
+            void* fn = nullptr;
+            cudaDriverEntryPointQueryResult q;
+            SBNN_CUDA_TRY(cudaGetDriverEntryPoint("cuTensorMapEncodeIm2col", &fn, cudaEnableDefault, &q));
+            if (!fn || q != cudaDriverEntryPointSuccess) return fail(SBNN_ERR_CUDA, "driver has no cuTensorMapEncodeIm2col");
+            encode = reinterpret_cast<EncodeIm2colFn>(fn);
+        }
+    }
+    const cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)N};
+    const cuuint64_t strides[3] = {(cuuint64_t)C * 4, (cuuint64_t)W * C * 4, (cuuint64_t)H * W * C * 4};
+    const int lower[2] = {-1, -1}, upper[2] = {-1, -1};
+    const cuuint32_t es[4] = {1, 1, 1, 1};
+    const CUresult cr = encode(static_cast<CUtensorMap*>(out), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<float*>(x), dims, strides, lower, upper,
+                               (cuuint32_t)channels, (cuuint32_t)pixels, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (cr != CUDA_SUCCESS) return fail(SBNN_ERR_CUDA, "cuTensorMapEncodeIm2col failed (%d)", (int)cr);
     return SBNN_OK;
 }
 
@@ -1067,10 +1094,16 @@ sbnn_status dwconv3x3_conv1x1_fused_cm(const sbnn_packed* pw, const float* dw_w,
 }
 
 sbnn_status encode_tiled_map(void* out, const void* base, int elem_bytes, int rank, const unsigned long long* dims,
-                             const unsigned long long* strides_bytes, const unsigned* box, bool swizzle128) {
-    if (swizzle128 && (size_t)box[0] * elem_bytes > 128) return fail(SBNN_ERR_SHAPE, "a swizzled box row is at most 128 bytes");
-    return encode_generic(out, base, elem_bytes, rank, dims, strides_bytes, box, swizzle128);
+                             const unsigned long long* strides_bytes, const unsigned* box, int swizzle) {
+    if (swizzle && box[0] * (unsigned)elem_bytes > (unsigned)swizzle) return fail(SBNN_ERR_SHAPE, "a swizzled box row is at most %d bytes", swizzle);
+    return encode_generic(out, base, elem_bytes, rank, dims, strides_bytes, box, swizzle);
 }
+
+sbnn_status encode_im2col_3x3_map(void* out, const float* x, int N, int H, int W, int C, int channels, int pixels) {
+    return encode_im2col(out, x, N, H, W, C, channels, pixels);
+}
+
+int device_sms() { return sm_count(); }
 
 sbnn_status prepare_default_cm(const sbnn_packed* p, long long M) {
     Stream1x1 s;
@@ -1179,6 +1212,10 @@ extern "C" sbnn_status sbnn_conv1x1_gs_cm(const sbnn_packed* w, const float* xt_
     sbnn_status st = check_packed_device(w);
     if (st != SBNN_OK) return st;
     if ((st = check_device()) != SBNN_OK) return st;
+    bool done = false;
+    if (!(P | GPW | NW | KC) && ((st = conv1x1_tc_cm(w, xt_dev, ldx, y_dev, ldy, M, flags & SBNN_RELU, out_cm, static_cast<cudaStream_t>(cuda_stream),
+                                                     &done)) != SBNN_OK || done))
+        return st;
     if (!(P | GPW | NW | KC) && few_tiles(w, M))
         return conv1x1_small(w, xt_dev, ldx, y_dev, ldy, M, flags & SBNN_RELU, out_cm, static_cast<cudaStream_t>(cuda_stream));
     const TileCfg c = (P | GPW | NW | KC) ? TileCfg{P, GPW, NW, KC} : default_cfg_cm(w, M);

@@ -437,6 +437,8 @@ extern "C" sbnn_status sbnn_conv1x1_gs(const sbnn_packed* w, const float* x_dev,
             return st;
         return conv1x1_bf16(w, x_dev, y_dev, (int)M, flags & SBNN_RELU, s);
     }
+    // (a layer is prepared for this route and, for calls with fewer pixels, the next one)
+    if ((st = conv1x1_tc(w, x_dev, y_dev, M, flags & SBNN_RELU, s, &done)) != SBNN_OK || (done && !prepare_only())) return st;
     if ((st = conv1x1_via_cm(w, x_dev, y_dev, (int)M, flags & SBNN_RELU, s, &done)) != SBNN_OK || done) return st;
     return dispatch(w, choose_cfg(w, M), x_dev, y_dev, (int)M, flags & SBNN_RELU, s);
 }

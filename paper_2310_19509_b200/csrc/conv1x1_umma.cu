@@ -35,72 +35,10 @@
 
 #include "common.h"
 #include "pipeline.cuh"
+#include "tcgen05.cuh"
 
 namespace sbnn {
 namespace {
-
-// ---- tcgen05 primitives ---------------------------------------------------------------------------
-__device__ __forceinline__ void tc_fence_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// Whole warp: reserves `cols` (a power of two >= 32) columns of tensor memory; the base address lands in *holder.
-__device__ __forceinline__ void tmem_alloc(uint32_t* holder_smem, uint32_t cols) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(holder_smem)), "r"(cols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t base, uint32_t cols) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "r"(cols) : "memory");
-}
-
-// Shared-memory operand descriptor: K-major tile whose rows are 128 bytes (64 bf16) written with the 128-byte
-// swizzle, rows 128 bytes apart, groups of 8 rows 1024 bytes apart; `addr` = shared address of the first row's
-// 16-byte chunk to start from (the tile itself is 1024-byte aligned, a K offset of 16 elements is +32 bytes).
-__device__ __forceinline__ uint64_t operand_desc(uint32_t addr) {
-    uint64_t d = (uint64_t)((addr & 0x3FFFFu) >> 4);   // bits  0-13: start address / 16
-    d |= (uint64_t)1 << 16;                            // bits 16-29: leading byte offset / 16 (not used by this layout)
-    d |= (uint64_t)(1024 >> 4) << 32;                  // bits 32-45: stride byte offset / 16
-    d |= (uint64_t)1 << 46;                            // bits 46-47: descriptor version of this architecture
-    d |= (uint64_t)2 << 61;                            // bits 61-63: 128-byte swizzle
-    return d;
-}
-
-// Instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, M = 128, N = n.
-__host__ __device__ constexpr uint32_t instr_desc(int n) {
-    return (1u << 4)                    // accumulator format fp32
-           | (1u << 7) | (1u << 10)     // A and B format bf16
-           | ((uint32_t)(n >> 3) << 17) // N / 8
-           | ((uint32_t)(128 >> 4) << 24);   // M / 16
-}
-
-// One thread: D[tmem] (+)= A[smem] * B[smem]^T, 128 x N x 16.
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %5, %5, %5}, p;\n\t}"
-        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(0u)
-        : "memory");
-}
-// The mbarrier receives one arrival once every MMA this thread has issued so far is complete.
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-// Whole warp: 32 consecutive fp32 columns of the warp's 32 tensor-memory lanes (lane l of the warp gets row l).
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
-          "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]),
-          "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
-          "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-        : "r"(taddr)
-        : "memory");
-}
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // ---- tile shape -----------------------------------------------------------------------------------
 template <int BN_>
@@ -347,20 +285,20 @@ sbnn_status launch_umma(const sbnn_packed* p, const DenseBf16& d, const __nv_bfl
         const unsigned long long dims[2] = {(unsigned long long)T::BK, (unsigned long long)mtiles * nkb * T::BM};
         const unsigned long long strides[1] = {(unsigned long long)T::BK * 2};
         const unsigned box[2] = {(unsigned)T::BK, (unsigned)T::BM};
-        if ((r = encode_tiled_map(&amap, xb, 2, 2, dims, strides, box, true)) != SBNN_OK) return r;
+        if ((r = encode_tiled_map(&amap, xb, 2, 2, dims, strides, box, 128)) != SBNN_OK) return r;
     }
     {   // B: [nkb * padded Cout rows][64 channels] bf16, a box = BN output channels of one channel step
         const unsigned long long dims[2] = {(unsigned long long)T::BK, (unsigned long long)nkb * ntiles_n * BN};
         const unsigned long long strides[1] = {(unsigned long long)T::BK * 2};
         const unsigned box[2] = {(unsigned)T::BK, (unsigned)BN};
-        if ((r = encode_tiled_map(&bmap, d.w, 2, 2, dims, strides, box, true)) != SBNN_OK) return r;
+        if ((r = encode_tiled_map(&bmap, d.w, 2, 2, dims, strides, box, 128)) != SBNN_OK) return r;
     }
     CUtensorMap ymap;
     {   // Y [M][Cout] fp32, stored in boxes of 32 pixels x 32 channels out of swizzled shared-memory tiles
         const unsigned long long dims[2] = {(unsigned long long)p->Cout, (unsigned long long)M};
         const unsigned long long strides[1] = {(unsigned long long)p->Cout * 4};
         const unsigned box[2] = {32u, 32u};
-        if ((r = encode_tiled_map(&ymap, y, 4, 2, dims, strides, box, true)) != SBNN_OK) return r;
+        if ((r = encode_tiled_map(&ymap, y, 4, 2, dims, strides, box, 128)) != SBNN_OK) return r;
     }
     const long long total = (long long)mtiles * ntiles_n;
     if (total > 0x7fffffffLL) return fail(SBNN_ERR_SHAPE, "too many tiles");

@@ -1306,6 +1306,8 @@ extern "C" sbnn_status sbnn_conv3x3_gs(const sbnn_packed* w, const float* x_dev,
     if (st != SBNN_OK) return st;
     if ((st = check_device()) != SBNN_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
+    bool on_tc = false;
+    if ((st = conv3x3_tc(w, x_dev, y_dev, N, H, W, flags & SBNN_RELU, s, &on_tc)) != SBNN_OK || (on_tc && !prepare_only())) return st;
     {
         // fast path: planes of the input in the per-device scratch buffer ([Cin][N*H][Wp], rows padded to a multiple of
         // 4 floats), then the copy-engine kernel

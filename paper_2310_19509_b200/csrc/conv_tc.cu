@@ -1,0 +1,685 @@
+// Group-sparse convolutions in fp32 on the 5th-generation tensor cores (tcgen05), 1x1 and 3x3.
+//
+//   Y[m][o] = act( bias[o] + sum_{t,c} W~[o][t][c] * X[pixel(m) + tap t][c] ),   W~ = W (.) M  (Section 3.1)
+//
+// Precision: fp32 operands, fp32 result.  Every fp32 number is the exact sum of three bf16 numbers (8 + 8 + 8
+// significand bits), x = xh + xm + xl, w = wh + wm + wl, and the product of two bf16 numbers is exact in fp32.  The
+// kernel adds the six products xl*wh, xh*wl, xm*wm, xm*wh, xh*wm, xh*wh; the three that are left out (m*l, l*m, l*l) are
+// together below 2^-25 |x*w|, because every image is rounded to nearest (|m| <= 2^-9, |l| <= 2^-18 of the number).
+// The tensor core truncates when it adds to its accumulator, so no long sum is left to it: a 64-channel step is summed in
+// a fresh accumulator, the five small products first, and added to the running sum in registers, rounded to nearest.
+// What the truncations of one step take from the magnitude of its sum on average, 5.4e-8 of it (measured for 64 to
+// 1024 channels, dense to 90 % pruned, 1x1 and 3x3, alone and in a network: 3.6e-8 to 5.9e-8), is put back in the weights,
+// which are scaled by kTruncation before they are split; without it the layers of a network lose the same fraction one
+// after the other.
+//
+// The contraction runs dense over the masked weights (pruned entries are zeros): a group shares its kept channels over
+// only G = 4..8 outputs, far too few for a 128-row MMA to gather for.  Six products per dense MAC still beat the FMA
+// pipe on kept MACs alone until most of the layer is pruned; the rule is tc_profits() below.
+//
+// Structure, one CTA per SM, persistent over tiles of 128 pixels x BN output channels, 20 warps in 5 warpgroups:
+//   warpgroups 0, 1  drain: tcgen05.ld of a finished step, added to the fp32 sums in registers, which start at the bias;
+//                    after the last step ReLU and stores;
+//   warpgroups 2, 3  split: a thread owns one pixel and 16 of the 32 channels of a staged fp32 tile, splits them and
+//                    writes the three bf16 images into tensor memory, where the MMAs read them as the A operand
+//                    (so either activation layout is read with conflict-free loads and nothing is transposed);
+//   warp 16          copies activations (tiled or im2col tensor-map copies of 32 channels x 128 pixels);
+//   warp 17          copies weights (one linear copy per step and 128 output channels: the three bf16 images,
+//                    stored in the swizzled order the MMA reads);
+//   warps 18, 19     issue the MMAs, each into its own accumulator: while one waits for its operands the other's MMAs run.
+// (With one issuing warp the waits between its batches of 24 MMAs, 740 cycles, came on top of the 1900 cycles a batch
+// takes; with one split warpgroup a step took 1300 cycles to split, as long as its MMAs.)
+// Every wait is bounded, as in the other pipelined kernels.
+#include <cuda_bf16.h>
+#include <stdint.h>
+
+#include <algorithm>
+#include <new>
+
+#include <cuda.h>   // CUtensorMap (type only)
+
+#include "common.h"
+#include "pipeline.cuh"
+#include "tcgen05.cuh"
+
+namespace sbnn {
+namespace {
+
+constexpr double kTruncation = 1.0 + 5.4e-8;
+
+enum Source { SRC_NHWC, SRC_CM, SRC_IM2COL };
+
+// Element strides of the activations and the arrays of the packed layer, for the outputs of pixels that hold a
+// non-finite value (see exact_pixel).
+struct ExactArgs {
+    const float* x;
+    long long pixel_stride, channel_stride;
+    const int32_t* group_ptr;
+    const int32_t* idx;
+    const float* val;
+    int G;
+};
+
+struct TcArgs {
+    const uint4* wts;      // [output tile of NUC][step][image][NUC rows][64] bf16, swizzled
+    const float* bias;
+    float* y;
+    int ldy;
+    int M, Cin, Cout;
+    int steps;             // 64-channel steps x taps (taps inner)
+    int ntiles_m, ntiles_n;
+    int dm, dn;            // a CTA's next tile: dm pixel tiles and dn channel tiles further (grid size divided by ntiles_n)
+    int W, H;              // image size (3x3 only)
+    int relu;
+    int sa, sb;            // stages of activations and of weights
+    int resident;          // every tile uses the same weights and all of them have a stage: they are loaded once
+    int* status;
+    ExactArgs ex;
+};
+
+template <int BN_, int SRC_, bool OUT_CM_>
+struct TC {
+    static constexpr int BM = 128, BN = BN_, BK = 64, SRC = SRC_;
+    static constexpr bool OUT_CM = OUT_CM_;
+    static constexpr int TAPS = SRC == SRC_IM2COL ? 9 : 1;
+    static constexpr int NUC = BN < 128 ? BN : 128;      // columns of one MMA
+    static constexpr int NU = BN / NUC;                  // MMA column blocks per tile
+    static constexpr int SUB = 32;                       // channels of one activation stage
+    static constexpr int A_BYTES = SUB * BM * 4;
+    static constexpr int B_BYTES = 3 * NUC * BK * 2;
+    static constexpr int OUT_BYTES = 8 * 2 * 2048;       // two staging tiles of 32 pixels x 16 channels for each drain warp
+    static constexpr int CTRL = 512;                     // mbarriers, tensor-memory base, abort flag
+    // Stages share what is left of 227 KB: weights that fit as a whole and serve every tile stay (see launch_tc), else
+    // SB stages of them; the rest goes to activations, up to SA_MAX stages.
+    static constexpr int SB = BN < 128 ? 4 : 3, SA_MAX = 12, SB_MAX = 6;
+    static constexpr int ROOM = 227 * 1024 - 1024 - CTRL - OUT_BYTES;
+    static_assert((2 * (SA_MAX + SB_MAX) + 8) * 8 + 8 <= CTRL && SB * B_BYTES + 3 * A_BYTES <= ROOM, "shared memory");
+    static constexpr int NT = 640;
+    // registers a thread of the drain, split and remaining warps: 2 x + 2 y + z = 5 x 96, what the launch reserves
+    static constexpr int LAUNCH_REGS = 96, DRAIN_REGS = BN == 256 ? 176 : 128, SPLIT_REGS = BN == 256 ? 48 : 80, AUX_REGS = BN == 256 ? 32 : 64;
+    static_assert(2 * DRAIN_REGS + 2 * SPLIT_REGS + AUX_REGS == 5 * LAUNCH_REGS, "register shares");
+    static constexpr int COLS = BN / 2;                  // output channels a drain thread sums
+    static constexpr int DEMPTY = NU == 2 ? 4 : 8;       // warps that drain one accumulator
+    static constexpr int A_COL0 = 256, A_COLS = 96;      // tensor-memory columns: accumulators 0-255, two A stages behind
+    static_assert(BN == 64 || BN == 128 || BN == 256, "tile width");
+};
+
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t join2(uint32_t lo, uint32_t hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
+    return r;
+}
+// (first, second) -> two bf16, rounded to nearest even, the first in the lower half.
+__device__ __forceinline__ uint32_t bf16x2(float first, float second) {
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(second), "f"(first));
+    return r;
+}
+
+// Splits two fp32 values into bf16 images packed as (first, second): x = h + m + l exactly (up to subnormal l).
+__device__ __forceinline__ void split2(float x0, float x1, uint32_t& h, uint32_t& m, uint32_t& l) {
+    h = bf16x2(x0, x1);
+    const float r0 = x0 - __uint_as_float(h << 16), r1 = x1 - __uint_as_float(h & 0xffff0000u);
+    m = bf16x2(r0, r1);
+    l = bf16x2(r0 - __uint_as_float(m << 16), r1 - __uint_as_float(m & 0xffff0000u));
+}
+
+// Position in a ring of `n` stages: the stage, and the parity of its current use.
+struct Ring {
+    int n, stage = 0, uses = 0;
+    uint32_t parity = 0;
+    __device__ explicit Ring(int stages) : n(stages) {}
+    __device__ bool reused() const { return uses > 0; }
+    __device__ void next() {
+        if (++stage == n) {
+            stage = 0;
+            parity ^= 1;
+            ++uses;
+        }
+    }
+    // A producer that gives up at `stage` lets the copies it has issued land before the shared memory is released.
+    __device__ void settle(uint64_t* full) const {
+        for (int s = 0; s < (uses ? n : stage); ++s) {
+            bool landed = false;
+            for (uint32_t i = 0; i < kWaitLimit && !landed; ++i) landed = mbar_try_wait(full + s, s < stage ? parity : parity ^ 1);
+        }
+    }
+};
+
+// The tiles of a CTA: every gridDim.x-th, channel tiles innermost.
+struct Tiles {
+    const TcArgs& a;
+    int m, n;
+    __device__ explicit Tiles(const TcArgs& args) : a(args), m(blockIdx.x / args.ntiles_n), n(blockIdx.x % args.ntiles_n) {}
+    __device__ bool left() const { return m < a.ntiles_m; }
+    __device__ void next() {
+        m += a.dm;
+        n += a.dn;
+        if (n >= a.ntiles_n) {
+            n -= a.ntiles_n;
+            ++m;
+        }
+    }
+};
+
+template <int REGS>
+__device__ __forceinline__ void regs_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS)); }
+template <int REGS>
+__device__ __forceinline__ void regs_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS)); }
+
+// Box of 128 consecutive output positions x 32 channels of the input shifted by (dx, dy): an im2col tensor map walks the
+// positions in (x, y, n) order and delivers zeros outside the image.
+__device__ __forceinline__ void im2col_g2s(void* dst_smem, const void* map, int c, int x, int y, int n, int dx, int dy, uint64_t* bar) {
+    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.im2col.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6], {%7, %8};"
+                 ::"r"(smem_u32(dst_smem)), "l"(map), "r"(c), "r"(x), "r"(y), "r"(n), "r"(smem_u32(bar)), "h"((short)dx), "h"((short)dy)
+                 : "memory");
+}
+
+// The outputs [n0, n1) of pixel m as a plain FMA chain over the kept units.  A pixel with an infinity or a NaN in any
+// channel spoils all its split products (0 * inf), also those of pruned weights, which must not see it; such pixels are
+// recomputed here and written over.
+template <class T>
+__device__ __noinline__ void exact_pixel(const TcArgs& a, int m, int n0, int n1) {
+    const ExactArgs& e = a.ex;
+    const int px = T::TAPS == 9 ? m % a.W : 0, py = T::TAPS == 9 ? (m / a.W) % a.H : 0;
+    for (int n = n0; n < n1; ++n) {
+        const int g = n / e.G, r = n % e.G;
+        float s = 0.0f;
+        for (int j = e.group_ptr[g]; j < e.group_ptr[g + 1]; ++j)
+            for (int t = 0; t < T::TAPS; ++t) {
+                const int dy = T::TAPS == 9 ? t / 3 - 1 : 0, dx = T::TAPS == 9 ? t % 3 - 1 : 0;
+                if (T::TAPS == 9 && (px + dx < 0 || px + dx >= a.W || py + dy < 0 || py + dy >= a.H)) continue;
+                const long long p = (long long)m + dy * a.W + dx;
+                s = fmaf(e.val[((size_t)j * T::TAPS + t) * e.G + r], e.x[p * e.pixel_stride + e.idx[j] * e.channel_stride], s);
+            }
+        s += a.bias[n];
+        if (a.relu) s = fmaxf(s, 0.0f);
+        a.y[T::OUT_CM ? (size_t)n * a.ldy + m : (size_t)m * a.ldy + n] = s;
+    }
+}
+
+template <class T>
+__global__ void __launch_bounds__(T::NT, 1)
+conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap ymap, const __grid_constant__ TcArgs a) {
+    constexpr int NUC = T::NUC, NU = T::NU, BN = T::BN;
+    const int SA = a.sa, SB = a.sb;
+    extern __shared__ unsigned char raw[];
+    const uint32_t raw_addr = smem_u32(raw);
+    unsigned char* bst = raw + (((raw_addr + 1023u) & ~1023u) - raw_addr);    // weight stages, 1024-byte aligned
+    unsigned char* ast = bst + (size_t)SB * T::B_BYTES;                       // activation stages
+    unsigned char* ost = ast + (size_t)SA * T::A_BYTES;                       // output staging
+    uint64_t* xfull = reinterpret_cast<uint64_t*>(ost + T::OUT_BYTES);
+    uint64_t* xempty = xfull + SA;
+    uint64_t* bfull = xempty + SA;
+    uint64_t* bempty = bfull + SB;
+    uint64_t* afull = bempty + SB;      // A images of a step are in tensor memory
+    uint64_t* aempty = afull + 2;
+    uint64_t* dfull = aempty + 2;       // accumulator of a step is complete
+    uint64_t* dempty = dfull + 2;
+    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(dempty + 2);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
+
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, wg = warp >> 2;
+    if (tid == 0) {
+        for (int s = 0; s < SA; ++s) { mbar_init(xfull + s, 1); mbar_init(xempty + s, 8); }
+        for (int s = 0; s < SB; ++s) { mbar_init(bfull + s, 1); mbar_init(bempty + s, 1); }
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(afull + s, 8); mbar_init(aempty + s, NU);
+            mbar_init(dfull + s, 1); mbar_init(dempty + s, T::DEMPTY);
+        }
+        *abort_flag = 0;
+        mbar_fence_init();
+    }
+    if (warp == 18) tmem_alloc(tmem_holder, 512);
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_holder, 0);
+
+    auto wait = [&](uint64_t* bar, uint32_t parity) {   // warp-uniform result
+        return (bool)__all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, a.status, SBNN_ERR_TIMEOUT));
+    };
+    // valid 32-channel halves of a step
+    auto subs = [&](int k) { return a.Cin - (k / T::TAPS) * 64 > 32 ? 2 : 1; };
+
+    if (wg >= 2) {
+        if (wg < 4) regs_dec<T::SPLIT_REGS>(); else regs_dec<T::AUX_REGS>();
+        if (warp == 16) {
+            // ---------------- activation copies ----------------
+            Ring ring(SA);
+            bool ok = true;
+            grid_dependency_wait();                       // X comes from the previous kernel of the stream
+            for (Tiles t(a); t.left() && ok; t.next()) {
+                const int m0 = t.m * T::BM;
+                int px = 0, py = 0, pn = 0;
+                if (T::SRC == SRC_IM2COL) { px = m0 % a.W; py = (m0 / a.W) % a.H; pn = m0 / (a.W * a.H); }
+                for (int k = 0; k < a.steps && ok; ++k) {
+                    const int c = k / T::TAPS, tap = k - c * T::TAPS;
+                    for (int h = 0; h < subs(k); ++h, ring.next()) {
+                        const int s = ring.stage;
+                        if (ring.reused() && !(ok = wait(xempty + s, ring.parity ^ 1))) break;
+                        if (lane == 0) {
+                            unsigned char* dst = ast + (size_t)s * T::A_BYTES;
+                            const int c0 = c * 64 + h * T::SUB;
+                            mbar_arrive_expect_tx(xfull + s, T::A_BYTES);
+                            if (T::SRC == SRC_CM) tensor_g2s_2d(dst, &amap, m0, c0, xfull + s);
+                            else if (T::SRC == SRC_NHWC) tensor_g2s_2d(dst, &amap, c0, m0, xfull + s);
+                            else im2col_g2s(dst, &amap, c0, px - 1, py - 1, pn, tap % 3, tap / 3, xfull + s);
+                        }
+                        __syncwarp();
+                    }
+                }
+            }
+            if (!ok) ring.settle(xfull);
+        } else if (warp == 17) {
+            // ---------------- weight copies ----------------
+            Ring ring(SB);
+            bool ok = true;
+            for (Tiles t(a); t.left() && ok; t.next()) {
+                const int nt = t.n * NU;
+                for (int k = 0; k < a.steps && ok; ++k)
+                    for (int u = 0; u < NU; ++u, ring.next()) {
+                        const int s = ring.stage;
+                        if (ring.reused() && !(ok = wait(bempty + s, ring.parity ^ 1))) break;
+                        if (lane == 0) {
+                            mbar_arrive_expect_tx(bfull + s, T::B_BYTES);
+                            bulk_g2s(bst + (size_t)s * T::B_BYTES, a.wts + ((size_t)(nt + u) * a.steps + k) * (T::B_BYTES / 16), T::B_BYTES, bfull + s);
+                        }
+                        __syncwarp();
+                    }
+                if (a.resident) break;
+            }
+            if (!ok) ring.settle(bfull);
+        } else if (warp >= 18) {
+            // ---------------- MMA issue ----------------
+            constexpr uint32_t idesc = instr_desc(NUC);
+            // (image of A, image of B), small products first: h = 0, m = 1, l = 2
+            constexpr int PA[6] = {2, 0, 1, 1, 0, 0}, PB[6] = {0, 2, 1, 0, 1, 0};
+            const int d = warp - 18;                        // this warp's accumulator: units d, d + 2, ...
+            int step = 0, unit = 0;
+            Ring ring(SB);
+            bool ok = true;
+            for (Tiles t(a); t.left() && ok; t.next()) {
+                for (int k0 = 0; k0 < a.steps && ok; ++k0, ++step)
+                    for (int u = 0; u < NU; ++u, ++unit, ring.next()) {
+                        if ((unit & 1) != d) continue;
+                        const int as = step & 1, s = ring.stage;
+                        if (unit >= 2 && !(ok = wait(dempty + d, ((unit >> 1) & 1) ^ 1))) break;
+                        if (!(ok = wait(bfull + s, ring.parity))) break;
+                        if (!(ok = wait(afull + as, (step >> 1) & 1))) break;
+                        tc_fence_after_sync();
+                        const uint32_t a_base = tmem + T::A_COL0 + as * T::A_COLS;
+                        const uint64_t b_desc = operand_desc(smem_u32(bst) + (uint32_t)s * T::B_BYTES);
+                        const bool whole = subs(k0) == 2;
+                        if (elect_one()) {
+                            if (whole) {
+#pragma unroll
+                                for (int i = 0; i < 24; ++i) {
+                                    const int p = i >> 2, k = i & 3;
+                                    umma_bf16_ta(tmem + d * 128, a_base + PA[p] * 32 + k * 8, b_desc + ((PB[p] * (NUC * 128) + k * 32) >> 4),
+                                                 idesc, i ? 1u : 0u);
+                                }
+                            } else {
+#pragma unroll
+                                for (int i = 0; i < 12; ++i) {
+                                    const int p = i >> 1, k = i & 1;
+                                    umma_bf16_ta(tmem + d * 128, a_base + PA[p] * 32 + k * 8, b_desc + ((PB[p] * (NUC * 128) + k * 32) >> 4),
+                                                 idesc, i ? 1u : 0u);
+                                }
+                            }
+                            if (!a.resident) umma_commit(bempty + s);
+                            umma_commit(dfull + d);
+                            umma_commit(aempty + as);
+                        }
+                        __syncwarp();
+                    }
+                if (a.resident) ring = Ring(SB);            // the same stages again, still full from the first round
+            }
+        } else if (wg < 4) {
+            // ---------------- split into bf16 images ----------------
+            const int half = wg - 2, q = warp & 3, p = q * 32 + lane;   // pixel of the tile = tensor-memory lane
+            const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16) + T::A_COL0;
+            int step = 0;
+            Ring ring(SA);
+            bool ok = true;
+            for (Tiles t(a); t.left() && ok; t.next())
+                for (int k0 = 0; k0 < a.steps && ok; ++k0, ++step) {
+                    const int as = step & 1;
+                    if (step >= 2 && !(ok = wait(aempty + as, ((step >> 1) & 1) ^ 1))) break;
+                    tc_fence_after_sync();
+                    for (int h = 0; h < subs(k0); ++h, ring.next()) {
+                        const int s = ring.stage;
+                        if (!(ok = wait(xfull + s, ring.parity))) break;
+                        const unsigned char* src = ast + (size_t)s * T::A_BYTES;
+                        float v[16];
+                        if (T::SRC == SRC_CM) {
+#pragma unroll
+                            for (int k = 0; k < 16; ++k) v[k] = reinterpret_cast<const float*>(src)[(half * 16 + k) * T::BM + p];
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j)
+                                *reinterpret_cast<float4*>(v + 4 * j) =
+                                    *reinterpret_cast<const float4*>(src + p * 128 + (((half * 4 + j) ^ (p & 7)) << 4));
+                        }
+                        uint32_t hh[8], mm[8], ll[8];
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) split2(v[2 * k], v[2 * k + 1], hh[k], mm[k], ll[k]);
+                        const uint32_t col = lane_base + as * T::A_COLS + h * 16 + half * 8;
+                        tmem_st8(col, hh);
+                        tmem_st8(col + 32, mm);
+                        tmem_st8(col + 64, ll);
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(xempty + s);
+                    }
+                    if (!ok) break;
+                    tmem_st_wait();
+                    tc_fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(afull + as);
+                }
+        }
+    } else {
+        // ---------------- drain and store ----------------
+        regs_inc<T::DRAIN_REGS>();
+        const int q = warp & 3;
+        const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16);
+        unsigned char* stage = ost + (size_t)warp * 4096;
+        int step = 0, copies = 0;                           // copies issued: the two tiles alternate between them
+        bool ok = true;
+        grid_dependency_wait();                             // Y may still be read by the previous kernel of the stream
+        grid_dependency_release();
+        for (Tiles t(a); t.left() && ok; t.next()) {
+            const int m0 = t.m * T::BM, n0 = t.n * BN + wg * T::COLS;
+            uint64_t acc[T::COLS / 2];                      // pairs of neighbouring channels, from the bias on
+#pragma unroll
+            for (int i = 0; i < T::COLS / 4; ++i) {
+                const ulonglong2 b = __ldg(reinterpret_cast<const ulonglong2*>(a.bias + n0) + i);
+                acc[2 * i] = b.x;
+                acc[2 * i + 1] = b.y;
+            }
+            for (int k = 0; k < a.steps; ++k, ++step) {
+                // two column blocks: a warpgroup drains its own; one block: both drain their half of every accumulator
+                const int unit = NU == 2 ? 2 * step + wg : step, d = unit & 1;
+                if (!(ok = wait(dfull + d, (unit >> 1) & 1))) break;
+                tc_fence_after_sync();
+                const uint32_t col = lane_base + d * 128 + (NU == 2 ? 0 : wg * T::COLS);
+#pragma unroll
+                for (int c0 = 0; c0 < T::COLS; c0 += 32) {
+                    uint32_t v[32];
+                    tmem_ld32(col + c0, v);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) acc[c0 / 2 + i] = add2(acc[c0 / 2 + i], join2(v[2 * i], v[2 * i + 1]));
+                }
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(dempty + d);
+            }
+            if (!ok) break;
+            const int m = m0 + q * 32 + lane;
+            float first, unused;
+            unpack2(acc[0], first, unused);
+            const bool redo = m < a.M && !(fabsf(first) <= 3.402823466e38f);
+            // 32 pixels x 16 channels at a time through one of the warp's two staging tiles, stored by tiled copies: rows of 32
+            // pixels (channel-major) or of 16 channels (64-byte swizzle).  Rows past Cout or M are clipped by the copy; the last
+            // pixels of a channel-major row are stored one by one, so that the padding behind them is left alone.
+            // (Stores straight from registers, one row of 32 pixels each, took 100 cycles apiece: 13700 cycles for a tile
+            // of 256 channels.)
+            const int mw = m0 + q * 32;
+#pragma unroll
+            for (int c0 = 0; c0 < T::COLS; c0 += 16) {
+                if (n0 + c0 < a.Cout && mw < a.M) {         // warp-uniform
+                    float o[16];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) unpack2(acc[c0 / 2 + i], o[2 * i], o[2 * i + 1]);
+                    if (a.relu) {
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) o[i] = fmaxf(o[i], 0.0f);
+                    }
+                    if (T::OUT_CM && mw + 32 > a.M) {
+#pragma unroll
+                        for (int i = 0; i < 16; ++i)
+                            if (m < a.M && n0 + c0 + i < a.Cout) a.y[(size_t)(n0 + c0 + i) * a.ldy + m] = o[i];
+                    } else {
+                        unsigned char* tile = stage + (copies++ & 1) * 2048;
+                        if (lane == 0) bulk_wait_read_pending1();   // the copy that last read this tile is done with it
+                        __syncwarp();
+                        if (T::OUT_CM) {
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) reinterpret_cast<float*>(tile)[i * 32 + lane] = o[i];
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j)
+                                *reinterpret_cast<float4*>(tile + lane * 64 + ((j ^ (lane >> 1 & 3)) << 4)) =
+                                    make_float4(o[4 * j], o[4 * j + 1], o[4 * j + 2], o[4 * j + 3]);
+                        }
+                        fence_async_smem();
+                        __syncwarp();
+                        if (lane == 0) {
+                            tensor_s2g_2d(&ymap, T::OUT_CM ? mw : n0 + c0, T::OUT_CM ? n0 + c0 : mw, tile);
+                            bulk_commit_group();
+                        }
+                    }
+                }
+            }
+            if (__any_sync(0xffffffffu, redo)) {
+                if (lane == 0) bulk_wait_all();
+                __syncwarp();
+                if (redo) exact_pixel<T>(a, m, n0, min(n0 + T::COLS, a.Cout));
+            }
+        }
+        if (lane == 0) bulk_wait_all();                     // this thread's copies are complete before the CTA gives up its shared memory
+    }
+    // common exit: nobody may still be using the tensor memory when it is released
+    tc_fence_before_sync();
+    __syncthreads();
+    if (warp == 18) tmem_dealloc(tmem, 512);
+}
+
+// One thread per (kept unit, tap, channel of the group): the weight's three bf16 images into their place in the tiles.
+__global__ void build_tc_weights_kernel(const int32_t* __restrict__ group_ptr, const int32_t* __restrict__ idx, const float* __restrict__ val,
+                                        int G, int taps, int csteps, int nuc, __nv_bfloat16* __restrict__ out) {
+    const int g = blockIdx.x, per_unit = taps * G;
+    const int lo = group_ptr[g];
+    const long long n = (long long)(group_ptr[g + 1] - lo) * per_unit;
+    for (long long i = threadIdx.x + (long long)blockIdx.y * blockDim.x; i < n; i += (long long)blockDim.x * gridDim.y) {
+        const int j = lo + (int)(i / per_unit), t = (int)(i % per_unit) / G, o = g * G + (int)(i % G), c = idx[j];
+        const double w = val[(size_t)j * per_unit + i % per_unit] * kTruncation;
+        // Round to nearest; magnitudes that would round up to infinity are truncated instead.
+        const __nv_bfloat16 h = fabs(w) > 3.3895e38 ? __float2bfloat16_rz(__double2float_rz(w)) : __float2bfloat16_rn((float)w);
+        const double r = w - (double)__bfloat162float(h);
+        const __nv_bfloat16 m = __float2bfloat16_rn((float)r);
+        const __nv_bfloat16 l = __float2bfloat16_rn((float)(r - (double)__bfloat162float(m)));
+        const int row = o % nuc, kk = c & 63;
+        const size_t block = (size_t)(o / nuc) * csteps * taps + (size_t)(c >> 6) * taps + t;
+        const size_t at = block * 3 * nuc * 64 + (size_t)row * 64 + ((((kk >> 3) ^ (row & 7)) << 3) | (kk & 7));
+        out[at] = h;
+        out[at + (size_t)nuc * 64] = m;
+        out[at + (size_t)2 * nuc * 64] = l;
+    }
+}
+
+// Weight images of a layer for MMA column blocks of `nuc` output channels, built on first use; NULL if that would be
+// while `st` is being captured, when nothing can be allocated.
+sbnn_status get_tc_weights(const sbnn_packed* p, int nuc, cudaStream_t st, uint4** out) {
+    std::lock_guard<std::mutex> lk(p->mu);
+    *out = nullptr;
+    auto it = p->tc_weights.find(nuc);
+    if (it != p->tc_weights.end()) {
+        *out = static_cast<uint4*>(it->second);
+        return SBNN_OK;
+    }
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (!prepare_only() && cudaStreamIsCapturing(st, &cs) != cudaSuccess) cudaGetLastError();
+    if (cs != cudaStreamCaptureStatusNone) return SBNN_OK;
+    const int taps = p->KH * p->KW, csteps = (p->Cin + 63) / 64, tiles = (p->Cout + 255) / 256 * 256 / nuc;
+    const size_t bytes = (size_t)tiles * csteps * taps * 3 * nuc * 64 * 2;
+    void* d = nullptr;
+    SBNN_CUDA_TRY(cudaMalloc(&d, bytes));
+    cudaError_t e = cudaMemset(d, 0, bytes);
+    if (e == cudaSuccess && p->nnz > 0) {
+        build_tc_weights_kernel<<<dim3((unsigned)p->ngroups, 4), 128>>>(p->d_group_ptr, p->d_idx, p->d_val, p->G, taps, csteps, nuc,
+                                                                       static_cast<__nv_bfloat16*>(d));
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+    if (e != cudaSuccess) {
+        cudaFree(d);
+        cudaGetLastError();
+        return fail(SBNN_ERR_CUDA, "building the tensor-core weights: %s", cudaGetErrorString(e));
+    }
+    p->tc_weights[nuc] = d;
+    *out = static_cast<uint4*>(d);
+    return SBNN_OK;
+}
+
+struct TcCall {
+    const float* x;
+    int ldx;           // channel-major sources
+    float* y;
+    int ldy;
+    long long M;
+    int N, H, W;       // 3x3
+    int relu;
+    cudaStream_t st;
+};
+
+bool tc_profits(const sbnn_packed* p, long long M) {
+    if (!p->finite || (double)p->nnz < 0.15 * p->ngroups * p->Cin) return false;
+    return M * p->Cout >= 128 * 64 * 74;
+}
+
+}  // namespace
+
+sbnn_status prepare_tc(const sbnn_packed* p, long long M) {
+    if (!tc_profits(p, M)) return SBNN_OK;
+    uint4* wts = nullptr;
+    PrepareScope scope;
+    for (int nuc : {64, 128}) {   // the tile width depends on the pixels: for calls with fewer, too
+        const sbnn_status r = get_tc_weights(p, nuc, nullptr, &wts);
+        if (r != SBNN_OK) return r;
+    }
+    return SBNN_OK;
+}
+
+namespace {
+
+template <class T>
+sbnn_status launch_tc(const sbnn_packed* p, const TcCall& c, bool* done) {
+    sbnn_status r = set_max_dyn_smem(reinterpret_cast<const void*>(&conv_tc_kernel<T>), 227 * 1024);
+    if (r != SBNN_OK) return r;
+    // The warpgroups' register shares add up to LAUNCH_REGS a thread: a build that starts with fewer must not be launched,
+    // since the drain warps would wait for registers that nobody returns.
+    static const int regs = [] {
+        cudaFuncAttributes fa = {};
+        return cudaFuncGetAttributes(&fa, conv_tc_kernel<T>) == cudaSuccess ? fa.numRegs : 0;
+    }();
+    if (regs != T::LAUNCH_REGS)
+        return fail(SBNN_ERR_UNSUPPORTED, "internal: the tensor-core kernel was built with %d registers a thread, not %d", regs, T::LAUNCH_REGS);
+    TcArgs a = {};
+    uint4* wts = nullptr;
+    if ((r = get_tc_weights(p, T::NUC, c.st, &wts)) != SBNN_OK || !wts) return r;
+    if ((r = async_status_word(&a.status)) != SBNN_OK) return r;
+    *done = true;
+    if (prepare_only()) return SBNN_OK;
+    const long long ntiles_n = (p->Cout + T::BN - 1) / T::BN, total = (c.M + T::BM - 1) / T::BM * ntiles_n;
+    if (total > 0x7fffffffLL) return fail(SBNN_ERR_SHAPE, "too many tiles");
+    a.wts = wts; a.bias = p->d_bias; a.y = c.y; a.ldy = c.ldy; a.M = (int)c.M; a.Cin = p->Cin; a.Cout = p->Cout;
+    a.steps = (p->Cin + 63) / 64 * T::TAPS; a.ntiles_m = (int)((c.M + T::BM - 1) / T::BM); a.ntiles_n = (int)ntiles_n;
+    a.W = c.W; a.H = c.H; a.relu = c.relu;
+    const bool cm = T::SRC == SRC_CM;
+    a.ex = {c.x, cm ? 1 : p->Cin, cm ? c.ldx : 1, p->d_group_ptr, p->d_idx, p->d_val, p->G};
+    CUtensorMap amap, ymap;
+    if (T::SRC == SRC_IM2COL) {
+        if ((r = encode_im2col_3x3_map(&amap, c.x, c.N, c.H, c.W, p->Cin, T::SUB, T::BM)) != SBNN_OK) return r;
+    } else if (cm) {
+        const unsigned long long dims[2] = {(unsigned long long)c.M, (unsigned long long)p->Cin};
+        const unsigned long long strides[1] = {(unsigned long long)c.ldx * 4};
+        const unsigned box[2] = {(unsigned)T::BM, (unsigned)T::SUB};
+        if ((r = encode_tiled_map(&amap, c.x, 4, 2, dims, strides, box)) != SBNN_OK) return r;
+    } else {
+        const unsigned long long dims[2] = {(unsigned long long)p->Cin, (unsigned long long)c.M};
+        const unsigned long long strides[1] = {(unsigned long long)p->Cin * 4};
+        const unsigned box[2] = {(unsigned)T::SUB, (unsigned)T::BM};
+        if ((r = encode_tiled_map(&amap, c.x, 4, 2, dims, strides, box, 128)) != SBNN_OK) return r;
+    }
+    {
+        const unsigned long long dims[2] = {(unsigned long long)(T::OUT_CM ? c.M : p->Cout), (unsigned long long)(T::OUT_CM ? p->Cout : c.M)};
+        const unsigned long long strides[1] = {(unsigned long long)c.ldy * 4};
+        const unsigned box[2] = {T::OUT_CM ? 32u : 16u, T::OUT_CM ? 16u : 32u};
+        if ((r = encode_tiled_map(&ymap, c.y, 4, 2, dims, strides, box, T::OUT_CM ? 0 : 64)) != SBNN_OK) return r;
+    }
+    const unsigned grid = (unsigned)std::min<long long>(total, device_sms());
+    a.dm = (int)(grid / (unsigned)ntiles_n);
+    a.dn = (int)(grid % (unsigned)ntiles_n);
+    a.resident = ntiles_n == 1 && a.steps * T::NU <= T::SB_MAX && a.steps * T::NU * T::B_BYTES + 3 * T::A_BYTES <= T::ROOM;
+    a.sb = a.resident ? a.steps * T::NU : T::SB;
+    a.sa = std::min(T::SA_MAX, (T::ROOM - a.sb * T::B_BYTES) / T::A_BYTES);
+    const size_t smem = (size_t)a.sb * T::B_BYTES + (size_t)a.sa * T::A_BYTES + T::OUT_BYTES + T::CTRL + 1024;
+    SBNN_CUDA_TRY(launch_kernel(conv_tc_kernel<T>, dim3(grid), dim3(T::NT), smem, c.st, amap, ymap, a));
+    return SBNN_OK;
+}
+
+// Cycles a launch takes with tiles of bn output channels: rounds of tiles x (steps x max(MMAs, copies from L2) + fill and store).
+double tc_cost(const sbnn_packed* p, long long M, int bn) {
+    const long long tiles = (M + 127) / 128 * ((p->Cout + bn - 1) / bn), sms = device_sms();
+    const double steps = (double)((p->Cin + 63) / 64) * p->KH * p->KW;
+    const double step = bn == 64 ? 1600.0 : 14.0 * bn;
+    return (double)((tiles + sms - 1) / sms) * (steps * step + 1000.0 + 12.0 * bn) + 4000.0;
+}
+int tc_width(const sbnn_packed* p, long long M) {
+    int best = 64;
+    for (int bn : {128, 256})
+        if (tc_cost(p, M, bn) < tc_cost(p, M, best)) best = bn;
+    return best;
+}
+
+template <int SRC, bool OUT_CM>
+sbnn_status dispatch_tc(const sbnn_packed* p, const TcCall& c, bool* done) {
+    if (prepare_only()) {
+        const sbnn_status r = prepare_tc(p, c.M);
+        if (r != SBNN_OK) return r;
+    }
+    switch (tc_width(p, c.M)) {
+        case 256: return launch_tc<TC<256, SRC, OUT_CM>>(p, c, done);
+        case 128: return launch_tc<TC<128, SRC, OUT_CM>>(p, c, done);
+        default: return launch_tc<TC<64, SRC, OUT_CM>>(p, c, done);
+    }
+}
+
+}  // namespace
+
+sbnn_status conv1x1_tc(const sbnn_packed* p, const float* x, float* y, long long M, int relu, cudaStream_t st, bool* done) {
+    *done = false;
+    if (p->Cin % 4 || p->Cout % 4 || !tc_profits(p, M)) return SBNN_OK;
+    const TcCall c{x, 0, y, p->Cout, M, 0, 0, 0, relu, st};
+    return dispatch_tc<SRC_NHWC, false>(p, c, done);
+}
+
+sbnn_status conv1x1_tc_cm(const sbnn_packed* p, const float* x, int ldx, float* y, int ldy, long long M, int relu, bool out_cm, cudaStream_t st,
+                          bool* done) {
+    *done = false;
+    if ((!out_cm && p->Cout % 4) || !tc_profits(p, M)) return SBNN_OK;
+    const TcCall c{x, ldx, y, ldy, M, 0, 0, 0, relu, st};
+    return out_cm ? dispatch_tc<SRC_CM, true>(p, c, done) : dispatch_tc<SRC_CM, false>(p, c, done);
+}
+
+sbnn_status conv3x3_tc(const sbnn_packed* p, const float* x, float* y, int N, int H, int W, int relu, cudaStream_t st, bool* done) {
+    *done = false;
+    const long long M = (long long)N * H * W;
+    if (p->Cin % 4 || p->Cout % 4 || M > 0x7fffffffLL - 128 || !tc_profits(p, M)) return SBNN_OK;
+    const TcCall c{x, 0, y, p->Cout, M, N, H, W, relu, st};
+    return dispatch_tc<SRC_IM2COL, false>(p, c, done);
+}
+
+void free_tc_weights(sbnn_packed* p) {
+    for (auto& kv : p->tc_weights) cudaFree(kv.second);
+    p->tc_weights.clear();
+}
+
+}  // namespace sbnn

@@ -119,6 +119,7 @@ extern "C" sbnn_status sbnn_mobilenet_v1_create(const sbnn_packed* const* pw, co
         if ((st = check_packed_device(pw[i])) != SBNN_OK) return st;
         const int hw = layer_table()[2 + 2 * i].hin;                 // the block's pointwise layer is entry 2 + 2*i
         if ((st = prepare_default_cm(pw[i], (long long)max_batch * hw * hw)) != SBNN_OK) return st;
+        if ((st = prepare_tc(pw[i], (long long)max_batch * hw * hw)) != SBNN_OK) return st;
         if ((st = prepare_default_cm(pw[i], (long long)hw * hw)) != SBNN_OK) return st;   // and the batch-1 choice
     }
     if ((st = check_packed_device(fc)) != SBNN_OK) return st;

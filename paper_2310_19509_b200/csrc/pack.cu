@@ -147,6 +147,15 @@ void detect_blocks(sbnn_packed* p) {
     p->gi = 4;
 }
 
+// The bias padded with zeros to whole tiles of 256 channels (kernels read it tile by tile).
+sbnn_status upload_bias(sbnn_packed* p) {
+    const size_t bytes = ((size_t)p->Cout + 255) / 256 * 256 * sizeof(float);
+    SBNN_CUDA_TRY(cudaMalloc(reinterpret_cast<void**>(&p->d_bias), bytes));
+    SBNN_CUDA_TRY(cudaMemset(p->d_bias, 0, bytes));
+    SBNN_CUDA_TRY(cudaMemcpy(p->d_bias, p->bias.data(), p->bias.size() * sizeof(float), cudaMemcpyHostToDevice));
+    return SBNN_OK;
+}
+
 // Last step of packing and of loading: device copies of the canonical arrays and the default private layouts, if
 // there is a device; *out owns p afterwards (on failure p is freed).
 sbnn_status finish_packed(sbnn_packed* p, sbnn_packed** out) {
@@ -156,6 +165,8 @@ sbnn_status finish_packed(sbnn_packed* p, sbnn_packed** out) {
         p->gi = 1;
         p->block_idx.clear();
     }
+    // (the difference of a value with itself is 0 unless the value is an infinity or a NaN)
+    p->finite = std::all_of(p->val.begin(), p->val.end(), [](float v) { return v - v == 0.0f; });
     int ndev = 0, dev = 0;
     if (cudaGetDeviceCount(&ndev) != cudaSuccess || ndev == 0 || cudaGetDevice(&dev) != cudaSuccess) {
         cudaGetLastError();
@@ -165,7 +176,7 @@ sbnn_status finish_packed(sbnn_packed* p, sbnn_packed** out) {
     sbnn_status st = SBNN_OK;
     p->device = dev;
     if ((st = upload(&p->d_group_ptr, p->group_ptr)) != SBNN_OK || (st = upload(&p->d_idx, p->idx)) != SBNN_OK ||
-        (st = upload(&p->d_val, p->val)) != SBNN_OK || (st = upload(&p->d_bias, p->bias)) != SBNN_OK) {
+        (st = upload(&p->d_val, p->val)) != SBNN_OK || (st = upload_bias(p)) != SBNN_OK) {
         sbnn_packed_free(p);
         return st;
     }
@@ -460,6 +471,7 @@ extern "C" sbnn_status sbnn_packed_free(sbnn_packed* p) {
         free_streams_cm(p);
         free_stream_bf16(p);
         free_umma_weights(p);
+        free_tc_weights(p);
         free_streams_3x3(p);
         cudaFree(p->d_group_ptr);
         cudaFree(p->d_idx);
