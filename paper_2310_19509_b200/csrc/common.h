@@ -40,22 +40,33 @@ struct ChainedLaunchScope {
     ~ChainedLaunchScope();
 };
 
-// Kernel launch that honours chained_launch().  Arguments are converted to the kernel's parameter types.
+// Kernel launch that honours chained_launch(), in clusters of `cluster` CTAs.  Arguments are converted to the kernel's
+// parameter types.
 template <class... Params, class... Args>
-cudaError_t launch_kernel(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+cudaError_t launch_kernel_cluster(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, unsigned cluster,
+                                  Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
+    cfg.attrs = attr;
     if (chained_launch()) {
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        attr[cfg.numAttrs].val.clusterDim.x = cluster;
+        attr[cfg.numAttrs].val.clusterDim.y = 1;
+        attr[cfg.numAttrs++].val.clusterDim.z = 1;
     }
     return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
+template <class... Params, class... Args>
+cudaError_t launch_kernel(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+    return launch_kernel_cluster(kernel, grid, block, smem, st, 1u, args...);
 }
 
 // Raises a kernel's dynamic shared-memory limit to `bytes` on the current device, once per (device, kernel) and size.
@@ -140,6 +151,11 @@ struct sbnn_packed {
     mutable void* umma_weights = nullptr; // dense bf16 copy of the masked weights, see conv1x1_umma.cu
     mutable std::map<int, void*> tc_weights;  // split bf16 images of the masked weights, see conv_tc.cu
     bool finite = true;                   // every stored weight is finite
+    struct TcChoice {                     // tile width (0: the FMA kernels are faster), CTAs that share a tile, estimated cycles
+        int bn, split;
+        double cost;
+    };
+    mutable std::map<long long, TcChoice> tc_choices;  // per pixel count and kind of call, see conv_tc.cu
 };
 
 namespace sbnn {
@@ -194,12 +210,18 @@ void free_stream_bf16(sbnn_packed* p);
 // conv1x1_umma.cu: bf16 mode as a dense contraction over the masked weights (tcgen05); *done = false if the shape is not taken
 sbnn_status conv1x1_umma(const sbnn_packed* w, const float* x, float* y, int M, int relu, cudaStream_t st, bool* done);
 void free_umma_weights(sbnn_packed* p);
+// True when the pipelined 1x1 kernel would get fewer tiles than half the SMs (the few-pixel kernel runs then).
+bool conv1x1_few_tiles(const sbnn_packed* p, long long M);
+// Taps kept over all units of a pattern layer.
+long long count_kept_taps(const sbnn_packed* p);
 // conv_tc.cu: fp32 layers on the tensor cores by a three-way bf16 split; *done = false (and SBNN_OK) when the shape or the
 // density is better served by the FMA kernels (or outside what the kernel takes)
 sbnn_status conv1x1_tc(const sbnn_packed* p, const float* x, float* y, long long M, int relu, cudaStream_t st, bool* done);
 sbnn_status conv1x1_tc_cm(const sbnn_packed* p, const float* x, int ldx, float* y, int ldy, long long M, int relu, bool out_cm, cudaStream_t st,
                           bool* done);
 sbnn_status conv3x3_tc(const sbnn_packed* p, const float* x, float* y, int N, int H, int W, int relu, cudaStream_t st, bool* done);
+sbnn_status conv3x3_tc_cm(const sbnn_packed* p, const float* x, int ldx, float* y, int ldy, int N, int H, int W, int relu, bool out_cm, cudaStream_t st,
+                          bool* done);
 // Builds the weight images for calls of up to M pixels.
 sbnn_status prepare_tc(const sbnn_packed* p, long long M);
 void free_tc_weights(sbnn_packed* p);

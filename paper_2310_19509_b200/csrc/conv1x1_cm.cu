@@ -1105,6 +1105,8 @@ sbnn_status encode_im2col_3x3_map(void* out, const float* x, int N, int H, int W
 
 int device_sms() { return sm_count(); }
 
+bool conv1x1_few_tiles(const sbnn_packed* p, long long M) { return few_tiles(p, M); }
+
 sbnn_status prepare_default_cm(const sbnn_packed* p, long long M) {
     Stream1x1 s;
     return get_stream_cm(p, default_cfg_cm(p, M), &s);

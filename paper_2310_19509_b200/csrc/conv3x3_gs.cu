@@ -759,14 +759,7 @@ int sm_count3() {
 // kept kernel, one tap" on config 4's shape, the whole-kernel loop with two output rows per lane about 35 us per tap
 // including the pruned ones (their stored weights are zeros), so lists pay below about five kept taps per kernel.
 bool use_tap_lists(const sbnn_packed* p) {
-    if (p->tap_mask.empty()) return false;
-    std::lock_guard<std::mutex> lk(p->mu);
-    if (p->kept_taps < 0) {
-        long long n = 0;
-        for (uint16_t m : p->tap_mask) n += __builtin_popcount(m);
-        p->kept_taps = n;
-    }
-    return (double)p->kept_taps < 4.8 * (double)p->tap_mask.size();
+    return !p->tap_mask.empty() && (double)count_kept_taps(p) < 4.8 * (double)p->tap_mask.size();
 }
 
 int pow2_ceil(int v) {
@@ -1270,6 +1263,16 @@ sbnn_status dispatch3(const sbnn_packed* p, const float* x, float* y, int N, int
 }
 }  // namespace
 
+long long count_kept_taps(const sbnn_packed* p) {
+    std::lock_guard<std::mutex> lk(p->mu);
+    if (p->kept_taps < 0) {
+        long long n = 0;
+        for (uint16_t m : p->tap_mask) n += __builtin_popcount(m);
+        p->kept_taps = n;
+    }
+    return p->kept_taps;
+}
+
 sbnn_status prepare_default_3x3(const sbnn_packed*) { return SBNN_OK; }  // the re-layout depends on the image width
 
 void free_streams_3x3(sbnn_packed* p) {
@@ -1390,6 +1393,8 @@ extern "C" sbnn_status sbnn_conv3x3_gs_cm(const sbnn_packed* w, const float* xt_
     if (st != SBNN_OK) return st;
     if ((st = check_device()) != SBNN_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
+    bool on_tc = false;
+    if ((st = conv3x3_tc_cm(w, xt_dev, ldx, y_dev, ldy, N, H, W, flags & SBNN_RELU, out_cm, s, &on_tc)) != SBNN_OK || on_tc) return st;
     // Widths that are not multiples of 4: the rows of the planes do not start on 16-byte boundaries, which the tiled
     // copy needs, so the planes are first copied into the scratch buffer with padded rows.
     const int Wp = (W + 3) / 4 * 4;

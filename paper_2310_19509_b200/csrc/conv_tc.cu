@@ -30,6 +30,10 @@
 // (With one issuing warp the waits between its batches of 24 MMAs, 740 cycles, came on top of the 1900 cycles a batch
 // takes; with one split warpgroup a step took 1300 cycles to split, as long as its MMAs.)
 // Every wait is bounded, as in the other pipelined kernels.
+//
+// Launches with too few tiles for the SMs (small batches, small maps) run with 64 output channels a tile and the steps of a
+// tile dealt to the CTAs of a cluster (SPLIT): each sums its share, then every CTA adds up a part of the channels, which
+// the others have written into its shared memory, in rank order, and stores it.
 #include <cuda_bf16.h>
 #include <stdint.h>
 
@@ -47,7 +51,9 @@ namespace {
 
 constexpr double kTruncation = 1.0 + 5.4e-8;
 
-enum Source { SRC_NHWC, SRC_CM, SRC_IM2COL };
+// SRC_CM3: 3x3 on channel-major activations.  A tap shifts the 128 pixels of a tile by dy * W + dx, so a copy of 136 pixels
+// (from a multiple of 4) serves the three taps of a kernel row; the split warps blank what lies outside the image.
+enum Source { SRC_NHWC, SRC_CM, SRC_IM2COL, SRC_CM3 };
 
 // Element strides of the activations and the arrays of the packed layer, for the outputs of pixels that hold a
 // non-finite value (see exact_pixel).
@@ -71,37 +77,43 @@ struct TcArgs {
     int dm, dn;            // a CTA's next tile: dm pixel tiles and dn channel tiles further (grid size divided by ntiles_n)
     int W, H;              // image size (3x3 only)
     int relu;
+    int split;             // CTAs of a cluster that share a tile's steps
     int sa, sb;            // stages of activations and of weights
     int resident;          // every tile uses the same weights and all of them have a stage: they are loaded once
     int* status;
     ExactArgs ex;
 };
 
-template <int BN_, int SRC_, bool OUT_CM_>
+template <int BN_, int SRC_, bool OUT_CM_, bool SPLIT_ = false>
 struct TC {
     static constexpr int BM = 128, BN = BN_, BK = 64, SRC = SRC_;
-    static constexpr bool OUT_CM = OUT_CM_;
-    static constexpr int TAPS = SRC == SRC_IM2COL ? 9 : 1;
+    static constexpr bool OUT_CM = OUT_CM_, SPLIT = SPLIT_;
+    static constexpr int TAPS = SRC == SRC_IM2COL || SRC == SRC_CM3 ? 9 : 1;
+    static constexpr int RUN = SRC == SRC_CM3 ? 3 : 1;   // steps that read the same activation stages
+    static constexpr int PIX = SRC == SRC_CM3 ? 136 : 128;   // pixels of a stage
     static constexpr int NUC = BN < 128 ? BN : 128;      // columns of one MMA
     static constexpr int NU = BN / NUC;                  // MMA column blocks per tile
     static constexpr int SUB = 32;                       // channels of one activation stage
-    static constexpr int A_BYTES = SUB * BM * 4;
+    static constexpr int A_BYTES = SUB * PIX * 4;
     static constexpr int B_BYTES = 3 * NUC * BK * 2;
     static constexpr int OUT_BYTES = 8 * 2 * 2048;       // two staging tiles of 32 pixels x 16 channels for each drain warp
     static constexpr int CTRL = 512;                     // mbarriers, tensor-memory base, abort flag
     // Stages share what is left of 227 KB: weights that fit as a whole and serve every tile stay (see launch_tc), else
     // SB stages of them; the rest goes to activations, up to SA_MAX stages.
-    static constexpr int SB = BN < 128 ? 4 : 3, SA_MAX = 12, SB_MAX = 6;
+    static constexpr int SB = BN < 128 ? 4 : (SRC == SRC_CM3 ? 2 : 3), SA_MAX = 12, SB_MAX = 6;
     static constexpr int ROOM = 227 * 1024 - 1024 - CTRL - OUT_BYTES;
-    static_assert((2 * (SA_MAX + SB_MAX) + 8) * 8 + 8 <= CTRL && SB * B_BYTES + 3 * A_BYTES <= ROOM, "shared memory");
+    static_assert((2 * (SA_MAX + SB_MAX) + 12) * 8 + 8 <= CTRL && SB * B_BYTES + (SRC == SRC_CM3 ? 4 : 3) * A_BYTES <= ROOM, "shared memory");
     static constexpr int NT = 640;
     // registers a thread of the drain, split and remaining warps: 2 x + 2 y + z = 5 x 96, what the launch reserves
     static constexpr int LAUNCH_REGS = 96, DRAIN_REGS = BN == 256 ? 176 : 128, SPLIT_REGS = BN == 256 ? 48 : 80, AUX_REGS = BN == 256 ? 32 : 64;
     static_assert(2 * DRAIN_REGS + 2 * SPLIT_REGS + AUX_REGS == 5 * LAUNCH_REGS, "register shares");
     static constexpr int COLS = BN / 2;                  // output channels a drain thread sums
     static constexpr int DEMPTY = NU == 2 ? 4 : 8;       // warps that drain one accumulator
-    static constexpr int A_COL0 = 256, A_COLS = 96;      // tensor-memory columns: accumulators 0-255, two A stages behind
+    // tensor-memory columns: two accumulators, behind them NA stages of A images
+    static constexpr int D_COLS = NUC, A_COL0 = 2 * D_COLS, A_COLS = 96, NA = BN == 64 ? 4 : 2;
+    static_assert(A_COL0 + NA * A_COLS <= 512, "tensor memory");
     static_assert(BN == 64 || BN == 128 || BN == 256, "tile width");
+    static_assert(!SPLIT || BN == 64, "the cluster's exchange takes 32 KB of the weight stages");
 };
 
 __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
@@ -122,11 +134,25 @@ __device__ __forceinline__ uint32_t bf16x2(float first, float second) {
 }
 
 // Splits two fp32 values into bf16 images packed as (first, second): x = h + m + l exactly (up to subnormal l).
-__device__ __forceinline__ void split2(float x0, float x1, uint32_t& h, uint32_t& m, uint32_t& l) {
-    h = bf16x2(x0, x1);
-    const float r0 = x0 - __uint_as_float(h << 16), r1 = x1 - __uint_as_float(h & 0xffff0000u);
-    m = bf16x2(r0, r1);
-    l = bf16x2(r0 - __uint_as_float(m << 16), r1 - __uint_as_float(m & 0xffff0000u));
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint32_t bf16_of(uint64_t x) {
+    float first, second;
+    unpack2(x, first, second);
+    return bf16x2(first, second);
+}
+__device__ __forceinline__ uint64_t widen(uint32_t b) { return join2(b << 16, b & 0xffff0000u); }
+__device__ __forceinline__ void split2(uint64_t x, uint32_t& h, uint32_t& m, uint32_t& l) {
+    h = bf16_of(x);
+    const uint64_t r = sub2(x, widen(h));
+    m = bf16_of(r);
+    l = bf16_of(sub2(r, widen(m)));
+}
+__device__ __forceinline__ void load_shared(uint32_t addr, uint64_t& a, uint64_t& b) {
+    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "r"(addr) : "memory");
 }
 
 // Position in a ring of `n` stages: the stage, and the parity of its current use.
@@ -151,11 +177,11 @@ struct Ring {
     }
 };
 
-// The tiles of a CTA: every gridDim.x-th, channel tiles innermost.
+// The tiles of a CTA: every gridDim.x-th, channel tiles innermost (a cluster that shares a tile has just that one).
 struct Tiles {
     const TcArgs& a;
     int m, n;
-    __device__ explicit Tiles(const TcArgs& args) : a(args), m(blockIdx.x / args.ntiles_n), n(blockIdx.x % args.ntiles_n) {}
+    __device__ explicit Tiles(const TcArgs& args) : a(args), m(blockIdx.x / args.split / args.ntiles_n), n(blockIdx.x / args.split % args.ntiles_n) {}
     __device__ bool left() const { return m < a.ntiles_m; }
     __device__ void next() {
         m += a.dm;
@@ -166,6 +192,26 @@ struct Tiles {
         }
     }
 };
+
+// All threads of the cluster: what any of them wrote before, to whose shared memory ever, is visible to all after.
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// Stores 16 bytes at the address that `addr` has in the shared memory of CTA `rank` of the cluster.
+__device__ __forceinline__ void store_remote(uint32_t addr, uint32_t rank, float4 v) {
+    asm volatile(
+        "{\n\t.reg .b32 r;\n\t"
+        "mapa.shared::cluster.u32 r, %0, %1;\n\t"
+        "st.shared::cluster.v4.f32 [r], {%2, %3, %4, %5};\n\t}"
+        ::"r"(addr), "r"(rank), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+        : "memory");
+}
 
 template <int REGS>
 __device__ __forceinline__ void regs_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS)); }
@@ -203,6 +249,57 @@ __device__ __noinline__ void exact_pixel(const TcArgs& a, int m, int n0, int n1)
     }
 }
 
+// Last step of a tile whose steps were shared by the `split` CTAs of a cluster, for the drain threads: chunk c of a
+// thread's channels (four of them) belongs to CTA c * split / CHUNKS.  Everybody writes its sums of the chunks of others into
+// their shared memory, [sender][chunk][thread], and then adds up and stores its own.  The weight stages hold the exchange:
+// every CTA's MMAs are complete when its drain threads reach the first barrier.
+template <class T>
+__device__ __forceinline__ void store_shared_tile(const TcArgs& a, uint64_t (&acc)[T::COLS / 2], uint32_t exchange, const unsigned char* mine, int m,
+                                                  int n0, int tid) {
+    constexpr int CHUNKS = T::COLS / 4;
+    const int rank = (int)cluster_rank(), own = CHUNKS / a.split;
+    __syncwarp();
+    cluster_sync();
+#pragma unroll
+    for (int c = 0; c < CHUNKS; ++c) {
+        const int owner = c / own;
+        float4 v;
+        unpack2(acc[2 * c], v.x, v.y);
+        unpack2(acc[2 * c + 1], v.z, v.w);
+        if (owner != rank) store_remote(exchange + ((rank * own + c - owner * own) * 256 + tid) * 16, owner, v);
+    }
+    cluster_sync();
+    bool redo = false;
+#pragma unroll
+    for (int c = 0; c < CHUNKS; ++c) {
+        if (c / own != rank) continue;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int s = 0; s < a.split; ++s) {
+            float4 o = reinterpret_cast<const float4*>(mine)[(s * own + c - rank * own) * 256 + tid];
+            if (s == rank) {
+                unpack2(acc[2 * c], o.x, o.y);
+                unpack2(acc[2 * c + 1], o.z, o.w);
+            }
+            v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
+        }
+        redo |= !(fabsf(v.x) <= 3.402823466e38f);
+        if (a.relu) v = make_float4(fmaxf(v.x, 0.f), fmaxf(v.y, 0.f), fmaxf(v.z, 0.f), fmaxf(v.w, 0.f));
+        const int n = n0 + 4 * c;
+        if (m < a.M && n < a.Cout) {
+            if (T::OUT_CM) {
+                float* yp = a.y + (size_t)n * a.ldy + m;
+                yp[0] = v.x;
+                if (n + 1 < a.Cout) yp[a.ldy] = v.y;
+                if (n + 2 < a.Cout) yp[2 * (size_t)a.ldy] = v.z;
+                if (n + 3 < a.Cout) yp[3 * (size_t)a.ldy] = v.w;
+            } else {
+                *reinterpret_cast<float4*>(a.y + (size_t)m * a.ldy + n) = v;   // Cout is a multiple of 4
+            }
+        }
+    }
+    if (redo && m < a.M) exact_pixel<T>(a, m, n0 + rank * own * 4, min(n0 + (rank + 1) * own * 4, a.Cout));
+}
+
 template <class T>
 __global__ void __launch_bounds__(T::NT, 1)
 conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap ymap, const __grid_constant__ TcArgs a) {
@@ -218,8 +315,8 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
     uint64_t* bfull = xempty + SA;
     uint64_t* bempty = bfull + SB;
     uint64_t* afull = bempty + SB;      // A images of a step are in tensor memory
-    uint64_t* aempty = afull + 2;
-    uint64_t* dfull = aempty + 2;       // accumulator of a step is complete
+    uint64_t* aempty = afull + T::NA;
+    uint64_t* dfull = aempty + T::NA;       // accumulator of a step is complete
     uint64_t* dempty = dfull + 2;
     uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(dempty + 2);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
@@ -229,9 +326,9 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
         for (int s = 0; s < SA; ++s) { mbar_init(xfull + s, 1); mbar_init(xempty + s, 8); }
         for (int s = 0; s < SB; ++s) { mbar_init(bfull + s, 1); mbar_init(bempty + s, 1); }
         for (int s = 0; s < 2; ++s) {
-            mbar_init(afull + s, 8); mbar_init(aempty + s, NU);
             mbar_init(dfull + s, 1); mbar_init(dempty + s, T::DEMPTY);
         }
+        for (int s = 0; s < T::NA; ++s) { mbar_init(afull + s, 8); mbar_init(aempty + s, NU); }
         *abort_flag = 0;
         mbar_fence_init();
     }
@@ -244,6 +341,13 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
     auto wait = [&](uint64_t* bar, uint32_t parity) {   // warp-uniform result
         return (bool)__all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, a.status, SBNN_ERR_TIMEOUT));
     };
+    // this CTA's steps of its tiles
+    int kb = 0, ke = a.steps;
+    if (T::SPLIT) {
+        const int rank = (int)cluster_rank(), runs = a.steps / T::RUN;
+        kb = runs * rank / a.split * T::RUN;
+        ke = runs * (rank + 1) / a.split * T::RUN;
+    }
     // valid 32-channel halves of a step
     auto subs = [&](int k) { return a.Cin - (k / T::TAPS) * 64 > 32 ? 2 : 1; };
 
@@ -258,7 +362,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                 const int m0 = t.m * T::BM;
                 int px = 0, py = 0, pn = 0;
                 if (T::SRC == SRC_IM2COL) { px = m0 % a.W; py = (m0 / a.W) % a.H; pn = m0 / (a.W * a.H); }
-                for (int k = 0; k < a.steps && ok; ++k) {
+                for (int k = kb; k < ke && ok; k += T::RUN) {
                     const int c = k / T::TAPS, tap = k - c * T::TAPS;
                     for (int h = 0; h < subs(k); ++h, ring.next()) {
                         const int s = ring.stage;
@@ -268,6 +372,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                             const int c0 = c * 64 + h * T::SUB;
                             mbar_arrive_expect_tx(xfull + s, T::A_BYTES);
                             if (T::SRC == SRC_CM) tensor_g2s_2d(dst, &amap, m0, c0, xfull + s);
+                            else if (T::SRC == SRC_CM3) tensor_g2s_2d(dst, &amap, (m0 + (tap / 3 - 1) * a.W - 1) & ~3, c0, xfull + s);
                             else if (T::SRC == SRC_NHWC) tensor_g2s_2d(dst, &amap, c0, m0, xfull + s);
                             else im2col_g2s(dst, &amap, c0, px - 1, py - 1, pn, tap % 3, tap / 3, xfull + s);
                         }
@@ -282,7 +387,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
             bool ok = true;
             for (Tiles t(a); t.left() && ok; t.next()) {
                 const int nt = t.n * NU;
-                for (int k = 0; k < a.steps && ok; ++k)
+                for (int k = kb; k < ke && ok; ++k)
                     for (int u = 0; u < NU; ++u, ring.next()) {
                         const int s = ring.stage;
                         if (ring.reused() && !(ok = wait(bempty + s, ring.parity ^ 1))) break;
@@ -305,13 +410,13 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
             Ring ring(SB);
             bool ok = true;
             for (Tiles t(a); t.left() && ok; t.next()) {
-                for (int k0 = 0; k0 < a.steps && ok; ++k0, ++step)
+                for (int k0 = kb; k0 < ke && ok; ++k0, ++step)
                     for (int u = 0; u < NU; ++u, ++unit, ring.next()) {
                         if ((unit & 1) != d) continue;
-                        const int as = step & 1, s = ring.stage;
+                        const int as = step % T::NA, s = ring.stage;
                         if (unit >= 2 && !(ok = wait(dempty + d, ((unit >> 1) & 1) ^ 1))) break;
                         if (!(ok = wait(bfull + s, ring.parity))) break;
-                        if (!(ok = wait(afull + as, (step >> 1) & 1))) break;
+                        if (!(ok = wait(afull + as, (step / T::NA) & 1))) break;
                         tc_fence_after_sync();
                         const uint32_t a_base = tmem + T::A_COL0 + as * T::A_COLS;
                         const uint64_t b_desc = operand_desc(smem_u32(bst) + (uint32_t)s * T::B_BYTES);
@@ -321,14 +426,14 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
 #pragma unroll
                                 for (int i = 0; i < 24; ++i) {
                                     const int p = i >> 2, k = i & 3;
-                                    umma_bf16_ta(tmem + d * 128, a_base + PA[p] * 32 + k * 8, b_desc + ((PB[p] * (NUC * 128) + k * 32) >> 4),
+                                    umma_bf16_ta(tmem + d * T::D_COLS, a_base + PA[p] * 32 + k * 8, b_desc + ((PB[p] * (NUC * 128) + k * 32) >> 4),
                                                  idesc, i ? 1u : 0u);
                                 }
                             } else {
 #pragma unroll
                                 for (int i = 0; i < 12; ++i) {
                                     const int p = i >> 1, k = i & 1;
-                                    umma_bf16_ta(tmem + d * 128, a_base + PA[p] * 32 + k * 8, b_desc + ((PB[p] * (NUC * 128) + k * 32) >> 4),
+                                    umma_bf16_ta(tmem + d * T::D_COLS, a_base + PA[p] * 32 + k * 8, b_desc + ((PB[p] * (NUC * 128) + k * 32) >> 4),
                                                  idesc, i ? 1u : 0u);
                                 }
                             }
@@ -347,41 +452,60 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
             int step = 0;
             Ring ring(SA);
             bool ok = true;
-            for (Tiles t(a); t.left() && ok; t.next())
-                for (int k0 = 0; k0 < a.steps && ok; ++k0, ++step) {
-                    const int as = step & 1;
-                    if (step >= 2 && !(ok = wait(aempty + as, ((step >> 1) & 1) ^ 1))) break;
+            for (Tiles t(a); t.left() && ok; t.next()) {
+                int px = 0, py = 0;                         // SRC_CM3: the pixel's place in its image
+                if (T::SRC == SRC_CM3) {
+                    const int m = t.m * T::BM + p;
+                    px = m % a.W;
+                    py = (m / a.W) % a.H;
+                }
+                for (int k0 = kb; k0 < ke && ok; ++k0, ++step) {
+                    const int as = step % T::NA, halves = subs(k0);
+                    const int tap = k0 % T::TAPS, dy = tap / 3 - 1, dx = tap % 3 - 1;
+                    const bool inside = T::SRC != SRC_CM3 || ((unsigned)(px + dx) < (unsigned)a.W && (unsigned)(py + dy) < (unsigned)a.H);
+                    const int shift = T::SRC == SRC_CM3 ? ((t.m * T::BM + dy * a.W - 1) & 3) + 1 + dx : 0;
+                    const uint32_t col = lane_base + as * T::A_COLS + half * 8;
+                    if (step >= T::NA && !(ok = wait(aempty + as, ((step / T::NA) & 1) ^ 1))) break;
                     tc_fence_after_sync();
-                    for (int h = 0; h < subs(k0); ++h, ring.next()) {
-                        const int s = ring.stage;
-                        if (!(ok = wait(xfull + s, ring.parity))) break;
+                    Ring at = ring;
+                    for (int h = 0; h < halves; ++h, at.next()) {
+                        const int s = at.stage;
+                        if (!(ok = wait(xfull + s, at.parity))) break;
                         const unsigned char* src = ast + (size_t)s * T::A_BYTES;
-                        float v[16];
-                        if (T::SRC == SRC_CM) {
+                        uint64_t v[8];                      // pairs of neighbouring channels
+                        if (T::SRC == SRC_CM || T::SRC == SRC_CM3) {
+                            const float* row = reinterpret_cast<const float*>(src) + half * 16 * T::PIX + shift + p;
 #pragma unroll
-                            for (int k = 0; k < 16; ++k) v[k] = reinterpret_cast<const float*>(src)[(half * 16 + k) * T::BM + p];
+                            for (int k = 0; k < 8; ++k)
+                                v[k] = inside ? pack2(row[2 * k * T::PIX], row[(2 * k + 1) * T::PIX]) : 0;
                         } else {
+                            // 16-byte chunk c of the pixel's row sits at chunk c ^ (p & 7)
+                            const uint32_t row = smem_u32(src) + p * 128 + ((p & 7) << 4);
 #pragma unroll
-                            for (int j = 0; j < 4; ++j)
-                                *reinterpret_cast<float4*>(v + 4 * j) =
-                                    *reinterpret_cast<const float4*>(src + p * 128 + (((half * 4 + j) ^ (p & 7)) << 4));
+                            for (int j = 0; j < 4; ++j) load_shared(row ^ ((half * 4 + j) << 4), v[2 * j], v[2 * j + 1]);
                         }
                         uint32_t hh[8], mm[8], ll[8];
 #pragma unroll
-                        for (int k = 0; k < 8; ++k) split2(v[2 * k], v[2 * k + 1], hh[k], mm[k], ll[k]);
-                        const uint32_t col = lane_base + as * T::A_COLS + h * 16 + half * 8;
-                        tmem_st8(col, hh);
-                        tmem_st8(col + 32, mm);
-                        tmem_st8(col + 64, ll);
+                        for (int k = 0; k < 8; ++k) split2(v[k], hh[k], mm[k], ll[k]);
+                        tmem_st8(col + h * 16, hh);
+                        tmem_st8(col + h * 16 + 32, mm);
+                        tmem_st8(col + h * 16 + 64, ll);
                         __syncwarp();
-                        if (lane == 0) mbar_arrive(xempty + s);
+                        if (lane == 0 && tap % T::RUN == T::RUN - 1) mbar_arrive(xempty + s);
                     }
                     if (!ok) break;
+                    if (tap % T::RUN == T::RUN - 1) ring = at;   // else the next tap reads the same stages
                     tmem_st_wait();
                     tc_fence_before_sync();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(afull + as);
                 }
+            }
+        }
+        if (T::SPLIT) {
+            __syncwarp();
+            cluster_sync();
+            cluster_sync();
         }
     } else {
         // ---------------- drain and store ----------------
@@ -398,16 +522,17 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
             uint64_t acc[T::COLS / 2];                      // pairs of neighbouring channels, from the bias on
 #pragma unroll
             for (int i = 0; i < T::COLS / 4; ++i) {
-                const ulonglong2 b = __ldg(reinterpret_cast<const ulonglong2*>(a.bias + n0) + i);
+                ulonglong2 b = __ldg(reinterpret_cast<const ulonglong2*>(a.bias + n0) + i);
+                if (T::SPLIT && kb) b = make_ulonglong2(0, 0);
                 acc[2 * i] = b.x;
                 acc[2 * i + 1] = b.y;
             }
-            for (int k = 0; k < a.steps; ++k, ++step) {
+            for (int k = kb; k < ke; ++k, ++step) {
                 // two column blocks: a warpgroup drains its own; one block: both drain their half of every accumulator
                 const int unit = NU == 2 ? 2 * step + wg : step, d = unit & 1;
                 if (!(ok = wait(dfull + d, (unit >> 1) & 1))) break;
                 tc_fence_after_sync();
-                const uint32_t col = lane_base + d * 128 + (NU == 2 ? 0 : wg * T::COLS);
+                const uint32_t col = lane_base + d * T::D_COLS + (NU == 2 ? 0 : wg * T::COLS);
 #pragma unroll
                 for (int c0 = 0; c0 < T::COLS; c0 += 32) {
                     uint32_t v[32];
@@ -419,6 +544,10 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                 tc_fence_before_sync();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(dempty + d);
+            }
+            if (T::SPLIT) {
+                store_shared_tile<T>(a, acc, smem_u32(bst), bst, m0 + q * 32 + lane, n0, tid);
+                break;
             }
             if (!ok) break;
             const int m = m0 + q * 32 + lane;
@@ -549,15 +678,120 @@ struct TcCall {
     cudaStream_t st;
 };
 
-bool tc_profits(const sbnn_packed* p, long long M) {
-    if (!p->finite || (double)p->nnz < 0.15 * p->ngroups * p->Cin) return false;
-    return M * p->Cout >= 128 * 64 * 74;
+// ---- which kernel, and how ------------------------------------------------------------------------
+// Cycles a launch takes with tiles of bn output channels: rounds of tiles x (steps + fill and store).  A step takes 14 cycles
+// a channel (24 MMAs at 70-75 cycles for 128 channels), 64 channels no less than it takes to split its activations.
+double tc_cost(const sbnn_packed* p, long long M, int bn) {
+    const long long tiles = (M + 127) / 128 * ((p->Cout + bn - 1) / bn), sms = device_sms();
+    const double steps = 0.5 * (double)((p->Cin + 31) / 32) * p->KH * p->KW;
+    const double step = bn == 64 ? 1600.0 : 14.0 * bn;
+    return (double)((tiles + sms - 1) / sms) * (steps * step + (bn == 64 ? 1300.0 : 1000.0 + 12.0 * bn)) + 6300.0;
+}
+
+// Clusters of `split` CTAs that the device runs at the same time (on 148 SMs 74 of 2, 33 of 4, 15 of 8).
+long long cluster_capacity(int split) {
+    static std::mutex mu;
+    static std::map<std::pair<int, int>, int> known;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    std::lock_guard<std::mutex> lk(mu);
+    auto it = known.find({dev, split});
+    if (it == known.end()) {
+        using T = TC<64, SRC_CM, true, true>;
+        int n = 0;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(device_sms() / split * split));
+        cfg.blockDim = dim3(T::NT);
+        cfg.dynamicSmemBytes = 227 * 1024;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)split;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if (set_max_dyn_smem(reinterpret_cast<const void*>(&conv_tc_kernel<T>), 227 * 1024) != SBNN_OK ||
+            cudaOccupancyMaxActiveClusters(&n, conv_tc_kernel<T>, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            n = 0;
+        }
+        it = known.emplace(std::make_pair(dev, split), n).first;
+    }
+    return it->second;
+}
+
+// The same for 64-channel tiles shared by `split` CTAs; infinite when they do not all run at the same time.
+double tc_split_cost(const sbnn_packed* p, long long M, int split, int run) {
+    const long long tiles = (M + 127) / 128 * ((p->Cout + 63) / 64), runs = (long long)((p->Cin + 63) / 64) * p->KH * p->KW / run;
+    if (runs < split || tiles * split > device_sms() || tiles > cluster_capacity(split)) return 1e30;
+    return (double)((runs + split - 1) / split * run) * 1600.0 + 11400.0;
+}
+
+using TcChoice = sbnn_packed::TcChoice;
+TcChoice tc_choose(const sbnn_packed* p, long long M, int run) {
+    TcChoice best{64, 1, tc_cost(p, M, 64)};
+    for (int bn : {128, 256})
+        if (tc_cost(p, M, bn) < best.cost) best = {bn, 1, tc_cost(p, M, bn)};
+    for (int split : {2, 4, 8})
+        if (tc_split_cost(p, M, split, run) < best.cost) best = {64, split, tc_split_cost(p, M, split, run)};
+    return best;
+}
+
+// Whether a call is faster here than on the FMA kernels, in microseconds of both, fitted to measured times.  Layers of
+// 64-1024 channels on 49 to 50176 pixels, G = 4 and 8, 0 / 50 / 70 / 90 % pruned: channel-major 1x1 calls gain up to 70 %
+// pruning (256 x 14 x 14, 1024 -> 1024: 1969 -> 404, 1025 -> 386, 669 -> 366 us; 9 x 14 x 14, 512 -> 512: 89 -> 12, 53 -> 12,
+// 39 -> 12 us) and lose where next to nothing is left to do (the same at 90 %: 313 and 338 us; one 56 x 56 image, 64 -> 128,
+// 50 %: 5.1 and 5.5 us); NHWC calls, which the FMA kernels convert first, and 3x3 calls gain nearly everywhere
+// (32 x 28 x 28, 256 -> 256: 305 -> 119 us at 50 %, 120 -> 111 at 90 %; in groups of 8 106 and 111).
+// `choice` is how; it is remembered with the layer for each kind of call and number of pixels.
+enum Call { CALL_1X1_NHWC, CALL_1X1_CM, CALL_3X3, CALL_3X3_CM };
+TcChoice decide(const sbnn_packed* p, long long M, Call call) {
+    TcChoice choice = {0, 0, 0.0};
+    if (!p->finite || p->nnz == 0) return choice;
+    const double bytes = 4.0 * M * (p->Cin + p->Cout), mem = bytes / 6.5e6;
+    const double dense = 1e-6 * M * p->Cin * p->Cout;                        // 1e6 multiply-adds of the unpruned layer, a tap
+    double kept = 1e-6 * M * p->nnz * p->G * (p->KH * p->KW);                // and of what is kept
+    if (!p->tap_mask.empty()) kept *= (double)count_kept_taps(p) / ((double)p->nnz * p->KH * p->KW);
+    double fma;
+    if (call == CALL_3X3 || call == CALL_3X3_CM) {
+        fma = 25.0 + kept * (p->G >= 8 ? 0.050 : 0.075);
+    } else if (call == CALL_1X1_CM && conv1x1_few_tiles(p, M)) {
+        fma = 2.7 + kept * (p->G >= 8 ? 0.18 : 0.22);
+    } else if (call == CALL_1X1_CM || (p->Cin >= 128 && M >= 2048)) {
+        fma = 5.0 + 0.034 * kept + 0.0026 * dense + 0.5 * mem;
+        if (call == CALL_1X1_NHWC) fma += 2.0 + 8.0 * M * p->Cin / 4.5e6;    // the conversion to channel-major
+    } else {
+        fma = 2.0 + (p->Cin >= 128 ? 2.0 : 0.0) + 0.012 * p->Cin + 0.1 * kept;
+    }
+    choice = tc_choose(p, M, call == CALL_3X3_CM ? 3 : 1);
+    if (std::max(choice.cost / 1750.0, mem) >= fma) choice.bn = 0;
+    return choice;
+}
+bool tc_profits(const sbnn_packed* p, long long M, Call call, TcChoice* choice = nullptr) {
+    const long long key = M * 4 + call;
+    {
+        std::lock_guard<std::mutex> lk(p->mu);
+        auto it = p->tc_choices.find(key);
+        if (it != p->tc_choices.end()) {
+            if (choice) *choice = it->second;
+            return it->second.bn != 0;
+        }
+    }
+    const TcChoice c = decide(p, M, call);
+    std::lock_guard<std::mutex> lk(p->mu);
+    if (p->tc_choices.size() > 64) p->tc_choices.clear();
+    p->tc_choices[key] = c;
+    if (choice) *choice = c;
+    return c.bn != 0;
 }
 
 }  // namespace
 
 sbnn_status prepare_tc(const sbnn_packed* p, long long M) {
-    if (!tc_profits(p, M)) return SBNN_OK;
+    // (a call with fewer pixels can be faster here although the largest is not)
+    bool any = false;
+    for (long long m = M; m > 0 && !any; m /= 2)
+        any = p->KH == 3 ? tc_profits(p, m, CALL_3X3) : tc_profits(p, m, CALL_1X1_NHWC) || tc_profits(p, m, CALL_1X1_CM);
+    if (!any) return SBNN_OK;
     uint4* wts = nullptr;
     PrepareScope scope;
     for (int nuc : {64, 128}) {   // the tile width depends on the pixels: for calls with fewer, too
@@ -570,7 +804,7 @@ sbnn_status prepare_tc(const sbnn_packed* p, long long M) {
 namespace {
 
 template <class T>
-sbnn_status launch_tc(const sbnn_packed* p, const TcCall& c, bool* done) {
+sbnn_status launch_tc(const sbnn_packed* p, const TcCall& c, int split, bool* done) {
     sbnn_status r = set_max_dyn_smem(reinterpret_cast<const void*>(&conv_tc_kernel<T>), 227 * 1024);
     if (r != SBNN_OK) return r;
     // The warpgroups' register shares add up to LAUNCH_REGS a thread: a build that starts with fewer must not be launched,
@@ -591,8 +825,8 @@ sbnn_status launch_tc(const sbnn_packed* p, const TcCall& c, bool* done) {
     if (total > 0x7fffffffLL) return fail(SBNN_ERR_SHAPE, "too many tiles");
     a.wts = wts; a.bias = p->d_bias; a.y = c.y; a.ldy = c.ldy; a.M = (int)c.M; a.Cin = p->Cin; a.Cout = p->Cout;
     a.steps = (p->Cin + 63) / 64 * T::TAPS; a.ntiles_m = (int)((c.M + T::BM - 1) / T::BM); a.ntiles_n = (int)ntiles_n;
-    a.W = c.W; a.H = c.H; a.relu = c.relu;
-    const bool cm = T::SRC == SRC_CM;
+    a.W = c.W; a.H = c.H; a.relu = c.relu; a.split = T::SPLIT ? split : 1;
+    const bool cm = T::SRC == SRC_CM || T::SRC == SRC_CM3;
     a.ex = {c.x, cm ? 1 : p->Cin, cm ? c.ldx : 1, p->d_group_ptr, p->d_idx, p->d_val, p->G};
     CUtensorMap amap, ymap;
     if (T::SRC == SRC_IM2COL) {
@@ -600,7 +834,7 @@ sbnn_status launch_tc(const sbnn_packed* p, const TcCall& c, bool* done) {
     } else if (cm) {
         const unsigned long long dims[2] = {(unsigned long long)c.M, (unsigned long long)p->Cin};
         const unsigned long long strides[1] = {(unsigned long long)c.ldx * 4};
-        const unsigned box[2] = {(unsigned)T::BM, (unsigned)T::SUB};
+        const unsigned box[2] = {(unsigned)T::PIX, (unsigned)T::SUB};
         if ((r = encode_tiled_map(&amap, c.x, 4, 2, dims, strides, box)) != SBNN_OK) return r;
     } else {
         const unsigned long long dims[2] = {(unsigned long long)p->Cin, (unsigned long long)c.M};
@@ -614,41 +848,24 @@ sbnn_status launch_tc(const sbnn_packed* p, const TcCall& c, bool* done) {
         const unsigned box[2] = {T::OUT_CM ? 32u : 16u, T::OUT_CM ? 16u : 32u};
         if ((r = encode_tiled_map(&ymap, c.y, 4, 2, dims, strides, box, T::OUT_CM ? 0 : 64)) != SBNN_OK) return r;
     }
-    const unsigned grid = (unsigned)std::min<long long>(total, device_sms());
-    a.dm = (int)(grid / (unsigned)ntiles_n);
-    a.dn = (int)(grid % (unsigned)ntiles_n);
-    a.resident = ntiles_n == 1 && a.steps * T::NU <= T::SB_MAX && a.steps * T::NU * T::B_BYTES + 3 * T::A_BYTES <= T::ROOM;
+    const unsigned grid = T::SPLIT ? (unsigned)(total * split) : (unsigned)std::min<long long>(total, device_sms());
+    a.dm = T::SPLIT ? a.ntiles_m : (int)(grid / (unsigned)ntiles_n);
+    a.dn = T::SPLIT ? 0 : (int)(grid % (unsigned)ntiles_n);
+    a.resident = !T::SPLIT && ntiles_n == 1 && a.steps * T::NU <= T::SB_MAX && a.steps * T::NU * T::B_BYTES + 3 * T::A_BYTES <= T::ROOM;
     a.sb = a.resident ? a.steps * T::NU : T::SB;
     a.sa = std::min(T::SA_MAX, (T::ROOM - a.sb * T::B_BYTES) / T::A_BYTES);
     const size_t smem = (size_t)a.sb * T::B_BYTES + (size_t)a.sa * T::A_BYTES + T::OUT_BYTES + T::CTRL + 1024;
-    SBNN_CUDA_TRY(launch_kernel(conv_tc_kernel<T>, dim3(grid), dim3(T::NT), smem, c.st, amap, ymap, a));
+    SBNN_CUDA_TRY(launch_kernel_cluster(conv_tc_kernel<T>, dim3(grid), dim3(T::NT), smem, c.st, (unsigned)a.split, amap, ymap, a));
     return SBNN_OK;
 }
 
-// Cycles a launch takes with tiles of bn output channels: rounds of tiles x (steps x max(MMAs, copies from L2) + fill and store).
-double tc_cost(const sbnn_packed* p, long long M, int bn) {
-    const long long tiles = (M + 127) / 128 * ((p->Cout + bn - 1) / bn), sms = device_sms();
-    const double steps = (double)((p->Cin + 63) / 64) * p->KH * p->KW;
-    const double step = bn == 64 ? 1600.0 : 14.0 * bn;
-    return (double)((tiles + sms - 1) / sms) * (steps * step + 1000.0 + 12.0 * bn) + 4000.0;
-}
-int tc_width(const sbnn_packed* p, long long M) {
-    int best = 64;
-    for (int bn : {128, 256})
-        if (tc_cost(p, M, bn) < tc_cost(p, M, best)) best = bn;
-    return best;
-}
-
 template <int SRC, bool OUT_CM>
-sbnn_status dispatch_tc(const sbnn_packed* p, const TcCall& c, bool* done) {
-    if (prepare_only()) {
-        const sbnn_status r = prepare_tc(p, c.M);
-        if (r != SBNN_OK) return r;
-    }
-    switch (tc_width(p, c.M)) {
-        case 256: return launch_tc<TC<256, SRC, OUT_CM>>(p, c, done);
-        case 128: return launch_tc<TC<128, SRC, OUT_CM>>(p, c, done);
-        default: return launch_tc<TC<64, SRC, OUT_CM>>(p, c, done);
+sbnn_status dispatch_tc(const sbnn_packed* p, const TcCall& c, const TcChoice& ch, bool* done) {
+    if (ch.split > 1) return launch_tc<TC<64, SRC, OUT_CM, true>>(p, c, ch.split, done);
+    switch (ch.bn) {
+        case 256: return launch_tc<TC<256, SRC, OUT_CM>>(p, c, 1, done);
+        case 128: return launch_tc<TC<128, SRC, OUT_CM>>(p, c, 1, done);
+        default: return launch_tc<TC<64, SRC, OUT_CM>>(p, c, 1, done);
     }
 }
 
@@ -656,25 +873,47 @@ sbnn_status dispatch_tc(const sbnn_packed* p, const TcCall& c, bool* done) {
 
 sbnn_status conv1x1_tc(const sbnn_packed* p, const float* x, float* y, long long M, int relu, cudaStream_t st, bool* done) {
     *done = false;
-    if (p->Cin % 4 || p->Cout % 4 || !tc_profits(p, M)) return SBNN_OK;
+    TcChoice ch;
+    sbnn_status r;
+    if (prepare_only() && (r = prepare_tc(p, M)) != SBNN_OK) return r;
+    if (p->Cin % 4 || p->Cout % 4 || !tc_profits(p, M, CALL_1X1_NHWC, &ch)) return SBNN_OK;
     const TcCall c{x, 0, y, p->Cout, M, 0, 0, 0, relu, st};
-    return dispatch_tc<SRC_NHWC, false>(p, c, done);
+    return dispatch_tc<SRC_NHWC, false>(p, c, ch, done);
 }
 
 sbnn_status conv1x1_tc_cm(const sbnn_packed* p, const float* x, int ldx, float* y, int ldy, long long M, int relu, bool out_cm, cudaStream_t st,
                           bool* done) {
     *done = false;
-    if ((!out_cm && p->Cout % 4) || !tc_profits(p, M)) return SBNN_OK;
+    TcChoice ch;
+    sbnn_status r;
+    if (prepare_only() && (r = prepare_tc(p, M)) != SBNN_OK) return r;
+    if (p->Cout % 4 || !tc_profits(p, M, CALL_1X1_CM, &ch)) return SBNN_OK;
     const TcCall c{x, ldx, y, ldy, M, 0, 0, 0, relu, st};
-    return out_cm ? dispatch_tc<SRC_CM, true>(p, c, done) : dispatch_tc<SRC_CM, false>(p, c, done);
+    return out_cm ? dispatch_tc<SRC_CM, true>(p, c, ch, done) : dispatch_tc<SRC_CM, false>(p, c, ch, done);
 }
 
 sbnn_status conv3x3_tc(const sbnn_packed* p, const float* x, float* y, int N, int H, int W, int relu, cudaStream_t st, bool* done) {
     *done = false;
+    TcChoice ch;
     const long long M = (long long)N * H * W;
-    if (p->Cin % 4 || p->Cout % 4 || M > 0x7fffffffLL - 128 || !tc_profits(p, M)) return SBNN_OK;
+    sbnn_status r;
+    if (prepare_only() && (r = prepare_tc(p, M)) != SBNN_OK) return r;
+    if (p->Cin % 4 || p->Cout % 4 || M > 0x7fffffffLL - 128 || !tc_profits(p, M, CALL_3X3, &ch)) return SBNN_OK;
     const TcCall c{x, 0, y, p->Cout, M, N, H, W, relu, st};
-    return dispatch_tc<SRC_IM2COL, false>(p, c, done);
+    return dispatch_tc<SRC_IM2COL, false>(p, c, ch, done);
+}
+
+sbnn_status conv3x3_tc_cm(const sbnn_packed* p, const float* x, int ldx, float* y, int ldy, int N, int H, int W, int relu, bool out_cm, cudaStream_t st,
+                          bool* done) {
+    *done = false;
+    TcChoice ch;
+    const long long M = (long long)N * H * W;
+    sbnn_status r;
+    if (prepare_only() && (r = prepare_tc(p, M)) != SBNN_OK) return r;
+    // (the entry point takes rows of up to 224 pixels)
+    if (W > 224 || ldy % 4 || p->Cout % 4 || M > 0x7fffffffLL - 1024 || !tc_profits(p, M, CALL_3X3_CM, &ch)) return SBNN_OK;
+    const TcCall c{x, ldx, y, ldy, M, N, H, W, relu, st};
+    return out_cm ? dispatch_tc<SRC_CM3, true>(p, c, ch, done) : dispatch_tc<SRC_CM3, false>(p, c, ch, done);
 }
 
 void free_tc_weights(sbnn_packed* p) {

@@ -124,6 +124,7 @@ extern "C" sbnn_status sbnn_mobilenet_v1_create(const sbnn_packed* const* pw, co
     }
     if ((st = check_packed_device(fc)) != SBNN_OK) return st;
     if ((st = prepare_default_cm(fc, max_batch)) != SBNN_OK) return st;
+    if ((st = prepare_tc(fc, max_batch)) != SBNN_OK) return st;
     sbnn_mbv1* n = new (std::nothrow) sbnn_mbv1;
     if (!n) return fail(SBNN_ERR_ALLOC, "out of host memory");
     for (int i = 0; i < SBNN_MBV1_NUM_BLOCKS; ++i) {

@@ -42,6 +42,11 @@ SHAPES = [
     (13, 14, 14, 516, 512, 8, 50),
     (64, 9, 9, 192, 256, 16, 50),
     (11, 23, 23, 128, 252, 2, 50),
+    # few tiles: the steps of a tile shared by the 2, 4 or 8 CTAs of a cluster
+    (1, 14, 14, 512, 512, 4, 0),
+    (4, 7, 7, 1024, 1000, 4, 0),
+    (2, 13, 11, 1000, 60, 4, 30),
+    (3, 14, 14, 200, 128, 8, 0),
 ]
 
 
@@ -83,6 +88,10 @@ def test_1x1_channel_major(n, h, w, cin, cout, g, pct, out_cm):
     (120, 7, 7, 100, 128, 4, 30),
     (1, 3, 250, 68, 900, 4, 50),
     (700, 1, 1, 64, 1000, 8, 50),
+    (5, 7, 7, 512, 512, 8, 70),
+    (1, 14, 14, 64, 64, 4, 50),
+    (2, 5, 28, 96, 72, 8, 0),
+    (1, 3, 4, 260, 12, 4, 50),
 ])
 def test_3x3(n, h, w, cin, cout, g, pct):
     d, p = layer(n, h, w, cin, cout, 3, g, pct, seed=2)
@@ -91,6 +100,18 @@ def test_3x3(n, h, w, cin, cout, g, pct):
     sbnn.conv3x3_gs(p, x, y, n, h, w)
     ref, s = reference(d)
     check(y.cpu().numpy(), ref, s)
+    m = n * h * w
+    ld = (m + 3) // 4 * 4 + 4
+    xt = torch.full((cin, ld), float("nan"), device="cuda")
+    xt[:, :m] = x.reshape(m, cin).T
+    for out_cm in (True, False) if w <= 224 else ():
+        y = torch.full((cout, ld) if out_cm else (m, cout), float("nan"), device="cuda")
+        sbnn.conv3x3_gs_cm(p, xt, ld, y, ld if out_cm else cout, n, h, w, sbnn.SBNN_RELU | (sbnn.SBNN_OUT_CM if out_cm else 0))
+        got = y.cpu().numpy()
+        if out_cm:
+            assert np.all(np.isnan(got[:, m:]))
+            got = got[:, :m].T
+        check(got.reshape(ref.shape), ref, s)
     sbnn.get_async_status()
 
 
@@ -107,13 +128,14 @@ def test_values_of_every_size():
 
 
 @pytest.mark.parametrize("k", [1, 3])
-def test_non_finite_activations_stay_where_they_belong(k):
+@pytest.mark.parametrize("h,w,cin", [(50, 41, 64), (18, 41, 520)])   # whole tiles; tiles shared by clusters
+def test_non_finite_activations_stay_where_they_belong(k, h, w, cin):
     """An infinity or a NaN reaches the outputs whose kept channels read it and no others."""
-    n, h, w, cin, cout, g = 5, 50, 41, 64, 128, 4
+    n, cout, g = 5 if cin == 64 else 1, 128, 4
     d, p = layer(n, h, w, cin, cout, k, g, 50, seed=4)
     d["x"][0, 0, 0, 3] = np.inf
-    d["x"][2, 17, 40, 9] = np.nan
-    d["x"][4, 49, 39, 63] = -np.inf
+    d["x"][n // 2, 17, 40, 9] = np.nan
+    d["x"][n - 1, h - 1, 39, 63] = -np.inf
     y = torch.empty((n, h, w, cout), device="cuda")
     (sbnn.conv1x1_gs if k == 1 else sbnn.conv3x3_gs)(p, torch.from_numpy(d["x"]).cuda(), y, n, h, w, 0)
     got = y.cpu().numpy()
