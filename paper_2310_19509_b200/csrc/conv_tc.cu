@@ -102,7 +102,7 @@ struct TC {
     // SB stages of them; the rest goes to activations, up to SA_MAX stages.
     static constexpr int SB = BN < 128 ? 4 : (SRC == SRC_CM3 ? 2 : 3), SA_MAX = 12, SB_MAX = 6;
     static constexpr int ROOM = 227 * 1024 - 1024 - CTRL - OUT_BYTES;
-    static_assert((2 * (SA_MAX + SB_MAX) + 12) * 8 + 8 <= CTRL && SB * B_BYTES + (SRC == SRC_CM3 ? 4 : 3) * A_BYTES <= ROOM, "shared memory");
+    static_assert((2 * SA_MAX + 3 * SB_MAX + 12) * 8 + 8 <= CTRL && SB * B_BYTES + (SRC == SRC_CM3 ? 4 : 3) * A_BYTES <= ROOM, "shared memory");
     static constexpr int NT = 640;
     // registers a thread of the drain, split and remaining warps: 2 x + 2 y + z = 5 x 96, what the launch reserves
     static constexpr int LAUNCH_REGS = 96, DRAIN_REGS = BN == 256 ? 176 : 128, SPLIT_REGS = BN == 256 ? 48 : 80, AUX_REGS = BN == 256 ? 32 : 64;
@@ -168,11 +168,18 @@ struct Ring {
             ++uses;
         }
     }
+    // The weight stages have two "full" barriers each, used in turn.  With an odd number of stages the two MMA warps take
+    // turns at a stage; a barrier for every second use is one that only the same warp waits for, once in each of its
+    // phases (the parity of a barrier that others complete in between would not tell its phases apart).
+    __device__ int turn() const { return stage + (uses & 1 ? n : 0); }
+    __device__ uint32_t turn_parity() const { return uses >> 1 & 1; }
     // A producer that gives up at `stage` lets the copies it has issued land before the shared memory is released.
-    __device__ void settle(uint64_t* full) const {
+    __device__ void settle(uint64_t* full, bool turns) const {
         for (int s = 0; s < (uses ? n : stage); ++s) {
+            const int use = s < stage ? uses : uses - 1;
             bool landed = false;
-            for (uint32_t i = 0; i < kWaitLimit && !landed; ++i) landed = mbar_try_wait(full + s, s < stage ? parity : parity ^ 1);
+            for (uint32_t i = 0; i < kWaitLimit && !landed; ++i)
+                landed = mbar_try_wait(full + s + (turns && (use & 1) ? n : 0), (turns ? use >> 1 : use) & 1);
         }
     }
 };
@@ -313,7 +320,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
     uint64_t* xfull = reinterpret_cast<uint64_t*>(ost + T::OUT_BYTES);
     uint64_t* xempty = xfull + SA;
     uint64_t* bfull = xempty + SA;
-    uint64_t* bempty = bfull + SB;
+    uint64_t* bempty = bfull + 2 * SB;
     uint64_t* afull = bempty + SB;      // A images of a step are in tensor memory
     uint64_t* aempty = afull + T::NA;
     uint64_t* dfull = aempty + T::NA;       // accumulator of a step is complete
@@ -324,7 +331,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, wg = warp >> 2;
     if (tid == 0) {
         for (int s = 0; s < SA; ++s) { mbar_init(xfull + s, 1); mbar_init(xempty + s, 8); }
-        for (int s = 0; s < SB; ++s) { mbar_init(bfull + s, 1); mbar_init(bempty + s, 1); }
+        for (int s = 0; s < SB; ++s) { mbar_init(bfull + s, 1); mbar_init(bfull + SB + s, 1); mbar_init(bempty + s, 1); }
         for (int s = 0; s < 2; ++s) {
             mbar_init(dfull + s, 1); mbar_init(dempty + s, T::DEMPTY);
         }
@@ -380,7 +387,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                     }
                 }
             }
-            if (!ok) ring.settle(xfull);
+            if (!ok) ring.settle(xfull, false);
         } else if (warp == 17) {
             // ---------------- weight copies ----------------
             Ring ring(SB);
@@ -392,14 +399,14 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                         const int s = ring.stage;
                         if (ring.reused() && !(ok = wait(bempty + s, ring.parity ^ 1))) break;
                         if (lane == 0) {
-                            mbar_arrive_expect_tx(bfull + s, T::B_BYTES);
-                            bulk_g2s(bst + (size_t)s * T::B_BYTES, a.wts + ((size_t)(nt + u) * a.steps + k) * (T::B_BYTES / 16), T::B_BYTES, bfull + s);
+                            mbar_arrive_expect_tx(bfull + ring.turn(), T::B_BYTES);
+                            bulk_g2s(bst + (size_t)s * T::B_BYTES, a.wts + ((size_t)(nt + u) * a.steps + k) * (T::B_BYTES / 16), T::B_BYTES, bfull + ring.turn());
                         }
                         __syncwarp();
                     }
                 if (a.resident) break;
             }
-            if (!ok) ring.settle(bfull);
+            if (!ok) ring.settle(bfull, true);
         } else if (warp >= 18) {
             // ---------------- MMA issue ----------------
             constexpr uint32_t idesc = instr_desc(NUC);
@@ -415,7 +422,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                         if ((unit & 1) != d) continue;
                         const int as = step % T::NA, s = ring.stage;
                         if (unit >= 2 && !(ok = wait(dempty + d, ((unit >> 1) & 1) ^ 1))) break;
-                        if (!(ok = wait(bfull + s, ring.parity))) break;
+                        if (!(ok = wait(bfull + ring.turn(), ring.turn_parity()))) break;
                         if (!(ok = wait(afull + as, (step / T::NA) & 1))) break;
                         tc_fence_after_sync();
                         const uint32_t a_base = tmem + T::A_COL0 + as * T::A_COLS;
