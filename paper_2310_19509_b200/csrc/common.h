@@ -148,8 +148,7 @@ struct sbnn_packed {
     mutable std::map<int, sbnn::Stream3x3> streams3x3;
     mutable std::map<long long, sbnn::Plan3x3> plans3x3;           // per (stream, row tiles of the launch, CTAs)
     mutable void* bf16_stream = nullptr;  // see conv1x1_bf16.cu
-    mutable void* umma_weights = nullptr; // dense bf16 copy of the masked weights, see conv1x1_umma.cu
-    mutable std::map<int, void*> tc_weights;  // split bf16 images of the masked weights, see conv_tc.cu
+    mutable std::map<std::pair<int, int>, void*> tc_weights;  // bf16 images of the masked weights, see conv_tc.cu
     bool finite = true;                   // every stored weight is finite
     struct TcChoice {                     // tile width (0: the FMA kernels are faster), CTAs that share a tile, estimated cycles
         int bn, split;
@@ -207,9 +206,6 @@ sbnn_status conv1x1_small(const sbnn_packed* p, const float* x, int ldx, float* 
 // conv1x1_bf16.cu
 sbnn_status conv1x1_bf16(const sbnn_packed* w, const float* x, float* y, int M, int relu, cudaStream_t st);
 void free_stream_bf16(sbnn_packed* p);
-// conv1x1_umma.cu: bf16 mode as a dense contraction over the masked weights (tcgen05); *done = false if the shape is not taken
-sbnn_status conv1x1_umma(const sbnn_packed* w, const float* x, float* y, int M, int relu, cudaStream_t st, bool* done);
-void free_umma_weights(sbnn_packed* p);
 // True when the pipelined 1x1 kernel would get fewer tiles than half the SMs (the few-pixel kernel runs then).
 bool conv1x1_few_tiles(const sbnn_packed* p, long long M);
 // Taps kept over all units of a pattern layer.
@@ -222,6 +218,8 @@ sbnn_status conv1x1_tc_cm(const sbnn_packed* p, const float* x, int ldx, float* 
 sbnn_status conv3x3_tc(const sbnn_packed* p, const float* x, float* y, int N, int H, int W, int relu, cudaStream_t st, bool* done);
 sbnn_status conv3x3_tc_cm(const sbnn_packed* p, const float* x, int ldx, float* y, int ldy, int N, int H, int W, int relu, bool out_cm, cudaStream_t st,
                           bool* done);
+// bf16 mode as a dense contraction over the masked weights; *done = false if the shape is not taken
+sbnn_status conv1x1_tc_bf16(const sbnn_packed* p, const float* x, float* y, long long M, int relu, cudaStream_t st, bool* done);
 // Builds the weight images for calls of up to M pixels.
 sbnn_status prepare_tc(const sbnn_packed* p, long long M);
 void free_tc_weights(sbnn_packed* p);

@@ -433,7 +433,7 @@ extern "C" sbnn_status sbnn_conv1x1_gs(const sbnn_packed* w, const float* x_dev,
     if (flags & SBNN_BF16_TC) {
         // dense over the masked weights on the tcgen05 tensor cores, unless the gathered warp-level kernel is asked
         // for or the shape is outside what the dense kernel takes
-        if (!(flags & SBNN_BF16_GATHER) && ((st = conv1x1_umma(w, x_dev, y_dev, (int)M, flags & SBNN_RELU, s, &done)) != SBNN_OK || done))
+        if (!(flags & SBNN_BF16_GATHER) && ((st = conv1x1_tc_bf16(w, x_dev, y_dev, M, flags & SBNN_RELU, s, &done)) != SBNN_OK || done))
             return st;
         return conv1x1_bf16(w, x_dev, y_dev, (int)M, flags & SBNN_RELU, s);
     }

@@ -26,10 +26,13 @@
 //   warp 16          copies activations (tiled or im2col tensor-map copies of 32 channels x 128 pixels);
 //   warp 17          copies weights (one linear copy per step and 128 output channels: the three bf16 images,
 //                    stored in the swizzled order the MMA reads);
-//   warps 18, 19     issue the MMAs, each into its own accumulator: while one waits for its operands the other's MMAs run.
+//   warps 18, 19     issue the MMAs, each into an accumulator of its own: while one waits for its operands the other's MMAs run.
 // (With one issuing warp the waits between its batches of 24 MMAs, 740 cycles, came on top of the 1900 cycles a batch
 // takes; with one split warpgroup a step took 1300 cycles to split, as long as its MMAs.)
 // Every wait is bounded, as in the other pipelined kernels.
+//
+// The bf16 mode (SBNN_BF16_TC: activations and weights rounded to bf16 once, fp32 sums) is the same kernel with one image
+// of each operand (IMAGES = 1): one product, summed over all steps of a tile in the accumulator and drained once.
 //
 // Launches with too few tiles for the SMs (small batches, small maps) run with 64 output channels a tile and the steps of a
 // tile dealt to the CTAs of a cluster (SPLIT): each sums its share, then every CTA adds up a part of the channels, which
@@ -84,10 +87,11 @@ struct TcArgs {
     ExactArgs ex;
 };
 
-template <int BN_, int SRC_, bool OUT_CM_, bool SPLIT_ = false>
+template <int BN_, int SRC_, bool OUT_CM_, bool SPLIT_ = false, int IMAGES_ = 3>
 struct TC {
     static constexpr int BM = 128, BN = BN_, BK = 64, SRC = SRC_;
     static constexpr bool OUT_CM = OUT_CM_, SPLIT = SPLIT_;
+    static constexpr int IMAGES = IMAGES_;
     static constexpr int TAPS = SRC == SRC_IM2COL || SRC == SRC_CM3 ? 9 : 1;
     static constexpr int RUN = SRC == SRC_CM3 ? 3 : 1;   // steps that read the same activation stages
     static constexpr int PIX = SRC == SRC_CM3 ? 136 : 128;   // pixels of a stage
@@ -95,25 +99,26 @@ struct TC {
     static constexpr int NU = BN / NUC;                  // MMA column blocks per tile
     static constexpr int SUB = 32;                       // channels of one activation stage
     static constexpr int A_BYTES = SUB * PIX * 4;
-    static constexpr int B_BYTES = 3 * NUC * BK * 2;
+    static constexpr int B_BYTES = IMAGES * NUC * BK * 2;
     static constexpr int OUT_BYTES = 8 * 2 * 2048;       // two staging tiles of 32 pixels x 16 channels for each drain warp
     static constexpr int CTRL = 512;                     // mbarriers, tensor-memory base, abort flag
     // Stages share what is left of 227 KB: weights that fit as a whole and serve every tile stay (see launch_tc), else
     // SB stages of them; the rest goes to activations, up to SA_MAX stages.
-    static constexpr int SB = BN < 128 ? 4 : (SRC == SRC_CM3 ? 2 : 3), SA_MAX = 12, SB_MAX = 6;
+    static constexpr int SB = IMAGES == 1 ? 6 : (BN < 128 ? 4 : (SRC == SRC_CM3 ? 2 : 3)), SA_MAX = 12, SB_MAX = 6;
     static constexpr int ROOM = 227 * 1024 - 1024 - CTRL - OUT_BYTES;
     static_assert((2 * SA_MAX + 3 * SB_MAX + 12) * 8 + 8 <= CTRL && SB * B_BYTES + (SRC == SRC_CM3 ? 4 : 3) * A_BYTES <= ROOM, "shared memory");
     static constexpr int NT = 640;
     // registers a thread of the drain, split and remaining warps: 2 x + 2 y + z = 5 x 96, what the launch reserves
-    static constexpr int LAUNCH_REGS = 96, DRAIN_REGS = BN == 256 ? 176 : 128, SPLIT_REGS = BN == 256 ? 48 : 80, AUX_REGS = BN == 256 ? 32 : 64;
+    static constexpr int LAUNCH_REGS = 96, DRAIN_REGS = BN == 256 ? 160 : 128, SPLIT_REGS = BN == 256 ? 56 : 80, AUX_REGS = BN == 256 ? 48 : 64;
     static_assert(2 * DRAIN_REGS + 2 * SPLIT_REGS + AUX_REGS == 5 * LAUNCH_REGS, "register shares");
     static constexpr int COLS = BN / 2;                  // output channels a drain thread sums
     static constexpr int DEMPTY = NU == 2 ? 4 : 8;       // warps that drain one accumulator
     // tensor-memory columns: two accumulators, behind them NA stages of A images
-    static constexpr int D_COLS = NUC, A_COL0 = 2 * D_COLS, A_COLS = 96, NA = BN == 64 ? 4 : 2;
+    static constexpr int D_COLS = NUC, A_COL0 = 2 * D_COLS, A_COLS = 32 * IMAGES, NA = BN == 64 || IMAGES == 1 ? 4 : 2;
     static_assert(A_COL0 + NA * A_COLS <= 512, "tensor memory");
     static_assert(BN == 64 || BN == 128 || BN == 256, "tile width");
-    static_assert(!SPLIT || BN == 64, "the cluster's exchange takes 32 KB of the weight stages");
+    static_assert(!SPLIT || (BN == 64 && SB * B_BYTES >= 32 * 1024), "the cluster's exchange takes 32 KB of the weight stages");
+    static_assert(IMAGES == 3 || (IMAGES == 1 && SRC == SRC_NHWC), "bf16 mode");
 };
 
 __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
@@ -304,7 +309,7 @@ __device__ __forceinline__ void store_shared_tile(const TcArgs& a, uint64_t (&ac
             }
         }
     }
-    if (redo && m < a.M) exact_pixel<T>(a, m, n0 + rank * own * 4, min(n0 + (rank + 1) * own * 4, a.Cout));
+    if (T::IMAGES == 3 && redo && m < a.M) exact_pixel<T>(a, m, n0 + rank * own * 4, min(n0 + (rank + 1) * own * 4, a.Cout));
 }
 
 template <class T>
@@ -345,8 +350,21 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
     tc_fence_after_sync();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_holder, 0);
 
-    auto wait = [&](uint64_t* bar, uint32_t parity) {   // warp-uniform result
-        return (bool)__all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, a.status, SBNN_ERR_TIMEOUT));
+    // Whole warp: until the barrier that each lane names has completed its phase; the same result in all lanes.  (A wait
+    // costs 60 to 100 cycles even when there is nothing to wait for, so a warp looks at all it needs at once, a barrier a lane.)
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+        uint32_t polls = 0;
+        while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) {
+            if (++polls > 64) {
+                if (__any_sync(0xffffffffu, polls > kWaitLimit || *abort_flag)) {
+                    *abort_flag = 1;
+                    atomicCAS(a.status, 0, SBNN_ERR_TIMEOUT);
+                    return false;
+                }
+                __nanosleep(64);
+            }
+        }
+        return true;
     };
     // this CTA's steps of its tiles
     int kb = 0, ke = a.steps;
@@ -412,44 +430,62 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
             constexpr uint32_t idesc = instr_desc(NUC);
             // (image of A, image of B), small products first: h = 0, m = 1, l = 2
             constexpr int PA[6] = {2, 0, 1, 1, 0, 0}, PB[6] = {0, 2, 1, 0, 1, 0};
-            const int d = warp - 18;                        // this warp's accumulator: units d, d + 2, ...
+            const int w = warp - 18;
             int step = 0, unit = 0;
             Ring ring(SB);
             bool ok = true;
+            // Three images: every step of a column block is a unit with an accumulator of its own, and the warps take turns.
+            // One image: a unit is a column block of a tile, warp u takes block u (with one block warp 0 takes all).
             for (Tiles t(a); t.left() && ok; t.next()) {
                 for (int k0 = kb; k0 < ke && ok; ++k0, ++step)
-                    for (int u = 0; u < NU; ++u, ++unit, ring.next()) {
-                        if ((unit & 1) != d) continue;
+                    for (int u = 0; u < NU; ++u, ring.next()) {
+                        if (T::IMAGES == 3) {
+                            if ((unit++ & 1) != w) continue;
+                        } else if (u != w) {
+                            continue;
+                        }
+                        const int mine = T::IMAGES == 3 ? unit - 1 : unit + w, d = mine & 1;
                         const int as = step % T::NA, s = ring.stage;
-                        if (unit >= 2 && !(ok = wait(dempty + d, ((unit >> 1) & 1) ^ 1))) break;
-                        if (!(ok = wait(bfull + ring.turn(), ring.turn_parity()))) break;
-                        if (!(ok = wait(afull + as, (step / T::NA) & 1))) break;
+                        // lane 0: the accumulator is drained, lane 1: the weights are here, others: so are the activations
+                        uint64_t* bar = afull + as;
+                        uint32_t parity = (step / T::NA) & 1;
+                        if (lane == 1) {
+                            bar = bfull + ring.turn();
+                            parity = ring.turn_parity();
+                        } else if (lane == 0 && (T::IMAGES == 3 || k0 == kb) && mine >= 2) {
+                            bar = dempty + d;
+                            parity = ((mine >> 1) & 1) ^ 1;
+                        }
+                        if (!(ok = wait(bar, parity))) break;
                         tc_fence_after_sync();
                         const uint32_t a_base = tmem + T::A_COL0 + as * T::A_COLS;
                         const uint64_t b_desc = operand_desc(smem_u32(bst) + (uint32_t)s * T::B_BYTES);
                         const bool whole = subs(k0) == 2;
+                        const uint32_t more = T::IMAGES == 1 && k0 > kb ? 1u : 0u;
+                        constexpr int P0 = T::IMAGES == 3 ? 0 : 5, NP = 6 - P0;      // one image: just h * h
                         if (elect_one()) {
                             if (whole) {
 #pragma unroll
-                                for (int i = 0; i < 24; ++i) {
-                                    const int p = i >> 2, k = i & 3;
+                                for (int i = 0; i < 4 * NP; ++i) {
+                                    const int p = P0 + (i >> 2), k = i & 3;
                                     umma_bf16_ta(tmem + d * T::D_COLS, a_base + PA[p] * 32 + k * 8, b_desc + ((PB[p] * (NUC * 128) + k * 32) >> 4),
-                                                 idesc, i ? 1u : 0u);
+                                                 idesc, i ? 1u : more);
                                 }
                             } else {
 #pragma unroll
-                                for (int i = 0; i < 12; ++i) {
-                                    const int p = i >> 1, k = i & 1;
+                                for (int i = 0; i < 2 * NP; ++i) {
+                                    const int p = P0 + (i >> 1), k = i & 1;
                                     umma_bf16_ta(tmem + d * T::D_COLS, a_base + PA[p] * 32 + k * 8, b_desc + ((PB[p] * (NUC * 128) + k * 32) >> 4),
-                                                 idesc, i ? 1u : 0u);
+                                                 idesc, i ? 1u : more);
                                 }
                             }
                             if (!a.resident) umma_commit(bempty + s);
-                            umma_commit(dfull + d);
+                            if (T::IMAGES == 3 || k0 == ke - 1) umma_commit(dfull + d);
                             umma_commit(aempty + as);
                         }
                         __syncwarp();
                     }
+                if (T::IMAGES == 1) unit += NU;
                 if (a.resident) ring = Ring(SB);            // the same stages again, still full from the first round
             }
         } else if (wg < 4) {
@@ -472,12 +508,23 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                     const bool inside = T::SRC != SRC_CM3 || ((unsigned)(px + dx) < (unsigned)a.W && (unsigned)(py + dy) < (unsigned)a.H);
                     const int shift = T::SRC == SRC_CM3 ? ((t.m * T::BM + dy * a.W - 1) & 3) + 1 + dx : 0;
                     const uint32_t col = lane_base + as * T::A_COLS + half * 8;
-                    if (step >= T::NA && !(ok = wait(aempty + as, ((step / T::NA) & 1) ^ 1))) break;
-                    tc_fence_after_sync();
+                    // lane 0: the place in tensor memory is free, lane 1: the second half of the step is here, others: the first
                     Ring at = ring;
+                    uint64_t* bar = xfull + at.stage;
+                    uint32_t parity = at.parity;
+                    if (lane == 1 && halves == 2) {
+                        Ring second = at;
+                        second.next();
+                        bar = xfull + second.stage;
+                        parity = second.parity;
+                    } else if (lane == 0 && step >= T::NA) {
+                        bar = aempty + as;
+                        parity = ((step / T::NA) & 1) ^ 1;
+                    }
+                    if (!(ok = wait(bar, parity))) break;
+                    tc_fence_after_sync();
                     for (int h = 0; h < halves; ++h, at.next()) {
                         const int s = at.stage;
-                        if (!(ok = wait(xfull + s, at.parity))) break;
                         const unsigned char* src = ast + (size_t)s * T::A_BYTES;
                         uint64_t v[8];                      // pairs of neighbouring channels
                         if (T::SRC == SRC_CM || T::SRC == SRC_CM3) {
@@ -492,15 +539,19 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                             for (int j = 0; j < 4; ++j) load_shared(row ^ ((half * 4 + j) << 4), v[2 * j], v[2 * j + 1]);
                         }
                         uint32_t hh[8], mm[8], ll[8];
+                        if (T::IMAGES == 3) {
 #pragma unroll
-                        for (int k = 0; k < 8; ++k) split2(v[k], hh[k], mm[k], ll[k]);
+                            for (int k = 0; k < 8; ++k) split2(v[k], hh[k], mm[k], ll[k]);
+                            tmem_st8(col + h * 16 + 32, mm);
+                            tmem_st8(col + h * 16 + 64, ll);
+                        } else {
+#pragma unroll
+                            for (int k = 0; k < 8; ++k) hh[k] = bf16_of(v[k]);
+                        }
                         tmem_st8(col + h * 16, hh);
-                        tmem_st8(col + h * 16 + 32, mm);
-                        tmem_st8(col + h * 16 + 64, ll);
                         __syncwarp();
                         if (lane == 0 && tap % T::RUN == T::RUN - 1) mbar_arrive(xempty + s);
                     }
-                    if (!ok) break;
                     if (tap % T::RUN == T::RUN - 1) ring = at;   // else the next tap reads the same stages
                     tmem_st_wait();
                     tc_fence_before_sync();
@@ -534,19 +585,20 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                 acc[2 * i] = b.x;
                 acc[2 * i + 1] = b.y;
             }
-            for (int k = kb; k < ke; ++k, ++step) {
+            for (int k = T::IMAGES == 3 ? kb : ke - 1; k < ke; ++k, ++step) {
                 // two column blocks: a warpgroup drains its own; one block: both drain their half of every accumulator
                 const int unit = NU == 2 ? 2 * step + wg : step, d = unit & 1;
                 if (!(ok = wait(dfull + d, (unit >> 1) & 1))) break;
                 tc_fence_after_sync();
                 const uint32_t col = lane_base + d * T::D_COLS + (NU == 2 ? 0 : wg * T::COLS);
+                constexpr int LD = T::BN == 256 ? 16 : 32;      // columns at a time: what registers there are left
 #pragma unroll
-                for (int c0 = 0; c0 < T::COLS; c0 += 32) {
-                    uint32_t v[32];
-                    tmem_ld32(col + c0, v);
+                for (int c0 = 0; c0 < T::COLS; c0 += LD) {
+                    uint32_t v[LD];
+                    tmem_ld(col + c0, v);
                     tmem_ld_wait();
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) acc[c0 / 2 + i] = add2(acc[c0 / 2 + i], join2(v[2 * i], v[2 * i + 1]));
+                    for (int i = 0; i < LD / 2; ++i) acc[c0 / 2 + i] = add2(acc[c0 / 2 + i], join2(v[2 * i], v[2 * i + 1]));
                 }
                 tc_fence_before_sync();
                 __syncwarp();
@@ -560,7 +612,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
             const int m = m0 + q * 32 + lane;
             float first, unused;
             unpack2(acc[0], first, unused);
-            const bool redo = m < a.M && !(fabsf(first) <= 3.402823466e38f);
+            const bool redo = T::IMAGES == 3 && m < a.M && !(fabsf(first) <= 3.402823466e38f);
             // 32 pixels x 16 channels at a time through one of the warp's two staging tiles, stored by tiled copies: rows of 32
             // pixels (channel-major) or of 16 channels (64-byte swizzle).  Rows past Cout or M are clipped by the copy; the last
             // pixels of a channel-major row are stored one by one, so that the padding behind them is left alone.
@@ -617,23 +669,27 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
     if (warp == 18) tmem_dealloc(tmem, 512);
 }
 
-// One thread per (kept unit, tap, channel of the group): the weight's three bf16 images into their place in the tiles.
+// One thread per (kept unit, tap, channel of the group): the weight's bf16 images into their place in the tiles.
 __global__ void build_tc_weights_kernel(const int32_t* __restrict__ group_ptr, const int32_t* __restrict__ idx, const float* __restrict__ val,
-                                        int G, int taps, int csteps, int nuc, __nv_bfloat16* __restrict__ out) {
+                                        int G, int taps, int csteps, int nuc, int images, __nv_bfloat16* __restrict__ out) {
     const int g = blockIdx.x, per_unit = taps * G;
     const int lo = group_ptr[g];
     const long long n = (long long)(group_ptr[g + 1] - lo) * per_unit;
     for (long long i = threadIdx.x + (long long)blockIdx.y * blockDim.x; i < n; i += (long long)blockDim.x * gridDim.y) {
         const int j = lo + (int)(i / per_unit), t = (int)(i % per_unit) / G, o = g * G + (int)(i % G), c = idx[j];
+        const int row = o % nuc, kk = c & 63;
+        const size_t block = (size_t)(o / nuc) * csteps * taps + (size_t)(c >> 6) * taps + t;
+        const size_t at = block * images * nuc * 64 + (size_t)row * 64 + ((((kk >> 3) ^ (row & 7)) << 3) | (kk & 7));
+        if (images == 1) {
+            out[at] = __float2bfloat16_rn(val[(size_t)j * per_unit + i % per_unit]);
+            continue;
+        }
         const double w = val[(size_t)j * per_unit + i % per_unit] * kTruncation;
         // Round to nearest; magnitudes that would round up to infinity are truncated instead.
         const __nv_bfloat16 h = fabs(w) > 3.3895e38 ? __float2bfloat16_rz(__double2float_rz(w)) : __float2bfloat16_rn((float)w);
         const double r = w - (double)__bfloat162float(h);
         const __nv_bfloat16 m = __float2bfloat16_rn((float)r);
         const __nv_bfloat16 l = __float2bfloat16_rn((float)(r - (double)__bfloat162float(m)));
-        const int row = o % nuc, kk = c & 63;
-        const size_t block = (size_t)(o / nuc) * csteps * taps + (size_t)(c >> 6) * taps + t;
-        const size_t at = block * 3 * nuc * 64 + (size_t)row * 64 + ((((kk >> 3) ^ (row & 7)) << 3) | (kk & 7));
         out[at] = h;
         out[at + (size_t)nuc * 64] = m;
         out[at + (size_t)2 * nuc * 64] = l;
@@ -642,10 +698,10 @@ __global__ void build_tc_weights_kernel(const int32_t* __restrict__ group_ptr, c
 
 // Weight images of a layer for MMA column blocks of `nuc` output channels, built on first use; NULL if that would be
 // while `st` is being captured, when nothing can be allocated.
-sbnn_status get_tc_weights(const sbnn_packed* p, int nuc, cudaStream_t st, uint4** out) {
+sbnn_status get_tc_weights(const sbnn_packed* p, int nuc, int images, cudaStream_t st, uint4** out) {
     std::lock_guard<std::mutex> lk(p->mu);
     *out = nullptr;
-    auto it = p->tc_weights.find(nuc);
+    auto it = p->tc_weights.find({nuc, images});
     if (it != p->tc_weights.end()) {
         *out = static_cast<uint4*>(it->second);
         return SBNN_OK;
@@ -654,12 +710,12 @@ sbnn_status get_tc_weights(const sbnn_packed* p, int nuc, cudaStream_t st, uint4
     if (!prepare_only() && cudaStreamIsCapturing(st, &cs) != cudaSuccess) cudaGetLastError();
     if (cs != cudaStreamCaptureStatusNone) return SBNN_OK;
     const int taps = p->KH * p->KW, csteps = (p->Cin + 63) / 64, tiles = (p->Cout + 255) / 256 * 256 / nuc;
-    const size_t bytes = (size_t)tiles * csteps * taps * 3 * nuc * 64 * 2;
+    const size_t bytes = (size_t)tiles * csteps * taps * images * nuc * 64 * 2;
     void* d = nullptr;
     SBNN_CUDA_TRY(cudaMalloc(&d, bytes));
     cudaError_t e = cudaMemset(d, 0, bytes);
     if (e == cudaSuccess && p->nnz > 0) {
-        build_tc_weights_kernel<<<dim3((unsigned)p->ngroups, 4), 128>>>(p->d_group_ptr, p->d_idx, p->d_val, p->G, taps, csteps, nuc,
+        build_tc_weights_kernel<<<dim3((unsigned)p->ngroups, 4), 128>>>(p->d_group_ptr, p->d_idx, p->d_val, p->G, taps, csteps, nuc, images,
                                                                        static_cast<__nv_bfloat16*>(d));
         e = cudaGetLastError();
     }
@@ -669,7 +725,7 @@ sbnn_status get_tc_weights(const sbnn_packed* p, int nuc, cudaStream_t st, uint4
         cudaGetLastError();
         return fail(SBNN_ERR_CUDA, "building the tensor-core weights: %s", cudaGetErrorString(e));
     }
-    p->tc_weights[nuc] = d;
+    p->tc_weights[{nuc, images}] = d;
     *out = static_cast<uint4*>(d);
     return SBNN_OK;
 }
@@ -688,11 +744,12 @@ struct TcCall {
 // ---- which kernel, and how ------------------------------------------------------------------------
 // Cycles a launch takes with tiles of bn output channels: rounds of tiles x (steps + fill and store).  A step takes 14 cycles
 // a channel (24 MMAs at 70-75 cycles for 128 channels), 64 channels no less than it takes to split its activations.
-double tc_cost(const sbnn_packed* p, long long M, int bn) {
+// One image (bf16 mode): the copies from L2 take longest, 32 KB of activations and 128 bytes a channel.
+double tc_step(int bn, int images) { return images == 1 ? 380.0 + 1.5 * bn : (bn == 64 ? 1600.0 : 14.0 * bn); }
+double tc_cost(const sbnn_packed* p, long long M, int bn, int images) {
     const long long tiles = (M + 127) / 128 * ((p->Cout + bn - 1) / bn), sms = device_sms();
     const double steps = 0.5 * (double)((p->Cin + 31) / 32) * p->KH * p->KW;
-    const double step = bn == 64 ? 1600.0 : 14.0 * bn;
-    return (double)((tiles + sms - 1) / sms) * (steps * step + (bn == 64 ? 1300.0 : 1000.0 + 12.0 * bn)) + 6300.0;
+    return (double)((tiles + sms - 1) / sms) * (steps * tc_step(bn, images) + (bn == 64 ? 1300.0 : 1000.0 + 12.0 * bn)) + 6300.0;
 }
 
 // Clusters of `split` CTAs that the device runs at the same time (on 148 SMs 74 of 2, 33 of 4, 15 of 8).
@@ -727,19 +784,23 @@ long long cluster_capacity(int split) {
 }
 
 // The same for 64-channel tiles shared by `split` CTAs; infinite when they do not all run at the same time.
-double tc_split_cost(const sbnn_packed* p, long long M, int split, int run) {
+double tc_split_cost(const sbnn_packed* p, long long M, int split, int run, int images) {
     const long long tiles = (M + 127) / 128 * ((p->Cout + 63) / 64), runs = (long long)((p->Cin + 63) / 64) * p->KH * p->KW / run;
     if (runs < split || tiles * split > device_sms() || tiles > cluster_capacity(split)) return 1e30;
-    return (double)((runs + split - 1) / split * run) * 1600.0 + 11400.0;
+    return (double)((runs + split - 1) / split * run) * tc_step(64, images) + 11400.0;
 }
 
 using TcChoice = sbnn_packed::TcChoice;
-TcChoice tc_choose(const sbnn_packed* p, long long M, int run) {
-    TcChoice best{64, 1, tc_cost(p, M, 64)};
-    for (int bn : {128, 256})
-        if (tc_cost(p, M, bn) < best.cost) best = {bn, 1, tc_cost(p, M, bn)};
-    for (int split : {2, 4, 8})
-        if (tc_split_cost(p, M, split, run) < best.cost) best = {64, split, tc_split_cost(p, M, split, run)};
+TcChoice tc_choose(const sbnn_packed* p, long long M, int run, int images) {
+    TcChoice best{64, 1, tc_cost(p, M, 64, images)};
+    for (int bn : {128, 256}) {
+        const double cost = tc_cost(p, M, bn, images);
+        if (cost < best.cost) best = {bn, 1, cost};
+    }
+    for (int split : {2, 4, 8}) {
+        const double cost = tc_split_cost(p, M, split, run, images);
+        if (cost < best.cost) best = {64, split, cost};
+    }
     return best;
 }
 
@@ -750,9 +811,10 @@ TcChoice tc_choose(const sbnn_packed* p, long long M, int run) {
 // 50 %: 5.1 and 5.5 us); NHWC calls, which the FMA kernels convert first, and 3x3 calls gain nearly everywhere
 // (32 x 28 x 28, 256 -> 256: 305 -> 119 us at 50 %, 120 -> 111 at 90 %; in groups of 8 106 and 111).
 // `choice` is how; it is remembered with the layer for each kind of call and number of pixels.
-enum Call { CALL_1X1_NHWC, CALL_1X1_CM, CALL_3X3, CALL_3X3_CM };
+enum Call { CALL_1X1_NHWC, CALL_1X1_CM, CALL_3X3, CALL_3X3_CM, CALL_BF16 };
 TcChoice decide(const sbnn_packed* p, long long M, Call call) {
     TcChoice choice = {0, 0, 0.0};
+    if (call == CALL_BF16) return tc_choose(p, M, 1, 1);
     if (!p->finite || p->nnz == 0) return choice;
     const double bytes = 4.0 * M * (p->Cin + p->Cout), mem = bytes / 6.5e6;
     const double dense = 1e-6 * M * p->Cin * p->Cout;                        // 1e6 multiply-adds of the unpruned layer, a tap
@@ -769,12 +831,12 @@ TcChoice decide(const sbnn_packed* p, long long M, Call call) {
     } else {
         fma = 2.0 + (p->Cin >= 128 ? 2.0 : 0.0) + 0.012 * p->Cin + 0.1 * kept;
     }
-    choice = tc_choose(p, M, call == CALL_3X3_CM ? 3 : 1);
+    choice = tc_choose(p, M, call == CALL_3X3_CM ? 3 : 1, 3);
     if (std::max(choice.cost / 1750.0, mem) >= fma) choice.bn = 0;
     return choice;
 }
 bool tc_profits(const sbnn_packed* p, long long M, Call call, TcChoice* choice = nullptr) {
-    const long long key = M * 4 + call;
+    const long long key = M * 8 + call;
     {
         std::lock_guard<std::mutex> lk(p->mu);
         auto it = p->tc_choices.find(key);
@@ -802,7 +864,7 @@ sbnn_status prepare_tc(const sbnn_packed* p, long long M) {
     uint4* wts = nullptr;
     PrepareScope scope;
     for (int nuc : {64, 128}) {   // the tile width depends on the pixels: for calls with fewer, too
-        const sbnn_status r = get_tc_weights(p, nuc, nullptr, &wts);
+        const sbnn_status r = get_tc_weights(p, nuc, 3, nullptr, &wts);
         if (r != SBNN_OK) return r;
     }
     return SBNN_OK;
@@ -824,7 +886,7 @@ sbnn_status launch_tc(const sbnn_packed* p, const TcCall& c, int split, bool* do
         return fail(SBNN_ERR_UNSUPPORTED, "internal: the tensor-core kernel was built with %d registers a thread, not %d", regs, T::LAUNCH_REGS);
     TcArgs a = {};
     uint4* wts = nullptr;
-    if ((r = get_tc_weights(p, T::NUC, c.st, &wts)) != SBNN_OK || !wts) return r;
+    if ((r = get_tc_weights(p, T::NUC, T::IMAGES, c.st, &wts)) != SBNN_OK || !wts) return r;
     if ((r = async_status_word(&a.status)) != SBNN_OK) return r;
     *done = true;
     if (prepare_only()) return SBNN_OK;
@@ -886,6 +948,29 @@ sbnn_status conv1x1_tc(const sbnn_packed* p, const float* x, float* y, long long
     if (p->Cin % 4 || p->Cout % 4 || !tc_profits(p, M, CALL_1X1_NHWC, &ch)) return SBNN_OK;
     const TcCall c{x, 0, y, p->Cout, M, 0, 0, 0, relu, st};
     return dispatch_tc<SRC_NHWC, false>(p, c, ch, done);
+}
+
+// bf16 mode, dense over the masked weights.  (Activations rounded to bf16 by a pass of their own and multiplied from shared
+// memory took 154 us for 1024 -> 1024 on 256 x 14 x 14, 40 of them for that pass.)
+sbnn_status conv1x1_tc_bf16(const sbnn_packed* p, const float* x, float* y, long long M, int relu, cudaStream_t st, bool* done) {
+    *done = false;
+    if (p->Cin % 4 || p->Cout % 4) return SBNN_OK;
+    if (prepare_only()) {   // the tile width depends on the pixels: for calls with fewer, too
+        uint4* wts = nullptr;
+        for (int nuc : {64, 128}) {
+            const sbnn_status r = get_tc_weights(p, nuc, 1, st, &wts);
+            if (r != SBNN_OK) return r;
+        }
+    }
+    TcChoice ch;
+    tc_profits(p, M, CALL_BF16, &ch);
+    const TcCall c{x, 0, y, p->Cout, M, 0, 0, 0, relu, st};
+    if (ch.split > 1) return launch_tc<TC<64, SRC_NHWC, false, true, 1>>(p, c, ch.split, done);
+    switch (ch.bn) {
+        case 256: return launch_tc<TC<256, SRC_NHWC, false, false, 1>>(p, c, 1, done);
+        case 128: return launch_tc<TC<128, SRC_NHWC, false, false, 1>>(p, c, 1, done);
+        default: return launch_tc<TC<64, SRC_NHWC, false, false, 1>>(p, c, 1, done);
+    }
 }
 
 sbnn_status conv1x1_tc_cm(const sbnn_packed* p, const float* x, int ldx, float* y, int ldy, long long M, int relu, bool out_cm, cudaStream_t st,
