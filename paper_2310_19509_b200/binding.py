@@ -91,24 +91,39 @@ def status_str(code: int) -> str:
 
 
 def _check(code):
-    if code != 0:
+    if code:
         L = lib()
         raise SbnnError(code, L.sbnn_status_str(code).decode(), L.sbnn_last_error().decode())
 
 
 def _ptr(t):
     """Device pointer of a torch tensor (or a raw int / None)."""
-    if t is None:
-        return None
-    if isinstance(t, int):
+    try:
+        return t.data_ptr()
+    except AttributeError:
         return t
-    return t.data_ptr()
+
+
+_current_stream = None
+
+
+def _find_current_stream():
+    """torch's current stream as an int.  The Stream object of the public call costs 3 us, as much as a launch, so later calls
+    ask for the raw handle where this version of torch has that."""
+    global _current_stream
+    import torch
+    handle = torch.cuda.current_stream().cuda_stream            # initialises CUDA
+    raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+    if raw and device:
+        _current_stream = lambda: raw(device())
+    else:
+        _current_stream = lambda: torch.cuda.current_stream().cuda_stream
+    return handle
 
 
 def _stream(stream):
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream() if _current_stream else _find_current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream

@@ -30,9 +30,9 @@ struct PrepareScope {
     ~PrepareScope();
 };
 
-// True while the calling thread is inside the MobileNet chain's forward pass: kernels are then launched with
-// programmatic stream serialization, i.e. a kernel may become resident and run its set-up while its predecessor in
-// the stream drains.  Every kernel launched this way executes grid_dependency_wait() (pipeline.cuh) before it reads or
+// True while the calling thread is inside the MobileNet chain's forward pass, or launches a kernel that before its wait
+// reads nothing but arrays the library owns: kernels are then launched with programmatic stream serialization, i.e. a
+// kernel may become resident and run its set-up while its predecessor in the stream drains.  Every kernel launched this way executes grid_dependency_wait() (pipeline.cuh) before it reads or
 // writes anything another kernel of the stream touches.
 bool chained_launch();
 struct ChainedLaunchScope {

@@ -888,6 +888,7 @@ sbnn_status launch_cm(const sbnn_packed* p, const Stream1x1& s, const float* x, 
     CUtensorMap xmap;
     r = encode_x_map(x, ldx, M, p->Cin, C::TM, C::KC, &xmap);
     if (r != SBNN_OK) return r;
+    ChainedLaunchScope early;   // before its waits the kernel reads the layer's own arrays only
     if (out_cm)
         SBNN_CUDA_TRY(launch_kernel(conv1x1_cm_kernel<C, true>, grid, C::NT, C::SMEM, st, xmap, y, ldy, p->d_bias, s.rec, s.blk_ptr, M,
                                     p->Cin, p->Cout, p->ngroups, s.nchunks, s.ntiles, total_tiles, relu, status));

@@ -26,6 +26,7 @@
 #include <algorithm>
 
 #include "common.h"
+#include "pipeline.cuh"
 
 namespace sbnn {
 namespace {
@@ -146,8 +147,10 @@ conv1x1_gs_kernel(const float* __restrict__ X, float* __restrict__ Y, const floa
         cp_async_commit();
     };
 
-    issue_x_loads(0);
     issue_w_loads(0, ws0);
+    grid_dependency_wait();       // X may come from the previous kernel of the stream, and Y may still be read by it
+    grid_dependency_release();
+    issue_x_loads(0);
     store_x(xs0);
     cp_async_wait_all();
     __syncthreads();
@@ -319,26 +322,17 @@ sbnn_status get_stream(const sbnn_packed* p, const TileCfg& c, Stream1x1* out) {
 
 template <class C>
 sbnn_status launch(const sbnn_packed* p, const Stream1x1& s, const float* x, float* y, int M, int relu, cudaStream_t st) {
-    static std::mutex mu;
-    static std::map<int, bool> configured;  // per device
-    {
-        std::lock_guard<std::mutex> lk(mu);
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (!configured[dev]) {
-            SBNN_CUDA_TRY(cudaFuncSetAttribute(conv1x1_gs_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM));
-            configured[dev] = true;
-        }
-    }
+    sbnn_status r = set_max_dyn_smem(reinterpret_cast<const void*>(&conv1x1_gs_kernel<C>), (int)C::SMEM);
+    if (r != SBNN_OK) return r;
     if (s.max_blk > C::WS_U4)
         return fail(SBNN_ERR_UNSUPPORTED, "internal: weight block %d exceeds buffer %d", s.max_blk, C::WS_U4);
     const long long nblk = (long long)((M + C::TM - 1) / C::TM) * s.ntiles;
     if (nblk > 0x7fffffffLL) return fail(SBNN_ERR_SHAPE, "too many tiles");
     if (prepare_only()) return SBNN_OK;
     dim3 grid((unsigned)nblk);
-    conv1x1_gs_kernel<C><<<grid, C::NT, C::SMEM, st>>>(x, y, p->d_bias, s.rec, s.blk_ptr, M, p->Cin, p->Cout,
-                                                       p->ngroups, s.nchunks, s.ntiles, relu);
-    SBNN_CUDA_TRY(cudaGetLastError());
+    ChainedLaunchScope early;   // before the wait the kernel reads the layer's own arrays only
+    SBNN_CUDA_TRY(launch_kernel(conv1x1_gs_kernel<C>, grid, C::NT, C::SMEM, st, x, y, p->d_bias, s.rec, s.blk_ptr, M, p->Cin, p->Cout,
+                                p->ngroups, s.nchunks, s.ntiles, relu));
     return SBNN_OK;
 }
 

@@ -140,6 +140,7 @@ template <int G, int KS, int PX>
 sbnn_status launch_small_ks(const sbnn_packed* p, const float* x, int ldx, float* y, int ldy, int M, int relu, bool out_cm,
                             cudaStream_t st) {
     dim3 grid((unsigned)((M + 32 * PX - 1) / (32 * PX)), (unsigned)p->ngroups);
+    ChainedLaunchScope early;   // before its wait the kernel reads the layer's own arrays only
     if (out_cm)
         SBNN_CUDA_TRY(launch_kernel(conv1x1_small_kernel<G, KS, true, PX>, grid, 32 * KS, 0, st, x, ldx, y, ldy, p->d_group_ptr, p->d_idx, p->d_val, p->d_bias, M, relu));
     else

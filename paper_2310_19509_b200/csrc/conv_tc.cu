@@ -924,6 +924,7 @@ sbnn_status launch_tc(const sbnn_packed* p, const TcCall& c, int split, bool* do
     a.sb = a.resident ? a.steps * T::NU : T::SB;
     a.sa = std::min(T::SA_MAX, (T::ROOM - a.sb * T::B_BYTES) / T::A_BYTES);
     const size_t smem = (size_t)a.sb * T::B_BYTES + (size_t)a.sa * T::A_BYTES + T::OUT_BYTES + T::CTRL + 1024;
+    ChainedLaunchScope early;   // before their waits the kernel's warps read the layer's own arrays only
     SBNN_CUDA_TRY(launch_kernel_cluster(conv_tc_kernel<T>, dim3(grid), dim3(T::NT), smem, c.st, (unsigned)a.split, amap, ymap, a));
     return SBNN_OK;
 }
