@@ -95,10 +95,10 @@ dwconv3x3_cm_vec_kernel(const float* __restrict__ w, const float* __restrict__ b
 template <int RR>
 __global__ void __launch_bounds__(128)
 dwconv3x3_cm_rows_kernel(const float* __restrict__ w, const float* __restrict__ b, const float* __restrict__ x, int ldx,
-                         float* __restrict__ y, int ldy, int items, int H, int W, int relu) {
-    const int c = blockIdx.y, C = gridDim.y;
+                         float* __restrict__ y, int ldy, int items, int C, int H, int W, int relu) {
+    const int c = blockIdx.x % C;
     const int spr = W >> 2;                                        // strips per row
-    const int t0 = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    const int t0 = (int)((gridDim.x - 1 - blockIdx.x) / C * blockDim.x + threadIdx.x), lane = threadIdx.x & 31;
     const bool live = t0 < items;
     const int t = live ? t0 : items - 1;
     const int strip = t % spr, f0 = (t / spr) * RR;                // first output row (batch-wide row number)
@@ -161,10 +161,10 @@ dwconv3x3_cm_rows_kernel(const float* __restrict__ w, const float* __restrict__ 
 template <int RR>
 __global__ void __launch_bounds__(128)
 dwconv3x3_cm_rows_s2_kernel(const float* __restrict__ w, const float* __restrict__ b, const float* __restrict__ x, int ldx,
-                            float* __restrict__ y, int ldy, int items, int Ho, int W, int relu) {
-    const int c = blockIdx.y, C = gridDim.y;
+                            float* __restrict__ y, int ldy, int items, int C, int Ho, int W, int relu) {
+    const int c = blockIdx.x % C;
     const int Wo = W >> 1, spr = Wo >> 2;
-    const int t0 = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    const int t0 = (int)((gridDim.x - 1 - blockIdx.x) / C * blockDim.x + threadIdx.x), lane = threadIdx.x & 31;
     const bool live = t0 < items;
     const int t = live ? t0 : items - 1;
     const int strip = t % spr, f0 = (t / spr) * RR;                // first output row (batch-wide row number)
@@ -698,13 +698,14 @@ sbnn_status launch_dwconv3x3_cm(const float* w, const float* b, const float* x, 
         dim3 grid((unsigned)((threads + 255) / 256), C);
         constexpr int RR = 4;
         const long long items = NHo / RR * (W / 4);
-        if (stride == 1 && H % RR == 0 && items > 0 && items < 0x7fffffffLL / 2) {
-            dim3 gr((unsigned)((items + 127) / 128), C);
-            SBNN_CUDA_TRY(launch_kernel(dwconv3x3_cm_rows_kernel<RR>, gr, 128, 0, st, w, b, x, ldx, y, ldy, (int)items, H, W, relu));
-        } else if (stride == 2 && Ho % 2 == 0 && NHo / 2 * (Wo / 4) > 0 && NHo / 2 * (Wo / 4) < 0x7fffffffLL / 2) {
+        if (stride == 1 && H % RR == 0 && items > 0 && items < 0x7fffffffLL / 2 && (items + 127) / 128 * C < 0x7fffffffLL) {
+            dim3 gr((unsigned)((items + 127) / 128 * C));
+            SBNN_CUDA_TRY(launch_kernel(dwconv3x3_cm_rows_kernel<RR>, gr, 128, 0, st, w, b, x, ldx, y, ldy, (int)items, C, H, W, relu));
+        } else if (stride == 2 && Ho % 2 == 0 && NHo / 2 * (Wo / 4) > 0 && NHo / 2 * (Wo / 4) < 0x7fffffffLL / 2 &&
+                   (NHo / 2 * (Wo / 4) + 127) / 128 * C < 0x7fffffffLL) {
             const long long items2 = NHo / 2 * (Wo / 4);
-            dim3 gr((unsigned)((items2 + 127) / 128), C);
-            SBNN_CUDA_TRY(launch_kernel(dwconv3x3_cm_rows_s2_kernel<2>, gr, 128, 0, st, w, b, x, ldx, y, ldy, (int)items2, Ho, W, relu));
+            dim3 gr((unsigned)((items2 + 127) / 128 * C));
+            SBNN_CUDA_TRY(launch_kernel(dwconv3x3_cm_rows_s2_kernel<2>, gr, 128, 0, st, w, b, x, ldx, y, ldy, (int)items2, C, Ho, W, relu));
         } else if (stride == 1) {
             SBNN_CUDA_TRY(launch_kernel(dwconv3x3_cm_vec_kernel<1>, grid, 256, 0, st, w, b, x, ldx, y, ldy, NHo, H, W, Ho, Wo, relu));
         } else {

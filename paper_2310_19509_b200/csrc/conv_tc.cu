@@ -334,6 +334,11 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, wg = warp >> 2;
+    grid_dependency_release();
+    if (warp == 16 && lane == 0) {
+        prefetch_map(&amap);
+        prefetch_map(&ymap);
+    }
     if (tid == 0) {
         for (int s = 0; s < SA; ++s) { mbar_init(xfull + s, 1); mbar_init(xempty + s, 8); }
         for (int s = 0; s < SB; ++s) { mbar_init(bfull + s, 1); mbar_init(bfull + SB + s, 1); mbar_init(bempty + s, 1); }
@@ -574,7 +579,6 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
         int step = 0, copies = 0;                           // copies issued: the two tiles alternate between them
         bool ok = true;
         grid_dependency_wait();                             // Y may still be read by the previous kernel of the stream
-        grid_dependency_release();
         for (Tiles t(a); t.left() && ok; t.next()) {
             const int m0 = t.m * T::BM, n0 = t.n * BN + wg * T::COLS;
             uint64_t acc[T::COLS / 2];                      // pairs of neighbouring channels, from the bias on

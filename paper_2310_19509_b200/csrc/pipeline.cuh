@@ -107,6 +107,11 @@ __device__ __forceinline__ void tensor_g2s_3d(void* dst_smem, const void* tensor
                  : "memory");
 }
 
+// Brings a tensor map (a kernel parameter) into the cache that the copies read it from.
+__device__ __forceinline__ void prefetch_map(const void* tensor_map) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(tensor_map) : "memory");
+}
+
 // ---- tiled copy shared -> global through a 2-D tensor map, tracked by the issuing thread's bulk groups ----
 // Stores the [box rows][box width] block at src_smem (laid out as the map's swizzle mode says, 128-byte aligned, 1024
 // with the 128-byte swizzle) to the box whose first element is (x, y); the part of the box outside the tensor is not
