@@ -48,12 +48,12 @@ dwconv3x3_cm_vec_kernel(const float* __restrict__ w, const float* __restrict__ b
     const int strip = (int)(t % spr);
     const long long f = t / spr;
     const int oy = (int)(f % Ho);
+    grid_dependency_wait();      // the activations come from the previous kernel of the stream
+    grid_dependency_release();
     float wk[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) wk[i] = __ldg(w + i * C + c);      // weights are [3][3][C]
     const float bias = b ? __ldg(b + c) : 0.0f;
-    grid_dependency_wait();      // the activations come from the previous kernel of the stream
-    grid_dependency_release();
     float acc[4] = {bias, bias, bias, bias};
     const float* xc = x + (size_t)c * ldx;
     const int ix0 = strip * 4 * S;                                 // first input column under the strip
@@ -103,6 +103,8 @@ dwconv3x3_cm_rows_kernel(const float* __restrict__ w, const float* __restrict__ 
     const int t = live ? t0 : items - 1;
     const int strip = t % spr, f0 = (t / spr) * RR;                // first output row (batch-wide row number)
     const int oy0 = f0 % H;
+    grid_dependency_wait();      // the activations come from the previous kernel of the stream
+    grid_dependency_release();
     float wk[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) wk[i] = __ldg(w + i * C + c);
@@ -112,8 +114,6 @@ dwconv3x3_cm_rows_kernel(const float* __restrict__ w, const float* __restrict__ 
     for (int o = 0; o < RR; ++o)
 #pragma unroll
         for (int i = 0; i < 4; ++i) acc[o][i] = bias;
-    grid_dependency_wait();      // the activations come from the previous kernel of the stream
-    grid_dependency_release();
     const float* xc = x + (size_t)c * ldx + (size_t)f0 * W + strip * 4;
     const bool first = strip == 0, last = strip == spr - 1;
     // all loads first (they are independent), so that a thread has RR + 2 rows in flight
@@ -169,6 +169,8 @@ dwconv3x3_cm_rows_s2_kernel(const float* __restrict__ w, const float* __restrict
     const int t = live ? t0 : items - 1;
     const int strip = t % spr, f0 = (t / spr) * RR;                // first output row (batch-wide row number)
     const int oy0 = f0 % Ho;
+    grid_dependency_wait();      // the activations come from the previous kernel of the stream
+    grid_dependency_release();
     float wk[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) wk[i] = __ldg(w + i * C + c);
@@ -178,8 +180,6 @@ dwconv3x3_cm_rows_s2_kernel(const float* __restrict__ w, const float* __restrict
     for (int o = 0; o < RR; ++o)
 #pragma unroll
         for (int i = 0; i < 4; ++i) acc[o][i] = bias;
-    grid_dependency_wait();      // the activations come from the previous kernel of the stream
-    grid_dependency_release();
     const float* xc = x + (size_t)c * ldx + (size_t)(2 * f0) * W + strip * 8;   // input row 2*f0, first column of the strip
     const bool first = strip == 0;
     float4 A[2 * RR + 1], B[2 * RR + 1];                           // all loads first: 2*RR + 1 rows in flight
@@ -242,6 +242,8 @@ dwconv3x3_cm_px_kernel(const float* __restrict__ w, const float* __restrict__ b,
     const int n0 = (blockIdx.x / QB) * NI;                           // first image of this thread
     if (q >= HoWo || cl >= CPB || c >= C) return;
     const int oy = q / Wo, ox = q - oy * Wo;
+    grid_dependency_wait();      // the activations come from the previous kernel of the stream
+    grid_dependency_release();
     float wk[9];
     bool ok[9];
 #pragma unroll
@@ -253,8 +255,6 @@ dwconv3x3_cm_px_kernel(const float* __restrict__ w, const float* __restrict__ b,
             wk[kh * 3 + kw] = __ldg(w + (kh * 3 + kw) * C + c);
         }
     const float bias = b ? __ldg(b + c) : 0.0f;
-    grid_dependency_wait();      // the activations come from the previous kernel of the stream
-    grid_dependency_release();
     const float* pc = x + (size_t)c * ldx + (size_t)n0 * HW + oy * S * W + ox * S;   // centre tap, first image
     float* yc = y + (size_t)c * ldy + (size_t)n0 * HoWo + q;
 #pragma unroll
@@ -293,12 +293,12 @@ dwconv3x3_cm_col7_kernel(const float* __restrict__ w, const float* __restrict__ 
     const int n0 = (blockIdx.x / QB) * NI;
     if (q >= items || cl >= CPB || c >= C) return;
     const int vs = q / W, ox = q - vs * W, oy0 = vs * 7;
+    grid_dependency_wait();      // the activations come from the previous kernel of the stream
+    grid_dependency_release();
     float wk[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) wk[i] = __ldg(w + i * C + c);
     const float bias = b ? __ldg(b + c) : 0.0f;
-    grid_dependency_wait();      // the activations come from the previous kernel of the stream
-    grid_dependency_release();
     const bool lok = ox > 0, rok = ox + 1 < W, top = oy0 > 0, bot = oy0 + 7 < H;
     const float* pc = x + (size_t)c * ldx + (size_t)n0 * H * W + (oy0 - 1) * W + ox;   // window origin (centre column)
     float* yc = y + (size_t)c * ldy + (size_t)n0 * H * W + oy0 * W + ox;
@@ -346,12 +346,12 @@ dwconv3x3_cm_w14_kernel(const float* __restrict__ w, const float* __restrict__ b
     const bool live = grp < 4 && c0 < C;
     const int c = c0 < C ? c0 : C - 1;
     const int oy0 = vs * 7, n0 = blockIdx.x * NI;
+    grid_dependency_wait();      // the activations come from the previous kernel of the stream
+    grid_dependency_release();
     float wk[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) wk[i] = __ldg(w + i * C + c);
     const float bias = b ? __ldg(b + c) : 0.0f;
-    grid_dependency_wait();      // the activations come from the previous kernel of the stream
-    grid_dependency_release();
     const float* pc = x + (size_t)c * ldx + (size_t)n0 * H * W + (oy0 - 1) * W + 2 * j;   // input row oy0 - 1, own pair
     float* yc = y + (size_t)c * ldy + (size_t)n0 * H * W + oy0 * W + 2 * j;
 #pragma unroll
@@ -407,6 +407,8 @@ dwconv3x3_cm_7x7_kernel(const float* __restrict__ w, const float* __restrict__ b
     const int tid = threadIdx.x, cl = tid >> 6, img = tid & 63;
     const int n0 = blockIdx.x * NI, nimg = min(NI, N - n0), c0 = blockIdx.y * 2;
     const int c = c0 + cl;
+    grid_dependency_wait();      // the activations come from the previous kernel of the stream
+    grid_dependency_release();
     float wk[9];
     float bias = 0.0f;
     if (c < C) {
@@ -414,8 +416,6 @@ dwconv3x3_cm_7x7_kernel(const float* __restrict__ w, const float* __restrict__ b
         for (int i = 0; i < 9; ++i) wk[i] = __ldg(w + i * C + c);
         bias = b ? __ldg(b + c) : 0.0f;
     }
-    grid_dependency_wait();      // the activations come from the previous kernel of the stream
-    grid_dependency_release();
     const int total = nimg * HW;                                    // floats per channel in this CTA
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
@@ -483,13 +483,13 @@ conv3x3_thin_cm32_kernel(const float* __restrict__ w, const float* __restrict__ 
                          float* __restrict__ y, int ldy, int N, int H, int W, int Cin, int Cout, int Ho, int Wo, int relu) {
     extern __shared__ __align__(16) float ws[];   // [9][Cin][32] of this CTA's channel group
     const int cg = blockIdx.y;
+    grid_dependency_wait();      // a caller's kernel in front of the network may write the image, and these weights
+    grid_dependency_release();
     for (int i = threadIdx.x; i < 9 * Cin * 32; i += blockDim.x) {
         const int o = i & 31, tc = i >> 5;
         ws[i] = w[(size_t)(cg * 32 + o) * 9 * Cin + tc];
     }
     __syncthreads();
-    grid_dependency_wait();      // the activations come from the previous kernel of the stream
-    grid_dependency_release();
     constexpr int TW = 2, IW = S * (TW - 1) + 3;
     const int strips = (Wo + TW - 1) / TW;
     const long long total = (long long)N * Ho * strips;
@@ -568,13 +568,13 @@ conv3x3_first_s2c3_kernel(const float* __restrict__ w, const float* __restrict__
     constexpr int Cin = 3;
     extern __shared__ __align__(16) float ws[];   // [9][3][32] of this CTA's channel group
     const int cg = blockIdx.y;
+    grid_dependency_wait();      // a caller's kernel in front of the network may write the image, and these weights
+    grid_dependency_release();
     for (int i = threadIdx.x; i < 9 * Cin * 32; i += blockDim.x) {
         const int o = i & 31, tc = i >> 5;
         ws[i] = w[(size_t)(cg * 32 + o) * 9 * Cin + tc];
     }
     __syncthreads();
-    grid_dependency_wait();      // the activations come from the previous kernel of the stream
-    grid_dependency_release();
     const int strips = Wo >> 1;
     const long long total = (long long)N * Ho * strips;
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;

@@ -410,7 +410,7 @@ conv1x1_cm_kernel(const __grid_constant__ CUtensorMap xmap, float* __restrict__ 
                     // (pixels past M and channels past Cin arrive as zeros and count towards the bytes).  The
                     // weights do not depend on the previous kernel of the stream, the activations do: the very
                     // first box is requested only once that kernel has finished.
-                    const int wbeg = bp[k], wn = bp[k + 1] - wbeg;
+                    const int wbeg = ld_early(bp + k), wn = ld_early(bp + k + 1) - wbeg;
                     mbar_arrive_expect_tx(full + s, (uint32_t)C::XS_BYTES + (uint32_t)wn * 16u);
                     bulk_g2s(ws0 + (size_t)s * C::WS_BYTES, rec + wbeg, (uint32_t)wn * 16u, full + s);
                     if (issued == 0) grid_dependency_wait();
@@ -469,7 +469,7 @@ dwpw_fused_kernel(const __grid_constant__ CUtensorMap rawmap, float* __restrict_
     float* dwsm = reinterpret_cast<float*>(raw_empty + RS) + 4;      // depthwise weights [9][Cin], then the bias [Cin]
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int i = tid; i < 10 * Cin; i += blockDim.x) dwsm[i] = i < 9 * Cin ? __ldg(dw_w + i) : (dw_b ? __ldg(dw_b + i - 9 * Cin) : 0.0f);
+    for (int i = tid; i < 10 * Cin; i += blockDim.x) dwsm[i] = i < 9 * Cin ? ld_early(dw_w + i) : (dw_b ? ld_early(dw_b + i - 9 * Cin) : 0.0f);
     if (tid == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(x_full + s, 1 + NDW);
@@ -733,6 +733,7 @@ sbnn_status build_stream_cm(const sbnn_packed* p, const TileCfg& c, Stream1x1* o
     cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&s.blk_ptr), blk.size() * 4);
     if (e == cudaSuccess && !rec.empty()) e = cudaMemcpy(s.rec, rec.data(), rec.size() * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(s.blk_ptr, blk.data(), blk.size() * 4, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);   // arrived, for every stream
     if (e != cudaSuccess) {
         cudaFree(s.rec);
         cudaFree(s.blk_ptr);

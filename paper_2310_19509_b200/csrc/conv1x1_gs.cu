@@ -109,7 +109,7 @@ conv1x1_gs_kernel(const float* __restrict__ X, float* __restrict__ Y, const floa
         const int g = tile * C::GT + warp * GPW + q;
 #pragma unroll
         for (int r = 0; r < G; ++r) {
-            const float b = (g < ngroups) ? bias[g * G + r] : 0.0f;
+            const float b = (g < ngroups) ? ld_early(bias + g * G + r) : 0.0f;
 #pragma unroll
             for (int p = 0; p < P / 2; ++p) acc[q][p][r] = pack2(b, b);
         }
@@ -142,7 +142,7 @@ conv1x1_gs_kernel(const float* __restrict__ X, float* __restrict__ Y, const floa
         }
     };
     auto issue_w_loads = [&](int k, uint4* ws) {
-        const int beg = bp[k], n = bp[k + 1] - beg;
+        const int beg = ld_early(bp + k), n = ld_early(bp + k + 1) - beg;
         for (int i = tid; i < n; i += C::NT) cp_async16(ws + i, rec + beg + i);
         cp_async_commit();
     };
@@ -299,6 +299,7 @@ sbnn_status build_stream(const sbnn_packed* p, const TileCfg& c, Stream1x1* out)
     }
     if (!rec.empty()) e = cudaMemcpy(s.rec, rec.data(), rec.size() * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(s.blk_ptr, blk.data(), blk.size() * 4, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);   // arrived, for every stream
     if (e != cudaSuccess) {
         cudaFree(s.rec);
         cudaFree(s.blk_ptr);

@@ -27,19 +27,19 @@ template <int G>
 __device__ __forceinline__ void fetch_unit(const int32_t* __restrict__ idx, const float* __restrict__ val, int u, int uend,
                                            UnitRegs<G>& r) {
     const bool ok = u < uend;
-    r.c = ok ? __ldg(idx + u) : 0;
+    r.c = ok ? ld_early(idx + u) : 0;
     const float* p = val + (size_t)(ok ? u : 0) * G;
     if constexpr (G % 4 == 0) {
 #pragma unroll
         for (int q = 0; q < G / 4; ++q) {
-            const float4 t = __ldg(reinterpret_cast<const float4*>(p) + q);
+            const float4 t = ld_early(reinterpret_cast<const float4*>(p) + q);
             r.w[4 * q] = t.x; r.w[4 * q + 1] = t.y; r.w[4 * q + 2] = t.z; r.w[4 * q + 3] = t.w;
         }
     } else if constexpr (G == 2) {
-        const float2 t = __ldg(reinterpret_cast<const float2*>(p));
+        const float2 t = ld_early(reinterpret_cast<const float2*>(p));
         r.w[0] = t.x; r.w[1] = t.y;
     } else {
-        r.w[0] = __ldg(p);
+        r.w[0] = ld_early(p);
     }
     if (!ok) {
 #pragma unroll
@@ -64,7 +64,7 @@ conv1x1_small_kernel(const float* __restrict__ X, int ldx, float* __restrict__ Y
         m[j] = (blockIdx.x * PX + j) * 32 + lane;
         xp[j] = X + (m[j] < M ? m[j] : M - 1);                     // lanes past the end read a valid pixel, store nothing
     }
-    const int beg = group_ptr[g], n = group_ptr[g + 1] - beg;
+    const int beg = ld_early(group_ptr + g), n = ld_early(group_ptr + g + 1) - beg;
     const int per = (n + KSPLIT - 1) / KSPLIT;
     const int u0 = beg + min(n, kq * per), uend = beg + min(n, (kq + 1) * per);
     float acc[PX][G];

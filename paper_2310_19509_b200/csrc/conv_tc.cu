@@ -746,15 +746,21 @@ struct TcCall {
 };
 
 // ---- which kernel, and how ------------------------------------------------------------------------
-// Cycles a launch takes with tiles of bn output channels: rounds of tiles x (steps + fill and store).  A step takes 14 cycles
-// a channel (24 MMAs at 70-75 cycles for 128 channels), 64 channels no less than it takes to split its activations.
-// One image (bf16 mode): the copies from L2 take longest, 32 KB of activations and 128 bytes a channel.
-double tc_step(int bn, int images) { return images == 1 ? 380.0 + 1.5 * bn : (bn == 64 ? 1600.0 : 14.0 * bn); }
+// Cycles a launch takes with tiles of bn output channels: rounds of tiles x (steps + fill and store).  A step of 128 or 256
+// channels takes about as long as its MMAs (64 cycles for 128 channels, 24 of them), 64 channels as long as the split of the
+// activations; one image (bf16 mode) as long as the copies and the barriers around them.  Fitted to launches of 1 to 72
+// steps on 1 to 112 CTAs (4.1 us for one step of 64 channels, 0.62 / 0.84 / 1.67 us for each further one of 64 / 128 / 256).
+double tc_step(int bn, int images) {
+    if (images == 1) return bn == 64 ? 600.0 : (bn == 128 ? 700.0 : 1150.0);
+    return bn == 64 ? 1150.0 : 12.5 * bn;
+}
 double tc_cost(const sbnn_packed* p, long long M, int bn, int images) {
     const long long tiles = (M + 127) / 128 * ((p->Cout + bn - 1) / bn), sms = device_sms();
     const double steps = 0.5 * (double)((p->Cin + 31) / 32) * p->KH * p->KW;
-    return (double)((tiles + sms - 1) / sms) * (steps * tc_step(bn, images) + (bn == 64 ? 1300.0 : 1000.0 + 12.0 * bn)) + 6300.0;
+    return (double)((tiles + sms - 1) / sms) * (steps * tc_step(bn, images) + (bn == 64 ? 1300.0 : 1000.0 + 12.0 * bn)) + 4700.0;
 }
+// Microseconds: long launches run at the clock that the power limit leaves them.
+double tc_us(double cycles) { return cycles / (cycles < 1e5 ? 1800.0 : 1600.0); }
 
 // Clusters of `split` CTAs that the device runs at the same time (on 148 SMs 74 of 2, 33 of 4, 15 of 8).
 long long cluster_capacity(int split) {
@@ -791,7 +797,7 @@ long long cluster_capacity(int split) {
 double tc_split_cost(const sbnn_packed* p, long long M, int split, int run, int images) {
     const long long tiles = (M + 127) / 128 * ((p->Cout + 63) / 64), runs = (long long)((p->Cin + 63) / 64) * p->KH * p->KW / run;
     if (runs < split || tiles * split > device_sms() || tiles > cluster_capacity(split)) return 1e30;
-    return (double)((runs + split - 1) / split * run) * tc_step(64, images) + 11400.0;
+    return (double)((runs + split - 1) / split * run) * (tc_step(64, images) + 50.0) + 9800.0;
 }
 
 using TcChoice = sbnn_packed::TcChoice;
@@ -828,15 +834,15 @@ TcChoice decide(const sbnn_packed* p, long long M, Call call) {
     if (call == CALL_3X3 || call == CALL_3X3_CM) {
         fma = 25.0 + kept * (p->G >= 8 ? 0.050 : 0.075);
     } else if (call == CALL_1X1_CM && conv1x1_few_tiles(p, M)) {
-        fma = 2.7 + kept * (p->G >= 8 ? 0.18 : 0.22);
+        fma = 2.7 + kept * std::max(1.0, 32.0 / M) * (p->G >= 8 ? 0.18 : 0.22);   // (a lane takes a pixel)
     } else if (call == CALL_1X1_CM || (p->Cin >= 128 && M >= 2048)) {
-        fma = 5.0 + 0.034 * kept + 0.0026 * dense + 0.5 * mem;
+        fma = 5.0 + 0.034 * kept + 0.0021 * dense + 0.6 * mem;
         if (call == CALL_1X1_NHWC) fma += 2.0 + 8.0 * M * p->Cin / 4.5e6;    // the conversion to channel-major
     } else {
         fma = 2.0 + (p->Cin >= 128 ? 2.0 : 0.0) + 0.012 * p->Cin + 0.1 * kept;
     }
     choice = tc_choose(p, M, call == CALL_3X3_CM ? 3 : 1, 3);
-    if (std::max(choice.cost / 1750.0, mem) >= fma) choice.bn = 0;
+    if (std::max(tc_us(choice.cost), mem) >= 0.95 * fma) choice.bn = 0;
     return choice;
 }
 bool tc_profits(const sbnn_packed* p, long long M, Call call, TcChoice* choice = nullptr) {

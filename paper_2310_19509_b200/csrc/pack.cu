@@ -181,6 +181,11 @@ sbnn_status finish_packed(sbnn_packed* p, sbnn_packed** out) {
         return st;
     }
     st = (p->KH == 1) ? prepare_default_1x1(p) : prepare_default_3x3(p);
+    // (a copy from pageable memory may return before it has arrived; streams that do not wait for the legacy one read it, too)
+    if (st == SBNN_OK && cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {
+        cudaGetLastError();
+        st = fail(SBNN_ERR_CUDA, "uploading the packed layer failed");
+    }
     if (st != SBNN_OK) {
         sbnn_packed_free(p);
         return st;

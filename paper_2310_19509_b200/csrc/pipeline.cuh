@@ -32,6 +32,10 @@ __device__ __forceinline__ void fma2(f32x2& d, f32x2 a, f32x2 b) {
 // touch memory no other kernel of the stream writes (weights, its own shared memory).  grid_dependency_release lets
 // the next kernel of the stream become resident as SM resources free up; that kernel still waits, in its own
 // grid_dependency_wait, for this one to finish.
+// Loads before grid_dependency_wait go past the L1 (ld_early): what an SM's L1 holds at that point may be from another
+// allocation that had the same addresses, and need not be dropped before the wait.
+template <class T>
+__device__ __forceinline__ T ld_early(const T* p) { return __ldcg(p); }
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependency_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
