@@ -397,7 +397,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                     for (int h = 0; h < subs(k); ++h, ring.next()) {
                         const int s = ring.stage;
                         if (ring.reused() && !(ok = wait(xempty + s, ring.parity ^ 1))) break;
-                        if (lane == 0) {
+                        if (elect_one()) {
                             unsigned char* dst = ast + (size_t)s * T::A_BYTES;
                             const int c0 = c * 64 + h * T::SUB;
                             mbar_arrive_expect_tx(xfull + s, T::A_BYTES);
@@ -421,7 +421,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                     for (int u = 0; u < NU; ++u, ring.next()) {
                         const int s = ring.stage;
                         if (ring.reused() && !(ok = wait(bempty + s, ring.parity ^ 1))) break;
-                        if (lane == 0) {
+                        if (elect_one()) {
                             mbar_arrive_expect_tx(bfull + ring.turn(), T::B_BYTES);
                             bulk_g2s(bst + (size_t)s * T::B_BYTES, a.wts + ((size_t)(nt + u) * a.steps + k) * (T::B_BYTES / 16), T::B_BYTES, bfull + ring.turn());
                         }
@@ -639,7 +639,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                             if (m < a.M && n0 + c0 + i < a.Cout) a.y[(size_t)(n0 + c0 + i) * a.ldy + m] = o[i];
                     } else {
                         unsigned char* tile = stage + (copies++ & 1) * 2048;
-                        if (lane == 0) bulk_wait_read_pending1();   // the copy that last read this tile is done with it
+                        if (elect_one()) bulk_wait_read_pending1();   // the copy that last read this tile is done with it
                         __syncwarp();
                         if (T::OUT_CM) {
 #pragma unroll
@@ -652,7 +652,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                         }
                         fence_async_smem();
                         __syncwarp();
-                        if (lane == 0) {
+                        if (elect_one()) {                  // (always the same lane)
                             tensor_s2g_2d(&ymap, T::OUT_CM ? mw : n0 + c0, T::OUT_CM ? n0 + c0 : mw, tile);
                             bulk_commit_group();
                         }
@@ -660,12 +660,12 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                 }
             }
             if (__any_sync(0xffffffffu, redo)) {
-                if (lane == 0) bulk_wait_all();
+                if (elect_one()) bulk_wait_all();
                 __syncwarp();
                 if (redo) exact_pixel<T>(a, m, n0, min(n0 + T::COLS, a.Cout));
             }
         }
-        if (lane == 0) bulk_wait_all();                     // this thread's copies are complete before the CTA gives up its shared memory
+        if (elect_one()) bulk_wait_all();                   // this thread's copies are complete before the CTA gives up its shared memory
     }
     // common exit: nobody may still be using the tensor memory when it is released
     tc_fence_before_sync();
