@@ -357,9 +357,9 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
 
     // Whole warp: until the barrier that each lane names has completed its phase; the same result in all lanes.  (A wait
     // costs 60 to 100 cycles even when there is nothing to wait for, so a warp looks at all it needs at once, a barrier a lane.)
-    auto wait = [&](uint64_t* bar, uint32_t parity) {
+    auto wait = [&](uint64_t* bar, uint32_t parity, bool needed = true) {
         uint32_t polls = 0;
-        while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) {
+        while (!__all_sync(0xffffffffu, (int)mbar_try_wait(bar, parity) | (int)!needed)) {
             if (++polls > 64) {
                 if (__any_sync(0xffffffffu, polls > kWaitLimit || *abort_flag)) {
                     *abort_flag = 1;
@@ -393,20 +393,29 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                 int px = 0, py = 0, pn = 0;
                 if (T::SRC == SRC_IM2COL) { px = m0 % a.W; py = (m0 / a.W) % a.H; pn = m0 / (a.W * a.H); }
                 for (int k = kb; k < ke && ok; k += T::RUN) {
-                    const int c = k / T::TAPS, tap = k - c * T::TAPS;
-                    for (int h = 0; h < subs(k); ++h, ring.next()) {
-                        const int s = ring.stage;
-                        if (ring.reused() && !(ok = wait(xempty + s, ring.parity ^ 1))) break;
+                    const int c = k / T::TAPS, tap = k - c * T::TAPS, halves = subs(k);
+                    // With stages enough both halves of a step are asked for after one wait: a wait and an issue take a warp
+                    // 370 cycles, which for 16 KB at a time is slower than the memory.
+                    const int batch = SA >= 4 ? halves : 1;
+                    for (int h = 0; h < halves && ok; h += batch) {
+                        Ring second = ring;
+                        second.next();
+                        const Ring& mine = lane == 1 && batch == 2 ? second : ring;   // lane 1 looks at the second stage
+                        if (second.reused() && !(ok = wait(xempty + mine.stage, mine.parity ^ 1, mine.reused()))) break;
                         if (elect_one()) {
-                            unsigned char* dst = ast + (size_t)s * T::A_BYTES;
-                            const int c0 = c * 64 + h * T::SUB;
-                            mbar_arrive_expect_tx(xfull + s, T::A_BYTES);
-                            if (T::SRC == SRC_CM) tensor_g2s_2d(dst, &amap, m0, c0, xfull + s);
-                            else if (T::SRC == SRC_CM3) tensor_g2s_2d(dst, &amap, (m0 + (tap / 3 - 1) * a.W - 1) & ~3, c0, xfull + s);
-                            else if (T::SRC == SRC_NHWC) tensor_g2s_2d(dst, &amap, c0, m0, xfull + s);
-                            else im2col_g2s(dst, &amap, c0, px - 1, py - 1, pn, tap % 3, tap / 3, xfull + s);
+                            for (int b = 0; b < batch; ++b) {
+                                const int s = b ? second.stage : ring.stage, c0 = c * 64 + (h + b) * T::SUB;
+                                unsigned char* dst = ast + (size_t)s * T::A_BYTES;
+                                mbar_arrive_expect_tx(xfull + s, T::A_BYTES);
+                                if (T::SRC == SRC_CM) tensor_g2s_2d(dst, &amap, m0, c0, xfull + s);
+                                else if (T::SRC == SRC_CM3) tensor_g2s_2d(dst, &amap, (m0 + (tap / 3 - 1) * a.W - 1) & ~3, c0, xfull + s);
+                                else if (T::SRC == SRC_NHWC) tensor_g2s_2d(dst, &amap, c0, m0, xfull + s);
+                                else im2col_g2s(dst, &amap, c0, px - 1, py - 1, pn, tap % 3, tap / 3, xfull + s);
+                            }
                         }
                         __syncwarp();
+                        ring.next();
+                        if (batch == 2) ring.next();
                     }
                 }
             }
@@ -417,15 +426,24 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
             bool ok = true;
             for (Tiles t(a); t.left() && ok; t.next()) {
                 const int nt = t.n * NU;
+                const int batch = SB >= 4 ? NU : 1;         // as above
                 for (int k = kb; k < ke && ok; ++k)
-                    for (int u = 0; u < NU; ++u, ring.next()) {
-                        const int s = ring.stage;
-                        if (ring.reused() && !(ok = wait(bempty + s, ring.parity ^ 1))) break;
+                    for (int u = 0; u < NU && ok; u += batch) {
+                        Ring second = ring;
+                        second.next();
+                        const Ring& mine = lane == 1 && batch == 2 ? second : ring;
+                        if (second.reused() && !(ok = wait(bempty + mine.stage, mine.parity ^ 1, mine.reused()))) break;
                         if (elect_one()) {
-                            mbar_arrive_expect_tx(bfull + ring.turn(), T::B_BYTES);
-                            bulk_g2s(bst + (size_t)s * T::B_BYTES, a.wts + ((size_t)(nt + u) * a.steps + k) * (T::B_BYTES / 16), T::B_BYTES, bfull + ring.turn());
+                            for (int b = 0; b < batch; ++b) {
+                                const Ring& r = b ? second : ring;
+                                mbar_arrive_expect_tx(bfull + r.turn(), T::B_BYTES);
+                                bulk_g2s(bst + (size_t)r.stage * T::B_BYTES, a.wts + ((size_t)(nt + u + b) * a.steps + k) * (T::B_BYTES / 16), T::B_BYTES,
+                                         bfull + r.turn());
+                            }
                         }
                         __syncwarp();
+                        ring.next();
+                        if (batch == 2) ring.next();
                     }
                 if (a.resident) break;
             }
