@@ -34,6 +34,8 @@ namespace {
 // Device status word: 0, or the sbnn_status of the first bounded wait that gave up.
 __device__ int g_async_status;
 
+constexpr size_t kMaxSmem = 227 * 1024;
+
 template <int G_, int P_, int GPW_, int NW_, int KC_, int STAGES_>
 struct K2 {
     static constexpr int G = G_, P = P_, GPW = GPW_, NW = NW_, KC = KC_, STAGES = STAGES_;
@@ -53,9 +55,9 @@ struct K2 {
     // (one all-zero end quad each).
     static constexpr int WS_U4 = UNION ? HDR + NW * (NQ * QUAD2 + 2 * QUAD) : HDR + GT * NQ * QUAD;
     static constexpr int WS_BYTES = WS_U4 * 16;
-    static constexpr size_t SMEM = (size_t)STAGES * (XS_BYTES + WS_BYTES) + 2 * STAGES * 8 + 16;
+    static constexpr size_t SMEM = (size_t)STAGES * (XS_BYTES + WS_BYTES) + 2 * STAGES * 8 + 16;   // with full lists
     static_assert(P % 4 == 0 && KC % 4 == 0, "tile shape");
-    static_assert(SMEM <= 227 * 1024, "shared memory");
+    static_assert(SMEM <= kMaxSmem, "shared memory");
 };
 
 template <int G>
@@ -228,21 +230,51 @@ __device__ __forceinline__ void run_list_v(uint32_t r, int n, uint32_t xs, f32x2
     }
 }
 
+// The stages of a launch.  Fixed: as many as fit with room for full lists, two of 64 channels.  Else as many as fit
+// with the room that the layer's largest weight block takes: three of 64 channels up to about half the units kept.
+// Two stages are one on its way while the other is used, and a copy of 64 channels takes some 2000 cycles, which short
+// lists do not last (101 x 14 x 14, 1024 -> 512, 90 % pruned: 89.4 -> 67.5 us; 256 x 14 x 14, 1024 -> 1024, G = 4: 317 -> 289).
+// Steps of 32 channels, of which four fit anyway, gain nothing from more (409 and 420 us for the latter), and long lists
+// of pairs of groups lose 5 % without the constants (50 %: 1024 and 1076 us).
+template <class C, bool FIXED>
+struct Stages {
+    int n, weights;                 // stages, and bytes of a stage for the weight block
+    __device__ int count() const { return FIXED ? C::STAGES : n; }
+    __device__ int weight_bytes() const { return FIXED ? C::WS_BYTES : weights; }
+};
+
+// Step of a warp in its ring of stages: the stage and the parity of its use.
+template <class C, bool FIXED>
+struct Step {
+    int k = 0, stage = 0;
+    uint32_t use = 0;
+    __device__ int s() const { return FIXED ? k % C::STAGES : stage; }
+    __device__ uint32_t parity() const { return FIXED ? (k / C::STAGES) & 1 : use & 1; }
+    __device__ bool reused() const { return FIXED ? k >= C::STAGES : use > 0; }
+    __device__ void next(int stages) {
+        ++k;
+        if (!FIXED && ++stage == stages) {
+            stage = 0;
+            ++use;
+        }
+    }
+};
+
 // The compute warps of the pipelined kernels: wait for a stage ("full": activations [KC][TM] at xs0, weight block at
 // ws0), run the warp's lists out of it, release it ("empty"), and write the tile's outputs.  Shared by the plain
 // kernel (stages filled by the copy engine) and the fused depthwise + pointwise kernel (activations written by the
 // CTA's own depthwise warps).
-template <class C, bool OUT_CM>
+template <class C, bool OUT_CM, bool FIXED>
 __device__ __forceinline__ void compute_warps(unsigned char* xs0, unsigned char* ws0, uint64_t* full, uint64_t* empty,
                                               volatile int* abort_flag, float* __restrict__ Y, int ldy,
                                               const float* __restrict__ bias, int M, int ngroups, int nchunks, int ntiles,
-                                              int total_tiles, int relu, int* status) {
-    constexpr int G = C::G, P = C::P, GPW = C::GPW, S = C::STAGES;
+                                              int total_tiles, int relu, int* status, Stages<C, FIXED> stages) {
+    constexpr int G = C::G, P = C::P, GPW = C::GPW;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     grid_dependency_wait();       // Y may still be read by the previous kernel of the stream
     grid_dependency_release();
     const unsigned lane_off = lane * 16;
-    int consumed = 0;
+    Step<C, FIXED> step;
     for (int t = blockIdx.x; t < total_tiles; t += gridDim.x) {
     const int tile = t % ntiles, m0 = (t / ntiles) * C::TM;
     f32x2 acc[GPW][P / 2][G];   // acc[q][p2][r]: pixels (2*p2, 2*p2+1) of the lane, channel r of group q
@@ -263,13 +295,13 @@ __device__ __forceinline__ void compute_warps(unsigned char* xs0, unsigned char*
     }
 
     bool ok = true;
-    for (int k = 0; k < nchunks; ++k, ++consumed) {
-        const int s = consumed % S;
-        ok = mbar_wait(full + s, (consumed / S) & 1, abort_flag, status, SBNN_ERR_TIMEOUT);
+    for (int k = 0; k < nchunks; ++k, step.next(stages.count())) {
+        const int s = step.s();
+        ok = mbar_wait(full + s, step.parity(), abort_flag, status, SBNN_ERR_TIMEOUT);
         if (!ok) break;
         if constexpr (G >= 8) {
             const uint32_t xs = smem_u32(xs0) + (uint32_t)s * C::XS_BYTES + lane_off;
-            const uint32_t ws = smem_u32(ws0) + (uint32_t)s * C::WS_BYTES;
+            const uint32_t ws = smem_u32(ws0) + (uint32_t)(s * stages.weight_bytes());
             const uint32_t hdr = ws + warp * C::NL * 8;             // (start in 16-byte units, kept units) per list
             static_assert(G < 8 || !C::UNION, "the G >= 8 instances have one list per group");
 #pragma unroll
@@ -279,7 +311,7 @@ __device__ __forceinline__ void compute_warps(unsigned char* xs0, unsigned char*
             }
         } else {
             const unsigned char* xs = xs0 + (size_t)s * C::XS_BYTES + lane_off;
-            const uint4* ws = reinterpret_cast<const uint4*>(ws0 + (size_t)s * C::WS_BYTES);
+            const uint4* ws = reinterpret_cast<const uint4*>(ws0 + (size_t)s * stages.weight_bytes());
             const int2* hdr = reinterpret_cast<const int2*>(ws) + warp * C::NL;   // (start, kept units) per list
             if constexpr (C::UNION) {
                 const int2 hb = hdr[0], h0 = hdr[1], h1 = hdr[2];
@@ -363,17 +395,18 @@ __device__ __forceinline__ void compute_warps(unsigned char* xs0, unsigned char*
     }   // tiles
 }
 
-template <class C, bool OUT_CM>
+template <class C, bool OUT_CM, bool FIXED>
 __global__ void __launch_bounds__(C::NT, 1)
 conv1x1_cm_kernel(const __grid_constant__ CUtensorMap xmap, float* __restrict__ Y, int ldy,
                   const float* __restrict__ bias, const uint4* __restrict__ rec,
                   const int32_t* __restrict__ blk_ptr, int M, int Cin, int Cout, int ngroups, int nchunks,
-                  int ntiles, int total_tiles, int relu, int* status) {
-    constexpr int G = C::G, P = C::P, GPW = C::GPW, NW = C::NW, KC = C::KC, S = C::STAGES;
+                  int ntiles, int total_tiles, int relu, int* status, Stages<C, FIXED> stages) {
+    constexpr int NW = C::NW, KC = C::KC;
+    const int S = stages.count(), ws_bytes = stages.weight_bytes();
     extern __shared__ __align__(128) unsigned char smem[];
     unsigned char* xs0 = smem;
     unsigned char* ws0 = smem + (size_t)S * C::XS_BYTES;
-    uint64_t* full = reinterpret_cast<uint64_t*>(ws0 + (size_t)S * C::WS_BYTES);
+    uint64_t* full = reinterpret_cast<uint64_t*>(ws0 + (size_t)S * ws_bytes);
     uint64_t* empty = full + S;
     volatile int* abort_flag = reinterpret_cast<volatile int*>(empty + S);
 
@@ -396,14 +429,14 @@ conv1x1_cm_kernel(const __grid_constant__ CUtensorMap xmap, float* __restrict__ 
 
     if (warp == NW) {
         // ---------------- producer warp ----------------
-        int issued = 0;
+        Step<C, FIXED> step;
         bool ok = true;
         for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x) {
             const int tile = t % ntiles, m0 = (t / ntiles) * C::TM;
             const int32_t* bp = blk_ptr + (size_t)tile * (nchunks + 1);
-            for (int k = 0; k < nchunks; ++k, ++issued) {
-                const int s = issued % S;
-                if (issued >= S) ok = mbar_wait(empty + s, ((issued / S) & 1) ^ 1, abort_flag, status, SBNN_ERR_TIMEOUT);
+            for (int k = 0; k < nchunks; ++k, step.next(S)) {
+                const int s = step.s();
+                if (step.reused()) ok = mbar_wait(empty + s, step.parity() ^ 1, abort_flag, status, SBNN_ERR_TIMEOUT);
                 if (!ok) break;
                 if (lane == 0) {
                     // a linear copy brings the step's weight block, one tiled copy the step's KC x TM box of X
@@ -412,24 +445,26 @@ conv1x1_cm_kernel(const __grid_constant__ CUtensorMap xmap, float* __restrict__ 
                     // first box is requested only once that kernel has finished.
                     const int wbeg = ld_early(bp + k), wn = ld_early(bp + k + 1) - wbeg;
                     mbar_arrive_expect_tx(full + s, (uint32_t)C::XS_BYTES + (uint32_t)wn * 16u);
-                    bulk_g2s(ws0 + (size_t)s * C::WS_BYTES, rec + wbeg, (uint32_t)wn * 16u, full + s);
-                    if (issued == 0) grid_dependency_wait();
+                    bulk_g2s(ws0 + (size_t)s * ws_bytes, rec + wbeg, (uint32_t)wn * 16u, full + s);
+                    if (step.k == 0) grid_dependency_wait();
                     tensor_g2s_2d(xs0 + (size_t)s * C::XS_BYTES, &xmap, m0, k * KC, full + s);
                 }
             }
         }
         if (!ok) {
             // gave up: let the copies already issued land before the CTA's shared memory is released
-            for (int k = max(0, issued - S); k < issued; ++k) {
+            // (every stage has one on its way or landed; those from the step's on were last filled a round ago)
+            for (int s = 0; s < S; ++s) {
                 bool landed = false;
-                for (uint32_t i = 0; i < kWaitLimit && !landed; ++i) landed = mbar_try_wait(full + k % S, (k / S) & 1);
+                for (uint32_t i = 0; i < kWaitLimit && !landed; ++i) landed = mbar_try_wait(full + s, step.parity() ^ (s >= step.s() ? 1 : 0));
             }
         }
         return;
     }
 
     // ---------------- compute warps ----------------
-    compute_warps<C, OUT_CM>(xs0, ws0, full, empty, abort_flag, Y, ldy, bias, M, ngroups, nchunks, ntiles, total_tiles, relu, status);
+    compute_warps<C, OUT_CM, FIXED>(xs0, ws0, full, empty, abort_flag, Y, ldy, bias, M, ngroups, nchunks, ntiles, total_tiles, relu, status,
+                                    stages);
 }
 
 // ---- depthwise 3x3 (stride 1, pad 1) fused into the pointwise kernel -----------------------------------------
@@ -605,7 +640,8 @@ dwpw_fused_kernel(const __grid_constant__ CUtensorMap rawmap, float* __restrict_
     }
 
     // ---------------- compute warps ----------------
-    compute_warps<C, true>(xs0, ws0, x_full, x_empty, abort_flag, Y, ldy, bias, M, ngroups, nchunks, ntiles, total_tiles, relu, status);
+    compute_warps<C, true, true>(xs0, ws0, x_full, x_empty, abort_flag, Y, ldy, bias, M, ngroups, nchunks, ntiles, total_tiles, relu, status,
+                                 Stages<C, true>{});
 }
 
 // Diagnostic: one warp waits, with a short cap, on an mbarrier that nothing ever completes.  Exercises the
@@ -872,31 +908,40 @@ sbnn_status encode_x_map(const float* x, int ldx, int M, int Cin, int box_px, in
     return encode_generic(out, x, 4, 2, dims, strides, box);
 }
 
-template <class C>
-sbnn_status launch_cm(const sbnn_packed* p, const Stream1x1& s, const float* x, int ldx, float* y, int ldy, int M,
-                      int relu, bool out_cm, cudaStream_t st) {
-    sbnn_status r = set_max_dyn_smem(reinterpret_cast<const void*>(&conv1x1_cm_kernel<C, false>), (int)C::SMEM);
-    if (r == SBNN_OK) r = set_max_dyn_smem(reinterpret_cast<const void*>(&conv1x1_cm_kernel<C, true>), (int)C::SMEM);
+template <class C, bool OUT_CM, bool FIXED>
+sbnn_status launch_cm_as(const sbnn_packed* p, const Stream1x1& s, const Stages<C, FIXED>& stages, size_t smem, const float* x, int ldx, float* y,
+                         int ldy, int M, int relu, cudaStream_t st) {
+    sbnn_status r = set_max_dyn_smem(reinterpret_cast<const void*>(&conv1x1_cm_kernel<C, OUT_CM, FIXED>), (int)kMaxSmem);
     if (r != SBNN_OK) return r;
-    if (s.max_blk > C::WS_U4) return fail(SBNN_ERR_UNSUPPORTED, "internal: weight block %d exceeds buffer %d", s.max_blk, C::WS_U4);
     int* status = nullptr;
     if ((r = status_word(&status)) != SBNN_OK) return r;
     if (prepare_only()) return SBNN_OK;
     const long long nblk = (long long)((M + C::TM - 1) / C::TM) * s.ntiles;
     if (nblk > 0x7fffffffLL) return fail(SBNN_ERR_SHAPE, "too many tiles");
-    const int total_tiles = (int)nblk;
-    dim3 grid((unsigned)std::min<long long>(nblk, sm_count()));
     CUtensorMap xmap;
-    r = encode_x_map(x, ldx, M, p->Cin, C::TM, C::KC, &xmap);
-    if (r != SBNN_OK) return r;
+    if ((r = encode_x_map(x, ldx, M, p->Cin, C::TM, C::KC, &xmap)) != SBNN_OK) return r;
     ChainedLaunchScope early;   // before its waits the kernel reads the layer's own arrays only
-    if (out_cm)
-        SBNN_CUDA_TRY(launch_kernel(conv1x1_cm_kernel<C, true>, grid, C::NT, C::SMEM, st, xmap, y, ldy, p->d_bias, s.rec, s.blk_ptr, M,
-                                    p->Cin, p->Cout, p->ngroups, s.nchunks, s.ntiles, total_tiles, relu, status));
-    else
-        SBNN_CUDA_TRY(launch_kernel(conv1x1_cm_kernel<C, false>, grid, C::NT, C::SMEM, st, xmap, y, ldy, p->d_bias, s.rec, s.blk_ptr, M,
-                                    p->Cin, p->Cout, p->ngroups, s.nchunks, s.ntiles, total_tiles, relu, status));
+    SBNN_CUDA_TRY(launch_kernel(conv1x1_cm_kernel<C, OUT_CM, FIXED>, dim3((unsigned)std::min<long long>(nblk, sm_count())), C::NT, smem, st, xmap, y,
+                                ldy, p->d_bias, s.rec, s.blk_ptr, M, p->Cin, p->Cout, p->ngroups, s.nchunks, s.ntiles, (int)nblk, relu, status,
+                                stages));
     return SBNN_OK;
+}
+
+template <class C>
+sbnn_status launch_cm(const sbnn_packed* p, const Stream1x1& s, const float* x, int ldx, float* y, int ldy, int M,
+                      int relu, bool out_cm, cudaStream_t st) {
+    if (s.max_blk > C::WS_U4) return fail(SBNN_ERR_UNSUPPORTED, "internal: weight block %d exceeds buffer %d", s.max_blk, C::WS_U4);
+    auto launch = [&](auto stages, size_t smem) {
+        sbnn_status r = SBNN_OK;
+        if (out_cm || prepare_only()) r = launch_cm_as<C, true>(p, s, stages, smem, x, ldx, y, ldy, M, relu, st);
+        if (r == SBNN_OK && (!out_cm || prepare_only())) r = launch_cm_as<C, false>(p, s, stages, smem, x, ldx, y, ldy, M, relu, st);
+        return r;
+    };
+    if constexpr (C::KC == 64) {   // see Stages
+        const int weights = (s.max_blk * 16 + 127) / 128 * 128, per_stage = C::XS_BYTES + weights + 16, n = (int)(kMaxSmem - 16) / per_stage;
+        if (n > C::STAGES) return launch(Stages<C, false>{n, weights}, (size_t)n * per_stage + 16);
+    }
+    return launch(Stages<C, true>{}, C::SMEM);
 }
 
 // Fused depthwise + pointwise launch (G = 4 layers, union lists, 8 warps, 32-channel steps, two stages).
@@ -990,9 +1035,11 @@ TileCfg choose_cfg_cm(const sbnn_packed* p, long long M) {
     // much per tile as twelve; three warps on a scheduler hide about 2 % more latency than two.
     // What a third warp on a scheduler hides of the per-list latencies grows as the lists get shorter: config 5,
     // 12 against 8 warps (whole launch, so including the 4 % of the 12-warp CTA): 50 % kept units 1033 / 1025 us,
-    // 30 % kept 670 / 684 us, 10 % kept 313 / 352 us.
+    // 30 % kept 670 / 684 us, 10 % kept 289 / 323 us.
     const double kept = (p->ngroups > 0 && p->Cin > 0) ? (double)p->nnz / ((double)p->ngroups * p->Cin) : 1.0;
-    const double hide3 = kept >= 0.5 ? 0.02 : (kept >= 0.3 ? 0.02 + 0.2 * (0.5 - kept) : 0.06 + 0.35 * (0.3 - kept));
+    // With one group of 8 per warp two warps leave a third little to hide (101 x 14 x 14, 1024 -> 512 at 10 % kept: 67.5 us
+    // with 8 warps, 78.4 with 12; 256 x 14 x 14, 1024 -> 1024: 275 and 282 us).
+    const double hide3 = p->G == 8 ? 0.03 : kept >= 0.5 ? 0.02 : (kept >= 0.3 ? 0.02 + 0.2 * (0.5 - kept) : 0.06 + 0.35 * (0.3 - kept));
     auto launch_cost = [&](const TileCfg& c) {
         const long long ptiles = (M + c.TM() - 1) / c.TM(), gtiles = (p->ngroups + c.GT() - 1) / c.GT();
         const long long sms = std::max(1, sm_count()), total = ptiles * gtiles;

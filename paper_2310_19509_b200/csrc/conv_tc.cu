@@ -15,7 +15,7 @@
 //
 // The contraction runs dense over the masked weights (pruned entries are zeros): a group shares its kept channels over
 // only G = 4..8 outputs, far too few for a 128-row MMA to gather for.  Six products per dense MAC still beat the FMA
-// pipe on kept MACs alone until most of the layer is pruned; the rule is tc_profits() below.
+// pipe on kept MACs alone until most of the layer is pruned; the rule is decide() below.
 //
 // Structure, one CTA per SM, persistent over tiles of 128 pixels x BN output channels, 20 warps in 5 warpgroups:
 //   warpgroups 0, 1  drain: tcgen05.ld of a finished step, added to the fp32 sums in registers, which start at the bias;
@@ -835,7 +835,7 @@ TcChoice tc_choose(const sbnn_packed* p, long long M, int run, int images) {
 // Whether a call is faster here than on the FMA kernels, in microseconds of both, fitted to measured times.  Layers of
 // 64-1024 channels on 49 to 50176 pixels, G = 4 and 8, 0 / 50 / 70 / 90 % pruned: channel-major 1x1 calls gain up to 70 %
 // pruning (256 x 14 x 14, 1024 -> 1024: 1969 -> 404, 1025 -> 386, 669 -> 366 us; 9 x 14 x 14, 512 -> 512: 89 -> 12, 53 -> 12,
-// 39 -> 12 us) and lose where next to nothing is left to do (the same at 90 %: 313 and 338 us; one 56 x 56 image, 64 -> 128,
+// 39 -> 12 us) and lose where next to nothing is left to do (the first at 90 %: 289 and 338 us; one 56 x 56 image, 64 -> 128,
 // 50 %: 5.1 and 5.5 us); NHWC calls, which the FMA kernels convert first, and 3x3 calls gain nearly everywhere
 // (32 x 28 x 28, 256 -> 256: 305 -> 119 us at 50 %, 120 -> 111 at 90 %; in groups of 8 106 and 111).
 // `choice` is how; it is remembered with the layer for each kind of call and number of pixels.
@@ -854,7 +854,7 @@ TcChoice decide(const sbnn_packed* p, long long M, Call call) {
     } else if (call == CALL_1X1_CM && conv1x1_few_tiles(p, M)) {
         fma = 2.7 + kept * std::max(1.0, 32.0 / M) * (p->G >= 8 ? 0.18 : 0.22);   // (a lane takes a pixel)
     } else if (call == CALL_1X1_CM || (p->Cin >= 128 && M >= 2048)) {
-        fma = 5.0 + 0.034 * kept + 0.0021 * dense + 0.6 * mem;
+        fma = 4.5 + 0.034 * kept + 0.0011 * dense + 0.65 * mem;
         if (call == CALL_1X1_NHWC) fma += 2.0 + 8.0 * M * p->Cin / 4.5e6;    // the conversion to channel-major
     } else {
         fma = 2.0 + (p->Cin >= 128 ? 2.0 : 0.0) + 0.012 * p->Cin + 0.1 * kept;
