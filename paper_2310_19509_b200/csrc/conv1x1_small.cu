@@ -15,8 +15,10 @@ namespace {
 
 
 // Index and weights of unit `u` for lane-parallel fetching: lane l of a warp fetches unit u0 + l (two coalesced
-// requests for 32 units), and the warp then hands them round by shuffle, so the only per-unit memory access
-// left is the activation row itself and 32 of those are independent.
+// requests for 32 units) and puts them into shared memory, from where the whole warp reads them, so the only per-unit
+// access to global memory left is the activation row itself and 16 of those are independent.
+// (Handing them round by shuffle, 1 + G for a unit, bound the launch: one pixel, 1024 -> 1000 dense, 10.1 -> 6.8 us; one
+// 14 x 14 image, 512 -> 512 at 50 %, G = 4 13 -> 7.5 us, 3 x 2 x 2 pixels, G = 8 4.0 -> 2.8.)
 template <int G>
 struct UnitRegs {
     int c;
@@ -48,13 +50,15 @@ __device__ __forceinline__ void fetch_unit(const int32_t* __restrict__ idx, cons
 }
 
 // KSPLIT = warps per CTA; each takes that fraction of the group's kept units.  PX = pixels per lane (the CTA covers
-// 32 * PX pixels): with two, a unit's index and weights, which reach the lanes by shuffle, serve twice the FMAs.
+// 32 * PX pixels): with two, a unit's index and weights, once read from shared memory, serve twice the FMAs.
 template <int G, int KSPLIT, bool OUT_CM, int PX>
 __global__ void __launch_bounds__(32 * KSPLIT)
 conv1x1_small_kernel(const float* __restrict__ X, int ldx, float* __restrict__ Y, int ldy, const int32_t* __restrict__ group_ptr,
                      const int32_t* __restrict__ idx, const float* __restrict__ val, const float* __restrict__ bias, int M,
                      int relu) {
     __shared__ float red[KSPLIT][G][32 * PX];
+    __shared__ __align__(16) float wsm[KSPLIT][32 * G];
+    __shared__ __align__(16) int csm[KSPLIT][32];
     const int lane = threadIdx.x & 31, kq = threadIdx.x >> 5;
     const int g = blockIdx.y;
     int m[PX];
@@ -77,6 +81,10 @@ conv1x1_small_kernel(const float* __restrict__ X, int ldx, float* __restrict__ Y
     grid_dependency_wait();      // X comes from the previous kernel of the stream; the weights above do not
     grid_dependency_release();
     for (int ub = u0; ub < uend; ub += 32) {
+        csm[kq][lane] = cur.c;
+#pragma unroll
+        for (int r = 0; r < G; ++r) wsm[kq][lane * G + r] = cur.w[r];
+        __syncwarp();
         fetch_unit<G>(idx, val, ub + 32 + lane, uend, nxt);        // the next 32 units, while these are consumed
         const int cnt = min(32, uend - ub);                        // warp-uniform
 #pragma unroll
@@ -84,20 +92,35 @@ conv1x1_small_kernel(const float* __restrict__ X, int ldx, float* __restrict__ Y
             if (h * 16 >= cnt) break;
             float xv[PX][16];
 #pragma unroll
-            for (int k = 0; k < 16; ++k) {
-                const int c = __shfl_sync(0xffffffffu, cur.c, h * 16 + k);
+            for (int k4 = 0; k4 < 4; ++k4) {
+                const int4 c4 = reinterpret_cast<const int4*>(csm[kq])[h * 4 + k4];
+                const int c[4] = {c4.x, c4.y, c4.z, c4.w};
 #pragma unroll
-                for (int j = 0; j < PX; ++j) xv[j][k] = (h * 16 + k < cnt) ? __ldg(xp[j] + (size_t)c * ldx) : 0.0f;
+                for (int e = 0; e < 4; ++e)
+#pragma unroll
+                    for (int j = 0; j < PX; ++j) xv[j][k4 * 4 + e] = (h * 16 + k4 * 4 + e < cnt) ? __ldg(xp[j] + (size_t)c[e] * ldx) : 0.0f;
             }
 #pragma unroll
-            for (int k = 0; k < 16; ++k)
+            for (int k = 0; k < 16; ++k) {
+                float w[G];
+                const float* wp = wsm[kq] + (h * 16 + k) * G;
+                if constexpr (G % 4 == 0) {
 #pragma unroll
-                for (int r = 0; r < G; ++r) {
-                    const float wr = __shfl_sync(0xffffffffu, cur.w[r], h * 16 + k);
+                    for (int q = 0; q < G / 4; ++q) {
+                        const float4 t = reinterpret_cast<const float4*>(wp)[q];
+                        w[4 * q] = t.x; w[4 * q + 1] = t.y; w[4 * q + 2] = t.z; w[4 * q + 3] = t.w;
+                    }
+                } else {
 #pragma unroll
-                    for (int j = 0; j < PX; ++j) acc[j][r] = fmaf(xv[j][k], wr, acc[j][r]);
+                    for (int r = 0; r < G; ++r) w[r] = wp[r];
                 }
+#pragma unroll
+                for (int r = 0; r < G; ++r)
+#pragma unroll
+                    for (int j = 0; j < PX; ++j) acc[j][r] = fmaf(xv[j][k], w[r], acc[j][r]);
+            }
         }
+        __syncwarp();                                              // before the next units take their place
         cur = nxt;
     }
 #pragma unroll
@@ -154,9 +177,10 @@ sbnn_status launch_small(const sbnn_packed* p, const float* x, int ldx, float* y
     // Long lists are split over more warps (shorter dependent chains); short ones are not worth the reduction.
     const long long avg = p->ngroups ? p->nnz / p->ngroups : 0;
     if (avg >= 256) {
-        // long lists and more than one 32-pixel block: two pixels per lane halve the shuffles per FMA (classifier at
-        // batch 64: 18.3 -> 14.9 us inside the step); groups of 16 channels would need 32 more accumulators and stay with one
-        if (G <= 8 && M > 32) return launch_small_ks<G, 8, 2>(p, x, ldx, y, ldy, M, relu, out_cm, st);
+        // long lists and more than one 32-pixel block: two pixels per lane halve the reads of weights per FMA (classifier at
+        // batch 64 when the weights still came by shuffle: 18.3 -> 14.9 us inside the step); groups of 16 channels would need 32 more accumulators and stay with one
+        if constexpr (G <= 8)
+            if (M > 32) return launch_small_ks<G, 8, 2>(p, x, ldx, y, ldy, M, relu, out_cm, st);
         return launch_small_ks<G, 8, 1>(p, x, ldx, y, ldy, M, relu, out_cm, st);
     }
     if (avg >= 96) return launch_small_ks<G, 4, 1>(p, x, ldx, y, ldy, M, relu, out_cm, st);

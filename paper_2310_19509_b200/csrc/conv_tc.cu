@@ -835,8 +835,8 @@ TcChoice tc_choose(const sbnn_packed* p, long long M, int run, int images) {
 // Whether a call is faster here than on the FMA kernels, in microseconds of both, fitted to measured times.  Layers of
 // 64-1024 channels on 49 to 50176 pixels, G = 4 and 8, 0 / 50 / 70 / 90 % pruned: channel-major 1x1 calls gain up to 70 %
 // pruning (256 x 14 x 14, 1024 -> 1024: 1969 -> 404, 1025 -> 386, 669 -> 366 us; 9 x 14 x 14, 512 -> 512: 89 -> 12, 53 -> 12,
-// 39 -> 12 us) and lose where next to nothing is left to do (the first at 90 %: 289 and 338 us; one 56 x 56 image, 64 -> 128,
-// 50 %: 5.1 and 5.5 us); NHWC calls, which the FMA kernels convert first, and 3x3 calls gain nearly everywhere
+// 39 -> 12 us) and lose where next to nothing is left to do (the first at 90 %: 289 and 338 us; one 14 x 14 image, 256 -> 512,
+// 50 %: 4.5 and 6.0 us); NHWC calls, which the FMA kernels convert first, and 3x3 calls gain nearly everywhere
 // (32 x 28 x 28, 256 -> 256: 305 -> 119 us at 50 %, 120 -> 111 at 90 %; in groups of 8 106 and 111).
 // `choice` is how; it is remembered with the layer for each kind of call and number of pixels.
 enum Call { CALL_1X1_NHWC, CALL_1X1_CM, CALL_3X3, CALL_3X3_CM, CALL_BF16 };
@@ -852,7 +852,7 @@ TcChoice decide(const sbnn_packed* p, long long M, Call call) {
     if (call == CALL_3X3 || call == CALL_3X3_CM) {
         fma = 25.0 + kept * (p->G >= 8 ? 0.050 : 0.075);
     } else if (call == CALL_1X1_CM && conv1x1_few_tiles(p, M)) {
-        fma = 2.7 + kept * std::max(1.0, 32.0 / M) * (p->G >= 8 ? 0.18 : 0.22);   // (a lane takes a pixel)
+        fma = 1.8 + kept * ((M + 31) / 32 * 32) / M * (p->G >= 8 ? 0.145 : 0.20);   // (a lane takes a pixel)
     } else if (call == CALL_1X1_CM || (p->Cin >= 128 && M >= 2048)) {
         fma = 4.5 + 0.034 * kept + 0.0011 * dense + 0.65 * mem;
         if (call == CALL_1X1_NHWC) fma += 2.0 + 8.0 * M * p->Cin / 4.5e6;    // the conversion to channel-major
