@@ -192,10 +192,14 @@ enum {
  * products are summed in fp32 on the tensor cores; bias and ReLU stay fp32.  By default the contraction then runs
  * densely over the masked weights (pruned weights are stored as zeros and multiplied: on the tcgen05 tensor cores
  * that is faster than skipping them, because a group of G <= 8 output channels is too narrow an MMA); this needs
- * Cin % 8 == 0 and Cout % 4 == 0, other shapes -- and every shape when SBNN_BF16_GATHER is added -- run the
- * gathered kernel, which visits kept units only.  Both give the same result up to the order of the fp32 sums.
+ * Cout % 4 == 0, other shapes -- and every shape when SBNN_BF16_GATHER is added -- run the gathered kernel, which
+ * visits kept units only.  Both give the same result up to the order of the fp32 sums.
  * The first call of a layer in either form builds a private re-layout of its weights (allocates and copies
- * synchronously), and both convert X to bf16 in the per-device scratch buffer first.
+ * synchronously); the gathered kernel converts X to bf16 in the per-device scratch buffer first.
+ * Without it the sums are fp32 sums of fp32 products.  Where that is faster (wide layers and whatever is not almost
+ * entirely pruned) they are formed on the tensor cores, from an exact split of every operand into three bf16 numbers;
+ * the error is that of an fp32 sum, and pixels that hold an infinity or a NaN are summed over the kept units alone.
+ * Which kernel runs depends on the layer and on N*H*W.
  */
 SBNN_API sbnn_status sbnn_conv1x1_gs(const sbnn_packed* w, const float* x_dev, float* y_dev,
                                      int N, int H, int W, int flags, void* cuda_stream);
@@ -222,11 +226,12 @@ SBNN_API sbnn_status sbnn_conv1x1_gs_tuned(const sbnn_packed* w, const float* x_
  *   shape whose tiles fill the SMs best for this M, or, when M is so small that even that leaves most SMs
  *   idle (the classifier, batch-1 layers), a kernel that splits the work by 32 pixels x one group instead.
  *   The order of the sums, hence the last bits of the result, can therefore depend on M.
- * sbnn_conv1x1_gs itself takes this path for wide layers (Cin >= 128, M >= 2048): it first copies X
- * into a channel-major scratch buffer kept per device, which it allocates or grows (synchronously) the
- * first time a size is seen.
+ * With the tile shape left open the layer may run on the tensor cores instead (see sbnn_conv1x1_gs).
+ * sbnn_conv1x1_gs itself takes this path for wide layers (Cin >= 128, M >= 2048) that do not run on the tensor
+ * cores: it first copies X into a channel-major scratch buffer kept per device, which it allocates or grows
+ * (synchronously) the first time a size is seen.
  * sbnn_to_channel_major converts x_dev [M][C] to xt_dev [C][ld].
- * The scratch buffer is one per device and is also used by the bf16 mode and by sbnn_conv3x3_gs: calls that
+ * The scratch buffer is one per device and is also used by SBNN_BF16_GATHER and by sbnn_conv3x3_gs: calls that
  * use it must be ordered on the GPU (same stream, or events); overlapping ones race on it.
  */
 SBNN_API sbnn_status sbnn_conv1x1_gs_cm(const sbnn_packed* w, const float* xt_dev, int ldx, float* y_dev, int ldy,
