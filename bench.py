@@ -521,7 +521,10 @@ def run_gpu(args, rank, world, local_rank):
     t_roof = lambda r: max(r["flops"] / (FP32_PEAK_TFLOPS * 1e12), r["bytes"] / (hbm_gbs * 1e9))  # noqa: E731
     total_layer_t = sum(r["s"] for r in per)
     roofline = {
-        "bound": "alu", "kernel": "conv1x1_cm_kernel (13 pointwise launches per step)",
+        "bound": "tensor", "kernel": "conv_tc_kernel (13 pointwise launches per step)",
+        "tensor_frac": 6 * pw_fl / (1 - args.sparsity / 100) / pw_t / 1e12 / bf16_tflops if bf16_tflops and args.sparsity < 100 else None,
+        "note": "achieved and frac count nonzero flops against the FP32 FMA peak; the kernel multiplies dense, six bf16 products for each "
+                "fp32 one, so frac can exceed 1: tensor_frac is those products against the measured bf16 rate",
         "achieved": pw_fl / pw_t / 1e12, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
         "frac": pw_fl / pw_t / 1e12 / FP32_PEAK_TFLOPS,
         "timing": "per layer: time of the chain's prefix up to and including the layer minus the prefix before it, each prefix a "
