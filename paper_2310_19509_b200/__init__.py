@@ -36,6 +36,8 @@ from .binding import (  # noqa: F401
     selftest_fma_rate,
     debug_set_packed_device,
     debug_check_packed,
+    debug_conv_gs,
+    debug_last_route,
     debug_plan_conv3x3,
     debug_poke_device_index,
     selftest_wait_timeout,

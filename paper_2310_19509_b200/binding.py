@@ -75,6 +75,8 @@ def lib():
         "sbnn_debug_set_packed_device": [P, I, P],
         "sbnn_debug_check_packed": [P, P],
         "sbnn_debug_poke_device_index": [P, C.c_longlong, I, P],
+        "sbnn_debug_last_route": [P, P],
+        "sbnn_debug_conv_gs": [P, P, I, P, I, I, I, I, I, I, I, P],
         "sbnn_debug_plan_conv3x3": [P, I, I, I, I, P, P, I, P, P, P],
     }
     for name, args in sig.items():
@@ -309,6 +311,18 @@ def debug_plan_conv3x3(block_ptr, nrow, ncta):
     _check(lib().sbnn_debug_plan_conv3x3(bp.ctypes.data, ntiles, nchunks, int(nrow), int(ncta), cta_ptr.ctypes.data,
                                          segs.ctypes.data, cap, C.byref(nsegs), C.byref(nslots), C.byref(ncounters)))
     return cta_ptr, segs[:nsegs.value].copy(), nslots.value, ncounters.value
+
+
+def debug_last_route():
+    """(tile, split) of this thread's latest convolution: tile 0 = FMA kernels, else channels of a tensor-core tile."""
+    tile, split = C.c_int(), C.c_int()
+    _check(lib().sbnn_debug_last_route(C.byref(tile), C.byref(split)))
+    return tile.value, split.value
+
+
+def debug_conv_gs(w: Packed, x, ldx, y, ldy, n, h, wd, flags, tile, split=1, stream=None):
+    """A 1x1 or 3x3 layer (ldx = ldy = 0: NHWC, else channel-major) on the kernel the caller names (see sbnn_debug_conv_gs)."""
+    _check(lib().sbnn_debug_conv_gs(w.handle, _ptr(x), ldx, _ptr(y), ldy, n, h, wd, flags, tile, split, _stream(stream)))
 
 
 def debug_poke_device_index(w: Packed, unit, value) -> int:

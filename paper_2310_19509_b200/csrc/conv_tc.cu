@@ -863,7 +863,16 @@ TcChoice decide(const sbnn_packed* p, long long M, Call call) {
     if (std::max(tc_us(choice.cost), mem) >= 0.95 * fma) choice.bn = 0;
     return choice;
 }
+// Test hooks (sbnn_debug_conv_gs, sbnn_debug_last_route), for the calling thread: how its calls have to run (bn = 0: on the
+// FMA kernels), and how the latest ran.
+thread_local const TcChoice* forced_choice = nullptr;
+thread_local TcChoice last_route = {0, 0, 0.0};
+
 bool tc_profits(const sbnn_packed* p, long long M, Call call, TcChoice* choice = nullptr) {
+    if (forced_choice) {
+        if (choice) *choice = *forced_choice;
+        return forced_choice->bn != 0;
+    }
     const long long key = M * 8 + call;
     {
         std::lock_guard<std::mutex> lk(p->mu);
@@ -952,6 +961,7 @@ sbnn_status launch_tc(const sbnn_packed* p, const TcCall& c, int split, bool* do
     a.sb = a.resident ? a.steps * T::NU : T::SB;
     a.sa = std::min(T::SA_MAX, (T::ROOM - a.sb * T::B_BYTES) / T::A_BYTES);
     const size_t smem = (size_t)a.sb * T::B_BYTES + (size_t)a.sa * T::A_BYTES + T::OUT_BYTES + T::CTRL + 1024;
+    last_route = {T::BN, a.split, 0.0};
     ChainedLaunchScope early;   // before their waits the kernel's warps read the layer's own arrays only
     SBNN_CUDA_TRY(launch_kernel_cluster(conv_tc_kernel<T>, dim3(grid), dim3(T::NT), smem, c.st, (unsigned)a.split, amap, ymap, a));
     return SBNN_OK;
@@ -971,6 +981,7 @@ sbnn_status dispatch_tc(const sbnn_packed* p, const TcCall& c, const TcChoice& c
 
 sbnn_status conv1x1_tc(const sbnn_packed* p, const float* x, float* y, long long M, int relu, cudaStream_t st, bool* done) {
     *done = false;
+    last_route = {0, 0, 0.0};
     TcChoice ch;
     sbnn_status r;
     if (prepare_only() && (r = prepare_tc(p, M)) != SBNN_OK) return r;
@@ -983,6 +994,7 @@ sbnn_status conv1x1_tc(const sbnn_packed* p, const float* x, float* y, long long
 // memory took 154 us for 1024 -> 1024 on 256 x 14 x 14, 40 of them for that pass.)
 sbnn_status conv1x1_tc_bf16(const sbnn_packed* p, const float* x, float* y, long long M, int relu, cudaStream_t st, bool* done) {
     *done = false;
+    last_route = {0, 0, 0.0};
     if (p->Cin % 4 || p->Cout % 4) return SBNN_OK;
     if (prepare_only()) {   // the tile width depends on the pixels: for calls with fewer, too
         uint4* wts = nullptr;
@@ -1005,6 +1017,7 @@ sbnn_status conv1x1_tc_bf16(const sbnn_packed* p, const float* x, float* y, long
 sbnn_status conv1x1_tc_cm(const sbnn_packed* p, const float* x, int ldx, float* y, int ldy, long long M, int relu, bool out_cm, cudaStream_t st,
                           bool* done) {
     *done = false;
+    last_route = {0, 0, 0.0};
     TcChoice ch;
     sbnn_status r;
     if (prepare_only() && (r = prepare_tc(p, M)) != SBNN_OK) return r;
@@ -1015,6 +1028,7 @@ sbnn_status conv1x1_tc_cm(const sbnn_packed* p, const float* x, int ldx, float* 
 
 sbnn_status conv3x3_tc(const sbnn_packed* p, const float* x, float* y, int N, int H, int W, int relu, cudaStream_t st, bool* done) {
     *done = false;
+    last_route = {0, 0, 0.0};
     TcChoice ch;
     const long long M = (long long)N * H * W;
     sbnn_status r;
@@ -1027,6 +1041,7 @@ sbnn_status conv3x3_tc(const sbnn_packed* p, const float* x, float* y, int N, in
 sbnn_status conv3x3_tc_cm(const sbnn_packed* p, const float* x, int ldx, float* y, int ldy, int N, int H, int W, int relu, bool out_cm, cudaStream_t st,
                           bool* done) {
     *done = false;
+    last_route = {0, 0, 0.0};
     TcChoice ch;
     const long long M = (long long)N * H * W;
     sbnn_status r;
@@ -1043,3 +1058,42 @@ void free_tc_weights(sbnn_packed* p) {
 }
 
 }  // namespace sbnn
+
+using namespace sbnn;
+
+extern "C" sbnn_status sbnn_debug_last_route(int* tile, int* split) {
+    clear_error();
+    if (!tile || !split) return fail(SBNN_ERR_NULL, "tile and split must not be NULL");
+    *tile = last_route.bn;
+    *split = last_route.split;
+    return SBNN_OK;
+}
+
+extern "C" sbnn_status sbnn_debug_conv_gs(const sbnn_packed* w, const float* x_dev, int ldx, float* y_dev, int ldy, int N, int H, int W, int flags,
+                                          int tile, int split, void* cuda_stream) {
+    clear_error();
+    if (!w) return fail(SBNN_ERR_NULL, "packed weights must not be NULL");
+    if (tile != 0 && tile != 64 && tile != 128 && tile != 256) return fail(SBNN_ERR_UNSUPPORTED, "tile=%d is not 0, 64, 128 or 256", tile);
+    if (split != 1 && !(tile == 64 && (split == 2 || split == 4 || split == 8)))
+        return fail(SBNN_ERR_UNSUPPORTED, "split=%d is not 1, or 2, 4 or 8 with 64-channel tiles", split);
+    const int runs = (w->Cin + 63) / 64 * w->KH * (ldx ? 1 : w->KW);   // (channel-major 3x3: the taps of a kernel row stay together)
+    if (runs < split) return fail(SBNN_ERR_UNSUPPORTED, "the layer has %d steps to split, not %d", runs, split);
+    const TcChoice choice = {tile, split, 0.0};
+    struct Scope {
+        explicit Scope(const TcChoice* c) { forced_choice = c; }
+        ~Scope() { forced_choice = nullptr; }
+    } scope(&choice);
+    last_route = {0, 0, 0.0};
+    sbnn_status r;
+    if (ldx == 0 && ldy == 0)
+        r = w->KH == 3 ? sbnn_conv3x3_gs(w, x_dev, y_dev, N, H, W, flags, cuda_stream) : sbnn_conv1x1_gs(w, x_dev, y_dev, N, H, W, flags, cuda_stream);
+    else if (w->KH == 3)
+        r = sbnn_conv3x3_gs_cm(w, x_dev, ldx, y_dev, ldy, N, H, W, flags, cuda_stream);
+    else if (N < 0 || H < 0 || W < 0 || (long long)N * H * W > 0x7fffffff)
+        r = fail(SBNN_ERR_SHAPE, "bad shape %dx%dx%d", N, H, W);
+    else
+        r = sbnn_conv1x1_gs_cm(w, x_dev, ldx, y_dev, ldy, N * H * W, flags, 0, 0, 0, 0, cuda_stream);
+    if (r == SBNN_OK && (last_route.bn != tile || (tile && last_route.split != split)))
+        return fail(SBNN_ERR_UNSUPPORTED, "the tensor-core kernel does not take this call; it ran on another kernel");
+    return r;
+}

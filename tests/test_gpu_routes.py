@@ -1,0 +1,207 @@
+"""Layers on a kernel that the test names: every instance of the tensor-core kernel, and the FMA kernels at shapes that the
+library's own choice gives to the tensor cores.
+
+Tolerance of the tensor-core kernel, per output: |gpu - ref| <= (4 * 2^-23 + (steps + 3) * 2^-24) * S, S = |b| + sum |w*x|.  A
+64-channel step adds its products in 24 MMAs of 16 channels, each of which cuts off less than a unit in the last place of the
+running sum; the 20 of them that add the small products have sums below 2^-7 S, so four count.  Steps are added in fp32,
+rounded to nearest; the three omitted products and the scale of the weights are within the remaining 3 * 2^-24.
+Over a whole output the 2-norm of the error is at most 4e-7 of the result's: measured 0.3e-7 to 0.9e-7 for 4 to 1024
+channels; without any one of the six products it is above 8e-7 (see test_a_missing_product_would_be_seen).
+FMA kernels: 1e-5 * S, as in their own tests (one rounding per kept product).
+"""
+import functools
+
+import numpy as np
+import pytest
+import torch
+
+import paper_2310_19509_b200 as sbnn
+from oracle import reference as R
+from sbnn_inputs import tap_pattern_mask
+from sbnn_inputs import workloads as WL
+
+gpu = pytest.mark.gpu
+RMS = 4e-7
+
+
+@functools.lru_cache(maxsize=None)
+def inputs(n, h, w, cin, cout, k, g, pct, bf16=False):
+    d = WL.single_conv_inputs(n, h, w, cin, cout, k, g, pct, 11, 0.05, 0.05)
+    ref, s = R.conv2d(d["x"], d["w"], d["mask"], d["bias"], relu=False, bf16=bf16)
+    return d, ref, s
+
+
+def run(p, d, layout, tile, split, flags=0):
+    """layout: 'nhwc', 'cm' (channel-major in, rows out) or 'cm-cm'.  Output as [M][Cout]; guards and padding are checked."""
+    n, h, w, cin = d["x"].shape
+    m, cout = n * h * w, d["w"].shape[0]
+    x = torch.from_numpy(d["x"]).cuda()
+    if layout == "nhwc":
+        y = torch.full((m * cout + 512,), float("nan"), device="cuda")
+        sbnn.debug_conv_gs(p, x, 0, y[256:], 0, n, h, w, flags, tile, split)
+        assert bool(torch.isnan(y[:256]).all()) and bool(torch.isnan(y[-256:]).all())
+        out = y[256:-256].view(m, cout)
+    else:
+        ld = (m + 3) // 4 * 4 + 8
+        xt = torch.full((cin, ld), float("nan"), device="cuda")
+        xt[:, :m] = x.reshape(m, cin).T
+        cm = layout == "cm-cm"
+        y = torch.full((cout, ld) if cm else (m, cout), float("nan"), device="cuda")
+        sbnn.debug_conv_gs(p, xt, ld, y, ld if cm else cout, n, h, w, flags | (sbnn.SBNN_OUT_CM if cm else 0), tile, split)
+        if cm:
+            assert bool(torch.isnan(y[:, m:]).all())
+        out = y[:, :m].T if cm else y
+    assert sbnn.debug_last_route() == ((tile, split) if tile else (0, 0))
+    sbnn.get_async_status()
+    return out.cpu().numpy()
+
+
+def check_tc(got, ref, s, steps):
+    ref, s = ref.reshape(got.shape), s.reshape(got.shape)
+    err = np.abs(got.astype(np.float64) - ref)
+    assert np.all(err <= (4 * 2.0 ** -23 + (steps + 3) * 2.0 ** -24) * s)
+    assert np.linalg.norm(err) <= RMS * np.linalg.norm(ref)
+
+
+INSTANCES = [(64, 1), (128, 1), (256, 1), (64, 2), (64, 4), (64, 8)]
+# ragged pixels, channels and output channels; nine steps for the splits; more tiles than SMs at every tile width
+SHAPES_1X1 = [(3, 17, 19, 516, 260, 4, 50), (7, 61, 63, 100, 516, 4, 30)]
+SHAPES_3X3 = [(2, 13, 14, 132, 260, 4, 50), (48, 14, 15, 132, 300, 4, 30)]
+
+
+@gpu
+@pytest.mark.parametrize("layout", ["nhwc", "cm", "cm-cm"])
+@pytest.mark.parametrize("k,shape,tile,split", [(k, s, *i) for k, shapes in ((1, SHAPES_1X1), (3, SHAPES_3X3)) for s in shapes for i in INSTANCES
+                                                if k == 3 or (s[3] + 63) // 64 >= i[1]])
+def test_every_tensor_core_instance(k, shape, tile, split, layout):
+    d, ref, s = inputs(*shape[:5], k, *shape[5:])
+    p = sbnn.pack_weights(d["w"], d["mask"], d["bias"], d["g"])
+    steps = (shape[3] + 63) // 64 * k * k
+    check_tc(run(p, d, layout, tile, split), ref, s, steps)
+    check_tc(run(p, d, layout, tile, split, sbnn.SBNN_RELU), np.maximum(ref, 0), s, steps)
+
+
+@gpu
+@pytest.mark.parametrize("tile,split", INSTANCES)
+def test_every_bf16_instance(tile, split):
+    """Operands rounded to bf16, exact products, sums cut off at most 4 * steps times: 36 * 2^-23 = 4.3e-6 of S."""
+    d, ref, s = inputs(*SHAPES_1X1[0][:5], 1, *SHAPES_1X1[0][5:], bf16=True)
+    p = sbnn.pack_weights(d["w"], d["mask"], d["bias"], d["g"])
+    got = run(p, d, "nhwc", tile, split, sbnn.SBNN_BF16_TC)
+    assert np.all(np.abs(got.astype(np.float64) - ref.reshape(got.shape)) <= 1e-5 * s.reshape(got.shape))
+
+
+@gpu
+@pytest.mark.parametrize("cin", [32, 64])
+def test_weights_that_stay_in_shared_memory(cin):
+    """One channel tile and no more steps than weight stages: the weights are loaded once and serve every tile."""
+    for tile, cout in ((64, 60), (128, 124), (256, 252)):
+        d, ref, s = inputs(7, 61, 63, cin, cout, 1, 4, 50)
+        p = sbnn.pack_weights(d["w"], d["mask"], d["bias"], d["g"])
+        for layout in ("nhwc", "cm-cm"):
+            check_tc(run(p, d, layout, tile, 1), ref, s, 1)
+
+
+@gpu
+@pytest.mark.parametrize("scale", [2.0 ** -60, 2.0 ** 60])
+def test_small_and_large_operands_keep_their_bits(scale):
+    """A pixel whose activations are all small (or large) must be as exact as any other: its own sum is the measure."""
+    d, ref, s = inputs(3, 17, 19, 516, 260, 1, 4, 50)
+    x = d["x"].copy()
+    x[:, 5, :, :] *= np.float32(scale)
+    d = dict(d, x=x, bias=np.zeros_like(d["bias"]))
+    ref, s = R.conv2d(d["x"], d["w"], d["mask"], d["bias"], relu=False)
+    p = sbnn.pack_weights(d["w"], d["mask"], d["bias"], d["g"])
+    got = run(p, d, "nhwc", 128, 1).reshape(ref.shape)
+    check_tc(got[:, 5], ref[:, 5], s[:, 5], 9)
+    check_tc(got, ref, s, 9)
+
+
+def bf16_images(v):
+    """Three bf16 numbers whose sum is v, each rounded to nearest even."""
+    out, r = [], np.asarray(v, np.float32)
+    for _ in range(3):
+        u = r.view(np.uint32)
+        h = ((u + 0x7FFF + ((u >> 16) & 1)) & np.uint32(0xFFFF0000)).astype(np.uint32).view(np.float32)
+        out.append(h.astype(np.float64))
+        r = (r - h).astype(np.float32)
+    return out
+
+
+@pytest.mark.parametrize("cin", [100, 516])
+def test_a_missing_product_would_be_seen(cin):
+    """The bound on the 2-norm is below the error of a sum without any one of the six products (a model in fp64)."""
+    rng = np.random.default_rng(cin)
+    x = rng.random((200, cin), dtype=np.float32)
+    w = rng.standard_normal((64, cin), dtype=np.float32) * np.float32(0.05) * (rng.random((64, cin)) < 0.5)
+    ref = x.astype(np.float64) @ w.astype(np.float64).T
+    xi, wi = bf16_images(x), bf16_images(w.astype(np.float32))
+    six = [(2, 0), (0, 2), (1, 1), (1, 0), (0, 1), (0, 0)]
+    err = lambda kept: np.linalg.norm(sum(xi[a] @ wi[b].T for a, b in kept) - ref) / np.linalg.norm(ref)  # noqa: E731
+    assert err(six) < RMS / 10
+    for gone in six:
+        assert err([q for q in six if q != gone]) > 2 * RMS
+
+
+# ---- the FMA 3x3 kernels: split tiles, tap lists, both numbers of rows per lane, every group size -----------------------
+@gpu
+@pytest.mark.parametrize("g,n,h,w,cin,cout", [
+    (4, 40, 14, 28, 64, 64), (4, 9, 7, 28, 40, 96), (8, 12, 14, 28, 64, 128), (2, 30, 8, 56, 32, 24), (1, 20, 10, 28, 24, 40),
+    (16, 6, 28, 28, 48, 64), (4, 200, 14, 28, 16, 32), (4, 20, 14, 28, 40, 72), (4, 3, 56, 56, 24, 120), (16, 20, 16, 8, 16, 32),
+    (4, 2, 5, 5, 20, 48), (8, 2, 9, 13, 20, 48), (2, 2, 14, 14, 20, 48), (4, 2, 3, 57, 20, 48), (8, 2, 6, 100, 20, 48), (4, 1, 5, 252, 20, 24),
+])
+def test_3x3_on_the_fma_kernels(g, n, h, w, cin, cout):
+    d, ref, s = inputs(n, h, w, cin, cout, 3, g, 50)
+    p = sbnn.pack_weights(d["w"], d["mask"], d["bias"], g)
+    for layout in ("nhwc", "cm", "cm-cm") if w <= 224 else ("nhwc",):
+        got = run(p, d, layout, 0, 1)
+        assert np.all(np.abs(got.astype(np.float64) - ref.reshape(got.shape)) <= 1e-5 * s.reshape(got.shape))
+        assert np.array_equal(got, run(p, d, layout, 0, 1))             # split tiles are summed in the same order every time
+
+
+@gpu
+@pytest.mark.parametrize("g", [1, 4, 8, 16])
+@pytest.mark.parametrize("taps", [2, 4, 7])
+def test_3x3_patterns_on_the_fma_kernels(g, taps):
+    """Tap lists (few taps) and the whole-kernel loop (many) on whole and odd heights."""
+    for n, h in ((6, 28), (5, 7)):
+        d = dict(inputs(n, h, 28, 40, 64, 3, g, 30)[0])
+        d["mask"] = tap_pattern_mask(2, 19, d["mask"][::g, 0, 0, :].astype(bool), g, taps)
+        p = sbnn.pack_weights(d["w"], d["mask"], d["bias"], g, tap_patterns=True)
+        ref, s = R.conv2d(d["x"], d["w"], d["mask"], d["bias"], relu=False)
+        for tile in (0, 64):
+            got = run(p, d, "nhwc", tile, 1)
+            assert np.all(np.abs(got.astype(np.float64) - ref.reshape(got.shape)) <= 1e-5 * s.reshape(got.shape))
+
+
+@gpu
+def test_the_library_s_own_choice():
+    """Wide and half-pruned layers run on the tensor cores, nearly empty ones and non-finite ones on the FMA kernels; a first
+    call during a capture cannot build the images and runs on the FMA kernels."""
+    def route(n, hw, cin, cout, k, g, pct, poke=None):
+        d = WL.single_conv_inputs(1, 1, 1, cin, cout, k, g, pct, 3, 0.05, 0.05)
+        if poke is not None:
+            d["w"][0, 0, 0, np.argmax(d["mask"][0, 0, 0])] = poke
+        p = sbnn.pack_weights(d["w"], d["mask"], d["bias"], g)
+        x, y = torch.zeros((n, hw, hw, cin), device="cuda"), torch.empty((n, hw, hw, cout), device="cuda")
+        (sbnn.conv1x1_gs if k == 1 else sbnn.conv3x3_gs)(p, x, y, n, hw, hw)
+        return sbnn.debug_last_route()
+
+    assert route(64, 14, 1024, 1024, 1, 4, 50)[0] in (128, 256)
+    assert route(8, 28, 256, 256, 3, 4, 50)[0] in (64, 128, 256)
+    assert route(5, 7, 512, 512, 3, 8, 70)[1] > 1
+    assert route(32, 28, 256, 256, 3, 8, 90) == (0, 0)
+    assert route(64, 14, 1024, 1024, 1, 4, 50, np.inf) == (0, 0)
+
+    d, ref, s = inputs(7, 61, 63, 64, 124, 1, 4, 50)
+    p = sbnn.pack_weights(d["w"], d["mask"], d["bias"], 4)
+    x, y = torch.from_numpy(d["x"]).cuda(), torch.empty(ref.shape, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=torch.cuda.Stream()):
+        sbnn.conv1x1_gs(p, x, y, 7, 61, 63, 0)
+        assert sbnn.debug_last_route() == (0, 0)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert np.all(np.abs(y.cpu().numpy().astype(np.float64) - ref) <= 1e-5 * s)
+    sbnn.conv1x1_gs(p, x, y, 7, 61, 63, 0)
+    assert sbnn.debug_last_route()[0] != 0
