@@ -99,11 +99,14 @@ def _check(code):
 
 
 def _ptr(t):
-    """Device pointer of a torch tensor (or a raw int / None)."""
+    """Device pointer of a torch tensor (or a raw int / None).  Nothing else: ctypes would take bytes, strings and ctypes arrays
+    for a pointer, too, and hand the kernels a host address."""
     try:
         return t.data_ptr()
     except AttributeError:
-        return t
+        if t is None or isinstance(t, int):
+            return t
+        raise
 
 
 _current_stream = None

@@ -551,3 +551,13 @@ def test_loading_a_pattern_layer_zeroes_the_weights_of_pruned_taps(tmp_path):
     got = q.view()
     assert np.array_equal(got["val"], want["val"]) and np.array_equal(got["tap_mask"], want["tap_mask"])
     q.free()
+
+
+@pytest.mark.parametrize("host", [b"0123456789abcdef", "text", bytearray(16), np.zeros(16, np.float32), (C.c_float * 16)(), C.c_void_p(256)])
+def test_only_tensors_and_addresses_are_taken_for_device_pointers(host):
+    """ctypes would convert bytes, strings, arrays and its own pointers to the address of host memory."""
+    p = sbnn.pack_weights(np.ones((8, 1, 1, 8), np.float32), np.ones((8, 1, 1, 8), np.uint8), None, 4)
+    with pytest.raises(AttributeError):
+        sbnn.conv1x1_gs(p, host, 512, 1, 1, 1, stream=0)
+    with pytest.raises(AttributeError):
+        sbnn.dwconv3x3(256, None, 512, host, 1, 4, 4, 8, 1, stream=0)
