@@ -369,6 +369,9 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                 __nanosleep(64);
             }
         }
+        // A wait makes the guarded memory visible to the lane that polled; the other lanes get it through this barrier (a vote
+        // orders no memory).
+        __syncwarp();
         return true;
     };
     // this CTA's steps of its tiles

@@ -92,6 +92,18 @@ def test_every_bf16_instance(tile, split):
 
 
 @gpu
+@pytest.mark.parametrize("k,layout", [(1, "nhwc"), (1, "cm"), (3, "nhwc"), (3, "cm")])
+@pytest.mark.parametrize("tile,split", INSTANCES)
+def test_same_bits_on_every_run(k, layout, tile, split):
+    """Stages, images and accumulators change hands hundreds of times in a launch; a reader that ran ahead would show."""
+    d, _, _ = inputs(48, 14, 15, 516, 140, 1, 4, 50) if k == 1 else inputs(*SHAPES_3X3[1][:5], 3, *SHAPES_3X3[1][5:])
+    p = sbnn.pack_weights(d["w"], d["mask"], d["bias"], d["g"])
+    first = run(p, d, layout, tile, split)
+    for _ in range(5):
+        assert np.array_equal(first, run(p, d, layout, tile, split))
+
+
+@gpu
 @pytest.mark.parametrize("cin", [32, 64])
 def test_weights_that_stay_in_shared_memory(cin):
     """One channel tile and no more steps than weight stages: the weights are loaded once and serve every tile."""
