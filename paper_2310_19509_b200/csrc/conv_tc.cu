@@ -334,7 +334,6 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, wg = warp >> 2;
-    grid_dependency_release();
     if (warp == 16 && lane == 0) {
         prefetch_map(&amap);
         prefetch_map(&ymap);
@@ -391,6 +390,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
             Ring ring(SA);
             bool ok = true;
             grid_dependency_wait();                       // X comes from the previous kernel of the stream
+            grid_dependency_release();                    // (only now: the next kernel must not run beside the one before this)
             for (Tiles t(a); t.left() && ok; t.next()) {
                 const int m0 = t.m * T::BM;
                 int px = 0, py = 0, pn = 0;
@@ -425,8 +425,10 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
             if (!ok) ring.settle(xfull, false);
         } else if (warp == 17) {
             // ---------------- weight copies ----------------
+            // The first round of stages is filled while the previous kernel of the stream drains.  No bounded wait starts before
+            // that kernel is done, here and in the warps below: its time must not count.
             Ring ring(SB);
-            bool ok = true;
+            bool ok = true, alone = false;
             for (Tiles t(a); t.left() && ok; t.next()) {
                 const int nt = t.n * NU;
                 const int batch = SB >= 4 ? NU : 1;         // as above
@@ -435,6 +437,10 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                         Ring second = ring;
                         second.next();
                         const Ring& mine = lane == 1 && batch == 2 ? second : ring;
+                        if (second.reused() && !alone) {
+                            grid_dependency_wait();
+                            alone = true;
+                        }
                         if (second.reused() && !(ok = wait(bempty + mine.stage, mine.parity ^ 1, mine.reused()))) break;
                         if (elect_one()) {
                             for (int b = 0; b < batch; ++b) {
@@ -460,6 +466,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
             int step = 0, unit = 0;
             Ring ring(SB);
             bool ok = true;
+            grid_dependency_wait();
             // Three images: every step of a column block is a unit with an accumulator of its own, and the warps take turns.
             // One image: a unit is a column block of a tile, warp u takes block u (with one block warp 0 takes all).
             for (Tiles t(a); t.left() && ok; t.next()) {
@@ -521,6 +528,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
             int step = 0;
             Ring ring(SA);
             bool ok = true;
+            grid_dependency_wait();
             for (Tiles t(a); t.left() && ok; t.next()) {
                 int px = 0, py = 0;                         // SRC_CM3: the pixel's place in its image
                 if (T::SRC == SRC_CM3) {

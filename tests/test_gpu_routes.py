@@ -104,6 +104,36 @@ def test_same_bits_on_every_run(k, layout, tile, split):
 
 
 @gpu
+@pytest.mark.parametrize("tile,split", [(64, 1), (64, 4), (256, 1)])
+def test_layers_back_to_back_on_two_buffers(tile, split):
+    """Depthwise and pointwise layers that write in turn what the other has just read, launched without a pause: each may start
+    early, but must not touch a buffer before the launch in front of it, and the one before that, are done with it."""
+    n, hw, c = 2, 14, 512
+    d, _, _ = inputs(n, hw, hw, c, c, 1, 4, 50)
+    p = sbnn.pack_weights(d["w"], d["mask"], d["bias"], 4)
+    m = n * hw * hw
+    dw_w, dw_b = torch.randn((3, 3, c), device="cuda") / 3, torch.zeros(c, device="cuda")
+    first = torch.rand((c, m), device="cuda")
+
+    def chain(pause):
+        a, b = first.clone(), torch.zeros((c, m), device="cuda")
+        for _ in range(12):
+            sbnn.dwconv3x3_cm(dw_w, dw_b, a, m, b, m, n, hw, hw, c, 1)
+            if pause:
+                torch.cuda.synchronize()
+            sbnn.debug_conv_gs(p, b, m, a, m, n, hw, hw, sbnn.SBNN_RELU | sbnn.SBNN_OUT_CM, tile, split)
+            if pause:
+                torch.cuda.synchronize()
+        return a
+
+    want = chain(True)
+    assert bool(torch.isfinite(want).all()) and float(want.abs().max()) > 0
+    for _ in range(20):
+        assert torch.equal(chain(False), want)
+    sbnn.get_async_status()
+
+
+@gpu
 @pytest.mark.parametrize("cin", [32, 64])
 def test_weights_that_stay_in_shared_memory(cin):
     """One channel tile and no more steps than weight stages: the weights are loaded once and serve every tile."""
