@@ -166,7 +166,8 @@ sbnn_status finish_packed(sbnn_packed* p, sbnn_packed** out) {
         p->block_idx.clear();
     }
     // (the difference of a value with itself is 0 unless the value is an infinity or a NaN)
-    p->finite = std::all_of(p->val.begin(), p->val.end(), [](float v) { return v - v == 0.0f; });
+    const auto finite = [](float v) { return v - v == 0.0f; };
+    p->finite = std::all_of(p->val.begin(), p->val.end(), finite) && std::all_of(p->bias.begin(), p->bias.end(), finite);
     int ndev = 0, dev = 0;
     if (cudaGetDeviceCount(&ndev) != cudaSuccess || ndev == 0 || cudaGetDevice(&dev) != cudaSuccess) {
         cudaGetLastError();

@@ -247,3 +247,20 @@ def test_the_library_s_own_choice():
     assert np.all(np.abs(y.cpu().numpy().astype(np.float64) - ref) <= 1e-5 * s)
     sbnn.conv1x1_gs(p, x, y, 7, 61, 63, 0)
     assert sbnn.debug_last_route()[0] != 0
+
+
+@gpu
+@pytest.mark.parametrize("value", [-np.inf, np.inf, np.nan])
+def test_a_bias_that_is_not_finite_costs_nothing(value):
+    """A channel switched off by its bias: the layer runs on the FMA kernels, where such a bias is a number like any other (on
+    the tensor cores it would look like a bad activation in every pixel, and have every pixel summed again)."""
+    d, ref, s = inputs(7, 61, 63, 64, 124, 1, 4, 50)
+    bias = d["bias"].copy()
+    bias[0] = value
+    p = sbnn.pack_weights(d["w"], d["mask"], bias, 4)
+    x, y = torch.from_numpy(d["x"]).cuda(), torch.empty(ref.shape, device="cuda")
+    sbnn.conv1x1_gs(p, x, y, 7, 61, 63, 0)
+    assert sbnn.debug_last_route() == (0, 0)
+    got = y.cpu().numpy()
+    assert np.array_equal(got[..., 0], np.full(got.shape[:-1], value, np.float32), equal_nan=True)
+    assert np.all(np.abs(got[..., 1:].astype(np.float64) - ref[..., 1:]) <= 1e-5 * s[..., 1:])
