@@ -59,7 +59,7 @@ constexpr double kTruncation = 1.0 + 5.4e-8;
 enum Source { SRC_NHWC, SRC_CM, SRC_IM2COL, SRC_CM3 };
 
 // Element strides of the activations and the arrays of the packed layer, for the outputs of pixels that hold a
-// non-finite value (see exact_pixel).
+// non-finite value (see sum_kept_units).
 struct ExactArgs {
     const float* x;
     long long pixel_stride, channel_stride;
@@ -238,26 +238,163 @@ __device__ __forceinline__ void im2col_g2s(void* dst_smem, const void* map, int 
                  : "memory");
 }
 
-// The outputs [n0, n1) of pixel m as a plain FMA chain over the kept units.  A pixel with an infinity or a NaN in any
-// channel spoils all its split products (0 * inf), also those of pruned weights, which must not see it; such pixels are
-// recomputed here and written over.
+// The 256 drain threads: a barrier among them, and whether any of them says so.
+__device__ __forceinline__ bool drain_any(bool mine) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 p, %1, 0;\n\t"
+        "barrier.cta.red.or.pred q, 1, 256, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"((uint32_t)mine)
+        : "memory");
+    return r != 0;
+}
+
+// All drain threads: sums pixels of the tile that starts at m0 once more, as fp32 FMAs over the kept units.  A pixel with an
+// infinity or a NaN in any channel spoils all its split products (0 * inf), also those of pruned weights, which must not see
+// it.  `bad` says which of the pixels m0 + 32 * q + lane (q = the warp's place in its warpgroup); a warpgroup wg has `len`
+// outputs from n0 + wg * T::COLS on.
+// Up to 32 pixels at a time go into shared memory, a row for every (channel, tap), and PS lanes of a warp take a pixel each,
+// the others share its units; a warp takes four outputs at a time.  Sums that span several stages of rows wait in `sums`.
+// Bound by the latency of the reads of 8 warps.  6 x 25 x 31, 1024 -> 516, half pruned, with three bad pixels: 89 us (a thread
+// a pixel, in the middle of the tile loop: 2800; the FMA kernels: 89); with a bad channel in every pixel: 372 us (9600; 88), or
+// 2500 with the activations read from global memory.
 template <class T>
-__device__ __noinline__ void exact_pixel(const TcArgs& a, int m, int n0, int n1) {
-    const ExactArgs& e = a.ex;
-    const int px = T::TAPS == 9 ? m % a.W : 0, py = T::TAPS == 9 ? (m / a.W) % a.H : 0;
-    for (int n = n0; n < n1; ++n) {
-        const int g = n / e.G, r = n % e.G;
-        float s = 0.0f;
-        for (int j = e.group_ptr[g]; j < e.group_ptr[g + 1]; ++j)
-            for (int t = 0; t < T::TAPS; ++t) {
-                const int dy = T::TAPS == 9 ? t / 3 - 1 : 0, dx = T::TAPS == 9 ? t % 3 - 1 : 0;
-                if (T::TAPS == 9 && (px + dx < 0 || px + dx >= a.W || py + dy < 0 || py + dy >= a.H)) continue;
-                const long long p = (long long)m + dy * a.W + dx;
-                s = fmaf(e.val[((size_t)j * T::TAPS + t) * e.G + r], e.x[p * e.pixel_stride + e.idx[j] * e.channel_stride], s);
+__device__ __noinline__ void sum_kept_units(const TcArgs& args, unsigned char* room, float* sums, int m0, bool bad, int n0, int len) {
+    const ExactArgs e = args.ex;
+    const int W = args.W, H = args.H, Cin = args.Cin, Cout = args.Cout, relu = args.relu, ldy = args.ldy;
+    float* const y = args.y;
+    const float* const bias = args.bias;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, width = e.G < 4 ? e.G : 4;
+    constexpr bool CM = T::SRC == SRC_CM || T::SRC == SRC_CM3;
+    uint32_t* const found = reinterpret_cast<uint32_t*>(room);
+    int* const list = reinterpret_cast<int*>(room + 64);
+    int* const where = reinterpret_cast<int*>(room + 1024) + warp * 32;        // 32 (unit, tap) pairs of a warp: place of the row,
+    float4* const weight = reinterpret_cast<float4*>(room + 2048) + warp * 32;  // and the weights of its four outputs
+    float* const rows = reinterpret_cast<float*>(room + 6144);
+    const int capacity = (args.sb * T::B_BYTES + args.sa * T::A_BYTES - 6144) / 4;
+
+    drain_any(false);                                          // nobody still uses the room
+    if (tid < 4) found[tid] = 0;
+    drain_any(false);
+    const uint32_t mine = __ballot_sync(0xffffffffu, bad);
+    if (lane == 0 && mine) atomicOr(found + (warp & 3), mine);
+    drain_any(false);
+    int count = 0;
+    for (int q = 0; q < 4; ++q) {
+        const uint32_t word = found[q];
+        if (warp == 0 && (word >> lane & 1)) list[count + __popc(word & ((1u << lane) - 1))] = m0 + q * 32 + lane;
+        count += __popc(word);
+    }
+    for (int first = 0; first < count; first += 32) {
+        const int pixels = min(32, count - first);
+        int PS = 1;
+        while (PS < pixels) PS *= 2;
+        const int p = lane & (PS - 1), us = 32 / PS, u = lane / PS;
+        const int stage = capacity / PS / T::TAPS;             // channels at a time
+        for (int c0 = 0; c0 < Cin; c0 += stage) {
+            const int c1 = min(Cin, c0 + stage);
+            drain_any(false);
+            // A row holds PS pixels, each moved by the channel's number so that neighbouring channels fall into different banks;
+            // eight loads of a thread are in flight.  NHWC: a warp reads the channels of a pixel's tap, channel-major: pixels.
+            auto place = [&](int c, int t, int i) { return rows + ((c - c0) * T::TAPS + t) * PS + (i ^ (c & (PS - 1))); };
+            auto source = [&](int i, int t) {                  // of channel 0; NULL outside the image
+                const int m = list[first + i], dy = T::TAPS == 9 ? t / 3 - 1 : 0, dx = T::TAPS == 9 ? t % 3 - 1 : 0;
+                const bool in = T::TAPS == 1 || ((unsigned)(m % W + dx) < (unsigned)W && (unsigned)(m / W % H + dy) < (unsigned)H);
+                return in ? e.x + ((long long)m + dy * W + dx) * e.pixel_stride : nullptr;
+            };
+            float v[8];
+            if (CM) {
+                for (int t = 0; t < T::TAPS; ++t) {
+                    const float* const x = p < pixels ? source(p, t) : nullptr;
+                    for (int c = c0 + warp * us + u; c < c1; c += 64 * us) {
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) v[k] = x && c + 8 * us * k < c1 ? x[(c + 8 * us * k) * e.channel_stride] : 0.0f;
+#pragma unroll
+                        for (int k = 0; k < 8; ++k)
+                            if (c + 8 * us * k < c1) *place(c + 8 * us * k, t, p) = v[k];
+                    }
+                }
+            } else {
+                for (int r = warp; r < PS * T::TAPS; r += 8) {
+                    const int i = r / T::TAPS, t = r % T::TAPS;
+                    const float* const x = i < pixels ? source(i, t) : nullptr;
+                    for (int c = c0 + lane; c < c1; c += 256) {
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) v[k] = x && c + 32 * k < c1 ? x[c + 32 * k] : 0.0f;
+#pragma unroll
+                        for (int k = 0; k < 8; ++k)
+                            if (c + 32 * k < c1) *place(c + 32 * k, t, i) = v[k];
+                    }
+                }
             }
-        s += a.bias[n];
-        if (a.relu) s = fmaxf(s, 0.0f);
-        a.y[T::OUT_CM ? (size_t)n * a.ldy + m : (size_t)m * a.ldy + n] = s;
+            drain_any(false);
+            const int chunks = 2 * len / width;
+            for (int i = warp; i < chunks; i += 8) {
+                const int wg = i * width / len, n = n0 + wg * T::COLS + i * width - wg * len;
+                if (n >= Cout) continue;
+                const int g = n / e.G;
+                auto first_unit = [&](int c) {                 // of the group, with a channel from c on
+                    int lo = e.group_ptr[g], hi = e.group_ptr[g + 1];
+                    while (lo < hi) {
+                        const int mid = (lo + hi) / 2;
+                        if (e.idx[mid] < c) lo = mid + 1; else hi = mid;
+                    }
+                    return lo;
+                };
+                const int lo = c0 > 0 ? first_unit(c0) : e.group_ptr[g], hi = c1 < Cin ? first_unit(c1) : e.group_ptr[g + 1];
+                const int items = (hi - lo) * T::TAPS;
+                const float* const v = e.val + (size_t)lo * T::TAPS * e.G + n % e.G;
+                float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                int c = 0;
+                float4 w = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                auto fetch = [&](int item) {                   // a lane's pair of the next 32, while the others are added up
+                    if (item >= items) return;
+                    c = e.idx[lo + item / T::TAPS];
+                    const float* from = v + (size_t)item * e.G;
+                    if (width == 4) w = __ldg(reinterpret_cast<const float4*>(from));
+                    else w = make_float4(__ldg(from), width > 1 ? __ldg(from + 1) : 0.0f, 0.0f, 0.0f);
+                };
+                fetch(lane);
+                for (int i0 = 0; i0 < items; i0 += 32) {
+                    const int limit = min(32, items - i0);
+                    __syncwarp();
+                    where[lane] = (((c - c0) * T::TAPS + (i0 + lane) % T::TAPS) * PS) | (c & (PS - 1));
+                    weight[lane] = w;
+                    __syncwarp();
+                    fetch(i0 + 32 + lane);
+                    auto add = [&](int k) {
+                        const float4 w = weight[k];
+                        const float x = rows[where[k] ^ p];
+                        s[0] = fmaf(w.x, x, s[0]); s[1] = fmaf(w.y, x, s[1]); s[2] = fmaf(w.z, x, s[2]); s[3] = fmaf(w.w, x, s[3]);
+                    };
+                    if (us == 1 && limit == 32) {
+#pragma unroll
+                        for (int k = 0; k < 32; ++k) add(k);
+                    } else {
+                        for (int k = u; k < limit; k += us) add(k);
+                    }
+                }
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    if (r >= width) break;
+                    for (int d = PS; d < 32; d *= 2) s[r] += __shfl_xor_sync(0xffffffffu, s[r], d);
+                    float* const sum = sums + (i * width + r) * 32 + p;
+                    if (lane >= pixels) continue;              // (u > 0 or no pixel)
+                    if (c0 > 0) s[r] += *sum;
+                    if (c1 < Cin) {
+                        *sum = s[r];
+                    } else {
+                        const int m = list[first + p];
+                        float out = s[r] + bias[n + r];
+                        if (relu) out = fmaxf(out, 0.0f);
+                        y[T::OUT_CM ? (size_t)(n + r) * ldy + m : (size_t)m * ldy + n + r] = out;
+                    }
+                }
+            }
+        }
     }
 }
 
@@ -266,9 +403,11 @@ __device__ __noinline__ void exact_pixel(const TcArgs& a, int m, int n0, int n1)
 // their shared memory, [sender][chunk][thread], and then adds up and stores its own.  The weight stages hold the exchange:
 // every CTA's MMAs are complete when its drain threads reach the first barrier.
 template <class T>
-__device__ __forceinline__ void store_shared_tile(const TcArgs& a, uint64_t (&acc)[T::COLS / 2], uint32_t exchange, const unsigned char* mine, int m,
-                                                  int n0, int tid) {
+__device__ __forceinline__ void store_shared_tile(const TcArgs& a, uint64_t (&acc)[T::COLS / 2], unsigned char* room, float* sums, int m0, int tid) {
     constexpr int CHUNKS = T::COLS / 4;
+    const uint32_t exchange = smem_u32(room);
+    const unsigned char* const mine = room;
+    const int m = m0 + (tid & 127), n00 = blockIdx.x / a.split % a.ntiles_n * T::BN, n0 = n00 + (tid >> 7) * T::COLS;
     const int rank = (int)cluster_rank(), own = CHUNKS / a.split;
     __syncwarp();
     cluster_sync();
@@ -309,7 +448,8 @@ __device__ __forceinline__ void store_shared_tile(const TcArgs& a, uint64_t (&ac
             }
         }
     }
-    if (T::IMAGES == 3 && redo && m < a.M) exact_pixel<T>(a, m, n0 + rank * own * 4, min(n0 + (rank + 1) * own * 4, a.Cout));
+    redo = redo && m < a.M;
+    if (T::IMAGES == 3 && drain_any(redo)) sum_kept_units<T>(a, room, sums, m0, redo, n00 + rank * own * 4, own * 4);
 }
 
 template <class T>
@@ -606,7 +746,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
         const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16);
         unsigned char* stage = ost + (size_t)warp * 4096;
         int step = 0, copies = 0;                           // copies issued: the two tiles alternate between them
-        bool ok = true;
+        bool ok = true, again = false;                      // again: some pixels have to be summed once more
         grid_dependency_wait();                             // Y may still be read by the previous kernel of the stream
         for (Tiles t(a); t.left() && ok; t.next()) {
             const int m0 = t.m * T::BM, n0 = t.n * BN + wg * T::COLS;
@@ -638,7 +778,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                 if (lane == 0) mbar_arrive(dempty + d);
             }
             if (T::SPLIT) {
-                store_shared_tile<T>(a, acc, smem_u32(bst), bst, m0 + q * 32 + lane, n0, tid);
+                store_shared_tile<T>(a, acc, bst, reinterpret_cast<float*>(ost), m0, tid);
                 break;
             }
             if (!ok) break;
@@ -646,6 +786,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
             float first, unused;
             unpack2(acc[0], first, unused);
             const bool redo = T::IMAGES == 3 && m < a.M && !(fabsf(first) <= 3.402823466e38f);
+            again |= __any_sync(0xffffffffu, redo);
             // 32 pixels x 16 channels at a time through one of the warp's two staging tiles, stored by tiled copies: rows of 32
             // pixels (channel-major) or of 16 channels (64-byte swizzle).  Rows past Cout or M are clipped by the copy; the last
             // pixels of a channel-major row are stored one by one, so that the padding behind them is left alone.
@@ -662,6 +803,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
 #pragma unroll
                         for (int i = 0; i < 16; ++i) o[i] = fmaxf(o[i], 0.0f);
                     }
+                    if (c0 == 0 && redo) o[0] = __int_as_float(0x7fffffff);   // marks the pixel for the second look below
                     if (T::OUT_CM && mw + 32 > a.M) {
 #pragma unroll
                         for (int i = 0; i < 16; ++i)
@@ -688,13 +830,20 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                     }
                 }
             }
-            if (__any_sync(0xffffffffu, redo)) {
-                if (elect_one()) bulk_wait_all();
-                __syncwarp();
-                if (redo) exact_pixel<T>(a, m, n0, min(n0 + T::COLS, a.Cout));
-            }
         }
         if (elect_one()) bulk_wait_all();                   // this thread's copies are complete before the CTA gives up its shared memory
+        // Pixels that hold an infinity or a NaN: only now, when no warp of the CTA is left in a bounded wait for these.
+        if (T::IMAGES == 3 && !T::SPLIT && drain_any(again && ok)) {
+            for (Tiles t(a); t.left(); t.next()) {
+                const int m = t.m * T::BM + q * 32 + lane, n0 = t.n * BN + wg * T::COLS;
+                bool bad = false;
+                if (n0 < a.Cout && m < a.M) {
+                    const float mark = __ldcg(a.y + (T::OUT_CM ? (size_t)n0 * a.ldy + m : (size_t)m * a.ldy + n0));
+                    bad = mark != mark;
+                }
+                if (drain_any(bad)) sum_kept_units<T>(a, bst, reinterpret_cast<float*>(ost), t.m * T::BM, bad, t.n * BN, T::COLS);
+            }
+        }
     }
     // common exit: nobody may still be using the tensor memory when it is released
     tc_fence_before_sync();

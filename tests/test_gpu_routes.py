@@ -264,3 +264,71 @@ def test_a_bias_that_is_not_finite_costs_nothing(value):
     got = y.cpu().numpy()
     assert np.array_equal(got[..., 0], np.full(got.shape[:-1], value, np.float32), equal_nan=True)
     assert np.all(np.abs(got[..., 1:].astype(np.float64) - ref[..., 1:]) <= 1e-5 * s[..., 1:])
+
+
+# ---- infinities, NaN and sums beyond fp32 ------------------------------------------------------------------------------
+def same_kind(got, want, s):
+    """NaN where `want` (the FMA kernels' result) has NaN, the same infinities, the rest within both kernels' bounds."""
+    assert np.array_equal(np.isnan(got), np.isnan(want))
+    assert np.array_equal(got[np.isinf(want)], want[np.isinf(want)])
+    f = np.isfinite(want)
+    assert np.all(np.abs(got[f].astype(np.float64) - want[f]) <= 2e-5 * s[f])
+
+
+def spoil(x, how):
+    rng = np.random.default_rng(5)
+    x = x.copy().reshape(-1, x.shape[-1])
+    if how == "all":
+        x[:] = np.nan
+    elif how == "one per pixel":
+        x[np.arange(len(x)), rng.integers(0, x.shape[1], len(x))] = np.inf
+    elif how == "both signs":
+        bad = rng.random(x.shape) < 0.01
+        x[bad] = np.where(rng.random(x.shape) < 0.5, np.inf, -np.inf)[bad]
+    else:
+        x[len(x) // 3, 1], x[len(x) // 2, 0], x[-1, -1] = np.nan, np.inf, -np.inf
+    return x
+
+
+@gpu
+@pytest.mark.parametrize("how", ["three", "one per pixel", "both signs", "all"])
+@pytest.mark.parametrize("k,layout,tile,split", [(1, "nhwc", 256, 1), (1, "cm-cm", 128, 1), (1, "cm", 64, 4), (3, "nhwc", 128, 1), (3, "cm-cm", 64, 1),
+                                                 (3, "nhwc", 64, 8)])
+def test_bad_activations_spoil_what_they_touch_and_little_time(k, layout, tile, split, how):
+    """The same outputs are infinite or NaN as on the FMA kernels, the others keep their values, and the call does not take
+    many times what it takes there (at most seven times, when every pixel has a bad channel; summed by a thread a pixel it was a hundred times)."""
+    n, h, w, cin, cout, g = (6, 25, 31, 1024, 516, 4) if k == 1 else (12, 28, 27, 260, 136, 8)
+    if split > 1:
+        n, h, w = 1, 17, 19
+    d = WL.single_conv_inputs(n, h, w, cin, cout, k, g, 50, 11, 0.05, 0.05)
+    p = sbnn.pack_weights(d["w"], d["mask"], d["bias"], g)
+    d = dict(d, x=spoil(d["x"], how).reshape(d["x"].shape))
+    want = run(p, d, layout, 0, 1)
+    s = np.broadcast_to(np.abs(d["bias"]) + np.abs(d["w"] * d["mask"]).reshape(cout, -1).sum(1), want.shape)      # (activations are below 1)
+    for flags in (0, sbnn.SBNN_RELU):
+        same_kind(run(p, d, layout, tile, split, flags), np.fmax(want, 0) if flags else want, s)
+    m = n * h * w
+    xt = torch.from_numpy(d["x"].reshape(m, cin)).cuda()
+    cm = layout != "nhwc"
+    ld = (m + 3) // 4 * 4
+    x = torch.zeros((cin, ld), device="cuda") if cm else xt
+    if cm:
+        x[:, :m] = xt.T
+    y = torch.empty(max(ld, m) * cout, device="cuda")
+    ldy = (ld if layout == "cm-cm" else cout) if cm else 0
+
+    def us(tile, split):
+        best = 1e30
+        for _ in range(3):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            sbnn.debug_conv_gs(p, x, ld if cm else 0, y, ldy, n, h, w, sbnn.SBNN_OUT_CM if layout == "cm-cm" else 0, tile, split)
+            b.record()
+            b.synchronize()
+            best = min(best, 1e3 * a.elapsed_time(b))
+        return best
+
+    base, bad = us(0, 1), us(tile, split)
+    print(f"{k} {layout} {tile} {split} {how}: FMA {base:.0f} us, tensor cores {bad:.0f} us")
+    assert bad <= 10 * base
+    sbnn.get_async_status()
