@@ -140,6 +140,7 @@ struct sbnn_packed {
     int32_t* d_idx = nullptr;
     float* d_val = nullptr;
     float* d_bias = nullptr;
+    uint16_t* d_taps = nullptr;           // tap_mask; NULL unless packed with tap patterns
     // kernel-private layouts, built on first use of a tile configuration
     mutable std::mutex mu;
     mutable std::map<sbnn::TileCfg, sbnn::Stream1x1> streams1x1;
@@ -208,8 +209,9 @@ sbnn_status conv1x1_bf16(const sbnn_packed* w, const float* x, float* y, int M, 
 void free_stream_bf16(sbnn_packed* p);
 // True when the pipelined 1x1 kernel would get fewer tiles than half the SMs (the few-pixel kernel runs then).
 bool conv1x1_few_tiles(const sbnn_packed* p, long long M);
-// Taps kept over all units of a pattern layer.
+// Taps kept over all units of a pattern layer, and whether its pruned taps are left out (few kept) or multiplied as zeros.
 long long count_kept_taps(const sbnn_packed* p);
+bool use_tap_lists(const sbnn_packed* p);
 // conv_tc.cu: fp32 layers on the tensor cores by a three-way bf16 split; *done = false (and SBNN_OK) when the shape or the
 // density is better served by the FMA kernels (or outside what the kernel takes)
 sbnn_status conv1x1_tc(const sbnn_packed* p, const float* x, float* y, long long M, int relu, cudaStream_t st, bool* done);

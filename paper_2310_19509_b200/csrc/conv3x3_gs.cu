@@ -755,13 +755,6 @@ int sm_count3() {
     return it->second;
 }
 
-// True if a layer packed with kernel patterns should run the tap-list kernel: a listed tap costs about 60 us per "every
-// kept kernel, one tap" on config 4's shape, the whole-kernel loop with two output rows per lane about 35 us per tap
-// including the pruned ones (their stored weights are zeros), so lists pay below about five kept taps per kernel.
-bool use_tap_lists(const sbnn_packed* p) {
-    return !p->tap_mask.empty() && (double)count_kept_taps(p) < 4.8 * (double)p->tap_mask.size();
-}
-
 int pow2_ceil(int v) {
     int p = 1;
     while (p < v) p <<= 1;
@@ -1271,6 +1264,13 @@ long long count_kept_taps(const sbnn_packed* p) {
         p->kept_taps = n;
     }
     return p->kept_taps;
+}
+
+// True if a layer packed with kernel patterns should run the tap-list kernel: a listed tap costs about 60 us per "every
+// kept kernel, one tap" on config 4's shape, the whole-kernel loop with two output rows per lane about 35 us per tap
+// including the pruned ones (their stored weights are zeros), so lists pay below about five kept taps per kernel.
+bool use_tap_lists(const sbnn_packed* p) {
+    return !p->tap_mask.empty() && (double)count_kept_taps(p) < 4.8 * (double)p->tap_mask.size();
 }
 
 sbnn_status prepare_default_3x3(const sbnn_packed*) { return SBNN_OK; }  // the re-layout depends on the image width

@@ -66,6 +66,7 @@ struct ExactArgs {
     const int32_t* group_ptr;
     const int32_t* idx;
     const float* val;
+    const uint16_t* taps;  // of the kept units, where the FMA kernels leave pruned taps out; else NULL
     int G;
 };
 
@@ -353,6 +354,7 @@ __device__ __noinline__ void sum_kept_units(const TcArgs& args, unsigned char* r
                 auto fetch = [&](int item) {                   // a lane's pair of the next 32, while the others are added up
                     if (item >= items) return;
                     c = e.idx[lo + item / T::TAPS];
+                    if (T::TAPS == 9 && e.taps && !(e.taps[lo + item / T::TAPS] >> item % T::TAPS & 1)) c = -1;
                     const float* from = v + (size_t)item * e.G;
                     if (width == 4) w = __ldg(reinterpret_cast<const float4*>(from));
                     else w = make_float4(__ldg(from), width > 1 ? __ldg(from + 1) : 0.0f, 0.0f, 0.0f);
@@ -361,11 +363,12 @@ __device__ __noinline__ void sum_kept_units(const TcArgs& args, unsigned char* r
                 for (int i0 = 0; i0 < items; i0 += 32) {
                     const int limit = min(32, items - i0);
                     __syncwarp();
-                    where[lane] = (((c - c0) * T::TAPS + (i0 + lane) % T::TAPS) * PS) | (c & (PS - 1));
+                    where[lane] = c < 0 ? -1 : (((c - c0) * T::TAPS + (i0 + lane) % T::TAPS) * PS) | (c & (PS - 1));
                     weight[lane] = w;
                     __syncwarp();
                     fetch(i0 + 32 + lane);
                     auto add = [&](int k) {
+                        if (T::TAPS == 9 && where[k] < 0) return;
                         const float4 w = weight[k];
                         const float x = rows[where[k] ^ p];
                         s[0] = fmaf(w.x, x, s[0]); s[1] = fmaf(w.y, x, s[1]); s[2] = fmaf(w.z, x, s[2]); s[3] = fmaf(w.w, x, s[3]);
@@ -1093,7 +1096,7 @@ sbnn_status launch_tc(const sbnn_packed* p, const TcCall& c, int split, bool* do
     a.steps = (p->Cin + 63) / 64 * T::TAPS; a.ntiles_m = (int)((c.M + T::BM - 1) / T::BM); a.ntiles_n = (int)ntiles_n;
     a.W = c.W; a.H = c.H; a.relu = c.relu; a.split = T::SPLIT ? split : 1;
     const bool cm = T::SRC == SRC_CM || T::SRC == SRC_CM3;
-    a.ex = {c.x, cm ? 1 : p->Cin, cm ? c.ldx : 1, p->d_group_ptr, p->d_idx, p->d_val, p->G};
+    a.ex = {c.x, cm ? 1 : p->Cin, cm ? c.ldx : 1, p->d_group_ptr, p->d_idx, p->d_val, use_tap_lists(p) ? p->d_taps : nullptr, p->G};
     CUtensorMap amap, ymap;
     if (T::SRC == SRC_IM2COL) {
         if ((r = encode_im2col_3x3_map(&amap, c.x, c.N, c.H, c.W, p->Cin, T::SUB, T::BM)) != SBNN_OK) return r;

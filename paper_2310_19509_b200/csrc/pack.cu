@@ -177,7 +177,8 @@ sbnn_status finish_packed(sbnn_packed* p, sbnn_packed** out) {
     sbnn_status st = SBNN_OK;
     p->device = dev;
     if ((st = upload(&p->d_group_ptr, p->group_ptr)) != SBNN_OK || (st = upload(&p->d_idx, p->idx)) != SBNN_OK ||
-        (st = upload(&p->d_val, p->val)) != SBNN_OK || (st = upload_bias(p)) != SBNN_OK) {
+        (st = upload(&p->d_val, p->val)) != SBNN_OK || (st = upload_bias(p)) != SBNN_OK ||
+        (!p->tap_mask.empty() && (st = upload(&p->d_taps, p->tap_mask)) != SBNN_OK)) {
         sbnn_packed_free(p);
         return st;
     }
@@ -482,6 +483,7 @@ extern "C" sbnn_status sbnn_packed_free(sbnn_packed* p) {
         cudaFree(p->d_idx);
         cudaFree(p->d_val);
         cudaFree(p->d_bias);
+        cudaFree(p->d_taps);
         if (sw) cudaSetDevice(cur);
         cudaGetLastError();
     }

@@ -332,3 +332,17 @@ def test_bad_activations_spoil_what_they_touch_and_little_time(k, layout, tile, 
     print(f"{k} {layout} {tile} {split} {how}: FMA {base:.0f} us, tensor cores {bad:.0f} us")
     assert bad <= 10 * base
     sbnn.get_async_status()
+
+
+@gpu
+@pytest.mark.parametrize("taps", [4, 7])
+@pytest.mark.parametrize("layout,tile,split", [("nhwc", 128, 1), ("cm-cm", 64, 1), ("nhwc", 64, 4)])
+def test_bad_activations_under_pruned_taps(layout, tile, split, taps):
+    """What a pruned tap sees: nothing in layers that run from tap lists (4 taps), its product with zero in others (7)."""
+    d, _, s = inputs(6, 28, 28, 40, 64, 3, 4, 30)
+    d = dict(d, mask=tap_pattern_mask(2, 19, d["mask"][::4, 0, 0, :].astype(bool), 4, taps), x=spoil(d["x"], "one per pixel").reshape(d["x"].shape))
+    d["x"].reshape(-1, 40)[::3] = 0.25
+    p = sbnn.pack_weights(d["w"], d["mask"], d["bias"], 4, tap_patterns=True)
+    want = run(p, d, layout, 0, 1)
+    assert np.isfinite(want).any() and not np.isfinite(want).all()
+    same_kind(run(p, d, layout, tile, split), want, s.reshape(want.shape))
