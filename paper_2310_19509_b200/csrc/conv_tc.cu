@@ -255,7 +255,7 @@ __device__ __forceinline__ bool drain_any(bool mine) {
 
 // All drain threads: sums pixels of the tile that starts at m0 once more, as fp32 FMAs over the kept units.  A pixel with an
 // infinity or a NaN in any channel spoils all its split products (0 * inf), also those of pruned weights, which must not see
-// it.  `bad` says which of the pixels m0 + 32 * q + lane (q = the warp's place in its warpgroup); a warpgroup wg has `len`
+// it; and sums near the end of the fp32 range may overflow here but not product after product with the bias last, as on the FMA kernels.  `bad` says which of the pixels m0 + 32 * q + lane (q = the warp's place in its warpgroup); a warpgroup wg has `len`
 // outputs from n0 + wg * T::COLS on.
 // Up to 32 pixels at a time go into shared memory, a row for every (channel, tap), and PS lanes of a warp take a pixel each,
 // the others share its units; a warp takes four outputs at a time.  Sums that span several stages of rows wait in `sums`.
@@ -436,7 +436,7 @@ __device__ __forceinline__ void store_shared_tile(const TcArgs& a, uint64_t (&ac
             }
             v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
         }
-        redo |= !(fabsf(v.x) <= 3.402823466e38f);
+        redo |= !(fmaf(v.x, 0.f, fmaf(v.y, 0.f, fmaf(v.z, 0.f, v.w * 0.f))) == 0.f);
         if (a.relu) v = make_float4(fmaxf(v.x, 0.f), fmaxf(v.y, 0.f), fmaxf(v.z, 0.f), fmaxf(v.w, 0.f));
         const int n = n0 + 4 * c;
         if (m < a.M && n < a.Cout) {
@@ -786,9 +786,17 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
             }
             if (!ok) break;
             const int m = m0 + q * 32 + lane;
-            float first, unused;
-            unpack2(acc[0], first, unused);
-            const bool redo = T::IMAGES == 3 && m < a.M && !(fabsf(first) <= 3.402823466e38f);
+            // Any sum that is not finite: a bad activation spoils them all, an overflow on the way, which another order of the
+            // additions may not have, only its own.  (0 * sum is NaN then, and stays it.)
+            bool redo = false;
+            if (T::IMAGES == 3) {
+                f32x2 probe[4] = {0, 0, 0, 0};
+                float lo, hi;
+#pragma unroll
+                for (int i = 0; i < T::COLS / 2; ++i) fma2(probe[i & 3], acc[i], 0);
+                unpack2(add2(add2(probe[0], probe[1]), add2(probe[2], probe[3])), lo, hi);
+                redo = m < a.M && !(lo + hi == 0.0f);
+            }
             again |= __any_sync(0xffffffffu, redo);
             // 32 pixels x 16 channels at a time through one of the warp's two staging tiles, stored by tiled copies: rows of 32
             // pixels (channel-major) or of 16 channels (64-byte swizzle).  Rows past Cout or M are clipped by the copy; the last

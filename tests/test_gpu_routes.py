@@ -346,3 +346,19 @@ def test_bad_activations_under_pruned_taps(layout, tile, split, taps):
     want = run(p, d, layout, 0, 1)
     assert np.isfinite(want).any() and not np.isfinite(want).all()
     same_kind(run(p, d, layout, tile, split), want, s.reshape(want.shape))
+
+
+@gpu
+@pytest.mark.parametrize("layout,tile,split", [("nhwc", 64, 1), ("nhwc", 256, 1), ("cm-cm", 128, 1), ("nhwc", 64, 2)])
+def test_sums_that_overflow_on_the_way(layout, tile, split):
+    """fp32 sums depend on their order near the end of the range: where the tensor cores' order overflows in any channel, the
+    order of the FMA kernels (products ascending, bias last) decides."""
+    d = WL.single_conv_inputs(3, 27, 29, 516, 260, 1, 4, 0, 3, 0.05, 0.05)       # (from 2048 pixels on the NHWC route adds the bias last, too)
+    w, x, bias = np.zeros_like(d["w"]), np.ones_like(d["x"]), np.zeros(260, np.float32)
+    for o in (5, 70, 131, 258):                                # 3e38 + (1e38 - 3e38): not finite from the left
+        w[o, 0, 0, 3], w[o, 0, 0, 300], bias[o] = 1e38, -3e38, 3e38
+    d = dict(d, w=w, x=x, bias=bias)
+    p = sbnn.pack_weights(w, d["mask"], bias, 4)
+    want = run(p, d, layout, 0, 1)
+    assert np.isfinite(want).all()
+    assert np.allclose(run(p, d, layout, tile, split), want, rtol=1e-5, atol=0)
