@@ -30,3 +30,24 @@ def test_matches_the_oracle(n, h, w, c, stride, relu):
     got = y.cpu().numpy()
     assert np.all(np.abs(got.astype(np.float64) - ref) <= 1e-5 * s)
     assert bool(torch.isnan(full[:256]).all()) and bool(torch.isnan(full[-256:]).all())
+
+
+@pytest.mark.parametrize("stride", [1, 2])
+@pytest.mark.parametrize("tap", [0, 1, 2])
+def test_taps_outside_the_image_are_not_multiplied(stride, tap):
+    """An infinite weight in the first or last kernel row: the outputs whose row lies outside the image stay finite, whichever
+    kernel the size selects (one image is too little for the kernel that slides)."""
+    n, h, w, c = 40, 13, 13, 516
+    rng = np.random.default_rng(stride)
+    x = torch.from_numpy(rng.random((n, h, w, c), dtype=np.float32) + np.float32(0.5)).cuda()
+    wt = rng.standard_normal((3, 3, c), dtype=np.float32)
+    wt[tap, 1, ::7] = np.inf
+    wt[tap, 1, 3::7] = np.nan
+    wt, b = torch.from_numpy(wt).cuda(), torch.zeros(c, device="cuda")
+    ho = (h - 1) // stride + 1
+    y, one = torch.empty((n, ho, ho, c), device="cuda"), torch.empty((n, ho, ho, c), device="cuda")
+    sbnn.dwconv3x3(wt, b, x, y, n, h, w, c, stride, 0)
+    for i in range(n):
+        sbnn.dwconv3x3(wt, b, x[i], one[i], 1, h, w, c, stride, 0)
+    assert bool(torch.isfinite(one).any()) and not bool(torch.isfinite(one).all())
+    torch.testing.assert_close(y, one, rtol=1e-5, atol=1e-5, equal_nan=True)
