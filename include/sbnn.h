@@ -501,6 +501,11 @@ SBNN_API sbnn_status sbnn_debug_poke_device_index(sbnn_packed* w, long long unit
 SBNN_API sbnn_status sbnn_debug_last_route(int* tile, int* split);
 SBNN_API sbnn_status sbnn_debug_conv_gs(const sbnn_packed* w, const float* x_dev, int ldx, float* y_dev, int ldy, int N, int H, int W,
                                         int flags, int tile, int split, void* cuda_stream);
+/*
+ * Test hook: from now on the layer's images for the tensor cores are treated as too large for the device where they take more
+ * than `bytes`; calls then run on the FMA kernels.
+ */
+SBNN_API sbnn_status sbnn_debug_limit_images(sbnn_packed* w, long long bytes);
 
 /*
  * Test hook: overwrite the device number recorded in a packed layer, so that the refusal of compute calls

@@ -38,6 +38,7 @@ from .binding import (  # noqa: F401
     debug_check_packed,
     debug_conv_gs,
     debug_last_route,
+    debug_limit_images,
     debug_plan_conv3x3,
     debug_poke_device_index,
     selftest_wait_timeout,

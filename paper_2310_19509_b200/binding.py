@@ -76,6 +76,7 @@ def lib():
         "sbnn_debug_check_packed": [P, P],
         "sbnn_debug_poke_device_index": [P, C.c_longlong, I, P],
         "sbnn_debug_last_route": [P, P],
+        "sbnn_debug_limit_images": [P, C.c_longlong],
         "sbnn_debug_conv_gs": [P, P, I, P, I, I, I, I, I, I, I, P],
         "sbnn_debug_plan_conv3x3": [P, I, I, I, I, P, P, I, P, P, P],
     }
@@ -321,6 +322,11 @@ def debug_last_route():
     tile, split = C.c_int(), C.c_int()
     _check(lib().sbnn_debug_last_route(C.byref(tile), C.byref(split)))
     return tile.value, split.value
+
+
+def debug_limit_images(w: Packed, nbytes):
+    """Test hook: larger images of the layer's weights are treated as too large for the device."""
+    _check(lib().sbnn_debug_limit_images(w.handle, int(nbytes)))
 
 
 def debug_conv_gs(w: Packed, x, ldx, y, ldy, n, h, wd, flags, tile, split=1, stream=None):

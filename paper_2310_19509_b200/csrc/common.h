@@ -150,6 +150,7 @@ struct sbnn_packed {
     mutable std::map<long long, sbnn::Plan3x3> plans3x3;           // per (stream, row tiles of the launch, CTAs)
     mutable void* bf16_stream = nullptr;  // see conv1x1_bf16.cu
     mutable std::map<std::pair<int, int>, void*> tc_weights;  // bf16 images of the masked weights, see conv_tc.cu
+    size_t tc_limit = SIZE_MAX;           // bytes that one of them may take (test hook)
     bool finite = true;                   // every stored weight and bias is finite
     struct TcChoice {                     // tile width (0: the FMA kernels are faster), CTAs that share a tile, estimated cycles
         int bn, split;

@@ -890,7 +890,8 @@ __global__ void build_tc_weights_kernel(const int32_t* __restrict__ group_ptr, c
 }
 
 // Weight images of a layer for MMA column blocks of `nuc` output channels, built on first use; NULL if that would be
-// while `st` is being captured, when nothing can be allocated.
+// while `st` is being captured, when nothing can be allocated, or if the device has no room for them (which is remembered:
+// they take six bytes for every weight of the unpruned layer, many times what is stored of a sparse one).
 sbnn_status get_tc_weights(const sbnn_packed* p, int nuc, int images, cudaStream_t st, uint4** out) {
     std::lock_guard<std::mutex> lk(p->mu);
     *out = nullptr;
@@ -905,8 +906,13 @@ sbnn_status get_tc_weights(const sbnn_packed* p, int nuc, int images, cudaStream
     const int taps = p->KH * p->KW, csteps = (p->Cin + 63) / 64, tiles = (p->Cout + 255) / 256 * 256 / nuc;
     const size_t bytes = (size_t)tiles * csteps * taps * images * nuc * 64 * 2;
     void* d = nullptr;
-    SBNN_CUDA_TRY(cudaMalloc(&d, bytes));
-    cudaError_t e = cudaMemset(d, 0, bytes);
+    cudaError_t e = bytes > p->tc_limit ? cudaErrorMemoryAllocation : cudaMalloc(&d, bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        p->tc_weights[{nuc, images}] = nullptr;
+        return SBNN_OK;
+    }
+    if (e == cudaSuccess) e = cudaMemset(d, 0, bytes);
     if (e == cudaSuccess && p->nnz > 0) {
         build_tc_weights_kernel<<<dim3((unsigned)p->ngroups, 4), 128>>>(p->d_group_ptr, p->d_idx, p->d_val, p->G, taps, csteps, nuc, images,
                                                                        static_cast<__nv_bfloat16*>(d));
@@ -1237,6 +1243,14 @@ extern "C" sbnn_status sbnn_debug_last_route(int* tile, int* split) {
     if (!tile || !split) return fail(SBNN_ERR_NULL, "tile and split must not be NULL");
     *tile = last_route.bn;
     *split = last_route.split;
+    return SBNN_OK;
+}
+
+extern "C" sbnn_status sbnn_debug_limit_images(sbnn_packed* w, long long bytes) {
+    clear_error();
+    if (!w) return fail(SBNN_ERR_NULL, "packed weights must not be NULL");
+    if (bytes < 0) return fail(SBNN_ERR_SHAPE, "bytes must not be negative");
+    w->tc_limit = (size_t)bytes;
     return SBNN_OK;
 }
 

@@ -362,3 +362,26 @@ def test_sums_that_overflow_on_the_way(layout, tile, split):
     want = run(p, d, layout, 0, 1)
     assert np.isfinite(want).all()
     assert np.allclose(run(p, d, layout, tile, split), want, rtol=1e-5, atol=0)
+
+
+@gpu
+@pytest.mark.parametrize("k", [1, 3])
+def test_images_that_do_not_fit_the_device(k):
+    """The images of a sparse layer can be many times its stored weights: without room for them it runs as it is stored."""
+    n, h, w, cin, cout, g, pct = SHAPES_3X3[1] if k == 3 else (7, 61, 63, 100, 516, 4, 30)
+    d, ref, s = inputs(n, h, w, cin, cout, k, g, pct)
+    p = sbnn.pack_weights(d["w"], d["mask"], d["bias"], g)
+    x, y = torch.from_numpy(d["x"]).cuda(), torch.empty(ref.shape, device="cuda")
+    call = sbnn.conv1x1_gs if k == 1 else sbnn.conv3x3_gs
+    call(p, x, y, n, h, w, 0)
+    assert sbnn.debug_last_route()[0] != 0
+    q = sbnn.pack_weights(d["w"], d["mask"], d["bias"], g)
+    sbnn.debug_limit_images(q, 1000)
+    sbnn.prepare(q, n, h, w)
+    call(q, x, y, n, h, w, 0)
+    assert sbnn.debug_last_route() == (0, 0)
+    assert np.all(np.abs(y.cpu().numpy().astype(np.float64) - ref) <= 1e-5 * s)
+    if k == 1:
+        call(q, x, y, n, h, w, sbnn.SBNN_BF16_TC)
+        assert sbnn.debug_last_route() == (0, 0)
+        assert np.all(np.abs(y.cpu().numpy().astype(np.float64) - ref) <= 1e-2 * s)
