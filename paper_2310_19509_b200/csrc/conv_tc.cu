@@ -41,6 +41,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <atomic>
 #include <new>
 
 #include <cuda.h>   // CUtensorMap (type only)
@@ -1091,13 +1092,15 @@ sbnn_status launch_tc(const sbnn_packed* p, const TcCall& c, int split, bool* do
     sbnn_status r = set_max_dyn_smem(reinterpret_cast<const void*>(&conv_tc_kernel<T>), 227 * 1024);
     if (r != SBNN_OK) return r;
     // The warpgroups' register shares add up to LAUNCH_REGS a thread: a build that starts with fewer must not be launched,
-    // since the drain warps would wait for registers that nobody returns.
-    static const int regs = [] {
+    // since the drain warps would wait for registers that nobody returns.  The FMA kernels run then.
+    static std::atomic<int> known{0};
+    int regs = known.load();
+    if (regs == 0) {
         cudaFuncAttributes fa = {};
-        return cudaFuncGetAttributes(&fa, conv_tc_kernel<T>) == cudaSuccess ? fa.numRegs : 0;
-    }();
-    if (regs != T::LAUNCH_REGS)
-        return fail(SBNN_ERR_UNSUPPORTED, "internal: the tensor-core kernel was built with %d registers a thread, not %d", regs, T::LAUNCH_REGS);
+        SBNN_CUDA_TRY(cudaFuncGetAttributes(&fa, conv_tc_kernel<T>));
+        known = regs = fa.numRegs;
+    }
+    if (regs != T::LAUNCH_REGS) return SBNN_OK;
     TcArgs a = {};
     uint4* wts = nullptr;
     if ((r = get_tc_weights(p, T::NUC, T::IMAGES, c.st, &wts)) != SBNN_OK || !wts) return r;
