@@ -160,9 +160,10 @@ SBNN_API sbnn_status sbnn_packed_load(const char* path, sbnn_packed** out);
  * does now everything that sbnn_conv1x1_gs / sbnn_conv1x1_gs_cm (KH = 1) or sbnn_conv3x3_gs (KH = 3) would
  * otherwise do on first use for activations of up to N x H x W pixels with these flags -- builds the kernels'
  * private weight layouts (for the 1x1 case those of every tile shape the library may choose, whatever the
- * pixel count), raises the kernels' shared-memory limits, and grows the per-device scratch buffer to what
- * the NHWC entry points need for this shape (with SBNN_BF16_TC: what the bf16 mode needs).  Allocates and
- * may synchronise; launches nothing; the activation buffers need not exist yet.  Afterwards compute calls of
+ * pixel count, and the images of the unpruned layer's weights, six bytes a weight for every tile
+ * width, where some call would run on the tensor cores), raises the kernels' shared-memory limits, and grows the per-device scratch buffer to what
+ * the NHWC entry points need for this shape (with SBNN_BF16_TC: what the bf16 mode needs).  Allocates,
+ * may launch kernels that lay the weights out, and synchronises; the activation buffers need not exist yet.  Afterwards compute calls of
  * this layer with no more pixels (3x3: the same W) only enqueue.  Call it once per layer and mode, outside
  * any stream capture.  The scratch buffer never shrinks and an outgrown one is kept until the process exits,
  * so a CUDA graph recorded over an entry point stays valid when a later, larger call makes the buffer grow;

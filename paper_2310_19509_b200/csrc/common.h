@@ -150,6 +150,7 @@ struct sbnn_packed {
     mutable std::map<long long, sbnn::Plan3x3> plans3x3;           // per (stream, row tiles of the launch, CTAs)
     mutable void* bf16_stream = nullptr;  // see conv1x1_bf16.cu
     mutable std::map<std::pair<int, int>, void*> tc_weights;  // bf16 images of the masked weights, see conv_tc.cu
+    mutable std::map<int, long long> tc_prepared;             // per number of images: pixels up to which calls build none
     size_t tc_limit = SIZE_MAX;           // bytes that one of them may take (test hook)
     bool finite = true;                   // every stored weight and bias is finite
     struct TcChoice {                     // tile width (0: the FMA kernels are faster), CTAs that share a tile, estimated cycles
@@ -223,8 +224,8 @@ sbnn_status conv3x3_tc_cm(const sbnn_packed* p, const float* x, int ldx, float* 
                           bool* done);
 // bf16 mode as a dense contraction over the masked weights; *done = false if the shape is not taken
 sbnn_status conv1x1_tc_bf16(const sbnn_packed* p, const float* x, float* y, long long M, int relu, cudaStream_t st, bool* done);
-// Builds the weight images for calls of up to M pixels.
-sbnn_status prepare_tc(const sbnn_packed* p, long long M);
+// Builds the weight images that calls of up to M pixels use (one image of every weight: the bf16 mode); such calls build none.
+sbnn_status prepare_tc(const sbnn_packed* p, long long M, int images = 3);
 void free_tc_weights(sbnn_packed* p);
 // conv3x3_gs.cu
 sbnn_status prepare_default_3x3(const sbnn_packed* p);

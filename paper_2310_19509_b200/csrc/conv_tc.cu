@@ -890,10 +890,18 @@ __global__ void build_tc_weights_kernel(const int32_t* __restrict__ group_ptr, c
     }
 }
 
+using TcChoice = sbnn_packed::TcChoice;
+
+// Test hooks (sbnn_debug_conv_gs, sbnn_debug_last_route), for the calling thread: how its calls have to run (bn = 0: on the
+// FMA kernels), and how the latest ran.
+thread_local const TcChoice* forced_choice = nullptr;
+thread_local TcChoice last_route = {0, 0, 0.0};
+
 // Weight images of a layer for MMA column blocks of `nuc` output channels, built on first use; NULL if that would be
-// while `st` is being captured, when nothing can be allocated, or if the device has no room for them (which is remembered:
-// they take six bytes for every weight of the unpruned layer, many times what is stored of a sparse one).
-sbnn_status get_tc_weights(const sbnn_packed* p, int nuc, int images, cudaStream_t st, uint4** out) {
+// in a call of M pixels the layer has been prepared for, which only enqueues, or while `st` is being captured, when nothing
+// can be allocated, or if the device has no room for them (which is remembered: they take six bytes for every weight of the
+// unpruned layer, many times what is stored of a sparse one).
+sbnn_status get_tc_weights(const sbnn_packed* p, int nuc, int images, long long M, cudaStream_t st, uint4** out) {
     std::lock_guard<std::mutex> lk(p->mu);
     *out = nullptr;
     auto it = p->tc_weights.find({nuc, images});
@@ -901,10 +909,13 @@ sbnn_status get_tc_weights(const sbnn_packed* p, int nuc, int images, cudaStream
         *out = static_cast<uint4*>(it->second);
         return SBNN_OK;
     }
+    auto prepared = p->tc_prepared.find(images);
+    if (!prepare_only() && !forced_choice && prepared != p->tc_prepared.end() && M <= prepared->second) return SBNN_OK;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (!prepare_only() && cudaStreamIsCapturing(st, &cs) != cudaSuccess) cudaGetLastError();
     if (cs != cudaStreamCaptureStatusNone) return SBNN_OK;
-    const int taps = p->KH * p->KW, csteps = (p->Cin + 63) / 64, tiles = (p->Cout + 255) / 256 * 256 / nuc;
+    const int taps = p->KH * p->KW, csteps = (p->Cin + 63) / 64;
+    const int tiles = nuc == 64 ? (p->Cout + 63) / 64 : (p->Cout + 255) / 256 * 2;    // (a tile of 256 channels reads two blocks of 128)
     const size_t bytes = (size_t)tiles * csteps * taps * images * nuc * 64 * 2;
     void* d = nullptr;
     cudaError_t e = bytes > p->tc_limit ? cudaErrorMemoryAllocation : cudaMalloc(&d, bytes);
@@ -996,7 +1007,6 @@ double tc_split_cost(const sbnn_packed* p, long long M, int split, int run, int 
     return (double)((runs + split - 1) / split * run) * (tc_step(64, images) + 50.0) + 9800.0;
 }
 
-using TcChoice = sbnn_packed::TcChoice;
 TcChoice tc_choose(const sbnn_packed* p, long long M, int run, int images) {
     TcChoice best{64, 1, tc_cost(p, M, 64, images)};
     for (int bn : {128, 256}) {
@@ -1041,11 +1051,6 @@ TcChoice decide(const sbnn_packed* p, long long M, Call call) {
     if (std::max(tc_us(choice.cost), mem) >= 0.95 * fma) choice.bn = 0;
     return choice;
 }
-// Test hooks (sbnn_debug_conv_gs, sbnn_debug_last_route), for the calling thread: how its calls have to run (bn = 0: on the
-// FMA kernels), and how the latest ran.
-thread_local const TcChoice* forced_choice = nullptr;
-thread_local TcChoice last_route = {0, 0, 0.0};
-
 bool tc_profits(const sbnn_packed* p, long long M, Call call, TcChoice* choice = nullptr) {
     if (forced_choice) {
         if (choice) *choice = *forced_choice;
@@ -1070,18 +1075,32 @@ bool tc_profits(const sbnn_packed* p, long long M, Call call, TcChoice* choice =
 
 }  // namespace
 
-sbnn_status prepare_tc(const sbnn_packed* p, long long M) {
-    // (a call with fewer pixels can be faster here although the largest is not)
-    bool any = false;
-    for (long long m = M; m > 0 && !any; m /= 2)
-        any = p->KH == 3 ? tc_profits(p, m, CALL_3X3) : tc_profits(p, m, CALL_1X1_NHWC) || tc_profits(p, m, CALL_1X1_CM);
-    if (!any) return SBNN_OK;
+// Calls with fewer pixels can be faster here although the largest is not, and in tiles of another width: what they choose is
+// looked up for every number of pixel tiles up to 512 and in steps of a 64th from there, with the fewest and with the most
+// pixels of these tiles.
+sbnn_status prepare_tc(const sbnn_packed* p, long long M, int images) {
+    bool wanted[2] = {false, false};                  // blocks of 64 and of 128 channels
+    auto look = [&](long long m) {
+        for (Call call : {CALL_1X1_NHWC, CALL_1X1_CM, CALL_3X3, CALL_BF16}) {   // (channel-major 3x3 calls gain no oftener than NHWC ones)
+            if (images == 1 ? call != CALL_BF16 : call == CALL_BF16 || (call == CALL_3X3) != (p->KH == 3)) continue;
+            const int bn = decide(p, m, call).bn;
+            if (bn) wanted[bn != 64] = true;
+        }
+    };
+    for (long long t = (M + 127) / 128; t > 0 && !(wanted[0] && (wanted[1] || p->Cout <= 64)); t -= t > 512 ? t / 64 : 1) {
+        look(std::min(M, 128 * t));
+        look(128 * (t - 1) + 1);
+    }
     uint4* wts = nullptr;
     PrepareScope scope;
-    for (int nuc : {64, 128}) {   // the tile width depends on the pixels: for calls with fewer, too
-        const sbnn_status r = get_tc_weights(p, nuc, 3, nullptr, &wts);
-        if (r != SBNN_OK) return r;
-    }
+    for (int k = 0; k < 2; ++k)
+        if (wanted[k]) {
+            const sbnn_status r = get_tc_weights(p, k ? 128 : 64, images, M, nullptr, &wts);
+            if (r != SBNN_OK) return r;
+        }
+    std::lock_guard<std::mutex> lk(p->mu);
+    long long& known = p->tc_prepared[images];
+    known = std::max(known, M);
     return SBNN_OK;
 }
 
@@ -1103,7 +1122,7 @@ sbnn_status launch_tc(const sbnn_packed* p, const TcCall& c, int split, bool* do
     if (regs != T::LAUNCH_REGS) return SBNN_OK;
     TcArgs a = {};
     uint4* wts = nullptr;
-    if ((r = get_tc_weights(p, T::NUC, T::IMAGES, c.st, &wts)) != SBNN_OK || !wts) return r;
+    if ((r = get_tc_weights(p, T::NUC, T::IMAGES, c.M, c.st, &wts)) != SBNN_OK || !wts) return r;
     if ((r = async_status_word(&a.status)) != SBNN_OK) return r;
     *done = true;
     if (prepare_only()) return SBNN_OK;
@@ -1176,12 +1195,9 @@ sbnn_status conv1x1_tc_bf16(const sbnn_packed* p, const float* x, float* y, long
     *done = false;
     last_route = {0, 0, 0.0};
     if (p->Cin % 4 || p->Cout % 4) return SBNN_OK;
-    if (prepare_only()) {   // the tile width depends on the pixels: for calls with fewer, too
-        uint4* wts = nullptr;
-        for (int nuc : {64, 128}) {
-            const sbnn_status r = get_tc_weights(p, nuc, 1, st, &wts);
-            if (r != SBNN_OK) return r;
-        }
+    if (prepare_only()) {
+        const sbnn_status r = prepare_tc(p, M, 1);
+        if (r != SBNN_OK) return r;
     }
     TcChoice ch;
     tc_profits(p, M, CALL_BF16, &ch);

@@ -385,3 +385,26 @@ def test_images_that_do_not_fit_the_device(k):
         call(q, x, y, n, h, w, sbnn.SBNN_BF16_TC)
         assert sbnn.debug_last_route() == (0, 0)
         assert np.all(np.abs(y.cpu().numpy().astype(np.float64) - ref) <= 1e-2 * s)
+
+
+@gpu
+def test_prepared_calls_build_nothing():
+    """A call prepared for some number of pixels runs the same way in a capture, where nothing can be built, as outside, for
+    every smaller number.  (The choice follows whole rounds of tiles: 96 -> 512 at 90 % gains on 2443 and 18749 pixels, say, but
+    not on 19256, nor a half or a quarter of that.)"""
+    for cin, cout, g, pct, top in ((96, 512, 4, 90, 19256), (80, 512, 8, 90, 4964), (96, 96, 8, 90, 37915)):
+        d = WL.single_conv_inputs(1, 1, 1, cin, cout, 1, g, pct, 3, 0.05, 0.05)
+        p = sbnn.pack_weights(d["w"], d["mask"], d["bias"], g)
+        sbnn.prepare(p, 1, 1, top)
+        ld = (top + 3) // 4 * 4
+        x, y = torch.zeros((cin, ld), device="cuda"), torch.empty((cout, ld), device="cuda")
+        for m in range(1, top, 331):
+            captured = []
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=torch.cuda.Stream()):
+                sbnn.conv1x1_gs_cm(p, x, ld, y, ld, m, sbnn.SBNN_OUT_CM)
+                captured.append(sbnn.debug_last_route())
+            del graph
+            sbnn.conv1x1_gs_cm(p, x, ld, y, ld, m, sbnn.SBNN_OUT_CM)
+            assert [sbnn.debug_last_route()] == captured, m
+        torch.cuda.synchronize()
