@@ -1178,13 +1178,16 @@ sbnn_status dispatch_tc(const sbnn_packed* p, const TcCall& c, const TcChoice& c
 
 }  // namespace
 
+// The kernel numbers pixels with ints and adds up to a tile and a row of 224 to them.
+constexpr long long kMaxPixels = 0x7fffffffLL - 1024;
+
 sbnn_status conv1x1_tc(const sbnn_packed* p, const float* x, float* y, long long M, int relu, cudaStream_t st, bool* done) {
     *done = false;
     last_route = {0, 0, 0.0};
     TcChoice ch;
     sbnn_status r;
     if (prepare_only() && (r = prepare_tc(p, M)) != SBNN_OK) return r;
-    if (p->Cin % 4 || p->Cout % 4 || !tc_profits(p, M, CALL_1X1_NHWC, &ch)) return SBNN_OK;
+    if (p->Cin % 4 || p->Cout % 4 || M > kMaxPixels || !tc_profits(p, M, CALL_1X1_NHWC, &ch)) return SBNN_OK;
     const TcCall c{x, 0, y, p->Cout, M, 0, 0, 0, relu, st};
     return dispatch_tc<SRC_NHWC, false>(p, c, ch, done);
 }
@@ -1194,7 +1197,7 @@ sbnn_status conv1x1_tc(const sbnn_packed* p, const float* x, float* y, long long
 sbnn_status conv1x1_tc_bf16(const sbnn_packed* p, const float* x, float* y, long long M, int relu, cudaStream_t st, bool* done) {
     *done = false;
     last_route = {0, 0, 0.0};
-    if (p->Cin % 4 || p->Cout % 4) return SBNN_OK;
+    if (p->Cin % 4 || p->Cout % 4 || M > kMaxPixels) return SBNN_OK;
     if (prepare_only()) {
         const sbnn_status r = prepare_tc(p, M, 1);
         if (r != SBNN_OK) return r;
@@ -1217,7 +1220,7 @@ sbnn_status conv1x1_tc_cm(const sbnn_packed* p, const float* x, int ldx, float* 
     TcChoice ch;
     sbnn_status r;
     if (prepare_only() && (r = prepare_tc(p, M)) != SBNN_OK) return r;
-    if (p->Cout % 4 || !tc_profits(p, M, CALL_1X1_CM, &ch)) return SBNN_OK;
+    if (p->Cout % 4 || M > kMaxPixels || !tc_profits(p, M, CALL_1X1_CM, &ch)) return SBNN_OK;
     const TcCall c{x, ldx, y, ldy, M, 0, 0, 0, relu, st};
     return out_cm ? dispatch_tc<SRC_CM, true>(p, c, ch, done) : dispatch_tc<SRC_CM, false>(p, c, ch, done);
 }
@@ -1229,7 +1232,7 @@ sbnn_status conv3x3_tc(const sbnn_packed* p, const float* x, float* y, int N, in
     const long long M = (long long)N * H * W;
     sbnn_status r;
     if (prepare_only() && (r = prepare_tc(p, M)) != SBNN_OK) return r;
-    if (p->Cin % 4 || p->Cout % 4 || M > 0x7fffffffLL - 128 || !tc_profits(p, M, CALL_3X3, &ch)) return SBNN_OK;
+    if (p->Cin % 4 || p->Cout % 4 || M > kMaxPixels || !tc_profits(p, M, CALL_3X3, &ch)) return SBNN_OK;
     const TcCall c{x, 0, y, p->Cout, M, N, H, W, relu, st};
     return dispatch_tc<SRC_IM2COL, false>(p, c, ch, done);
 }
@@ -1243,7 +1246,7 @@ sbnn_status conv3x3_tc_cm(const sbnn_packed* p, const float* x, int ldx, float* 
     sbnn_status r;
     if (prepare_only() && (r = prepare_tc(p, M)) != SBNN_OK) return r;
     // (the entry point takes rows of up to 224 pixels)
-    if (W > 224 || ldy % 4 || p->Cout % 4 || M > 0x7fffffffLL - 1024 || !tc_profits(p, M, CALL_3X3_CM, &ch)) return SBNN_OK;
+    if (W > 224 || ldy % 4 || p->Cout % 4 || M > kMaxPixels || !tc_profits(p, M, CALL_3X3_CM, &ch)) return SBNN_OK;
     const TcCall c{x, ldx, y, ldy, M, N, H, W, relu, st};
     return out_cm ? dispatch_tc<SRC_CM3, true>(p, c, ch, done) : dispatch_tc<SRC_CM3, false>(p, c, ch, done);
 }
