@@ -1,4 +1,4 @@
-// Thin wrappers of the tcgen05 instructions (5th-generation tensor cores, tensor memory) that the kernels share.
+// Thin wrappers of the tcgen05 instructions (5th-generation tensor cores, tensor memory) that conv_tc.cu issues.
 #pragma once
 
 #include <stdint.h>
@@ -49,21 +49,13 @@ __host__ __device__ constexpr uint32_t instr_desc(int n) {
            | ((uint32_t)(128 >> 4) << 24);   // M / 16
 }
 
-// One thread: D[tmem] (+)= A[smem] * B[smem]^T, 128 x N x 16.
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %5, %5, %5}, p;\n\t}"
-        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(0u)
-        : "memory");
-}
 // The mbarrier receives one arrival once every MMA this thread has issued so far is complete.
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
-// The same with the A operand in tensor memory: lane = row, a 32-bit column = two consecutive K elements (lower half first).
+// One thread: D[tmem] (+)= A[tmem] * B[smem]^T, 128 x N x 16.  A in tensor memory: lane = row, a 32-bit column = two consecutive
+// K elements (lower half first).
 __device__ __forceinline__ void umma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
