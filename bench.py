@@ -34,7 +34,7 @@ METRIC = "mobilenet_v1_images_per_s"
 # the figure is reported only while the kernel source still has that hash.
 PW_DRAM_BYTES_PER_STEP = 746.4e6
 PW_DRAM_KERNEL_SHA1 = "9f06514dd1cb76d2bf0745dbbaa788580eeabf86"
-PW_KERNEL_SOURCES = ("paper_2310_19509_b200/csrc/conv1x1_cm.cu", "paper_2310_19509_b200/csrc/pipeline.cuh")
+PW_KERNEL_SOURCES = tuple("paper_2310_19509_b200/csrc/" + f for f in ("conv_tc.cu", "tcgen05.cuh", "conv1x1_cm.cu", "pipeline.cuh"))
 
 
 def kernel_source_sha1():
@@ -206,7 +206,9 @@ def time_layers(sbnn, torch, net, layers, batch, reps, flush):
             ev1.synchronize()
             ts.append(ev0.elapsed_time(ev1) * 1e-3)
         fl, by = layer_work(L, batch)
-        res.append({"name": L["name"], "kind": L["kind"], "s": float(np.median(ts)), "flops": fl, "bytes": by})
+        sparse = L["kind"] in ("pw", "fc")
+        res.append({"name": L["name"], "kind": L["kind"], "s": float(np.median(ts)), "flops": fl, "bytes": by,
+                    "tile": sbnn.debug_last_route()[0] if sparse else 0, "dense_flops": 2.0 * batch * hout * hout * cin * cout if sparse else 0.0})
         del xin, yout
     return res
 
@@ -314,7 +316,8 @@ def dense_library_us(torch, m, cin, cout, k, shape4, reps, flush):
 def single_layer_lines(sbnn, torch, flush, hbm_gbs, bf16_tflops, reps):
     """The single-layer configurations (config 1, config 4, the ten config-5 cases in fp32 and in the bf16 tensor-core
     mode) through the NHWC entry points, beside dense cuDNN / cuBLAS of the same shape.  fp32 fractions are against
-    max(nonzero flop / FP32 peak, bytes / HBM); bf16 fractions against max(nonzero flop / bf16 tensor peak, bytes / HBM)."""
+    max(flops, bytes / HBM), flops = the nonzero ones / FP32 peak, or those of the unpruned layer / a sixth of the bf16 peak where
+    that is less; bf16 fractions against max(nonzero flop / bf16 tensor peak, bytes / HBM)."""
     from sbnn_inputs import workloads as WL
     out, dense = [], {}
 
@@ -336,11 +339,15 @@ def single_layer_lines(sbnn, torch, flush, hbm_gbs, bf16_tflops, reps):
         taps = k * k if tap_mask is None else int(tap_mask.sum()) / float(g * units)   # kept taps per kept kernel
         flops = 2.0 * m * g * taps * units
         byts = 4.0 * (m * (cin + cout) + units * (1 + g * taps) + cout + cout // g + 1)
-        peak = bf16_tflops if mode == "bf16_tc" else FP32_PEAK_TFLOPS
-        t_alu, t_hbm = flops / (peak * 1e12), byts / (hbm_gbs * 1e9)
+        tile = sbnn.debug_last_route()[0]
+        t_hbm = byts / (hbm_gbs * 1e9)
+        t_fma, t_tensor = flops / (FP32_PEAK_TFLOPS * 1e12), 6 * 2.0 * m * cin * cout * k * k / (bf16_tflops * 1e12)
+        t_alu = flops / (bf16_tflops * 1e12) if mode == "bf16_tc" else min(t_fma, t_tensor)
+        limit = "tensor" if mode == "bf16_tc" or t_tensor < t_fma else "alu"
         rec = {"case": name, "mode": mode, "G": g, "sparsity_pct": d["sparsity_pct"], "us": round(t * 1e6, 1),
                "tflops_nonzero": round(flops / t / 1e12, 2), "roofline_us": round(max(t_alu, t_hbm) * 1e6, 1),
-               "frac": round(max(t_alu, t_hbm) / t, 3), "bound": ("tensor" if mode == "bf16_tc" else "alu") if t_alu > t_hbm else "hbm"}
+               "frac": round(max(t_alu, t_hbm) / t, 3), "bound": limit if t_alu > t_hbm else "hbm",
+               "kernel": "FMA" if not tile and mode == "fp32" else ("gathered bf16" if not tile else f"conv_tc, {tile} channels a tile")}
         if k == 1 and mode == "fp32" and cin >= 128:
             # the same layer in the kernel's own layout (channel-major in and out, as the MobileNet chain calls it): no
             # conversion pass, row-contiguous output
@@ -518,34 +525,45 @@ def run_gpu(args, rank, world, local_rank):
     pw = [r for r in per if r["kind"] == "pw"]
     pw_t, pw_fl, pw_by = sum(r["s"] for r in pw), sum(r["flops"] for r in pw), sum(r["bytes"] for r in pw)
     pw_t_cold = sum(r["s_cold"] for r in pw)
-    t_roof = lambda r: max(r["flops"] / (FP32_PEAK_TFLOPS * 1e12), r["bytes"] / (hbm_gbs * 1e9))  # noqa: E731
+    # Least time of a layer: its bytes, or its flops -- the kept ones on the FP32 pipe, or all of them, six bf16 products each,
+    # on the tensor cores, whichever is less.
+    tc_peak = bf16_tflops / 6
+    t_flops = lambda r: min([r["flops"] / (FP32_PEAK_TFLOPS * 1e12)] + ([r["dense_flops"] / (tc_peak * 1e12)] if r["dense_flops"] else []))  # noqa: E731
+    t_roof = lambda r: max(t_flops(r), r["bytes"] / (hbm_gbs * 1e9))  # noqa: E731
     total_layer_t = sum(r["s"] for r in per)
+    on_tc, on_fma = [r for r in pw if r["tile"]], [r for r in pw if not r["tile"]]
+    tc_t, tc_fl = sum(r["s"] for r in on_tc), sum(r["dense_flops"] for r in on_tc)
+    tensor = tc_t > 0.5 * pw_t
+    achieved, peak = (tc_fl / tc_t / 1e12, tc_peak) if tensor else (pw_fl / pw_t / 1e12, FP32_PEAK_TFLOPS)
     roofline = {
-        "bound": "tensor", "kernel": "conv_tc_kernel (13 pointwise launches per step)",
-        "tensor_frac": 6 * pw_fl / (1 - args.sparsity / 100) / pw_t / 1e12 / bf16_tflops if bf16_tflops and args.sparsity < 100 else None,
-        "note": "achieved and frac count nonzero flops against the FP32 FMA peak; the kernel multiplies dense, six bf16 products for each "
-                "fp32 one, so frac can exceed 1: tensor_frac is those products against the measured bf16 rate",
-        "achieved": pw_fl / pw_t / 1e12, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
-        "frac": pw_fl / pw_t / 1e12 / FP32_PEAK_TFLOPS,
+        "bound": "tensor" if tensor else "alu",
+        "kernel": f"conv_tc_kernel ({len(on_tc)} of the 13 pointwise launches per step)" if tensor
+                  else f"FMA kernels ({len(on_fma)} of the 13 pointwise launches per step)",
+        "launches_on_tensor_cores": len(on_tc), "launches_on_fma_kernels": len(on_fma),
+        "note": "tensor: flops of the unpruned layers, which is what the kernel multiplies, against a sixth of the measured bf16 rate (six "
+                "bf16 products make an fp32 one), over the launches that run there; alu: nonzero flops of all 13 against the FP32 FMA peak",
+        "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
+        "nonzero_tflops": pw_fl / pw_t / 1e12, "nonzero_frac_of_fp32_fma_peak": pw_fl / pw_t / 1e12 / FP32_PEAK_TFLOPS,
         "timing": "per layer: time of the chain's prefix up to and including the layer minus the prefix before it, each prefix a "
                   "CUDA graph replayed back to back under CUDA events (forward's launches and buffers, no flush); the 29 "
                   "figures add up to one whole forward",
-        "frac_cold": pw_fl / pw_t_cold / 1e12 / FP32_PEAK_TFLOPS,
+        "frac_cold": (sum(r["dense_flops"] for r in on_tc) / sum(r["s_cold"] for r in on_tc) if tensor else pw_fl / pw_t_cold) / 1e12 / peak,
         "frac_cold_note": "each layer launched alone after a 256 MB write has flushed L2",
-        "peak_source": "derived: 148 SMs x 128 FP32 lanes x 2 x 1.965 GHz",
-        "peak_measured": fma_measured,
-        "peak_measured_note": "register-only fma.rn.f32x2 kernel of the library (sbnn_selftest_fma_rate) timed in this run",
-        "frac_of_measured_peak": pw_fl / pw_t / 1e12 / fma_measured if fma_measured > 0 else None,
+        "peak_source": f"bf16 rate, {peak_kind}, divided by six" if tensor else "derived: 148 SMs x 128 FP32 lanes x 2 x 1.965 GHz",
+        "fp32_fma_peak": FP32_PEAK_TFLOPS, "fp32_fma_peak_source": "derived: 148 SMs x 128 FP32 lanes x 2 x 1.965 GHz",
+        "fp32_fma_measured": fma_measured,
+        "fp32_fma_measured_note": "register-only fma.rn.f32x2 kernel of the library (sbnn_selftest_fma_rate) timed in this run",
         "traffic": PW_DRAM_BYTES_PER_STEP if (batch == 64 and args.sparsity == 50 and PW_DRAM_KERNEL_SHA1 == kernel_source_sha1()) else None,
         "algorithmic_bytes": pw_by,
         "mixed_frac": sum(t_roof(r) for r in pw) / pw_t,
-        "mixed_note": f"sum over layers of max(nonzero flops/FP32 peak, bytes/{hbm_gbs:.0f} GB/s {peak_kind}) / measured",
+        "mixed_note": f"sum over layers of max(min(nonzero flops/FP32 peak, flops/tensor peak), bytes/{hbm_gbs:.0f} GB/s {peak_kind}) / measured",
         "hbm_achieved_gbs": pw_by / pw_t / 1e9,
         "share_of_step": pw_t / total_layer_t,
         "whole_chain_frac": sum(t_roof(r) for r in per) / total_layer_t,
     }
     layers_out = [{"name": r["name"], "us": round(r["s"] * 1e6, 2), "us_cold": round(r["s_cold"] * 1e6, 2), "tflops": round(r["flops"] / r["s"] / 1e12, 2),
-                   "gbs": round(r["bytes"] / r["s"] / 1e9, 1), "frac": round(t_roof(r) / r["s"], 3)} for r in per]
+                   "gbs": round(r["bytes"] / r["s"] / 1e9, 1), "frac": round(t_roof(r) / r["s"], 3),
+                   **({"tensor_core_tile": r["tile"]} if r["kind"] in ("pw", "fc") else {})} for r in per]
 
     if not args.no_dense:
         seen = {}
