@@ -7,8 +7,9 @@
  * that connect one input channel to one group — is either kept or removed as a
  * whole (the paper's connectivity group pruning, Section 3.2 and Eq. 2, with an
  * input-channel group size of 1).  The result is by definition the ordinary
- * convolution with W~ = W (.) M (Section 3.1); the kernels reach it by visiting
- * kept units only (Algorithm 1).
+ * convolution with W~ = W (.) M (Section 3.1).  The FMA kernels reach it by visiting
+ * kept units only (Algorithm 1); the tensor-core kernel, which runs where that is
+ * faster, multiplies the pruned weights as zeros.
  *
  * Conventions that hold for every entry point
  *   - Tensors: activations [N][H][W][C] fp32 (NHWC), weights [Cout][KH][KW][Cin]
@@ -104,7 +105,8 @@ SBNN_API sbnn_status sbnn_pack_weights(const float* W_host, const uint8_t* mask_
  * identical for the G filters of a group (the pattern is shared by the group), a unit is kept if any of its
  * KH*KW taps is, pruned taps are stored as 0.0f in val, and the view's tap_mask records which taps were kept,
  * so that sbnn_unpack_weights returns the mask exactly.  The convolution entry points take the result like
- * any other packed layer (pruned taps are multiplied as zeros; they are not skipped).
+ * any other packed layer.  Where less than 4.8 of 9 taps are kept on average, an infinity or a NaN under a pruned tap does
+ * not reach the output; with more, pruned taps are multiplied as zeros.
  */
 SBNN_API sbnn_status sbnn_pack_weights_pattern(const float* W_host, const uint8_t* mask_host, const float* bias_host,
                                                int Cout, int KH, int KW, int Cin, int G, sbnn_packed** out);
@@ -160,11 +162,12 @@ SBNN_API sbnn_status sbnn_packed_load(const char* path, sbnn_packed** out);
  * does now everything that sbnn_conv1x1_gs / sbnn_conv1x1_gs_cm (KH = 1) or sbnn_conv3x3_gs (KH = 3) would
  * otherwise do on first use for activations of up to N x H x W pixels with these flags -- builds the kernels'
  * private weight layouts (for the 1x1 case those of every tile shape the library may choose, whatever the
- * pixel count, and the images of the unpruned layer's weights, six bytes a weight for every tile
- * width, where some call would run on the tensor cores), raises the kernels' shared-memory limits, and grows the per-device scratch buffer to what
- * the NHWC entry points need for this shape (with SBNN_BF16_TC: what the bf16 mode needs).  Allocates,
- * may launch kernels that lay the weights out, and synchronises; the activation buffers need not exist yet.  Afterwards compute calls of
- * this layer with no more pixels (3x3: the same W) only enqueue.  Call it once per layer and mode, outside
+ * pixel count; and, where some call would run on the tensor cores, images of the unpruned layer's weights: six bytes
+ * a weight, two in the bf16 mode, for each of the one or two tile widths in use, with Cin rounded up to 64 and Cout
+ * to 64 or 256), raises the kernels' shared-memory limits, and grows the per-device scratch buffer to what
+ * the NHWC entry points need for this shape (with SBNN_BF16_TC: what the bf16 mode needs).  Allocates, may launch
+ * kernels that lay the weights out, and synchronises; the activation buffers need not exist yet.  Afterwards compute
+ * calls of this layer with no more pixels (3x3: the same W) only enqueue.  Call it once per layer and mode, outside
  * any stream capture.  The scratch buffer never shrinks and an outgrown one is kept until the process exits,
  * so a CUDA graph recorded over an entry point stays valid when a later, larger call makes the buffer grow;
  * growth during a capture is refused with SBNN_ERR_UNSUPPORTED.
@@ -198,9 +201,13 @@ enum {
  * The first call of a layer in either form builds a private re-layout of its weights (allocates and copies
  * synchronously); the gathered kernel converts X to bf16 in the per-device scratch buffer first.
  * Without it the sums are fp32 sums of fp32 products.  Where that is faster (wide layers and whatever is not almost
- * entirely pruned) they are formed on the tensor cores, from an exact split of every operand into three bf16 numbers;
- * the error is that of an fp32 sum, and pixels that hold an infinity or a NaN are summed over the kept units alone.
- * Which kernel runs depends on the layer and on N*H*W.
+ * entirely pruned) they are formed on the tensor cores, from a split of every operand into three bf16 numbers.  The error is
+ * that of an fp32 sum: 0.3e-7 to 0.9e-7 of the result (2-norm) for 4 to 1024 channels.  Two things differ from a chain of FMAs:
+ * the weights are scaled by 1 + 5.4e-8, which makes up on average for what the tensor cores cut off, and operands below
+ * 2^-109 lose bits (below 2^-133 all of them), so that an output can be off by 2^-133 times the operands they meet.
+ * Pixels that hold an infinity or a NaN, or a sum that overflows, are summed over the kept units alone; layers with a weight
+ * or bias that is not finite run on the FMA kernels.  A call in which every pixel holds a bad activation takes up to seven
+ * times as long as on those.  Which kernel runs depends on the layer and on N*H*W.
  */
 SBNN_API sbnn_status sbnn_conv1x1_gs(const sbnn_packed* w, const float* x_dev, float* y_dev,
                                      int N, int H, int W, int flags, void* cuda_stream);
@@ -243,9 +250,10 @@ SBNN_API sbnn_status sbnn_to_channel_major(const float* x_dev, float* xt_dev, in
  * 3x3, stride 1, pad 1:
  * Y[n][y][x][g*G + r] = act( bias + sum_j sum_{kh,kw} val[g][j][kh*3+kw][r] * X[n][y+kh-1][x+kw-1][idx[g][j]] ),
  * X taken as zero outside the image.  Shapes as above with KH = KW = 3.  SBNN_BF16_TC is not accepted.
- * W <= 256 and Cin a multiple of 4, else SBNN_ERR_UNSUPPORTED.  The first call with a new image width
- * builds a private re-layout of the weights (allocates and copies synchronously); later calls only enqueue.
- * The input is first copied, channel by channel (image rows padded to a multiple of 4 floats), into a scratch buffer
+ * W <= 256 and Cin a multiple of 4, else SBNN_ERR_UNSUPPORTED.  The layer runs on the tensor cores where that is faster
+ * (see sbnn_conv1x1_gs).  Else the first call with a new image width
+ * builds a private re-layout of the weights (allocates and copies synchronously), later calls only enqueue, and
+ * the input is first copied, channel by channel (image rows padded to a multiple of 4 floats), into a scratch buffer
  * kept per device (allocated or grown synchronously the first time a size is seen).
  */
 SBNN_API sbnn_status sbnn_conv3x3_gs(const sbnn_packed* w, const float* x_dev, float* y_dev,

@@ -11,7 +11,10 @@
 // What the truncations of one step take from the magnitude of its sum on average, 5.4e-8 of it (measured for 64 to
 // 1024 channels, dense to 90 % pruned, 1x1 and 3x3, alone and in a network: 3.6e-8 to 5.9e-8), is put back in the weights,
 // which are scaled by kTruncation before they are split; without it the layers of a network lose the same fraction one
-// after the other.
+// after the other.  What remains is -0.6e-8 to 1.0e-8 for 64 to 1024 channels and up to 1.6e-8 for 4 to 48, whose steps are
+// half as long, against 3e-8 to 9e-8 of rounding.
+// Small operands: bf16 ends at 2^-133, so the third image of a number below 2^-109 loses bits, and a number below 2^-133 is
+// lost: an output is then off by up to 2^-133 times the other operands (the FMA kernels: 2^-149).
 //
 // The contraction runs dense over the masked weights (pruned entries are zeros): a group shares its kept channels over
 // only G = 4..8 outputs, far too few for a 128-row MMA to gather for.  Six products per dense MAC still beat the FMA
@@ -140,7 +143,7 @@ __device__ __forceinline__ uint32_t bf16x2(float first, float second) {
     return r;
 }
 
-// Splits two fp32 values into bf16 images packed as (first, second): x = h + m + l exactly (up to subnormal l).
+// Splits two fp32 values into bf16 images packed as (first, second): x = h + m + l exactly, down to 2^-109 (see above).
 __device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
     uint64_t r;
     asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
@@ -750,7 +753,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
         const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16);
         unsigned char* stage = ost + (size_t)warp * 4096;
         int step = 0, copies = 0;                           // copies issued: the two tiles alternate between them
-        bool ok = true, again = false;                      // again: some pixels have to be summed once more
+        bool ok = true, again = false;                      // again: some of this lane's pixels have to be summed once more
         grid_dependency_wait();                             // Y may still be read by the previous kernel of the stream
         for (Tiles t(a); t.left() && ok; t.next()) {
             const int m0 = t.m * T::BM, n0 = t.n * BN + wg * T::COLS;
@@ -798,7 +801,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                 unpack2(add2(add2(probe[0], probe[1]), add2(probe[2], probe[3])), lo, hi);
                 redo = m < a.M && !(lo + hi == 0.0f);
             }
-            again |= __any_sync(0xffffffffu, redo);
+            again |= redo;
             // 32 pixels x 16 channels at a time through one of the warp's two staging tiles, stored by tiled copies: rows of 32
             // pixels (channel-major) or of 16 channels (64-byte swizzle).  Rows past Cout or M are clipped by the copy; the last
             // pixels of a channel-major row are stored one by one, so that the padding behind them is left alone.
@@ -1021,7 +1024,8 @@ TcChoice tc_choose(const sbnn_packed* p, long long M, int run, int images) {
 }
 
 // Whether a call is faster here than on the FMA kernels, in microseconds of both, fitted to measured times.  Layers of
-// 64-1024 channels on 49 to 50176 pixels, G = 4 and 8, 0 / 50 / 70 / 90 % pruned: channel-major 1x1 calls gain up to 70 %
+// 64-1024 channels on 49 to 50176 pixels, G = 4 and 8, 0 / 50 / 70 / 90 % pruned, in short bursts (in a long loop the largest
+// run at the power limit, 460 us instead of 390 here): channel-major 1x1 calls gain up to 70 %
 // pruning (256 x 14 x 14, 1024 -> 1024: 1969 -> 404, 1025 -> 386, 669 -> 366 us; 9 x 14 x 14, 512 -> 512: 89 -> 12, 53 -> 12,
 // 39 -> 12 us) and lose where next to nothing is left to do (the first at 90 %: 289 and 338 us; one 14 x 14 image, 256 -> 512,
 // 50 %: 4.5 and 6.0 us); NHWC calls, which the FMA kernels convert first, and 3x3 calls gain nearly everywhere

@@ -159,6 +159,24 @@ def test_small_and_large_operands_keep_their_bits(scale):
     check_tc(got, ref, s, 9)
 
 
+@gpu
+@pytest.mark.parametrize("exponent", [-100, -120, -140])
+def test_operands_near_the_end_of_bf16(exponent):
+    """Down to 2^-109 an operand keeps all its bits; below, each of its three images is rounded to multiples of 2^-133, which
+    leaves at most 2^-134 of it out (and a smaller operand whole)."""
+    d, _, _ = inputs(3, 17, 19, 516, 260, 1, 4, 50)
+    x, w = np.ldexp(d["x"], exponent).astype(np.float32), np.ldexp(d["w"], 60).astype(np.float32)
+    d = dict(d, x=x, w=w, bias=np.zeros_like(d["bias"]))
+    ref, s = R.conv2d(x, w, d["mask"], d["bias"], relu=False)
+    p = sbnn.pack_weights(w, d["mask"], d["bias"], d["g"])
+    got = run(p, d, "nhwc", 128, 1)
+    if exponent == -100:
+        check_tc(got, ref, s, 9)
+    lost = 2.0 ** -133 * np.abs(w * d["mask"]).astype(np.float64).reshape(260, -1).sum(1)
+    err = np.abs(got.astype(np.float64) - ref.reshape(got.shape))
+    assert np.all(err <= lost + (4 * 2.0 ** -23 + 12 * 2.0 ** -24) * s.reshape(got.shape))
+
+
 def bf16_images(v):
     """Three bf16 numbers whose sum is v, each rounded to nearest even."""
     out, r = [], np.asarray(v, np.float32)

@@ -116,7 +116,7 @@ def test_3x3(n, h, w, cin, cout, g, pct):
 
 
 def test_values_of_every_size():
-    """Products from 1e-30 to 1e30 in one sum: the split must not lose the bits of small or large operands."""
+    """Products from 1e-16 to 1e14 in one sum: the split must not lose the bits of small or large operands."""
     d, _ = layer(5, 50, 41, 64, 128, 1, 4, 50, seed=3)
     scale = np.float32(2.0) ** np.random.default_rng(0).integers(-50, 50, 64).astype(np.float32)
     d["x"] = np.ascontiguousarray(d["x"] * scale).astype(np.float32)
