@@ -504,7 +504,7 @@ SBNN_API sbnn_status sbnn_debug_poke_device_index(sbnn_packed* w, long long unit
  * the layer and the number of pixels.  sbnn_debug_last_route tells what the calling thread's latest convolution ran on: *tile
  * = 0 the FMA kernels (or the gathered bf16 kernel), else the output channels of a tensor-core tile (64, 128 or 256), and
  * *split the CTAs that shared a tile's steps.  sbnn_debug_conv_gs is sbnn_conv1x1_gs / sbnn_conv3x3_gs (ldx = ldy = 0) or their
- * channel-major variants with that choice made by the caller: tile 0, 64, 128 or 256; split 1, or 2, 4 or 8 with tile = 64.
+ * channel-major variants with that choice made by the caller: tile 0, 64, 128 or 256; split 1, or up to 8 with tile = 64.
  * SBNN_ERR_UNSUPPORTED if the tensor-core kernel does not take the call (the output may have been written all the same).
  */
 SBNN_API sbnn_status sbnn_debug_last_route(int* tile, int* split);

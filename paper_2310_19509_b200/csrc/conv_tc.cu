@@ -122,7 +122,8 @@ struct TC {
     static constexpr int D_COLS = NUC, A_COL0 = 2 * D_COLS, A_COLS = 32 * IMAGES, NA = BN == 64 || IMAGES == 1 ? 4 : 2;
     static_assert(A_COL0 + NA * A_COLS <= 512, "tensor memory");
     static_assert(BN == 64 || BN == 128 || BN == 256, "tile width");
-    static_assert(!SPLIT || (BN == 64 && SB * B_BYTES >= 32 * 1024), "the cluster's exchange takes 32 KB of the weight stages");
+    // (shared by 7, the most for an exchange: 7 senders of up to 2 of a thread's 8 chunks)
+    static_assert(!SPLIT || (BN == 64 && SB * B_BYTES + 3 * A_BYTES >= 7 * 2 * 256 * 16), "the cluster's exchange");
     static_assert(IMAGES == 3 || (IMAGES == 1 && SRC == SRC_NHWC), "bf16 mode");
 };
 
@@ -406,34 +407,35 @@ __device__ __noinline__ void sum_kept_units(const TcArgs& args, unsigned char* r
 }
 
 // Last step of a tile whose steps were shared by the `split` CTAs of a cluster, for the drain threads: chunk c of a
-// thread's channels (four of them) belongs to CTA c * split / CHUNKS.  Everybody writes its sums of the chunks of others into
-// their shared memory, [sender][chunk][thread], and then adds up and stores its own.  The weight stages hold the exchange:
-// every CTA's MMAs are complete when its drain threads reach the first barrier.
+// thread's channels (four of them) belongs to the last CTA r with r * CHUNKS / split <= c.  Everybody writes its sums of the
+// chunks of others into their shared memory, [sender][chunk][thread], and then adds up and stores its own.  The stages hold the
+// exchange: every CTA's MMAs are complete when its drain threads reach the first barrier.
 template <class T>
 __device__ __forceinline__ void store_shared_tile(const TcArgs& a, uint64_t (&acc)[T::COLS / 2], unsigned char* room, float* sums, int m0, int tid) {
     constexpr int CHUNKS = T::COLS / 4;
     const uint32_t exchange = smem_u32(room);
     const unsigned char* const mine = room;
     const int m = m0 + (tid & 127), n00 = blockIdx.x / a.split % a.ntiles_n * T::BN, n0 = n00 + (tid >> 7) * T::COLS;
-    const int rank = (int)cluster_rank(), own = CHUNKS / a.split;
+    const int rank = (int)cluster_rank(), slots = (CHUNKS + a.split - 1) / a.split;
+    const int first = rank * CHUNKS / a.split, own = (rank + 1) * CHUNKS / a.split - first;
     __syncwarp();
     cluster_sync();
 #pragma unroll
     for (int c = 0; c < CHUNKS; ++c) {
-        const int owner = c / own;
+        const int owner = ((c + 1) * a.split - 1) / CHUNKS;
         float4 v;
         unpack2(acc[2 * c], v.x, v.y);
         unpack2(acc[2 * c + 1], v.z, v.w);
-        if (owner != rank) store_remote(exchange + ((rank * own + c - owner * own) * 256 + tid) * 16, owner, v);
+        if (owner != rank) store_remote(exchange + ((rank * slots + c - owner * CHUNKS / a.split) * 256 + tid) * 16, owner, v);
     }
     cluster_sync();
     bool redo = false;
 #pragma unroll
     for (int c = 0; c < CHUNKS; ++c) {
-        if (c / own != rank) continue;
+        if (c < first || c >= first + own) continue;
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
         for (int s = 0; s < a.split; ++s) {
-            float4 o = reinterpret_cast<const float4*>(mine)[(s * own + c - rank * own) * 256 + tid];
+            float4 o = reinterpret_cast<const float4*>(mine)[(s * slots + c - first) * 256 + tid];
             if (s == rank) {
                 unpack2(acc[2 * c], o.x, o.y);
                 unpack2(acc[2 * c + 1], o.z, o.w);
@@ -456,7 +458,7 @@ __device__ __forceinline__ void store_shared_tile(const TcArgs& a, uint64_t (&ac
         }
     }
     redo = redo && m < a.M;
-    if (T::IMAGES == 3 && drain_any(redo)) sum_kept_units<T>(a, room, sums, m0, redo, n00 + rank * own * 4, own * 4);
+    if (T::IMAGES == 3 && drain_any(redo)) sum_kept_units<T>(a, room, sums, m0, redo, n00 + first * 4, own * 4);
 }
 
 template <class T>
@@ -1016,7 +1018,9 @@ TcChoice tc_choose(const sbnn_packed* p, long long M, int run, int images) {
         const double cost = tc_cost(p, M, bn, images);
         if (cost < best.cost) best = {bn, 1, cost};
     }
-    for (int split : {2, 4, 8}) {
+    // (every number: a layer of 16 tiles gets no clusters of 8, of which 15 run at a time, but clusters of 6.  5 x 7 x 7, 512 -> 512
+    // 3x3, 72 steps: 17.9 us shared by 4, 15.0 by 6)
+    for (int split = 2; split <= 8; ++split) {
         const double cost = tc_split_cost(p, M, split, run, images);
         if (cost < best.cost) best = {64, split, cost};
     }
@@ -1285,8 +1289,8 @@ extern "C" sbnn_status sbnn_debug_conv_gs(const sbnn_packed* w, const float* x_d
     clear_error();
     if (!w) return fail(SBNN_ERR_NULL, "packed weights must not be NULL");
     if (tile != 0 && tile != 64 && tile != 128 && tile != 256) return fail(SBNN_ERR_UNSUPPORTED, "tile=%d is not 0, 64, 128 or 256", tile);
-    if (split != 1 && !(tile == 64 && (split == 2 || split == 4 || split == 8)))
-        return fail(SBNN_ERR_UNSUPPORTED, "split=%d is not 1, or 2, 4 or 8 with 64-channel tiles", split);
+    if (split < 1 || split > 8 || (split > 1 && tile != 64))
+        return fail(SBNN_ERR_UNSUPPORTED, "split=%d is not 1, or up to 8 with 64-channel tiles", split);
     const int runs = (w->Cin + 63) / 64 * w->KH * (ldx ? 1 : w->KW);   // (channel-major 3x3: the taps of a kernel row stay together)
     if (runs < split) return fail(SBNN_ERR_UNSUPPORTED, "the layer has %d steps to split, not %d", runs, split);
     const TcChoice choice = {tile, split, 0.0};
