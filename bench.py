@@ -216,6 +216,7 @@ def time_layers(sbnn, torch, net, layers, batch, reps, flush):
 def time_layers_in_chain(sbnn, torch, net, layers, batch, xd, reps):
     """Cost of every layer inside a step: T(layers 0..l) - T(layers 0..l-1), where each prefix of the chain is recorded
     into a CUDA graph (the way forward runs) and replayed back to back, CUDA events around `reps` replays, median of 3.
+    A pointwise layer that runs in one launch with the depthwise layer in front gets the time of both, that layer zero.
     The 29 figures add up to the time of the whole chain, so they include what a kernel costs its neighbours (launch
     gap, cold pipeline) and nothing that a step does not pay."""
     r4 = lambda v: (v + 3) // 4 * 4  # noqa: E731
@@ -242,7 +243,19 @@ def time_layers_in_chain(sbnn, torch, net, layers, batch, xd, reps):
         prefix.append(float(np.median(runs)))
         del g
     # (a difference can come out at or below zero when timing noise exceeds a very short layer: floor of 10 ns)
-    return [max(prefix[0], 1e-8)] + [max(prefix[l] - prefix[l - 1], 1e-8) for l in range(1, len(layers))]
+    times = [max(prefix[0], 1e-8)] + [max(prefix[l] - prefix[l - 1], 1e-8) for l in range(1, len(layers))]
+    for l in joined_layers(net, layers, batch):
+        times[l - 1], times[l] = 0.0, prefix[l] - prefix[l - 2]
+    return times
+
+
+def joined_layers(net, layers, batch):
+    """Pointwise layers that forward runs in one launch with the depthwise layer in front of them."""
+    return [l for l, L in enumerate(layers) if L["kind"] == "pw" and net.debug_launches(batch, l) == net.debug_launches(batch, l - 2) + 1]
+
+
+def layer_pixels(sbnn, l):
+    return sbnn.mobilenet_v1_layer_shape(l)[0] ** 2
 
 
 def sweep_oracle_lines():
@@ -520,6 +533,10 @@ def run_gpu(args, rank, world, local_rank):
     chain_t = time_layers_in_chain(sbnn, torch, net, layers, batch, xd, max(args.layer_reps, 10))
     for r, t in zip(per, chain_t):
         r["s_cold"], r["s"] = r["s"], t          # the roofline uses the in-step durations; the cold ones are reported beside
+    for l in joined_layers(net, layers, batch):  # one launch: the depthwise layer's output is not moved
+        per[l]["bytes"] += per[l - 1]["bytes"] - 8.0 * batch * layer_pixels(sbnn, l) * sbnn.mobilenet_v1_layer_shape(l)[1]
+        per[l]["s_cold"] += per[l - 1]["s_cold"]
+        per[l - 1].update(bytes=0.0, flops=0.0)
     hbm_gbs, bf16_tflops, peak_kind = measured_peaks()
     fma_measured = measure_fma_peak(sbnn, torch)
     pw = [r for r in per if r["kind"] == "pw"]
@@ -546,7 +563,8 @@ def run_gpu(args, rank, world, local_rank):
         "nonzero_tflops": pw_fl / pw_t / 1e12, "nonzero_frac_of_fp32_fma_peak": pw_fl / pw_t / 1e12 / FP32_PEAK_TFLOPS,
         "timing": "per layer: time of the chain's prefix up to and including the layer minus the prefix before it, each prefix a "
                   "CUDA graph replayed back to back under CUDA events (forward's launches and buffers, no flush); the 29 "
-                  "figures add up to one whole forward",
+                  "figures add up to one whole forward; a pointwise layer that runs in one launch with the depthwise layer in front "
+                  "(us 0) has the time of both, us_cold apart",
         "frac_cold": (sum(r["dense_flops"] for r in on_tc) / sum(r["s_cold"] for r in on_tc) if tensor else pw_fl / pw_t_cold) / 1e12 / peak,
         "frac_cold_note": "each layer launched alone after a 256 MB write has flushed L2",
         "peak_source": f"bf16 rate, {peak_kind}, divided by six" if tensor else "derived: 148 SMs x 128 FP32 lanes x 2 x 1.965 GHz",
@@ -561,8 +579,8 @@ def run_gpu(args, rank, world, local_rank):
         "share_of_step": pw_t / total_layer_t,
         "whole_chain_frac": sum(t_roof(r) for r in per) / total_layer_t,
     }
-    layers_out = [{"name": r["name"], "us": round(r["s"] * 1e6, 2), "us_cold": round(r["s_cold"] * 1e6, 2), "tflops": round(r["flops"] / r["s"] / 1e12, 2),
-                   "gbs": round(r["bytes"] / r["s"] / 1e9, 1), "frac": round(t_roof(r) / r["s"], 3),
+    layers_out = [{"name": r["name"], "us": round(r["s"] * 1e6, 2), "us_cold": round(r["s_cold"] * 1e6, 2), "tflops": round(r["flops"] / max(r["s"], 1e-8) / 1e12, 2),
+                   "gbs": round(r["bytes"] / max(r["s"], 1e-8) / 1e9, 1), "frac": round(t_roof(r) / max(r["s"], 1e-8), 3),
                    **({"tensor_core_tile": r["tile"]} if r["kind"] in ("pw", "fc") else {})} for r in per]
 
     if not args.no_dense:
@@ -598,7 +616,7 @@ def run_gpu(args, rank, world, local_rank):
         "effective_gflops_nonzero": sum(r["flops"] for r in per) / (elapsed / args.steps) / 1e9,
         "e2e": {"value": imgs / e2e_elapsed, "unit": "images/s", "h2d_bytes_per_step": int(x.nbytes),
                 "d2h_bytes_per_step": int(batch * 1000 * 4)},
-        "gpu_launches": 29 * args.steps,
+        "gpu_launches": net.debug_launches(batch) * args.steps,
         "clocks": clocks, "roofline": roofline, "layers": layers_out,
     }
     if single is not None:

@@ -377,7 +377,7 @@ SBNN_API sbnn_status sbnn_mobilenet_v1_create(const sbnn_packed* const* pw, cons
  * conv0 -> 13 x (depthwise 3x3 -> group-sparse 1x1) -> average pool -> classifier.
  *   x_dev [N][224][224][3] fp32 (4-byte aligned is enough), logits_dev [N][1000] fp32.
  * Every conv but the classifier applies ReLU.  No host synchronisation.
- * The second call with the same (x_dev, logits_dev, N) records the 29 launches into a CUDA graph (captured on a
+ * The second call with the same (x_dev, logits_dev, N) records the launches (one for each layer, or for each block of a depthwise and a pointwise one) into a CUDA graph (captured on a
  * stream the network owns; nothing of the caller's stream is touched) and from then on such calls launch that
  * graph on cuda_stream, which shortens the gaps between the kernels; up to 8 triples are kept.  If recording
  * fails, or if cuda_stream is itself being captured, the launches are issued one by one as on the first call.
@@ -406,8 +406,9 @@ SBNN_API sbnn_status sbnn_mobilenet_v1_run_layer_cm(sbnn_mbv1* net, int layer, c
 
 /*
  * The first last_layer + 1 layers of the forward pass (Section 3.5), launched exactly as sbnn_mobilenet_v1_forward
- * launches them (same kernels, same workspaces, no CUDA graph of the library's own), with the output of layer
- * last_layer written to out_dev in the chain's layout: channel-major [Cout][ld], ld = N*side*side rounded up to 4
+ * launches them (same kernels, same workspaces, no CUDA graph of the library's own); a depthwise layer that forward does in one
+ * launch with the pointwise layer behind it runs alone where it is the last.  The output of layer
+ * last_layer is written to out_dev in the chain's layout: channel-major [Cout][ld], ld = N*side*side rounded up to 4
  * (the pool: [1024][N rounded up to 4]; layer 28: the logits [N][1000]).  Gives access to every intermediate
  * activation of the chain, and, by timing consecutive prefixes, to the cost of each layer inside a step.  The call
  * only enqueues; it may be captured into a caller's CUDA graph.  out_dev: 16-byte aligned device memory of the caller.
@@ -510,6 +511,15 @@ SBNN_API sbnn_status sbnn_debug_poke_device_index(sbnn_packed* w, long long unit
 SBNN_API sbnn_status sbnn_debug_last_route(int* tile, int* split);
 SBNN_API sbnn_status sbnn_debug_conv_gs(const sbnn_packed* w, const float* x_dev, int ldx, float* y_dev, int ldy, int N, int H, int W,
                                         int flags, int tile, int split, void* cuda_stream);
+/*
+ * Test hook: block `block` (1 to 13: a depthwise layer and the pointwise layer behind it) of the network in one launch on the
+ * tensor-core kernel, with tiles of `tile` output channels (64, 128 or 256) shared by `split` CTAs as above; activations as for
+ * sbnn_mobilenet_v1_run_layer_cm.  SBNN_ERR_UNSUPPORTED where there is no such kernel.  sbnn_debug_mobilenet_v1_launches: kernel
+ * launches of layers 0 .. last_layer of N images, which are fewer than layers where blocks run in one.
+ */
+SBNN_API sbnn_status sbnn_debug_mobilenet_v1_launches(const sbnn_mbv1* net, int N, int last_layer, int* launches);
+SBNN_API sbnn_status sbnn_debug_mobilenet_v1_block(sbnn_mbv1* net, int block, const float* in_dev, float* out_dev, int N, int tile, int split,
+                                                   void* cuda_stream);
 /*
  * Test hook: from now on the layer's images for the tensor cores are treated as too large for the device where they take more
  * than `bytes`; calls then run on the FMA kernels.

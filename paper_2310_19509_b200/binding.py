@@ -78,6 +78,8 @@ def lib():
         "sbnn_debug_last_route": [P, P],
         "sbnn_debug_limit_images": [P, C.c_longlong],
         "sbnn_debug_conv_gs": [P, P, I, P, I, I, I, I, I, I, I, P],
+        "sbnn_debug_mobilenet_v1_launches": [P, I, I, P],
+        "sbnn_debug_mobilenet_v1_block": [P, I, P, P, I, I, I, P],
         "sbnn_debug_plan_conv3x3": [P, I, I, I, I, P, P, I, P, P, P],
     }
     for name, args in sig.items():
@@ -388,6 +390,16 @@ class MobileNetV1:
     def run_layer_cm(self, layer, x, y, n, stream=None):
         """One layer on the chain's channel-major buffers (no layout conversion)."""
         _check(lib().sbnn_mobilenet_v1_run_layer_cm(self._h, layer, _ptr(x), _ptr(y), n, _stream(stream)))
+
+    def debug_launches(self, n, last_layer=28) -> int:
+        """Kernel launches of layers 0..last_layer of n images."""
+        count = C.c_int()
+        _check(lib().sbnn_debug_mobilenet_v1_launches(self._h, n, int(last_layer), C.byref(count)))
+        return count.value
+
+    def debug_block(self, block, x, y, n, tile, split=1, stream=None):
+        """One block (depthwise and pointwise layer) in one launch, on the tiles the caller names (see sbnn_debug_mobilenet_v1_block)."""
+        _check(lib().sbnn_debug_mobilenet_v1_block(self._h, block, _ptr(x), _ptr(y), n, tile, split, _stream(stream)))
 
     def free(self):
         if self._h:

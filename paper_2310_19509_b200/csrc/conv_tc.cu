@@ -37,6 +37,9 @@
 // The bf16 mode (SBNN_BF16_TC: activations and weights rounded to bf16 once, fp32 sums) is the same kernel with one image
 // of each operand (IMAGES = 1): one product, summed over all steps of a tile in the accumulator and drained once.
 //
+// A launch can do the depthwise 3x3 layer in front of a 1x1 layer as well (SRC_DW, see DwShape), whose output then never reaches
+// memory: the split warps compute it from the staged input, in fp32, and split it.
+//
 // Launches with too few tiles for the SMs (small batches, small maps) run with 64 output channels a tile and the steps of a
 // tile dealt to the CTAs of a cluster (SPLIT): each sums its share, then every CTA adds up a part of the channels, which
 // the others have written into its shared memory, in rank order, and stores it.
@@ -46,6 +49,7 @@
 #include <algorithm>
 #include <atomic>
 #include <new>
+#include <type_traits>
 
 #include <cuda.h>   // CUtensorMap (type only)
 
@@ -60,7 +64,9 @@ constexpr double kTruncation = 1.0 + 5.4e-8;
 
 // SRC_CM3: 3x3 on channel-major activations.  A tap shifts the 128 pixels of a tile by dy * W + dx, so a copy of 136 pixels
 // (from a multiple of 4) serves the three taps of a kernel row; the split warps blank what lies outside the image.
-enum Source { SRC_NHWC, SRC_CM, SRC_IM2COL, SRC_CM3 };
+// SRC_DW: 1x1 on the result of a depthwise 3x3 (stride 1 or 2, bias, ReLU) of channel-major square images, which the split
+// warps compute on the way (see DwShape).
+enum Source { SRC_NHWC, SRC_CM, SRC_IM2COL, SRC_CM3, SRC_DW };
 
 // Element strides of the activations and the arrays of the packed layer, for the outputs of pixels that hold a
 // non-finite value (see sum_kept_units).
@@ -91,10 +97,48 @@ struct TcArgs {
     int* status;
     ExactArgs ex;
 };
+struct DwArgs : TcArgs {
+    CUtensorMap wmap;      // the depthwise weights [9][Cin]
+    const float* dw_w;
+    const float* dw_b;
+    long long M_in;        // pixels of the depthwise layer's input
+};
 
-template <int BN_, int SRC_, bool OUT_CM_, bool SPLIT_ = false, int IMAGES_ = 3>
+// What a stage holds for the depthwise layer in front of a 1x1 layer (SRC_DW), for images of WI x WI input pixels, 112 to 28: of
+// SUB channels every input pixel that the 128 output pixels of a tile need, as BOXES tiled copies of PB consecutive pixels each
+// (box-major, then channel, then pixel), behind them the nine rows of weights and the bias of these channels.
+// Stride 1: the 128 pixels and a row and a pixel more on both sides are one run, except for 112 pixels a row, where a box
+// holds the run of one kernel row (408 pixels, where one run would take 360 and two boxes).
+// Stride 2: the input rows of the output rows that the tile touches, BR rows to a box.
+// A box has LEAD pixels in front of the tile's, so that it starts at a multiple of 4 pixels and four pixels of a row at one; PB / 4
+// is odd, so that 16-byte loads of 8 channels fall into different banks.
+template <int WI_, int S_>
+struct DwShape {
+    static constexpr int WI = WI_, S = S_, WO = WI / S, SUB = S == 1 ? 16 : 8;
+    static constexpr bool ROWS3 = S == 1 && WI == 112;
+    static constexpr int BR = WI == 112 ? 1 : 2;         // (stride 2)
+    static constexpr int LEAD = S == 2 ? 0 : (ROWS3 ? 4 : WI + 4);
+    static constexpr int RUN = S == 2 ? BR * WI : (ROWS3 ? 133 : 128 + WI + 1 + LEAD);
+    static constexpr int PB = (RUN + 3) / 4 * 4 + ((RUN + 3) / 4 % 2 ? 0 : 4);
+    static constexpr int BOXES = S == 2 ? (2 * ((126 + WO) / WO) + 3 + BR - 1) / BR : (ROWS3 ? 3 : 1);
+    static constexpr int BOX = SUB * PB;                 // floats
+    static constexpr int X_BYTES = BOXES * BOX * 4, COPIED = X_BYTES + 10 * SUB * 4, STAGE = (COPIED + 127) / 128 * 128;
+    // The depthwise output of a stage on its way from lanes that own channels to lanes that own pixels, of each split warpgroup.
+    static constexpr int PITCH = 132, OUTPUT = 2 * SUB * PITCH * 4;
+    static constexpr int ZEROS = 16;                     // what is read outside the image
+    static_assert(WI % 4 == 0 && WO % 4 == 0 && PB <= 256 && PB / 4 % 2 == 1 && BOX * 4 % 128 == 0, "boxes");
+};
+template <>
+struct DwShape<0, 1> {
+    static constexpr int SUB = 32, COPIED = 0, STAGE = 0, OUTPUT = 0, ZEROS = 0, S = 1;
+};
+
+template <int BN_, int SRC_, bool OUT_CM_, bool SPLIT_ = false, int IMAGES_ = 3, int WI_ = 0, int STRIDE_ = 1>
 struct TC {
     static constexpr int BM = 128, BN = BN_, BK = 64, SRC = SRC_;
+    static constexpr bool FUSED = SRC == SRC_DW;
+    using DW = DwShape<WI_, STRIDE_>;
+    using Args = std::conditional_t<FUSED, DwArgs, TcArgs>;
     static constexpr bool OUT_CM = OUT_CM_, SPLIT = SPLIT_;
     static constexpr int IMAGES = IMAGES_;
     static constexpr int TAPS = SRC == SRC_IM2COL || SRC == SRC_CM3 ? 9 : 1;
@@ -102,16 +146,18 @@ struct TC {
     static constexpr int PIX = SRC == SRC_CM3 ? 136 : 128;   // pixels of a stage
     static constexpr int NUC = BN < 128 ? BN : 128;      // columns of one MMA
     static constexpr int NU = BN / NUC;                  // MMA column blocks per tile
-    static constexpr int SUB = 32;                       // channels of one activation stage
-    static constexpr int A_BYTES = SUB * PIX * 4;
+    static constexpr int SUB = DW::SUB;                  // channels of one activation stage
+    static constexpr int A_COPIED = FUSED ? DW::COPIED : SUB * PIX * 4, A_BYTES = FUSED ? DW::STAGE : A_COPIED;
     static constexpr int B_BYTES = IMAGES * NUC * BK * 2;
-    static constexpr int OUT_BYTES = 8 * 2 * 2048;       // two staging tiles of 32 pixels x 16 channels for each drain warp
-    static constexpr int CTRL = 512;                     // mbarriers, tensor-memory base, abort flag
+    static constexpr int OUT_TILES = DW::S == 2 ? 1 : 2;      // staging tiles of 32 pixels x 16 channels for each drain warp
+    static constexpr int OUT_BYTES = 8 * OUT_TILES * 2048;
+    static constexpr int CTRL = 512;                     // mbarriers, tensor-memory base, abort flag; zeros for SRC_DW
     // Stages share what is left of 227 KB: weights that fit as a whole and serve every tile stay (see launch_tc), else
     // SB stages of them; the rest goes to activations, up to SA_MAX stages.
-    static constexpr int SB = IMAGES == 1 ? 6 : (BN < 128 ? 4 : (SRC == SRC_CM3 ? 2 : 3)), SA_MAX = 12, SB_MAX = 6;
-    static constexpr int ROOM = 227 * 1024 - 1024 - CTRL - OUT_BYTES;
-    static_assert((2 * SA_MAX + 3 * SB_MAX + 12) * 8 + 8 <= CTRL && SB * B_BYTES + (SRC == SRC_CM3 ? 4 : 3) * A_BYTES <= ROOM, "shared memory");
+    static constexpr int SB = IMAGES == 1 ? 6 : (BN < 128 ? (WI_ == 112 ? 2 : 4) : (WI_ == 112 ? 1 : (SRC == SRC_CM3 || FUSED ? 2 : 3))), SA_MAX = 12, SB_MAX = 6;
+    static constexpr int ROOM = 227 * 1024 - 1024 - CTRL - OUT_BYTES - DW::OUTPUT;
+    static constexpr int SA_MIN = SRC == SRC_CM3 || FUSED ? 4 : 3;
+    static_assert((2 * SA_MAX + 3 * SB_MAX + 12) * 8 + 8 + 16 + DW::ZEROS <= CTRL && SB * B_BYTES + SA_MIN * A_BYTES <= ROOM, "shared memory");
     static constexpr int NT = 640;
     // registers a thread of the drain, split and remaining warps: 2 x + 2 y + z = 5 x 96, what the launch reserves
     static constexpr int LAUNCH_REGS = 96, DRAIN_REGS = BN == 256 ? 160 : 128, SPLIT_REGS = BN == 256 ? 56 : 80, AUX_REGS = BN == 256 ? 48 : 64;
@@ -123,7 +169,7 @@ struct TC {
     static_assert(A_COL0 + NA * A_COLS <= 512, "tensor memory");
     static_assert(BN == 64 || BN == 128 || BN == 256, "tile width");
     // (shared by 7, the most for an exchange: 7 senders of up to 2 of a thread's 8 chunks)
-    static_assert(!SPLIT || (BN == 64 && SB * B_BYTES + 3 * A_BYTES >= 7 * 2 * 256 * 16), "the cluster's exchange");
+    static_assert(!SPLIT || (BN == 64 && SB * B_BYTES + SA_MIN * A_BYTES >= 7 * 2 * 256 * 16), "the cluster's exchange");
     static_assert(IMAGES == 3 || (IMAGES == 1 && SRC == SRC_NHWC), "bf16 mode");
 };
 
@@ -258,6 +304,21 @@ __device__ __forceinline__ bool drain_any(bool mine) {
     return r != 0;
 }
 
+// One output of the depthwise layer in front (SRC_DW), straight from global memory: for the few pixels that are summed again.
+template <class T>
+__device__ __noinline__ float depthwise_output(const DwArgs& a, int m, int c) {
+    constexpr int WI = T::DW::WI, WO = T::DW::WO, S = T::DW::S;
+    const int x = m % WO, f = m / WO, y = f % WO;
+    const float* const from = a.ex.x + c * a.ex.channel_stride + ((long long)f * S - 1) * WI + x * S - 1;
+    float sum = a.dw_b[c];
+    for (int t = 0; t < 9; ++t) {
+        const int iy = y * S + t / 3 - 1, ix = x * S + t % 3 - 1;
+        const float v = (unsigned)iy < (unsigned)WI && (unsigned)ix < (unsigned)WI ? from[t / 3 * WI + t % 3] : 0.0f;
+        sum = fmaf(v, a.dw_w[t * a.Cin + c], sum);
+    }
+    return fmaxf(sum, 0.0f);
+}
+
 // All drain threads: sums pixels of the tile that starts at m0 once more, as fp32 FMAs over the kept units.  A pixel with an
 // infinity or a NaN in any channel spoils all its split products (0 * inf), also those of pruned weights, which must not see
 // it; and sums near the end of the fp32 range may overflow here but not product after product with the bias last, as on the FMA kernels.  `bad` says which of the pixels m0 + 32 * q + lane (q = the warp's place in its warpgroup); a warpgroup wg has `len`
@@ -268,13 +329,13 @@ __device__ __forceinline__ bool drain_any(bool mine) {
 // a pixel, in the middle of the tile loop: 2800; the FMA kernels: 89); with a bad channel in every pixel: 372 us (9600; 88), or
 // 2500 with the activations read from global memory.
 template <class T>
-__device__ __noinline__ void sum_kept_units(const TcArgs& args, unsigned char* room, float* sums, int m0, bool bad, int n0, int len) {
+__device__ __noinline__ void sum_kept_units(const typename T::Args& args, unsigned char* room, float* sums, int m0, bool bad, int n0, int len) {
     const ExactArgs e = args.ex;
     const int W = args.W, H = args.H, Cin = args.Cin, Cout = args.Cout, relu = args.relu, ldy = args.ldy;
     float* const y = args.y;
     const float* const bias = args.bias;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, width = e.G < 4 ? e.G : 4;
-    constexpr bool CM = T::SRC == SRC_CM || T::SRC == SRC_CM3;
+    constexpr bool CM = T::SRC == SRC_CM || T::SRC == SRC_CM3 || T::FUSED;
     uint32_t* const found = reinterpret_cast<uint32_t*>(room);
     int* const list = reinterpret_cast<int*>(room + 64);
     int* const where = reinterpret_cast<int*>(room + 1024) + warp * 32;        // 32 (unit, tap) pairs of a warp: place of the row,
@@ -316,6 +377,12 @@ __device__ __noinline__ void sum_kept_units(const TcArgs& args, unsigned char* r
                 for (int t = 0; t < T::TAPS; ++t) {
                     const float* const x = p < pixels ? source(p, t) : nullptr;
                     for (int c = c0 + warp * us + u; c < c1; c += 64 * us) {
+                        if constexpr (T::FUSED) {
+#pragma unroll 1
+                            for (int k = 0; k < 8; ++k)
+                                if (c + 8 * us * k < c1) *place(c + 8 * us * k, 0, p) = x ? depthwise_output<T>(args, list[first + p], c + 8 * us * k) : 0.0f;
+                            continue;
+                        }
 #pragma unroll
                         for (int k = 0; k < 8; ++k) v[k] = x && c + 8 * us * k < c1 ? x[(c + 8 * us * k) * e.channel_stride] : 0.0f;
 #pragma unroll
@@ -411,7 +478,7 @@ __device__ __noinline__ void sum_kept_units(const TcArgs& args, unsigned char* r
 // chunks of others into their shared memory, [sender][chunk][thread], and then adds up and stores its own.  The stages hold the
 // exchange: every CTA's MMAs are complete when its drain threads reach the first barrier.
 template <class T>
-__device__ __forceinline__ void store_shared_tile(const TcArgs& a, uint64_t (&acc)[T::COLS / 2], unsigned char* room, float* sums, int m0, int tid) {
+__device__ __forceinline__ void store_shared_tile(const typename T::Args& a, uint64_t (&acc)[T::COLS / 2], unsigned char* room, float* sums, int m0, int tid) {
     constexpr int CHUNKS = T::COLS / 4;
     const uint32_t exchange = smem_u32(room);
     const unsigned char* const mine = room;
@@ -461,9 +528,179 @@ __device__ __forceinline__ void store_shared_tile(const TcArgs& a, uint64_t (&ac
     if (T::IMAGES == 3 && drain_any(redo)) sum_kept_units<T>(a, room, sums, m0, redo, n00 + first * 4, own * 4);
 }
 
+__device__ __forceinline__ float shared_f1(uint32_t addr) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ float4 shared_f4(uint32_t addr) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ void store_relu(uint32_t addr, const float (&s)[4]) {
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};"
+                 ::"r"(addr), "f"(fmaxf(s[0], 0.0f)), "f"(fmaxf(s[1], 0.0f)), "f"(fmaxf(s[2], 0.0f)), "f"(fmaxf(s[3], 0.0f))
+                 : "memory");
+}
+
+// A thread of the split warpgroups in a launch with a depthwise layer (SRC_DW): lanes 8 * i .. 8 * i + 7 of warp q own 8 channels
+// of a run of pixels, which they take four at a time.
+template <class D>
+struct DwThread {
+    static constexpr int BLOCKS = D::SUB / 8, GROUPS = D::SUB / 4;    // blocks of 8 channels, groups of 4 pixels
+    int c, p0;
+    int x, y, r;                                                      // of the tile's first group: its place in the image, and (stride 2) in the stage
+    __device__ DwThread(int q, int lane) : c(q % BLOCKS * 8 + (lane & 7)), p0(q / BLOCKS * 32 * BLOCKS + (lane >> 3) * 4 * GROUPS) {}
+    __device__ void tile(int m0) {
+        const int m = m0 + p0, f = m / D::WO;
+        x = m % D::WO;
+        y = f % D::WO;
+        r = 2 * (f - m0 / D::WO);                                     // box rows r, r + 1, r + 2
+    }
+    // A stage's depthwise output, bias first and the taps in order as in the depthwise kernels, then ReLU; `zeros`: what is outside.
+    // Bound by the latency of one warp's instructions: a stage of 16 channels takes a warpgroup 1000 cycles, 500 more the split.
+    // (With a pixel a lane, for every tap a load of each channel and its weight, a 64-channel step took 6000 cycles instead of 4400:
+    // the loads fill 11 values for each output.  Four split warpgroups with stages of 8 channels: 82 instead of 69 us for 64
+    // images of 56 x 56, 128 -> 128; the columns beside a group summed apart, to save selects: 73.)
+    __device__ __forceinline__ void run(uint32_t stage, uint32_t out, uint32_t zeros) const {
+        float w[9];
+#pragma unroll
+        for (int t = 0; t < 9; ++t) w[t] = shared_f1(stage + D::X_BYTES + (t * D::SUB + c) * 4);
+        const float bias = shared_f1(stage + D::X_BYTES + (9 * D::SUB + c) * 4);
+        const uint32_t to = out + (c * D::PITCH + p0) * 4;
+        int x = this->x, y = this->y;
+        if constexpr (D::S == 1) {
+            uint32_t row[3];                                          // of the first group
+#pragma unroll
+            for (int i = 0; i < 3; ++i) row[i] = stage + (c * D::PB + D::LEAD + p0 + (D::ROWS3 ? i * D::BOX : (i - 1) * D::WI)) * 4;
+            auto at = [&](int i, int y, uint32_t addr) { return i == 1 || (i == 0 ? y > 0 : y < D::WO - 1) ? addr : zeros; };
+            float left[3];
+            float4 here[3];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                here[i] = shared_f4(at(i, y, row[i]));
+                left[i] = shared_f1(at(i, y, row[i] - 4));
+            }
+#pragma unroll
+            for (int g = 0; g < GROUPS; ++g) {
+                const bool first = x == 0, last = x == D::WO - 4;
+                const int yn = !last ? y : (y == D::WO - 1 ? 0 : y + 1);
+                float4 next[3];
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    if (g < GROUPS - 1) next[i] = shared_f4(at(i, yn, row[i] + 16 * g + 16));
+                    else next[i].x = shared_f1(at(i, y, row[i] + 16 * g + 16));
+                }
+                float s[4] = {bias, bias, bias, bias};
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    const float v[6] = {first ? 0.0f : left[i], here[i].x, here[i].y, here[i].z, here[i].w, last ? 0.0f : next[i].x};
+#pragma unroll
+                    for (int t = 0; t < 3; ++t)
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) s[k] = fmaf(v[k + t], w[3 * i + t], s[k]);
+                    left[i] = here[i].w;
+                    here[i] = next[i];
+                }
+                store_relu(to + 16 * g, s);
+                x = last ? 0 : x + 4;
+                y = yn;
+            }
+        } else {
+            int r = this->r;
+            float left[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll
+            for (int g = 0; g < GROUPS; ++g) {
+                const bool first = x == 0;
+                float s[4] = {bias, bias, bias, bias};
+                float4 a[3], b[3];
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    const uint32_t row = stage + ((r + i) / D::BR * D::BOX + c * D::PB + (r + i) % D::BR * D::WI + 2 * x) * 4;
+                    const bool in = i > 0 || y > 0;
+                    a[i] = shared_f4(in ? row : zeros);
+                    b[i] = shared_f4(in ? row + 16 : zeros);
+                    if (g == 0) left[i] = shared_f1(in && !first ? row - 4 : zeros);
+                }
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    const float v[9] = {first ? 0.0f : left[i], a[i].x, a[i].y, a[i].z, a[i].w, b[i].x, b[i].y, b[i].z, b[i].w};
+#pragma unroll
+                    for (int t = 0; t < 3; ++t)
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) s[k] = fmaf(v[2 * k + t], w[3 * i + t], s[k]);
+                    left[i] = b[i].w;
+                }
+                store_relu(to + 16 * g, s);
+                x += 4;
+                if (x == D::WO) {
+                    x = 0;
+                    r += 2;
+                    y = y == D::WO - 1 ? 0 : y + 1;
+                }
+            }
+        }
+    }
+};
+
+// The split warps of a launch whose activations are the output of a depthwise layer (SRC_DW).  The two warpgroups take the
+// stages in turn (an even number of them, so that a stage always belongs to the same one): depthwise output into shared
+// memory, then as for other sources, a pixel a lane, into bf16 images.  A warp that gave up still joins its warpgroup's barriers.
+// `wait`, `stages`: as in the kernel.
+template <class T, class Stages, class Wait>
+__device__ __forceinline__ bool depthwise_split(const DwArgs& a, const unsigned char* ast, float* out, const float4* zeros, Ring ring, uint64_t* xfull,
+                                                uint64_t* xempty, uint64_t* afull, uint64_t* aempty, uint32_t lane_base, int half, int q, int lane,
+                                                int kb, int ke, Stages stages, Wait wait) {
+    using D = typename T::DW;
+    auto together = [&] { asm volatile("barrier.cta.sync %0, 128;" ::"r"(2 + half) : "memory"); };
+    const float* const pixel = out + q * 32 + lane;
+    DwThread<D> thread(q, lane);
+    int step = 0;
+    bool ok = true;
+    if (half) ring.next();
+    for (Tiles t(a); t.left(); t.next()) {
+        thread.tile(t.m * T::BM);
+        for (int k0 = kb; k0 < ke; ++k0, ++step) {
+            const int as = step % T::NA, n = stages(k0);
+            for (int i = half; i < n; i += 2) {
+                // lane 0: the place in tensor memory is free, others: the stage is here
+                const bool place = lane == 0 && i == half && step >= T::NA;
+                ok = ok && wait(place ? aempty + as : xfull + ring.stage, place ? ((step / T::NA) & 1) ^ 1 : ring.parity);
+                if (ok) {
+                    tc_fence_after_sync();
+                    thread.run(smem_u32(ast) + ring.stage * T::A_BYTES, smem_u32(out), smem_u32(zeros));
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(xempty + ring.stage);
+                }
+                together();
+                if (ok) {
+                    const uint32_t col = lane_base + as * T::A_COLS + i * D::SUB / 2;
+                    uint32_t h[D::SUB / 2], md[D::SUB / 2], lo[D::SUB / 2];
+#pragma unroll
+                    for (int k = 0; k < D::SUB / 2; ++k)
+                        split2(pack2(pixel[2 * k * D::PITCH], pixel[(2 * k + 1) * D::PITCH]), h[k], md[k], lo[k]);
+                    tmem_st(col + 32, md);
+                    tmem_st(col + 64, lo);
+                    tmem_st(col, h);
+                }
+                together();
+                ring.next();
+                ring.next();
+            }
+            if (!ok) continue;
+            tmem_st_wait();
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(afull + as);
+        }
+    }
+    return ok;
+}
+
 template <class T>
 __global__ void __launch_bounds__(T::NT, 1)
-conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap ymap, const __grid_constant__ TcArgs a) {
+conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap ymap, const __grid_constant__ typename T::Args a) {
     constexpr int NUC = T::NUC, NU = T::NU, BN = T::BN;
     const int SA = a.sa, SB = a.sb;
     extern __shared__ unsigned char raw[];
@@ -483,12 +720,15 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, wg = warp >> 2;
+    float* const dwout = reinterpret_cast<float*>(ost + T::OUT_BYTES + T::CTRL);   // SRC_DW: see DwShape
+    float4* const zeros = reinterpret_cast<float4*>(ost + T::OUT_BYTES + T::CTRL - 16);
+    if (T::FUSED && tid == 0) *zeros = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (warp == 16 && lane == 0) {
         prefetch_map(&amap);
         prefetch_map(&ymap);
     }
     if (tid == 0) {
-        for (int s = 0; s < SA; ++s) { mbar_init(xfull + s, 1); mbar_init(xempty + s, 8); }
+        for (int s = 0; s < SA; ++s) { mbar_init(xfull + s, 1); mbar_init(xempty + s, T::FUSED ? 4 : 8); }
         for (int s = 0; s < SB; ++s) { mbar_init(bfull + s, 1); mbar_init(bfull + SB + s, 1); mbar_init(bempty + s, 1); }
         for (int s = 0; s < 2; ++s) {
             mbar_init(dfull + s, 1); mbar_init(dempty + s, T::DEMPTY);
@@ -529,8 +769,9 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
         kb = runs * rank / a.split * T::RUN;
         ke = runs * (rank + 1) / a.split * T::RUN;
     }
-    // valid 32-channel halves of a step
+    // valid 32-channel halves of a step, and its activation stages
     auto subs = [&](int k) { return a.Cin - (k / T::TAPS) * 64 > 32 ? 2 : 1; };
+    auto stages = [&](int k) { return subs(k) * (32 / T::SUB); };
 
     if (wg >= 2) {
         if (wg < 4) regs_dec<T::SPLIT_REGS>(); else regs_dec<T::AUX_REGS>();
@@ -545,10 +786,10 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                 int px = 0, py = 0, pn = 0;
                 if (T::SRC == SRC_IM2COL) { px = m0 % a.W; py = (m0 / a.W) % a.H; pn = m0 / (a.W * a.H); }
                 for (int k = kb; k < ke && ok; k += T::RUN) {
-                    const int c = k / T::TAPS, tap = k - c * T::TAPS, halves = subs(k);
+                    const int c = k / T::TAPS, tap = k - c * T::TAPS, halves = stages(k);
                     // With stages enough both halves of a step are asked for after one wait: a wait and an issue take a warp
                     // 370 cycles, which for 16 KB at a time is slower than the memory.
-                    const int batch = SA >= 4 ? halves : 1;
+                    const int batch = SA >= 4 ? (T::FUSED ? 2 : halves) : 1;
                     for (int h = 0; h < halves && ok; h += batch) {
                         Ring second = ring;
                         second.next();
@@ -558,7 +799,17 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                             for (int b = 0; b < batch; ++b) {
                                 const int s = b ? second.stage : ring.stage, c0 = c * 64 + (h + b) * T::SUB;
                                 unsigned char* dst = ast + (size_t)s * T::A_BYTES;
-                                mbar_arrive_expect_tx(xfull + s, T::A_BYTES);
+                                mbar_arrive_expect_tx(xfull + s, T::A_COPIED);
+                                if constexpr (T::FUSED) {
+                                    using D = typename T::DW;
+                                    const int first = D::S == 2 ? (2 * (m0 / D::WO) - 1) * D::WI - D::LEAD : (D::ROWS3 ? m0 - D::WI : m0) - D::LEAD;
+#pragma unroll
+                                    for (int i = 0; i < D::BOXES; ++i)
+                                        tensor_g2s_2d(dst + i * D::SUB * D::PB * 4, &amap, first + i * (D::S == 2 ? D::BR : 1) * D::WI, c0, xfull + s);
+                                    tensor_g2s_2d(dst + D::X_BYTES, &a.wmap, c0, 0, xfull + s);
+                                    bulk_g2s(dst + D::X_BYTES + 9 * D::SUB * 4, a.dw_b + c0, D::SUB * 4, xfull + s);
+                                    continue;
+                                }
                                 if (T::SRC == SRC_CM) tensor_g2s_2d(dst, &amap, m0, c0, xfull + s);
                                 else if (T::SRC == SRC_CM3) tensor_g2s_2d(dst, &amap, (m0 + (tap / 3 - 1) * a.W - 1) & ~3, c0, xfull + s);
                                 else if (T::SRC == SRC_NHWC) tensor_g2s_2d(dst, &amap, c0, m0, xfull + s);
@@ -678,6 +929,10 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
             Ring ring(SA);
             bool ok = true;
             grid_dependency_wait();
+            if constexpr (T::FUSED) {
+                ok = depthwise_split<T>(a, ast, dwout + half * T::DW::SUB * T::DW::PITCH, zeros, ring, xfull, xempty, afull, aempty, lane_base, half, q, lane, kb,
+                                        ke, stages, wait);
+            } else
             for (Tiles t(a); t.left() && ok; t.next()) {
                 int px = 0, py = 0;                         // SRC_CM3: the pixel's place in its image
                 if (T::SRC == SRC_CM3) {
@@ -709,7 +964,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                     for (int h = 0; h < halves; ++h, at.next()) {
                         const int s = at.stage;
                         const unsigned char* src = ast + (size_t)s * T::A_BYTES;
-                        uint64_t v[8];                      // pairs of neighbouring channels
+                        uint64_t v[8];                // pairs of neighbouring channels
                         if (T::SRC == SRC_CM || T::SRC == SRC_CM3) {
                             const float* row = reinterpret_cast<const float*>(src) + half * 16 * T::PIX + shift + p;
 #pragma unroll
@@ -725,13 +980,13 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                         if (T::IMAGES == 3) {
 #pragma unroll
                             for (int k = 0; k < 8; ++k) split2(v[k], hh[k], mm[k], ll[k]);
-                            tmem_st8(col + h * 16 + 32, mm);
-                            tmem_st8(col + h * 16 + 64, ll);
+                            tmem_st(col + h * 16 + 32, mm);
+                            tmem_st(col + h * 16 + 64, ll);
                         } else {
 #pragma unroll
                             for (int k = 0; k < 8; ++k) hh[k] = bf16_of(v[k]);
                         }
-                        tmem_st8(col + h * 16, hh);
+                        tmem_st(col + h * 16, hh);
                         __syncwarp();
                         if (lane == 0 && tap % T::RUN == T::RUN - 1) mbar_arrive(xempty + s);
                     }
@@ -753,7 +1008,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
         regs_inc<T::DRAIN_REGS>();
         const int q = warp & 3;
         const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16);
-        unsigned char* stage = ost + (size_t)warp * 4096;
+        unsigned char* stage = ost + (size_t)warp * (T::OUT_TILES * 2048);
         int step = 0, copies = 0;                           // copies issued: the two tiles alternate between them
         bool ok = true, again = false;                      // again: some of this lane's pixels have to be summed once more
         grid_dependency_wait();                             // Y may still be read by the previous kernel of the stream
@@ -826,8 +1081,10 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                         for (int i = 0; i < 16; ++i)
                             if (m < a.M && n0 + c0 + i < a.Cout) a.y[(size_t)(n0 + c0 + i) * a.ldy + m] = o[i];
                     } else {
-                        unsigned char* tile = stage + (copies++ & 1) * 2048;
-                        if (elect_one()) bulk_wait_read_pending1();   // the copy that last read this tile is done with it
+                        unsigned char* tile = stage + (copies++ & (T::OUT_TILES - 1)) * 2048;
+                        if (elect_one()) {                  // the copy that last read this tile is done with it
+                            if (T::OUT_TILES == 2) bulk_wait_read_pending1(); else bulk_wait_read_all();
+                        }
                         __syncwarp();
                         if (T::OUT_CM) {
 #pragma unroll
@@ -955,6 +1212,9 @@ struct TcCall {
     int N, H, W;       // 3x3
     int relu;
     cudaStream_t st;
+    const float* dw_w;  // SRC_DW: the depthwise layer in front, and the pixels of its input
+    const float* dw_b;
+    long long M_in;
 };
 
 // ---- which kernel, and how ------------------------------------------------------------------------
@@ -1036,28 +1296,61 @@ TcChoice tc_choose(const sbnn_packed* p, long long M, int run, int images) {
 // (32 x 28 x 28, 256 -> 256: 305 -> 119 us at 50 %, 120 -> 111 at 90 %; in groups of 8 106 and 111).
 // `choice` is how; it is remembered with the layer for each kind of call and number of pixels.
 enum Call { CALL_1X1_NHWC, CALL_1X1_CM, CALL_3X3, CALL_3X3_CM, CALL_BF16 };
-TcChoice decide(const sbnn_packed* p, long long M, Call call) {
-    TcChoice choice = {0, 0, 0.0};
-    if (call == CALL_BF16) return tc_choose(p, M, 1, 1);
-    if (!p->finite || p->nnz == 0) return choice;
+double fma_us(const sbnn_packed* p, long long M, Call call) {
     const double bytes = 4.0 * M * (p->Cin + p->Cout), mem = bytes / 6.5e6;
     const double dense = 1e-6 * M * p->Cin * p->Cout;                        // 1e6 multiply-adds of the unpruned layer, a tap
     double kept = 1e-6 * M * p->nnz * p->G * (p->KH * p->KW);                // and of what is kept
     if (!p->tap_mask.empty()) kept *= (double)count_kept_taps(p) / ((double)p->nnz * p->KH * p->KW);
-    double fma;
-    if (call == CALL_3X3 || call == CALL_3X3_CM) {
-        fma = 25.0 + kept * (p->G >= 8 ? 0.050 : 0.075);
-    } else if (call == CALL_1X1_CM && conv1x1_few_tiles(p, M)) {
-        fma = 1.8 + kept * ((M + 31) / 32 * 32) / M * (p->G >= 8 ? 0.145 : 0.20);   // (a lane takes a pixel)
-    } else if (call == CALL_1X1_CM || (p->Cin >= 128 && M >= 2048)) {
-        fma = 4.5 + 0.034 * kept + 0.0011 * dense + 0.65 * mem;
-        if (call == CALL_1X1_NHWC) fma += 2.0 + 8.0 * M * p->Cin / 4.5e6;    // the conversion to channel-major
-    } else {
-        fma = 2.0 + (p->Cin >= 128 ? 2.0 : 0.0) + 0.012 * p->Cin + 0.1 * kept;
+    if (call == CALL_3X3 || call == CALL_3X3_CM) return 25.0 + kept * (p->G >= 8 ? 0.050 : 0.075);
+    if (call == CALL_1X1_CM && conv1x1_few_tiles(p, M)) {
+        return 1.8 + kept * ((M + 31) / 32 * 32) / M * (p->G >= 8 ? 0.145 : 0.20);   // (a lane takes a pixel)
     }
+    if (call == CALL_1X1_CM || (p->Cin >= 128 && M >= 2048)) {
+        const double conversion = call == CALL_1X1_NHWC ? 2.0 + 8.0 * M * p->Cin / 4.5e6 : 0.0;   // to channel-major
+        return 4.5 + 0.034 * kept + 0.0011 * dense + 0.65 * mem + conversion;
+    }
+    return 2.0 + (p->Cin >= 128 ? 2.0 : 0.0) + 0.012 * p->Cin + 0.1 * kept;
+}
+TcChoice decide(const sbnn_packed* p, long long M, Call call) {
+    TcChoice choice = {0, 0, 0.0};
+    if (call == CALL_BF16) return tc_choose(p, M, 1, 1);
+    if (!p->finite || p->nnz == 0) return choice;
     choice = tc_choose(p, M, call == CALL_3X3_CM ? 3 : 1, 3);
-    if (std::max(tc_us(choice.cost), mem) >= 0.95 * fma) choice.bn = 0;
+    if (std::max(tc_us(choice.cost), 4.0 * M * (p->Cin + p->Cout) / 6.5e6) >= 0.95 * fma_us(p, M, call)) choice.bn = 0;
     return choice;
+}
+
+// A block of the network (a depthwise layer with images of `side` pixels a row and the 1x1 layer behind it, N images): the
+// tile of the launch that does both, bn = 0 where two launches are faster.  Microseconds, in one launch and apart (alone, back to
+// back), half pruned: 64 images of 112 x 112, 32 -> 64: 68 and 101; 112 -> 56, 64 -> 128: 61 and 73; 56 x 56, 128 -> 128: 69 and 78;
+// 56 -> 28, 128 -> 256: 39 and 48; 28 x 28, 256 -> 256: 46 and 53; 9 images 12.4 and 15.6, 12.9 and 12.7, 16.0 and 15.4, 11.4 and
+// 11.4, 15.4 and 13.4; one image 4.8 and 6.6, 6.9 and 6.9, 8.1 and 7.7, 9.2 and 7.8, 8.5 and 8.7.  The network at batch 64: 774 ->
+// 695 us.  The depthwise layer is computed again for every tile of output channels, on the split warps, so a step takes 2400 (128
+// channels a tile) to 3300 cycles longer than without (twice that at stride 2, whose stages hold 8 channels); layers with
+// smaller maps, more channels and less to move (14 x 14, 512 -> 512: 9 + 30 us) stay apart.
+double block_step(int bn, int stride) { return stride == 2 ? (bn == 256 ? 8700.0 : 6500.0) : (bn == 256 ? 5500.0 : 4400.0); }
+TcChoice decide_block(const sbnn_packed* p, int N, int side, int stride) {
+    const long long out = side / stride, M = N * out * out, M_in = (long long)N * side * side, sms = device_sms();
+    TcChoice best = {0, 0, 0.0};
+    if (!p->finite || p->nnz == 0 || side < 28 || out < 28) return best;
+    const double depthwise = 4.0 * (M_in + M) * p->Cin;              // bytes of the depthwise launch
+    const double steps = p->Cin / 64.0, mem = 4.0 * (M_in * p->Cin + M * p->Cout) / 5.0e6;
+    double us = 0.0;
+    for (int bn : {64, 128, 256}) {
+        if (bn > p->Cout || (bn == 256 && out > 28)) continue;
+        const long long tiles = (M + 127) / 128 * ((p->Cout + bn - 1) / bn);
+        const double cycles = (double)((tiles + sms - 1) / sms) * (steps * block_step(bn, stride) + (bn == 64 ? 1300.0 : 1000.0 + 12.0 * bn)) + 4700.0;
+        const double t = std::max(cycles / 1800.0, mem);
+        if (best.bn == 0 || t < us) {
+            best = {bn, 1, cycles};
+            us = t;
+        }
+    }
+    const TcChoice layer = decide(p, M, CALL_1X1_CM);
+    const double apart = (layer.bn ? std::max(tc_us(layer.cost), 4.0 * M * (p->Cin + p->Cout) / 6.5e6) : fma_us(p, M, CALL_1X1_CM)) + 2.0 +
+                         depthwise / (depthwise < 1e8 ? 5.0e6 : 4.6e6);
+    if (us >= 0.95 * apart) best.bn = 0;
+    return best;
 }
 bool tc_profits(const sbnn_packed* p, long long M, Call call, TcChoice* choice = nullptr) {
     if (forced_choice) {
@@ -1128,7 +1421,7 @@ sbnn_status launch_tc(const sbnn_packed* p, const TcCall& c, int split, bool* do
         known = regs = fa.numRegs;
     }
     if (regs != T::LAUNCH_REGS) return SBNN_OK;
-    TcArgs a = {};
+    typename T::Args a = {};
     uint4* wts = nullptr;
     if ((r = get_tc_weights(p, T::NUC, T::IMAGES, c.M, c.st, &wts)) != SBNN_OK || !wts) return r;
     if ((r = async_status_word(&a.status)) != SBNN_OK) return r;
@@ -1139,10 +1432,18 @@ sbnn_status launch_tc(const sbnn_packed* p, const TcCall& c, int split, bool* do
     a.wts = wts; a.bias = p->d_bias; a.y = c.y; a.ldy = c.ldy; a.M = (int)c.M; a.Cin = p->Cin; a.Cout = p->Cout;
     a.steps = (p->Cin + 63) / 64 * T::TAPS; a.ntiles_m = (int)((c.M + T::BM - 1) / T::BM); a.ntiles_n = (int)ntiles_n;
     a.W = c.W; a.H = c.H; a.relu = c.relu; a.split = T::SPLIT ? split : 1;
-    const bool cm = T::SRC == SRC_CM || T::SRC == SRC_CM3;
+    const bool cm = T::SRC == SRC_CM || T::SRC == SRC_CM3 || T::FUSED;
     a.ex = {c.x, cm ? 1 : p->Cin, cm ? c.ldx : 1, p->d_group_ptr, p->d_idx, p->d_val, use_tap_lists(p) ? p->d_taps : nullptr, p->G};
     CUtensorMap amap, ymap;
-    if (T::SRC == SRC_IM2COL) {
+    if constexpr (T::FUSED) {
+        using D = typename T::DW;
+        a.dw_w = c.dw_w; a.dw_b = c.dw_b; a.M_in = c.M_in;
+        const unsigned long long dims[2] = {(unsigned long long)c.M_in, (unsigned long long)p->Cin}, wdims[2] = {(unsigned long long)p->Cin, 9};
+        const unsigned long long strides[1] = {(unsigned long long)c.ldx * 4}, wstrides[1] = {(unsigned long long)p->Cin * 4};
+        const unsigned box[2] = {(unsigned)D::PB, (unsigned)D::SUB}, wbox[2] = {(unsigned)D::SUB, 9u};
+        if ((r = encode_tiled_map(&amap, c.x, 4, 2, dims, strides, box)) != SBNN_OK) return r;
+        if ((r = encode_tiled_map(&a.wmap, c.dw_w, 4, 2, wdims, wstrides, wbox)) != SBNN_OK) return r;
+    } else if (T::SRC == SRC_IM2COL) {
         if ((r = encode_im2col_3x3_map(&amap, c.x, c.N, c.H, c.W, p->Cin, T::SUB, T::BM)) != SBNN_OK) return r;
     } else if (cm) {
         const unsigned long long dims[2] = {(unsigned long long)c.M, (unsigned long long)p->Cin};
@@ -1164,10 +1465,11 @@ sbnn_status launch_tc(const sbnn_packed* p, const TcCall& c, int split, bool* do
     const unsigned grid = T::SPLIT ? (unsigned)(total * split) : (unsigned)std::min<long long>(total, device_sms());
     a.dm = T::SPLIT ? a.ntiles_m : (int)(grid / (unsigned)ntiles_n);
     a.dn = T::SPLIT ? 0 : (int)(grid % (unsigned)ntiles_n);
-    a.resident = !T::SPLIT && ntiles_n == 1 && a.steps * T::NU <= T::SB_MAX && a.steps * T::NU * T::B_BYTES + 3 * T::A_BYTES <= T::ROOM;
+    a.resident = !T::SPLIT && ntiles_n == 1 && a.steps * T::NU <= T::SB_MAX && a.steps * T::NU * T::B_BYTES + (T::FUSED ? T::SA_MIN : 3) * T::A_BYTES <= T::ROOM;
     a.sb = a.resident ? a.steps * T::NU : T::SB;
     a.sa = std::min(T::SA_MAX, (T::ROOM - a.sb * T::B_BYTES) / T::A_BYTES);
-    const size_t smem = (size_t)a.sb * T::B_BYTES + (size_t)a.sa * T::A_BYTES + T::OUT_BYTES + T::CTRL + 1024;
+    if (T::FUSED) a.sa &= ~1;   // (see depthwise_split)
+    const size_t smem = (size_t)a.sb * T::B_BYTES + (size_t)a.sa * T::A_BYTES + T::OUT_BYTES + T::CTRL + T::DW::OUTPUT + 1024;
     last_route = {T::BN, a.split, 0.0};
     ChainedLaunchScope early;   // before their waits the kernel's warps read the layer's own arrays only
     SBNN_CUDA_TRY(launch_kernel_cluster(conv_tc_kernel<T>, dim3(grid), dim3(T::NT), smem, c.st, (unsigned)a.split, amap, ymap, a));
@@ -1259,6 +1561,65 @@ sbnn_status conv3x3_tc_cm(const sbnn_packed* p, const float* x, int ldx, float* 
     return out_cm ? dispatch_tc<SRC_CM3, true>(p, c, ch, done) : dispatch_tc<SRC_CM3, false>(p, c, ch, done);
 }
 
+namespace {
+template <int WI, int S>
+sbnn_status dispatch_dw(const sbnn_packed* p, const TcCall& c, const TcChoice& ch, bool* done) {
+    if constexpr (WI < 112) {                     // (steps to share)
+        if (ch.split > 1) return launch_tc<TC<64, SRC_DW, true, true, 3, WI, S>>(p, c, ch.split, done);
+    }
+    if constexpr (WI / S <= 28) {                 // 256 outputs
+        if (ch.bn == 256) return launch_tc<TC<256, SRC_DW, true, false, 3, WI, S>>(p, c, 1, done);
+    }
+    if constexpr (WI / S < 112) {
+        if (ch.bn == 128) return launch_tc<TC<128, SRC_DW, true, false, 3, WI, S>>(p, c, 1, done);
+    }
+    return ch.bn == 64 ? launch_tc<TC<64, SRC_DW, true, false, 3, WI, S>>(p, c, 1, done) : SBNN_OK;
+}
+}  // namespace
+
+sbnn_status dwconv3x3_conv1x1_tc_cm(const sbnn_packed* p, const float* dw_w, const float* dw_b, const float* x, int ldx, float* y, int ldy, int N,
+                                    int side, int stride, cudaStream_t st, bool* done) {
+    *done = false;
+    last_route = {0, 0, 0.0};
+    const int out = side / stride;
+    const long long M = (long long)N * out * out, M_in = (long long)N * side * side;
+    if ((p->Cin != 32 && p->Cin % 64) || p->Cout % 4 || M_in > kMaxPixels || !aligned16(x) || !aligned16(y) || !aligned16(dw_w) || !aligned16(dw_b)) return SBNN_OK;
+    TcChoice ch;
+    if (forced_choice) ch = *forced_choice;
+    else ch = decide_block(p, N, side, stride);
+    if (ch.split > (p->Cin + 63) / 64) return SBNN_OK;
+    const TcCall c{x, ldx, y, ldy, M, N, out, out, 1, st, dw_w, dw_b, M_in};
+    switch (side * 4 + stride) {
+        case 112 * 4 + 1: return dispatch_dw<112, 1>(p, c, ch, done);
+        case 112 * 4 + 2: return dispatch_dw<112, 2>(p, c, ch, done);
+        case 56 * 4 + 1: return dispatch_dw<56, 1>(p, c, ch, done);
+        case 56 * 4 + 2: return dispatch_dw<56, 2>(p, c, ch, done);
+        case 28 * 4 + 1: return dispatch_dw<28, 1>(p, c, ch, done);
+        default: return SBNN_OK;
+    }
+}
+
+bool block_in_one_launch(const sbnn_packed* p, int N, int side, int stride) { return decide_block(p, N, side, stride).bn != 0; }
+
+sbnn_status prepare_block_tc(const sbnn_packed* p, int max_batch, int side, int stride) {
+    bool wanted[2] = {false, false};                  // blocks of 64 and of 128 channels
+    for (int n = max_batch; n > 0; n -= n > 64 ? n / 64 : 1) {
+        const int bn = decide_block(p, n, side, stride).bn;
+        if (bn) wanted[bn != 64] = true;
+    }
+    uint4* wts = nullptr;
+    PrepareScope scope;
+    for (int k = 0; k < 2; ++k)
+        if (wanted[k]) {
+            const sbnn_status r = get_tc_weights(p, k ? 128 : 64, 3, 0, nullptr, &wts);
+            if (r != SBNN_OK) return r;
+        }
+    return SBNN_OK;
+}
+
+ForcedChoiceScope::ForcedChoiceScope(int tile, int split) : choice{tile, split, 0.0} { forced_choice = &choice; }
+ForcedChoiceScope::~ForcedChoiceScope() { forced_choice = nullptr; }
+
 void free_tc_weights(sbnn_packed* p) {
     for (auto& kv : p->tc_weights) cudaFree(kv.second);
     p->tc_weights.clear();
@@ -1293,11 +1654,7 @@ extern "C" sbnn_status sbnn_debug_conv_gs(const sbnn_packed* w, const float* x_d
         return fail(SBNN_ERR_UNSUPPORTED, "split=%d is not 1, or up to 8 with 64-channel tiles", split);
     const int runs = (w->Cin + 63) / 64 * w->KH * (ldx ? 1 : w->KW);   // (channel-major 3x3: the taps of a kernel row stay together)
     if (runs < split) return fail(SBNN_ERR_UNSUPPORTED, "the layer has %d steps to split, not %d", runs, split);
-    const TcChoice choice = {tile, split, 0.0};
-    struct Scope {
-        explicit Scope(const TcChoice* c) { forced_choice = c; }
-        ~Scope() { forced_choice = nullptr; }
-    } scope(&choice);
+    const ForcedChoiceScope scope(tile, split);
     last_route = {0, 0, 0.0};
     sbnn_status r;
     if (ldx == 0 && ldy == 0)

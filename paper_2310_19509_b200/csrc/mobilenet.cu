@@ -1,7 +1,8 @@
 // MobileNet-v1 (width 1.0, 224x224x3) forward chain: the engine's forward pass of Section 3.5
 // with the 13 pointwise layers group-sparse (the layers Tables 3 and 4 prune) and everything
 // else dense.  Launches only: conv0 -> 13 x (depthwise, pointwise) -> pool -> classifier on one
-// stream over two ping-pong workspaces.  Between the image and the pooled features every
+// stream over two ping-pong workspaces; depthwise layers on wide maps run in the launch of the pointwise
+// layer behind them where that is faster.  Between the image and the pooled features every
 // activation is kept channel-major ([C][ld], the pixels of a channel contiguous), the layout in
 // which the group-sparse 1x1 kernel's tiles are plain row copies; no layer transposes anything.
 #include <new>
@@ -56,7 +57,7 @@ struct sbnn_mbv1 {
     int max_batch;
     int device;
     float* ws[2];  // ping-pong activation buffers
-    // Forward calls replay a CUDA graph of the 29 launches once a (x, logits, N) triple has been seen twice:
+    // Forward calls replay a CUDA graph of their launches once a (x, logits, N) triple has been seen twice:
     // the first call runs plainly (and builds whatever is built lazily), the second is captured on a private
     // stream and instantiated, later ones only launch the graph on the caller's stream.
     struct GraphKey {
@@ -121,6 +122,8 @@ extern "C" sbnn_status sbnn_mobilenet_v1_create(const sbnn_packed* const* pw, co
         if ((st = prepare_default_cm(pw[i], (long long)max_batch * hw * hw)) != SBNN_OK) return st;
         if ((st = prepare_tc(pw[i], (long long)max_batch * hw * hw)) != SBNN_OK) return st;
         if ((st = prepare_default_cm(pw[i], (long long)hw * hw)) != SBNN_OK) return st;   // and the batch-1 choice
+        const LayerShape& D = layer_table()[1 + 2 * i];
+        if ((st = prepare_block_tc(pw[i], max_batch, D.hin, D.stride)) != SBNN_OK) return st;
     }
     if ((st = check_packed_device(fc)) != SBNN_OK) return st;
     if ((st = prepare_default_cm(fc, max_batch)) != SBNN_OK) return st;
@@ -225,6 +228,42 @@ extern "C" sbnn_status sbnn_mobilenet_v1_run_layer_cm(sbnn_mbv1* net, int layer,
     return run_cm(net, layer, in, outp, N, stream);
 }
 
+// Layers 2 * block - 1 and 2 * block (depthwise, pointwise) in one launch; *done = false when separate launches are faster.
+static sbnn_status run_block_cm(sbnn_mbv1* net, int block, const float* in, float* out, int N, void* stream, bool* done) {
+    const LayerShape &D = layer_table()[2 * block - 1], &P = layer_table()[2 * block];
+    return dwconv3x3_conv1x1_tc_cm(net->pw[block - 1], net->dw_w[block - 1], net->dw_b[block - 1], in, round4((long long)N * D.hin * D.hin), out,
+                                   round4((long long)N * P.hout * P.hout), N, D.hin, D.stride, static_cast<cudaStream_t>(stream), done);
+}
+
+extern "C" sbnn_status sbnn_debug_mobilenet_v1_launches(const sbnn_mbv1* net, int N, int last_layer, int* launches) {
+    clear_error();
+    if (!net || !launches) return fail(SBNN_ERR_NULL, "net and launches must not be NULL");
+    if (last_layer < 0 || last_layer >= SBNN_MBV1_NUM_LAYERS) return fail(SBNN_ERR_SHAPE, "layer %d out of range", last_layer);
+    if (N <= 0 || N > net->max_batch) return fail(SBNN_ERR_SHAPE, "N=%d outside [1, max_batch=%d]", N, net->max_batch);
+    *launches = last_layer + 1;
+    for (int block = 1; 2 * block <= last_layer && block <= SBNN_MBV1_NUM_BLOCKS; ++block) {
+        const LayerShape& D = layer_table()[2 * block - 1];
+        *launches -= block_in_one_launch(net->pw[block - 1], N, D.hin, D.stride);
+    }
+    return SBNN_OK;
+}
+
+extern "C" sbnn_status sbnn_debug_mobilenet_v1_block(sbnn_mbv1* net, int block, const float* in, float* outp, int N, int tile, int split,
+                                                     void* stream) {
+    clear_error();
+    if (!net || !in || !outp) return fail(SBNN_ERR_NULL, "net, in_dev and out_dev must not be NULL");
+    if (block < 1 || block > SBNN_MBV1_NUM_BLOCKS) return fail(SBNN_ERR_SHAPE, "block %d out of range", block);
+    if (N < 0 || N > net->max_batch) return fail(SBNN_ERR_SHAPE, "N=%d outside [0, max_batch=%d]", N, net->max_batch);
+    if (!aligned16(in) || !aligned16(outp)) return fail(SBNN_ERR_ALIGN, "in_dev and out_dev must be 16-byte aligned");
+    if (N == 0) return SBNN_OK;
+    sbnn_status r = check_net_device(net);
+    if (r != SBNN_OK) return r;
+    bool done = false;
+    const ForcedChoiceScope scope(tile, split);
+    if ((r = run_block_cm(net, block, in, outp, N, stream, &done)) != SBNN_OK) return r;
+    return done ? SBNN_OK : fail(SBNN_ERR_UNSUPPORTED, "block %d does not run in one launch with tile=%d and split=%d", block, tile, split);
+}
+
 namespace {
 
 // Layers 0 .. last on the ping-pong workspaces; the output of layer `last` goes to out_dev.
@@ -235,8 +274,20 @@ sbnn_status forward_plain(sbnn_mbv1* net, const float* x_dev, float* out_dev, in
     // predecessor's completion before it touches an activation buffer.
     ChainedLaunchScope chained;
     const float* cur = x_dev;
-    for (int l = 0; l <= last; ++l) {
-        float* dst = (l == last) ? out_dev : net->ws[l & 1];
+    for (int l = 0, launch = 0; l <= last; ++l, ++launch) {
+        float* const free_ws = net->ws[launch & 1];   // (the other one holds `cur`)
+        if (layer_table()[l].kind == 1 && l < last) {
+            float* const dst = l + 1 == last ? out_dev : free_ws;
+            bool done = false;
+            sbnn_status st = run_block_cm(net, (l + 1) / 2, cur, dst, N, stream, &done);
+            if (st != SBNN_OK) return st;
+            if (done) {
+                ++l;
+                cur = dst;
+                continue;
+            }
+        }
+        float* const dst = l == last ? out_dev : free_ws;
         sbnn_status st = run_cm(net, l, cur, dst, N, stream);
         if (st != SBNN_OK) return st;
         cur = dst;

@@ -130,6 +130,7 @@ __device__ __forceinline__ void tensor_s2g_2d(const void* tensor_map, int x, int
 __device__ __forceinline__ void bulk_commit_group() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 // Waits until all but the most recent one of the calling thread's bulk groups have finished READING their shared-memory source.
 __device__ __forceinline__ void bulk_wait_read_pending1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 // Waits until the calling thread's bulk groups have completed altogether (their global writes are performed).
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
