@@ -1265,11 +1265,15 @@ long long cluster_capacity(int split) {
     return it->second;
 }
 
-// The same for 64-channel tiles shared by `split` CTAs; infinite when they do not all run at the same time.
-double tc_split_cost(const sbnn_packed* p, long long M, int split, int run, int images) {
+// The same for 64-channel tiles shared by `split` CTAs; infinite when that is not below `limit` or they do not all run at the same time.
+double tc_split_cost(const sbnn_packed* p, long long M, int split, int run, int images, double limit) {
     const long long tiles = (M + 127) / 128 * ((p->Cout + 63) / 64), runs = (long long)((p->Cin + 63) / 64) * p->KH * p->KW / run;
-    if (runs < split || tiles * split > device_sms() || tiles > cluster_capacity(split)) return 1e30;
-    return (double)((runs + split - 1) / split * run) * (tc_step(64, images) + 50.0) + 9800.0;
+    if (runs < split || tiles * split > device_sms()) return 1e30;
+    // Clusters of 5 to 7 start later: one 14 x 14 image, 512 -> 512, two steps a CTA in clusters of 4, 5, 6: 6.8, 7.3, 7.6 us; 2 x 28 x
+    // 28, 128 -> 128 3x3, 18 steps in clusters of 4 and 5: 9.7 and 10.2.
+    const double late = split > 4 && split < 8 ? 1500.0 : 0.0;
+    const double cost = (double)((runs + split - 1) / split * run) * (tc_step(64, images) + 50.0) + 9800.0 + late;
+    return cost < limit && tiles <= cluster_capacity(split) ? cost : 1e30;
 }
 
 TcChoice tc_choose(const sbnn_packed* p, long long M, int run, int images) {
@@ -1281,7 +1285,7 @@ TcChoice tc_choose(const sbnn_packed* p, long long M, int run, int images) {
     // (every number: a layer of 16 tiles gets no clusters of 8, of which 15 run at a time, but clusters of 6.  5 x 7 x 7, 512 -> 512
     // 3x3, 72 steps: 17.9 us shared by 4, 15.0 by 6)
     for (int split = 2; split <= 8; ++split) {
-        const double cost = tc_split_cost(p, M, split, run, images);
+        const double cost = tc_split_cost(p, M, split, run, images, best.cost);
         if (cost < best.cost) best = {64, split, cost};
     }
     return best;
