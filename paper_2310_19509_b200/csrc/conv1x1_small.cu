@@ -51,8 +51,12 @@ __device__ __forceinline__ void fetch_unit(const int32_t* __restrict__ idx, cons
 
 // KSPLIT = warps per CTA; each takes that fraction of the group's kept units.  PX = pixels per lane (the CTA covers
 // 32 * PX pixels): with two, a unit's index and weights, once read from shared memory, serve twice the FMAs.
+// The eight-warp instances say that one CTA an SM is enough: the compiler then takes 96 registers instead of 64 and has more of a
+// round's loads in flight (G = 4; 7 x 7 pixels, 1024 -> 1024 at 30 / 50 / 70 %: 11.6 -> 8.0, 8.5 -> 6.0, 6.6 -> 4.9 us; 512 -> 1024 at
+// 30 % 6.7 -> 5.1; 64 pixels, 1024 -> 1000 dense 15.2 -> 10.1).  With fewer warps it costs more CTAs than it gains (14 x 14,
+// 256 -> 512 at 50 %, four warps: 4.6 -> 5.1).  Sixteen warps are no faster than eight (1 pixel, 1024 -> 1000: 6.9 and 6.6).
 template <int G, int KSPLIT, bool OUT_CM, int PX>
-__global__ void __launch_bounds__(32 * KSPLIT)
+__global__ void __launch_bounds__(32 * KSPLIT, KSPLIT == 8 ? 1 : 0)
 conv1x1_small_kernel(const float* __restrict__ X, int ldx, float* __restrict__ Y, int ldy, const int32_t* __restrict__ group_ptr,
                      const int32_t* __restrict__ idx, const float* __restrict__ val, const float* __restrict__ bias, int M,
                      int relu) {
