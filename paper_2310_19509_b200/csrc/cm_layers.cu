@@ -92,8 +92,11 @@ dwconv3x3_cm_vec_kernel(const float* __restrict__ w, const float* __restrict__ b
 // by instruction issue).  The values left and right of the strip come from the neighbouring lanes by
 // shuffle; only the first and last lane of a warp fetch theirs from memory.  No thread leaves before the
 // shuffles: threads past the end work on a clamped position and store nothing.
+// One CTA an SM is stated to be enough (here, at stride 2 and for the narrow maps below): the compiler then keeps all rows' loads in
+// flight, with 68 registers instead of 48.  64 images of 112 x 112 x 32 38.6 -> 35.4 us, of 56 x 56 x 128 39.1 -> 36.1; 112 x 112 x 64 at
+// stride 2 43.0 -> 38.8, 56 x 56 x 128 24.6 -> 21.0; one image of 112 x 112 x 32 2.9 -> 2.4; 9 images of 28 x 28 x 256 at stride 2 5.1 -> 4.5.
 template <int RR>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, 1)
 dwconv3x3_cm_rows_kernel(const float* __restrict__ w, const float* __restrict__ b, const float* __restrict__ x, int ldx,
                          float* __restrict__ y, int ldy, int items, int C, int H, int W, int relu) {
     const int c = blockIdx.x % C;
@@ -159,7 +162,7 @@ dwconv3x3_cm_rows_kernel(const float* __restrict__ w, const float* __restrict__ 
 // The same for stride 2 (W a multiple of 8, Ho a multiple of RR): 4 output columns x RR output rows per thread,
 // 2*RR + 1 input rows of 8 columns each plus the column left of them, which is the left neighbour's last.
 template <int RR>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, 1)
 dwconv3x3_cm_rows_s2_kernel(const float* __restrict__ w, const float* __restrict__ b, const float* __restrict__ x, int ldx,
                             float* __restrict__ y, int ldy, int items, int C, int Ho, int W, int relu) {
     const int c = blockIdx.x % C;
@@ -228,7 +231,7 @@ dwconv3x3_cm_rows_s2_kernel(const float* __restrict__ w, const float* __restrict
 // turns the 9 tap offsets into immediates of the load instructions (the kernel is bound by
 // instruction issue, not by memory).
 template <int S, int NI, int WT>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 1)
 dwconv3x3_cm_px_kernel(const float* __restrict__ w, const float* __restrict__ b, const float* __restrict__ x, int ldx,
                        float* __restrict__ y, int ldy, int N, int H, int Wrt, int C, int QB, int relu) {
     const int W = WT ? WT : Wrt;
@@ -334,7 +337,7 @@ dwconv3x3_cm_col7_kernel(const float* __restrict__ w, const float* __restrict__ 
 // was limited by the number of load requests in flight, not by bytes.)  A warp holds 4 such strips in 28 lanes;
 // lanes 28-31 only take part in the shuffles.  A CTA of 4 warps covers 8 channels x 2 strips.
 template <int NI>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, 1)
 dwconv3x3_cm_w14_kernel(const float* __restrict__ w, const float* __restrict__ b, const float* __restrict__ x, int ldx,
                         float* __restrict__ y, int ldy, int N, int C, int relu) {
     constexpr int W = 14, H = 14;
@@ -562,7 +565,10 @@ conv3x3_thin_cm32_kernel(const float* __restrict__ w, const float* __restrict__ 
 // boundary, so four aligned 16-byte loads per row fetch them, and all twelve are issued before the first FMA
 // (the generic kernel above issues 45 scalar loads in nine dependent batches).  Otherwise as above: 2 output
 // columns x 32 output channels per thread, packed FMAs over channel pairs, weights broadcast from shared memory.
-__global__ void __launch_bounds__(128)
+// WIDE, for launches of few CTAs: 156 registers instead of 102, for more loads in flight (1 image 5.0 -> 4.4 us, 9 images 8.1 -> 7.9; 24
+// images, three waves of CTAs, 16.7 -> 17.0, 64 images 43.6 -> 45.0).
+template <bool WIDE>
+__global__ void __launch_bounds__(128, WIDE ? 1 : 0)
 conv3x3_first_s2c3_kernel(const float* __restrict__ w, const float* __restrict__ b, const float* __restrict__ x,
                           float* __restrict__ y, int ldy, int N, int H, int W, int Cout, int Ho, int Wo, int relu) {
     constexpr int Cin = 3;
@@ -758,7 +764,8 @@ sbnn_status launch_conv3x3_thin_cm(const float* w, const float* b, const float* 
         dim3 grid((unsigned)blocks, Cout / 32);
         const size_t smem = sizeof(float) * 9 * Cin * 32;
         if (stride == 2 && Cin == 3 && W % 4 == 0 && H % 2 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0) {
-            SBNN_CUDA_TRY(launch_kernel(conv3x3_first_s2c3_kernel, grid, 128, smem, st, w, b, x, y, ldy, N, H, W, Cout, Ho, Wo, relu));
+            auto* const kernel = blocks <= 3 * device_sms() ? conv3x3_first_s2c3_kernel<true> : conv3x3_first_s2c3_kernel<false>;
+            SBNN_CUDA_TRY(launch_kernel(kernel, grid, 128, smem, st, w, b, x, y, ldy, N, H, W, Cout, Ho, Wo, relu));
         } else if (stride == 1) {
             SBNN_CUDA_TRY(launch_kernel(conv3x3_thin_cm32_kernel<1>, grid, 128, smem, st, w, b, x, y, ldy, N, H, W, Cin, Cout, Ho, Wo, relu));
         } else {

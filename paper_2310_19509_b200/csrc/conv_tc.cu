@@ -1326,9 +1326,9 @@ TcChoice decide(const sbnn_packed* p, long long M, Call call) {
 
 // A block of the network (a depthwise layer with images of `side` pixels a row and the 1x1 layer behind it, N images): the
 // tile of the launch that does both, bn = 0 where two launches are faster.  Microseconds, in one launch and apart (alone, back to
-// back), half pruned: 64 images of 112 x 112, 32 -> 64: 68 and 101; 112 -> 56, 64 -> 128: 61 and 73; 56 x 56, 128 -> 128: 69 and 78;
-// 56 -> 28, 128 -> 256: 39 and 48; 28 x 28, 256 -> 256: 46 and 53; 9 images 12.4 and 15.6, 12.9 and 12.7, 16.0 and 15.4, 11.4 and
-// 11.4, 15.4 and 13.4; one image 4.8 and 6.6, 6.9 and 6.9, 8.1 and 7.7, 9.2 and 7.8, 8.5 and 8.7.  The network at batch 64: 774 ->
+// back), half pruned: 64 images of 112 x 112, 32 -> 64: 68 and 98; 112 -> 56, 64 -> 128: 61 and 68; 56 x 56, 128 -> 128: 69 and 75;
+// 56 -> 28, 128 -> 256: 39 and 44; 28 x 28, 256 -> 256: 46 and 53; 9 images 12.4 and 15.2, 12.9 and 12.8, 16.0 and 15.0, 11.4 and
+// 11.2, 15.4 and 13.1; one image 4.8 and 6.4, 6.9 and 6.7, 8.1 and 7.3, 9.2 and 7.3, 8.5 and 8.4.  The network at batch 64: 774 ->
 // 695 us.  The depthwise layer is computed again for every tile of output channels, on the split warps, so a step takes 2400 (128
 // channels a tile) to 3300 cycles longer than without (twice that at stride 2, whose stages hold 8 channels); layers with
 // smaller maps, more channels and less to move (14 x 14, 512 -> 512: 9 + 30 us) stay apart.

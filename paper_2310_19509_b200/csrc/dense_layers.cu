@@ -10,8 +10,10 @@ namespace {
 // ---- depthwise 3x3 --------------------------------------------------------------------------
 // One thread: 4 channels x TW consecutive output columns of one output row.  The 3 x (S*(TW-1)+3)
 // input window is read once into registers and slides across the TW outputs.
-template <int S, int TW>
-__global__ void __launch_bounds__(256)
+// WIDE: 92 registers instead of 66 (96, 78 at stride 2), for more loads in flight, where two CTAs an SM take the whole launch (1 x 13 x
+// 13 x 40 3.6 -> 3.2 us, 2 x 28 x 28 x 256 at stride 2 4.0 -> 3.4); with more it loses (9 x 28 x 28 x 256, 441 CTAs, 5.1 -> 6.6).
+template <int S, int TW, bool WIDE>
+__global__ void __launch_bounds__(256, WIDE ? 1 : 0)
 dwconv3x3_kernel(const float* __restrict__ w, const float* __restrict__ b, const float* __restrict__ x,
                  float* __restrict__ y, int N, int H, int W, int C, int Ho, int Wo, int relu) {
     const int C4 = C >> 2;
@@ -321,10 +323,12 @@ extern "C" sbnn_status sbnn_dwconv3x3(const float* w_dev, const float* b_dev, co
         dwconv3x3_slide_kernel<1, 3, SR1><<<(unsigned)b1, 256, 0, s>>>(w_dev, b_dev, x_dev, y_dev, N, H, W, C, Ho, Wo, relu);
     else if (stride == 2 && b2 >= 2 * device_sms() && b2 <= 0xffffff)
         dwconv3x3_slide_kernel<2, 2, SR2><<<(unsigned)b2, 256, 0, s>>>(w_dev, b_dev, x_dev, y_dev, N, H, W, C, Ho, Wo, relu);
-    else if (stride == 1)
-        dwconv3x3_kernel<1, TW><<<(unsigned)blocks, 256, 0, s>>>(w_dev, b_dev, x_dev, y_dev, N, H, W, C, Ho, Wo, relu);
-    else
-        dwconv3x3_kernel<2, TW><<<(unsigned)blocks, 256, 0, s>>>(w_dev, b_dev, x_dev, y_dev, N, H, W, C, Ho, Wo, relu);
+    else {
+        const bool wide = blocks <= 2 * device_sms();
+        auto* const kernel = stride == 1 ? (wide ? dwconv3x3_kernel<1, TW, true> : dwconv3x3_kernel<1, TW, false>)
+                                         : (wide ? dwconv3x3_kernel<2, TW, true> : dwconv3x3_kernel<2, TW, false>);
+        kernel<<<(unsigned)blocks, 256, 0, s>>>(w_dev, b_dev, x_dev, y_dev, N, H, W, C, Ho, Wo, relu);
+    }
     SBNN_CUDA_TRY(cudaGetLastError());
     return SBNN_OK;
 }
