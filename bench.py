@@ -558,7 +558,7 @@ def run_gpu(args, rank, world, local_rank):
                   else f"FMA kernels ({len(on_fma)} of the 13 pointwise launches per step)",
         "launches_on_tensor_cores": len(on_tc), "launches_on_fma_kernels": len(on_fma),
         "note": "tensor: flops of the unpruned layers, which is what the kernel multiplies, against a sixth of the measured bf16 rate (six "
-                "bf16 products make an fp32 one), over the launches that run there; alu: nonzero flops of all 13 against the FP32 FMA peak",
+                "bf16 products make an fp32 one), over the launches that run there, some of which compute a depthwise layer as well; alu: nonzero flops of all 13 against the FP32 FMA peak",
         "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
         "nonzero_tflops": pw_fl / pw_t / 1e12, "nonzero_frac_of_fp32_fma_peak": pw_fl / pw_t / 1e12 / FP32_PEAK_TFLOPS,
         "timing": "per layer: time of the chain's prefix up to and including the layer minus the prefix before it, each prefix a "
