@@ -51,12 +51,12 @@ __device__ __forceinline__ void fetch_unit(const int32_t* __restrict__ idx, cons
 
 // KSPLIT = warps per CTA; each takes that fraction of the group's kept units.  PX = pixels per lane (the CTA covers
 // 32 * PX pixels): with two, a unit's index and weights, once read from shared memory, serve twice the FMAs.
-// The eight-warp instances say that one CTA an SM is enough: the compiler then takes 96 registers instead of 64 and has more of a
-// round's loads in flight (G = 4; 7 x 7 pixels, 1024 -> 1024 at 30 / 50 / 70 %: 11.6 -> 8.0, 8.5 -> 6.0, 6.6 -> 4.9 us; 512 -> 1024 at
-// 30 % 6.7 -> 5.1; 64 pixels, 1024 -> 1000 dense 15.2 -> 10.1).  With fewer warps it costs more CTAs than it gains (14 x 14,
-// 256 -> 512 at 50 %, four warps: 4.6 -> 5.1).  Sixteen warps are no faster than eight (1 pixel, 1024 -> 1000: 6.9 and 6.6).
-template <int G, int KSPLIT, bool OUT_CM, int PX>
-__global__ void __launch_bounds__(32 * KSPLIT, KSPLIT == 8 ? 1 : 0)
+// WIDE (eight warps): one CTA an SM is stated to be enough; the compiler then takes more registers (G = 4: 96 instead of 64, with two
+// pixels 104 instead of 79) and has more of a round's loads in flight, but fewer CTAs are resident, see wide_limit.  With four warps it
+// costs more than it gains at any size (14 x 14, 256 -> 512 at 50 %: 4.6 -> 5.1 us).  Sixteen warps are no faster than eight (1 pixel,
+// 1024 -> 1000: 6.9 and 6.6).
+template <int G, int KSPLIT, bool OUT_CM, int PX, bool WIDE>
+__global__ void __launch_bounds__(32 * KSPLIT, WIDE ? 1 : 0)
 conv1x1_small_kernel(const float* __restrict__ X, int ldx, float* __restrict__ Y, int ldy, const int32_t* __restrict__ group_ptr,
                      const int32_t* __restrict__ idx, const float* __restrict__ val, const float* __restrict__ bias, int M,
                      int relu) {
@@ -163,16 +163,40 @@ conv1x1_small_kernel(const float* __restrict__ X, int ldx, float* __restrict__ Y
     }
 }
 
+// CTAs an SM up to which a launch of eight warps takes the WIDE instance.  Measured without and with it, us: G = 4, two pixels a lane,
+// 1024 -> 1024 at 50 %: 256 CTAs 8.4 and 5.9, 512 11.4 and 11.0, 1792 31.7 and 32.1; 512 -> 512 at 50 %: 256 CTAs 4.9 and 3.8, 1280 13.5
+// and 14.3; one pixel: 128 CTAs 2.2 and 2.1, 256 4.0 and 4.1, 512 (1024 -> 2048) 6.5 and 7.4.  G = 2, 1024 -> 256 at 50 %: one pixel, 128
+// CTAs 3.2 and 2.8; two pixels, 256 CTAs 7.0 and 5.3, 896 14.5 and 15.7; 512 -> 512, one pixel, 256 CTAs 3.4 and 4.2.  G = 1, 512 -> 512 at
+// 50 %: one pixel, 512 CTAs 3.7 and 3.3, two pixels, 5.2 and 5.8, 1024 CTAs 8.6 and 10.1.  G = 8 gains 1 to 4 % up to 832 CTAs (1024 ->
+// 2048, one pixel: 7.0 and 5.7) and loses up to 6 % above; G = 16 gains 0 to 10 % everywhere.
+template <int G, int PX>
+constexpr long long wide_limit() {
+    if (G == 8) return 6;
+    if (PX == 2) return G == 4 ? 4 : 2;
+    return G == 1 ? 4 : 1;
+}
+
+template <int G, int KS, int PX, bool WIDE>
+sbnn_status launch_small_as(const sbnn_packed* p, dim3 grid, const float* x, int ldx, float* y, int ldy, int M, int relu, bool out_cm,
+                            cudaStream_t st) {
+    ChainedLaunchScope early;   // before its wait the kernel reads the layer's own arrays only
+    auto* const kernel = out_cm ? conv1x1_small_kernel<G, KS, true, PX, WIDE> : conv1x1_small_kernel<G, KS, false, PX, WIDE>;
+    SBNN_CUDA_TRY(launch_kernel(kernel, grid, 32 * KS, 0, st, x, ldx, y, ldy, p->d_group_ptr, p->d_idx, p->d_val, p->d_bias, M, relu));
+    return SBNN_OK;
+}
 template <int G, int KS, int PX>
 sbnn_status launch_small_ks(const sbnn_packed* p, const float* x, int ldx, float* y, int ldy, int M, int relu, bool out_cm,
                             cudaStream_t st) {
-    dim3 grid((unsigned)((M + 32 * PX - 1) / (32 * PX)), (unsigned)p->ngroups);
-    ChainedLaunchScope early;   // before its wait the kernel reads the layer's own arrays only
-    if (out_cm)
-        SBNN_CUDA_TRY(launch_kernel(conv1x1_small_kernel<G, KS, true, PX>, grid, 32 * KS, 0, st, x, ldx, y, ldy, p->d_group_ptr, p->d_idx, p->d_val, p->d_bias, M, relu));
-    else
-        SBNN_CUDA_TRY(launch_kernel(conv1x1_small_kernel<G, KS, false, PX>, grid, 32 * KS, 0, st, x, ldx, y, ldy, p->d_group_ptr, p->d_idx, p->d_val, p->d_bias, M, relu));
-    return SBNN_OK;
+    const dim3 grid((unsigned)((M + 32 * PX - 1) / (32 * PX)), (unsigned)p->ngroups);
+    if constexpr (KS == 8 && G == 16) {
+        return launch_small_as<G, KS, PX, true>(p, grid, x, ldx, y, ldy, M, relu, out_cm, st);
+    } else {
+        if constexpr (KS == 8) {
+            if ((long long)grid.x * grid.y <= wide_limit<G, PX>() * device_sms())
+                return launch_small_as<G, KS, PX, true>(p, grid, x, ldx, y, ldy, M, relu, out_cm, st);
+        }
+        return launch_small_as<G, KS, PX, false>(p, grid, x, ldx, y, ldy, M, relu, out_cm, st);
+    }
 }
 
 template <int G>

@@ -1,0 +1,31 @@
+"""The few-pixel 1x1 kernel with eight warps: both instances, by the number of CTAs of a launch, for every group size."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2310_19509_b200 as sbnn
+from oracle import reference as R
+from sbnn_inputs import workloads as WL
+
+gpu = pytest.mark.gpu
+
+
+# Groups x blocks of 32 or 64 pixels just below and above the line between the instances on 148 SMs, with one and with two pixels a
+# lane; 516 channels half pruned are more than 256 a group.
+@gpu
+@pytest.mark.parametrize("g,cout,m", [(1, 592, 32), (1, 593, 32), (1, 148, 65), (1, 149, 65), (2, 296, 17), (2, 298, 17), (2, 592, 64), (2, 594, 64),
+                                      (4, 592, 32), (4, 596, 1), (4, 592, 197), (4, 596, 225), (8, 2368, 33), (8, 1192, 325), (16, 1200, 33), (16, 64, 1)])
+def test_both_instances(g, cout, m):
+    """1e-5 * S: the tolerance of every kernel (S = |b| + sum |w*x|)."""
+    d = WL.single_conv_inputs(1, 1, m, 516, cout, 1, g, 50, 7, 0.05, 0.05)
+    ref, s = R.conv2d(d["x"], d["w"], d["mask"], d["bias"], relu=True)
+    p = sbnn.pack_weights(d["w"], d["mask"], d["bias"], g)
+    ld = (m + 3) // 4 * 4
+    x = torch.zeros((516, ld), device="cuda")
+    x[:, :m] = torch.from_numpy(d["x"].reshape(m, 516).T.copy())
+    y = torch.full((cout, ld + 4), float("nan"), device="cuda")
+    sbnn.debug_conv_gs(p, x, ld, y, ld + 4, 1, 1, m, sbnn.SBNN_RELU | sbnn.SBNN_OUT_CM, 0, 1)
+    assert bool(torch.isnan(y[:, m:]).all())
+    err = np.abs(y[:, :m].T.cpu().numpy().astype(np.float64) - ref.reshape(m, cout))
+    assert np.all(err <= 1e-5 * s.reshape(m, cout))
+    p.free()
