@@ -96,6 +96,8 @@ struct TcArgs {
     int resident;          // every tile uses the same weights and all of them have a stage: they are loaded once
     int* status;
     ExactArgs ex;
+    int slots;             // the most of a drain thread's chunks of outputs that one CTA of the cluster stores
+    int share;             // chunks of a CTA in units of 2^-16, rounded up: the first of CTA r is r * share >> 16
 };
 struct DwArgs : TcArgs {
     CUtensorMap wmap;      // the depthwise weights [9][Cin]
@@ -474,7 +476,8 @@ __device__ __noinline__ void sum_kept_units(const typename T::Args& args, unsign
 }
 
 // Last step of a tile whose steps were shared by the `split` CTAs of a cluster, for the drain threads: chunk c of a
-// thread's channels (four of them) belongs to the last CTA r with r * CHUNKS / split <= c.  Everybody writes its sums of the
+// thread's channels (four of them) belongs to the last CTA r with r * CHUNKS / split <= c (quotients by a factor that comes
+// with the launch: with divisions here tiles shared by 8 took 0.1 to 0.2 us longer).  Everybody writes its sums of the
 // chunks of others into their shared memory, [sender][chunk][thread], and then adds up and stores its own.  The stages hold the
 // exchange: every CTA's MMAs are complete when its drain threads reach the first barrier.
 template <class T>
@@ -483,8 +486,9 @@ __device__ __forceinline__ void store_shared_tile(const typename T::Args& a, uin
     const uint32_t exchange = smem_u32(room);
     const unsigned char* const mine = room;
     const int m = m0 + (tid & 127), n00 = blockIdx.x / a.split % a.ntiles_n * T::BN, n0 = n00 + (tid >> 7) * T::COLS;
-    const int rank = (int)cluster_rank(), slots = (CHUNKS + a.split - 1) / a.split;
-    const int first = rank * CHUNKS / a.split, own = (rank + 1) * CHUNKS / a.split - first;
+    auto first_of = [&](int r) { return r * a.share >> 16; };
+    const int rank = (int)cluster_rank(), slots = a.slots;
+    const int first = first_of(rank), own = first_of(rank + 1) - first;
     __syncwarp();
     cluster_sync();
 #pragma unroll
@@ -493,7 +497,7 @@ __device__ __forceinline__ void store_shared_tile(const typename T::Args& a, uin
         float4 v;
         unpack2(acc[2 * c], v.x, v.y);
         unpack2(acc[2 * c + 1], v.z, v.w);
-        if (owner != rank) store_remote(exchange + ((rank * slots + c - owner * CHUNKS / a.split) * 256 + tid) * 16, owner, v);
+        if (owner != rank) store_remote(exchange + ((rank * slots + c - first_of(owner)) * 256 + tid) * 16, owner, v);
     }
     cluster_sync();
     bool redo = false;
@@ -1436,6 +1440,11 @@ sbnn_status launch_tc(const sbnn_packed* p, const TcCall& c, int split, bool* do
     a.wts = wts; a.bias = p->d_bias; a.y = c.y; a.ldy = c.ldy; a.M = (int)c.M; a.Cin = p->Cin; a.Cout = p->Cout;
     a.steps = (p->Cin + 63) / 64 * T::TAPS; a.ntiles_m = (int)((c.M + T::BM - 1) / T::BM); a.ntiles_n = (int)ntiles_n;
     a.W = c.W; a.H = c.H; a.relu = c.relu; a.split = T::SPLIT ? split : 1;
+    if (T::SPLIT) {
+        constexpr int CHUNKS = T::COLS / 4;
+        a.slots = (CHUNKS + split - 1) / split;
+        a.share = CHUNKS * 65536 / split + 1;   // (r * share / 65536 = r * CHUNKS / split for all r <= split <= 8)
+    }
     const bool cm = T::SRC == SRC_CM || T::SRC == SRC_CM3 || T::FUSED;
     a.ex = {c.x, cm ? 1 : p->Cin, cm ? c.ldx : 1, p->d_group_ptr, p->d_idx, p->d_val, use_tap_lists(p) ? p->d_taps : nullptr, p->G};
     CUtensorMap amap, ymap;

@@ -63,7 +63,7 @@ def check_tc(got, ref, s, steps):
     assert np.linalg.norm(err) <= RMS * np.linalg.norm(ref)
 
 
-INSTANCES = [(64, 1), (128, 1), (256, 1), (64, 2), (64, 4), (64, 8)]
+INSTANCES = [(64, 1), (128, 1), (256, 1)] + [(64, split) for split in range(2, 9)]
 # ragged pixels, channels and output channels; nine steps for the splits; more tiles than SMs at every tile width
 SHAPES_1X1 = [(3, 17, 19, 516, 260, 4, 50), (7, 61, 63, 100, 516, 4, 30)]
 SHAPES_3X3 = [(2, 13, 14, 132, 260, 4, 50), (48, 14, 15, 132, 300, 4, 30)]
