@@ -206,6 +206,7 @@ sbnn_status launch_avgpool_cm(const float* x, int ldx, float* y, int ldy, int N,
 // conv1x1_small.cu: kernel for launches with few pixels; reads the canonical packed arrays (no private layout)
 sbnn_status conv1x1_small(const sbnn_packed* p, const float* x, int ldx, float* y, int ldy, int M, int relu, bool out_cm,
                           cudaStream_t st);
+double conv1x1_small_us(const sbnn_packed* p, long long M);   // what it takes, modelled
 // conv1x1_bf16.cu
 sbnn_status conv1x1_bf16(const sbnn_packed* w, const float* x, float* y, int M, int relu, cudaStream_t st);
 void free_stream_bf16(sbnn_packed* p);

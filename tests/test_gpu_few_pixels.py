@@ -29,3 +29,29 @@ def test_both_instances(g, cout, m):
     err = np.abs(y[:, :m].T.cpu().numpy().astype(np.float64) - ref.reshape(m, cout))
     assert np.all(err <= 1e-5 * s.reshape(m, cout))
     p.free()
+
+
+# Pixels, channels, group, pruned: which side was the faster one by 10 % and more, tensor cores or FMA (us: tensor cores and FMA)
+@gpu
+@pytest.mark.parametrize("m,cin,cout,g,pct,tensor", [
+    (49, 1024, 1024, 8, 30, False),      # 8.2, 7.4
+    (49, 512, 1024, 4, 0, False),        # 6.9, 6.0
+    (49, 1024, 1024, 4, 50, False),      # 8.2, 5.9
+    (1, 1024, 1000, 4, 0, False),        # 8.1, 6.6
+    (17, 64, 128, 4, 50, False),         # 4.2, 1.7
+    (183, 768, 256, 1, 30, True),        # 6.9, 13.3
+    (879, 56, 320, 1, 90, True),         # 4.3, 10.2
+    (396, 52, 1040, 2, 70, True),        # 4.5, 7.9
+    (1286, 32, 720, 4, 90, True),        # 4.1, 8.5
+    (49, 1296, 256, 8, 0, True),         # 7.3, 11.3
+    (34, 1472, 160, 16, 0, True),        # 7.4, 13.6
+    (784, 256, 256, 4, 0, True),
+    (196, 512, 512, 4, 0, True),
+])
+def test_the_faster_kernel_is_picked(m, cin, cout, g, pct, tensor):
+    d = WL.single_conv_inputs(1, 1, 1, cin, cout, 1, g, pct, 3, 0.05, 0.05)
+    p = sbnn.pack_weights(d["w"], d["mask"], d["bias"], g)
+    ld = (m + 3) // 4 * 4
+    sbnn.conv1x1_gs_cm(p, torch.zeros((cin, ld), device="cuda"), ld, torch.empty((cout, ld), device="cuda"), ld, m, sbnn.SBNN_RELU | sbnn.SBNN_OUT_CM)
+    assert (sbnn.debug_last_route()[0] != 0) == tensor
+    p.free()
