@@ -1277,7 +1277,12 @@ double tc_split_cost(const sbnn_packed* p, long long M, int split, int run, int 
     // 28, 128 -> 128 3x3, 18 steps in clusters of 4 and 5: 9.7 and 10.2.
     const double late = split > 4 && split < 8 ? 1500.0 : 0.0;
     const double cost = (double)((runs + split - 1) / split * run) * (tc_step(64, images) + 50.0) + 9800.0 + late;
-    return cost < limit && tiles <= cluster_capacity(split) ? cost : 1e30;
+    if (cost >= limit) return 1e30;
+    // Behind another launch the last clusters of 3 and of 5 of a full device find no place before others have ended.  In clusters of 3, of
+    // which 45 run at a time: 9 x 5 tiles of 6 steps 10.3 us (unshared 7.5), 5 x 9 of 10 steps 11.9 (of 2: 9.6), 44 tiles of 4 steps 9.0, 43
+    // and fewer take what they are modelled at.  26 tiles of 17 steps in clusters of 5: 10.6 (of 4: 9.0).
+    const long long capacity = cluster_capacity(split), spare = split == 3 || split == 5 ? capacity / 16 : 0;
+    return tiles <= capacity - spare ? cost : 1e30;
 }
 
 TcChoice tc_choose(const sbnn_packed* p, long long M, int run, int images) {

@@ -55,3 +55,17 @@ def test_the_faster_kernel_is_picked(m, cin, cout, g, pct, tensor):
     sbnn.conv1x1_gs_cm(p, torch.zeros((cin, ld), device="cuda"), ld, torch.empty((cout, ld), device="cuda"), ld, m, sbnn.SBNN_RELU | sbnn.SBNN_OUT_CM)
     assert (sbnn.debug_last_route()[0] != 0) == tensor
     p.free()
+
+
+# 45 tiles of 64 channels fit the device in clusters of 3, but not behind another launch (10.3 us; unshared 7.5), 12.0 (of 2: 9.6);
+# 42 tiles of 15 steps: 9.8 us in clusters of 3, 11.6 of 2
+@gpu
+@pytest.mark.parametrize("m,cin,cout,fits", [(1072, 384, 288, False), (621, 608, 576, False), (349, 608, 912, False), (1674, 940, 176, True)])
+def test_clusters_that_fit_behind_another_launch(m, cin, cout, fits):
+    d = WL.single_conv_inputs(1, 1, 1, cin, cout, 1, 4, 0, 3, 0.05, 0.05)
+    p = sbnn.pack_weights(d["w"], d["mask"], d["bias"], 4)
+    ld = (m + 3) // 4 * 4
+    sbnn.conv1x1_gs_cm(p, torch.zeros((cin, ld), device="cuda"), ld, torch.empty((cout, ld), device="cuda"), ld, m, sbnn.SBNN_RELU | sbnn.SBNN_OUT_CM)
+    tile, split = sbnn.debug_last_route()
+    assert tile == 64 and (split == 3) == fits
+    p.free()
