@@ -336,9 +336,8 @@ dwconv3x3_cm_col7_kernel(const float* __restrict__ w, const float* __restrict__ 
 // its neighbours by shuffle: 9 load requests for 14 outputs.  (With one scalar load per tap the kernel above
 // was limited by the number of load requests in flight, not by bytes.)  A warp holds 4 such strips in 28 lanes;
 // lanes 28-31 only take part in the shuffles.  A CTA of 4 warps covers 8 channels x 2 strips.
-// WIDE: 48 registers instead of 40, see launch_dwconv3x3_cm.
-template <int NI, bool WIDE>
-__global__ void __launch_bounds__(128, WIDE ? 1 : 0)
+template <int NI>
+__global__ void __launch_bounds__(128, 1)
 dwconv3x3_cm_w14_kernel(const float* __restrict__ w, const float* __restrict__ b, const float* __restrict__ x, int ldx,
                         float* __restrict__ y, int ldy, int N, int C, int relu) {
     constexpr int W = 14, H = 14;
@@ -736,10 +735,7 @@ sbnn_status launch_dwconv3x3_cm(const float* w, const float* b, const float* x, 
             if (W == 14 && H == 14 && ldx % 2 == 0 && ldy % 2 == 0) {
                 constexpr int NI2 = 2;
                 dim3 g14((unsigned)((N + NI2 - 1) / NI2), (C + 7) / 8);
-                // Few CTAs leave room for more registers, and loads in flight: 512 channels, 4 images (128 CTAs) 2.45 -> 2.32 us, 12 images (384)
-                // 3.25 -> 3.21; with more it loses: 20 images (640) 4.02 -> 4.27, 48 (1536) 7.20 -> 7.54, from 64 images on the same.
-                auto* const kernel = (long long)g14.x * g14.y <= 3 * device_sms() ? dwconv3x3_cm_w14_kernel<NI2, true> : dwconv3x3_cm_w14_kernel<NI2, false>;
-                SBNN_CUDA_TRY(launch_kernel(kernel, g14, 128, 0, st, w, b, x, ldx, y, ldy, N, C, relu));
+                SBNN_CUDA_TRY(launch_kernel(dwconv3x3_cm_w14_kernel<NI2>, g14, 128, 0, st, w, b, x, ldx, y, ldy, N, C, relu));
             } else if (W == 14 && H % 7 == 0) SBNN_DW_C7(14)
             else if (W == 7 && H == 7 && ldx % 4 == 0 && ldy % 4 == 0) {
                 dim3 g77((unsigned)((N + 63) / 64), (unsigned)((C + 1) / 2));
