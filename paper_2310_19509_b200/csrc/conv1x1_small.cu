@@ -167,15 +167,16 @@ conv1x1_small_kernel(const float* __restrict__ X, int ldx, float* __restrict__ Y
 
 // CTAs an SM up to which a launch of eight warps takes the WIDE instance.  Measured without and with it, us: G = 4, two pixels a lane,
 // 1024 -> 1024 at 50 %: 256 CTAs 8.4 and 5.9, 512 11.4 and 11.0, 1792 31.7 and 32.1; 512 -> 512 at 50 %: 256 CTAs 4.9 and 3.8, 1280 13.5
-// and 14.3; one pixel: 128 CTAs 2.2 and 2.1, 256 4.0 and 4.1, 512 (1024 -> 2048) 6.5 and 7.4.  G = 2, 1024 -> 256 at 50 %: one pixel, 128
-// CTAs 3.2 and 2.8; two pixels, 256 CTAs 7.0 and 5.3, 896 14.5 and 15.7; 512 -> 512, one pixel, 256 CTAs 3.4 and 4.2.  G = 1, 512 -> 512 at
-// 50 %: one pixel, 512 CTAs 3.7 and 3.3, two pixels, 5.2 and 5.8, 1024 CTAs 8.6 and 10.1.  G = 8 gains 1 to 4 % up to 832 CTAs (1024 ->
-// 2048, one pixel: 7.0 and 5.7) and loses up to 6 % above; G = 16 gains 0 to 10 % everywhere.
+// and 14.3; one pixel: 128 CTAs 2.2 and 2.1, 256 4.0 and 4.1, 512 (1024 -> 2048) 6.5 and 7.4 (but the network, whose classifier is a
+// launch of 250 behind another, takes 120.6 us on one image at 30 % without and 117.7 with it).  G = 2, 1024 -> 256 at 50 %: one pixel,
+// 128 CTAs 3.2 and 2.8; two pixels, 256 CTAs 7.0 and 5.3, 896 14.5 and 15.7; 512 -> 512, one pixel, 256 CTAs 3.4 and 4.2.  G = 1, 512 ->
+// 512 at 50 %: one pixel, 512 CTAs 3.7 and 3.3, two pixels, 5.2 and 5.8, 1024 CTAs 8.6 and 10.1.  G = 8 gains 1 to 4 % up to 832 CTAs
+// (1024 -> 2048, one pixel: 7.0 and 5.7) and loses up to 6 % above; G = 16 gains 0 to 10 % everywhere.
 template <int G, int PX>
 constexpr long long wide_limit() {
     if (G == 8) return 6;
     if (PX == 2) return G == 4 ? 4 : 2;
-    return G == 1 ? 4 : 1;
+    return G == 1 ? 4 : (G == 4 ? 2 : 1);
 }
 
 template <int G, int KS, int PX, bool WIDE>

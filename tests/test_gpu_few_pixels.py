@@ -14,7 +14,7 @@ gpu = pytest.mark.gpu
 # lane; 516 channels half pruned are more than 256 a group.
 @gpu
 @pytest.mark.parametrize("g,cout,m", [(1, 592, 32), (1, 593, 32), (1, 148, 65), (1, 149, 65), (2, 296, 17), (2, 298, 17), (2, 592, 64), (2, 594, 64),
-                                      (4, 592, 32), (4, 596, 1), (4, 592, 197), (4, 596, 225), (8, 2368, 33), (8, 1192, 325), (16, 1200, 33), (16, 64, 1)])
+                                      (4, 1184, 32), (4, 1188, 1), (4, 592, 197), (4, 596, 225), (8, 2368, 33), (8, 1192, 325), (16, 1200, 33), (16, 64, 1)])
 def test_both_instances(g, cout, m):
     """1e-5 * S: the tolerance of every kernel (S = |b| + sum |w*x|)."""
     d = WL.single_conv_inputs(1, 1, m, 516, cout, 1, g, 50, 7, 0.05, 0.05)
