@@ -1335,20 +1335,31 @@ TcChoice decide(const sbnn_packed* p, long long M, Call call) {
 }
 
 // A block of the network (a depthwise layer with images of `side` pixels a row and the 1x1 layer behind it, N images): the
-// tile of the launch that does both, bn = 0 where two launches are faster.  Microseconds, in one launch and apart (alone, back to
-// back), half pruned: 64 images of 112 x 112, 32 -> 64: 68 and 98; 112 -> 56, 64 -> 128: 61 and 68; 56 x 56, 128 -> 128: 69 and 75;
-// 56 -> 28, 128 -> 256: 39 and 44; 28 x 28, 256 -> 256: 46 and 53; 9 images 12.4 and 15.2, 12.9 and 12.8, 16.0 and 15.0, 11.4 and
-// 11.2, 15.4 and 13.1; one image 4.8 and 6.4, 6.9 and 6.7, 8.1 and 7.3, 9.2 and 7.3, 8.5 and 8.4.  The network at batch 64: 774 ->
-// 695 us.  The depthwise layer is computed again for every tile of output channels, on the split warps, so a step takes 2400 (128
+// tile of the launch that does both, bn = 0 where two launches are faster.  What one launch saves of the time of the network whose other
+// blocks run as the rule has them, in microseconds, mean of 0 to 70 % pruned, at 1, 4, 6, 9, 12, 16, 28, 40 and 64 images (of 114, 158,
+// 168, 200, 222, 263, 407, 467 and 668):
+//   112 x 112, 32 -> 64           1.5   2.1   2.4   2.1   2.9   3.1   6.4  12.2  20.8
+//   112 -> 56, 64 -> 128         -1.3   0.7   2.5   0.1   2.9   1.8  -0.3   2.7   7.7
+//   56 x 56, 128 -> 128          -2.1   1.0   1.5  -0.6   2.3   2.1  -0.2   3.5  16.7
+//   56 -> 28, 128 -> 256         -4.4  -1.9  -2.1   0.0   0.8   2.2  -2.7  10.6  23.6
+//   28 x 28, 256 -> 256          -6.6  -3.7  -5.8  -2.8  -1.5   1.1  -6.2   5.1   8.9
+// (Whole rounds of tiles on both sides make it go up and down, and a launch less saves more in a chain than the same pair called again
+// and again: three of these were slower in one launch by that measure.)  Over 89 batch sizes and densities the rule is 0.06 us off the
+// better side on average for a block, at most 1.9.  Tiles of 64 channels shared by 2 to 4 CTAs, for few images, save nothing: +2.0 to
+// -2.1 at one image, -3 to -9 at two.
+// The depthwise layer is computed again for every tile of output channels, on the split warps, so a step takes 3000 (64 or 128
 // channels a tile) to 3300 cycles longer than without (twice that at stride 2, whose stages hold 8 channels); layers with
-// smaller maps, more channels and less to move (14 x 14, 512 -> 512: 9 + 30 us) stay apart.
-double block_step(int bn, int stride) { return stride == 2 ? (bn == 256 ? 8700.0 : 6500.0) : (bn == 256 ? 5500.0 : 4400.0); }
+// smaller maps, more channels and less to move (14 x 14, 512 -> 512: 9 + 30 us at 64 images) stay apart.
+double block_step(int bn, int stride) {
+    if (stride == 2) return bn == 64 ? 6500.0 : (bn == 128 ? 7200.0 : 9500.0);
+    return bn == 64 ? 4400.0 : (bn == 128 ? 5000.0 : 5600.0);
+}
 TcChoice decide_block(const sbnn_packed* p, int N, int side, int stride) {
     const long long out = side / stride, M = N * out * out, M_in = (long long)N * side * side, sms = device_sms();
     TcChoice best = {0, 0, 0.0};
     if (!p->finite || p->nnz == 0 || side < 28 || out < 28) return best;
     const double depthwise = 4.0 * (M_in + M) * p->Cin;              // bytes of the depthwise launch
-    const double steps = p->Cin / 64.0, mem = 4.0 * (M_in * p->Cin + M * p->Cout) / 5.0e6;
+    const double steps = p->Cin / 64.0, mem = 4.0 * (M_in * p->Cin + M * p->Cout) / 5.2e6;
     double us = 0.0;
     for (int bn : {64, 128, 256}) {
         if (bn > p->Cout || (bn == 256 && out > 28)) continue;
@@ -1362,8 +1373,8 @@ TcChoice decide_block(const sbnn_packed* p, int N, int side, int stride) {
     }
     const TcChoice layer = decide(p, M, CALL_1X1_CM);
     const double apart = (layer.bn ? std::max(tc_us(layer.cost), 4.0 * M * (p->Cin + p->Cout) / 6.5e6) : fma_us(p, M, CALL_1X1_CM)) + 2.0 +
-                         depthwise / (depthwise < 1e8 ? 5.0e6 : 4.6e6);
-    if (us >= 0.95 * apart) best.bn = 0;
+                         depthwise / (depthwise < 1e8 ? 4.2e6 : 4.4e6);
+    if (us >= 0.94 * apart) best.bn = 0;
     return best;
 }
 bool tc_profits(const sbnn_packed* p, long long M, Call call, TcChoice* choice = nullptr) {

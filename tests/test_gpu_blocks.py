@@ -104,3 +104,25 @@ def test_forward_runs_the_blocks_that_it_says(net):
             net.run_layer_cm(last, mid, want, n)
             sbnn.get_async_status()
             assert float((got - want).norm() / want.norm()) < 1e-6      # (2-norm of an fp32 layer's error: below 5.5e-7 on any kernel)
+
+
+# Which blocks run in one launch: what each saves of the time of the network is in csrc/conv_tc.cu.  (At 9 images the third would cost 0.6 us.)
+JOINED = {1: [1], 2: [1, 2], 4: [1, 2, 3], 6: [1, 2, 3], 9: [1, 2], 12: [1, 2, 3, 4], 16: [1, 2, 3, 4, 5], 40: [1, 2, 3, 4, 5], 64: [1, 2, 3, 4, 5]}
+
+
+def make_net(batch, limit=None):
+    """The network of `net` for up to `batch` images; limit: bytes of the first pointwise layer's images for the tensor cores."""
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()  # noqa: E731
+    of = lambda kind: [L for L in layers() if L["kind"] == kind]  # noqa: E731
+    pw, (fc,) = ([sbnn.pack_weights(L["w"], L["mask"], L["bias"], L["g"]) for L in of(kind)] for kind in ("pw", "fc"))
+    if limit is not None:
+        sbnn.debug_limit_images(pw[0], limit)
+    return sbnn.MobileNetV1(pw, fc, [t(L["w"]) for L in of("dw")], [t(L["bias"]) for L in of("dw")], t(layers()[0]["w"]), t(layers()[0]["bias"]), batch)
+
+
+def test_the_blocks_that_are_joined():
+    big = make_net(64)
+    for n, blocks in JOINED.items():
+        got = [b for b in range(1, 14) if big.debug_launches(n, 2 * b) == big.debug_launches(n, 2 * b - 2) + 1]
+        assert got == blocks, n
+    big.free()
