@@ -244,7 +244,9 @@ sbnn_status conv1x1_small(const sbnn_packed* p, const float* x, int ldx, float* 
 
 // Microseconds a call takes: a fixed part, a warp's chain of kept units, and for every round of CTAs over the SMs, how many of them
 // an SM works through, their units and their warps.  Fitted to 2472 calls of random sizes (1 to 3200 pixels, 32 to 2048 channels in, 16
-// to 1536 out, all group sizes, dense to 90 % pruned): 90 % of them are within 17 % below and 15 % above what was measured.
+// to 1536 out, all group sizes, dense to 90 % pruned): 90 % of them are within 17 % below and 15 % above what was measured.  With more
+// than 64 pixels a call takes no less than 0.19 us (0.138 in groups of 8 and 16) for a million multiply-adds of whole blocks of 32
+// pixels: without that limit ten calls of 4924 left the tensor cores, eight of which are 17 % slower here on average.
 double conv1x1_small_us(const sbnn_packed* p, long long M) {
     static constexpr double cost[5][3][4] = {   // G = 1, 2, 4, 8, 16; fewer than eight warps, eight, eight with two pixels a lane
         {{1.19, 0.016, 0.017, 0.076}, {0.66, 0.018, 0.035, 0.045}, {1.48, 0.007, 0.086, 0.043}},
@@ -256,7 +258,9 @@ double conv1x1_small_us(const sbnn_packed* p, long long M) {
     const double* const c = cost[p->G == 1 ? 0 : p->G == 2 ? 1 : p->G == 4 ? 2 : p->G == 8 ? 3 : 4][s.px == 2 ? 2 : s.warps == 8];
     const long long ctas = (M + 32 * s.px - 1) / (32 * s.px) * p->ngroups, sms = std::max(1, device_sms());
     const double units = p->ngroups ? (double)p->nnz / p->ngroups : 0.0, rounds = (double)((ctas + sms - 1) / sms);
-    return c[0] + c[1] * units / s.warps + rounds * (c[2] * units / 32 + c[3] * s.warps);
+    const double us = c[0] + c[1] * units / s.warps + rounds * (c[2] * units / 32 + c[3] * s.warps);
+    const double macs = 1e-6 * (double)((M + 31) / 32 * 32) * p->nnz * p->G;
+    return M > 64 ? std::max(us, 1.7 + macs * (p->G >= 8 ? 0.138 : 0.19)) : us;
 }
 
 }  // namespace sbnn

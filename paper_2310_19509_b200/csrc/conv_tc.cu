@@ -1327,8 +1327,8 @@ TcChoice decide(const sbnn_packed* p, long long M, Call call) {
     if (call == CALL_BF16) return tc_choose(p, M, 1, 1);
     if (!p->finite || p->nnz == 0) return choice;
     choice = tc_choose(p, M, call == CALL_3X3_CM ? 3 : 1, 3);
-    // (Few-pixel calls need no margin between the two models: of 2472 timed on both sides 59 run on the one that is more than 3 % slower,
-    // with 0.95 74; the other FMA kernels' model is rougher.)
+    // (Few-pixel calls need no margin between the two models: of 4924 timed on both sides 36 run on a side that is more than 3 % slower
+    // than the one an older model had picked, and 266 on one that is faster by that; the other FMA kernels' model is rougher.)
     const double least = call == CALL_1X1_CM && conv1x1_few_tiles(p, M) ? 1.0 : 0.95;
     if (std::max(tc_us(choice.cost), 4.0 * M * (p->Cin + p->Cout) / 6.5e6) >= least * fma_us(p, M, call)) choice.bn = 0;
     return choice;

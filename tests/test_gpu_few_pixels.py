@@ -31,7 +31,7 @@ def test_both_instances(g, cout, m):
     p.free()
 
 
-# Pixels, channels, group, pruned: which side was the faster one by 10 % and more, tensor cores or FMA (us: tensor cores and FMA)
+# Pixels, channels, group, pruned: which side is the faster one, tensor cores or FMA kernel (us: tensor cores and FMA)
 @gpu
 @pytest.mark.parametrize("m,cin,cout,g,pct,tensor", [
     (49, 1024, 1024, 8, 30, False),      # 8.2, 7.4
@@ -45,8 +45,9 @@ def test_both_instances(g, cout, m):
     (1286, 32, 720, 4, 90, True),        # 4.1, 8.5
     (49, 1296, 256, 8, 0, True),         # 7.3, 11.3
     (34, 1472, 160, 16, 0, True),        # 7.4, 13.6
-    (784, 256, 256, 4, 0, True),
-    (196, 512, 512, 4, 0, True),
+    (392, 640, 232, 4, 50, True),        # 7.6, 7.8
+    (733, 512, 512, 16, 70, True),       # 8.9, 10.9
+    (171, 428, 576, 4, 30, True),        # 7.0, 7.6
 ])
 def test_the_faster_kernel_is_picked(m, cin, cout, g, pct, tensor):
     d = WL.single_conv_inputs(1, 1, 1, cin, cout, 1, g, pct, 3, 0.05, 0.05)
