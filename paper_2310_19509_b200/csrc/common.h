@@ -224,11 +224,11 @@ sbnn_status conv3x3_tc(const sbnn_packed* p, const float* x, float* y, int N, in
 sbnn_status conv3x3_tc_cm(const sbnn_packed* p, const float* x, int ldx, float* y, int ldy, int N, int H, int W, int relu, bool out_cm, cudaStream_t st,
                           bool* done);
 // Depthwise 3x3 (stride 1 or 2, padding 1, bias, ReLU) of square images of `side` pixels a row and the 1x1 layer behind it (bias,
-// ReLU) in one launch, channel-major; *done as above.  The network's shapes: sides of 112 to 7, an even side with stride 2.
+// ReLU) in one launch, channel-major; *done as above.  Taken: sides of 112 and 56 with both strides, 28 with stride 1.  `ask`: nothing
+// is launched or built, *done says whether the call would run.
 sbnn_status dwconv3x3_conv1x1_tc_cm(const sbnn_packed* p, const float* dw_w, const float* dw_b, const float* x, int ldx, float* y, int ldy, int N,
-                                    int side, int stride, cudaStream_t st, bool* done);
-// Whether that is how N images run, and the weight images that calls of up to `max_batch` of them use.
-bool block_in_one_launch(const sbnn_packed* p, int N, int side, int stride);
+                                    int side, int stride, cudaStream_t st, bool* done, bool ask = false);
+// Builds the weight images that such calls of up to `max_batch` images use.
 sbnn_status prepare_block_tc(const sbnn_packed* p, int max_batch, int side, int stride);
 // While one is alive, the calls of its thread run on tensor-core tiles of this width, shared by that many CTAs (tests; tile 0: the FMA kernels).
 struct ForcedChoiceScope {

@@ -1166,8 +1166,8 @@ thread_local TcChoice last_route = {0, 0, 0.0};
 // Weight images of a layer for MMA column blocks of `nuc` output channels, built on first use; NULL if that would be
 // in a call of M pixels the layer has been prepared for, which only enqueues, or while `st` is being captured, when nothing
 // can be allocated, or if the device has no room for them (which is remembered: they take six bytes for every weight of the
-// unpruned layer, many times what is stored of a sparse one).
-sbnn_status get_tc_weights(const sbnn_packed* p, int nuc, int images, long long M, cudaStream_t st, uint4** out) {
+// unpruned layer, many times what is stored of a sparse one).  `ask`: nothing is built, either.
+sbnn_status get_tc_weights(const sbnn_packed* p, int nuc, int images, long long M, cudaStream_t st, uint4** out, bool ask = false) {
     std::lock_guard<std::mutex> lk(p->mu);
     *out = nullptr;
     auto it = p->tc_weights.find({nuc, images});
@@ -1175,6 +1175,7 @@ sbnn_status get_tc_weights(const sbnn_packed* p, int nuc, int images, long long 
         *out = static_cast<uint4*>(it->second);
         return SBNN_OK;
     }
+    if (ask) return SBNN_OK;
     auto prepared = p->tc_prepared.find(images);
     if (!prepare_only() && !forced_choice && prepared != p->tc_prepared.end() && M <= prepared->second) return SBNN_OK;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -1219,6 +1220,7 @@ struct TcCall {
     const float* dw_w;  // SRC_DW: the depthwise layer in front, and the pixels of its input
     const float* dw_b;
     long long M_in;
+    bool ask;          // launch and build nothing, only say whether the call runs here
 };
 
 // ---- which kernel, and how ------------------------------------------------------------------------
@@ -1448,10 +1450,10 @@ sbnn_status launch_tc(const sbnn_packed* p, const TcCall& c, int split, bool* do
     if (regs != T::LAUNCH_REGS) return SBNN_OK;
     typename T::Args a = {};
     uint4* wts = nullptr;
-    if ((r = get_tc_weights(p, T::NUC, T::IMAGES, c.M, c.st, &wts)) != SBNN_OK || !wts) return r;
+    if ((r = get_tc_weights(p, T::NUC, T::IMAGES, c.M, c.st, &wts, c.ask)) != SBNN_OK || !wts) return r;
     if ((r = async_status_word(&a.status)) != SBNN_OK) return r;
     *done = true;
-    if (prepare_only()) return SBNN_OK;
+    if (prepare_only() || c.ask) return SBNN_OK;
     const long long ntiles_n = (p->Cout + T::BN - 1) / T::BN, total = (c.M + T::BM - 1) / T::BM * ntiles_n;
     if (total > 0x7fffffffLL) return fail(SBNN_ERR_SHAPE, "too many tiles");
     a.wts = wts; a.bias = p->d_bias; a.y = c.y; a.ldy = c.ldy; a.M = (int)c.M; a.Cin = p->Cin; a.Cout = p->Cout;
@@ -1608,9 +1610,9 @@ sbnn_status dispatch_dw(const sbnn_packed* p, const TcCall& c, const TcChoice& c
 }  // namespace
 
 sbnn_status dwconv3x3_conv1x1_tc_cm(const sbnn_packed* p, const float* dw_w, const float* dw_b, const float* x, int ldx, float* y, int ldy, int N,
-                                    int side, int stride, cudaStream_t st, bool* done) {
+                                    int side, int stride, cudaStream_t st, bool* done, bool ask) {
     *done = false;
-    last_route = {0, 0, 0.0};
+    if (!ask) last_route = {0, 0, 0.0};
     const int out = side / stride;
     const long long M = (long long)N * out * out, M_in = (long long)N * side * side;
     if ((p->Cin != 32 && p->Cin % 64) || p->Cout % 4 || M_in > kMaxPixels || !aligned16(x) || !aligned16(y) || !aligned16(dw_w) || !aligned16(dw_b)) return SBNN_OK;
@@ -1618,7 +1620,7 @@ sbnn_status dwconv3x3_conv1x1_tc_cm(const sbnn_packed* p, const float* dw_w, con
     if (forced_choice) ch = *forced_choice;
     else ch = decide_block(p, N, side, stride);
     if (ch.split > (p->Cin + 63) / 64) return SBNN_OK;
-    const TcCall c{x, ldx, y, ldy, M, N, out, out, 1, st, dw_w, dw_b, M_in};
+    const TcCall c{x, ldx, y, ldy, M, N, out, out, 1, st, dw_w, dw_b, M_in, ask};
     switch (side * 4 + stride) {
         case 112 * 4 + 1: return dispatch_dw<112, 1>(p, c, ch, done);
         case 112 * 4 + 2: return dispatch_dw<112, 2>(p, c, ch, done);
@@ -1628,8 +1630,6 @@ sbnn_status dwconv3x3_conv1x1_tc_cm(const sbnn_packed* p, const float* dw_w, con
         default: return SBNN_OK;
     }
 }
-
-bool block_in_one_launch(const sbnn_packed* p, int N, int side, int stride) { return decide_block(p, N, side, stride).bn != 0; }
 
 sbnn_status prepare_block_tc(const sbnn_packed* p, int max_batch, int side, int stride) {
     bool wanted[2] = {false, false};                  // blocks of 64 and of 128 channels

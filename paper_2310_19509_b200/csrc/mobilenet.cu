@@ -228,11 +228,12 @@ extern "C" sbnn_status sbnn_mobilenet_v1_run_layer_cm(sbnn_mbv1* net, int layer,
     return run_cm(net, layer, in, outp, N, stream);
 }
 
-// Layers 2 * block - 1 and 2 * block (depthwise, pointwise) in one launch; *done = false when separate launches are faster.
-static sbnn_status run_block_cm(sbnn_mbv1* net, int block, const float* in, float* out, int N, void* stream, bool* done) {
+// Layers 2 * block - 1 and 2 * block (depthwise, pointwise) in one launch; *done = false when separate launches are faster, or the only
+// way.  `ask`: only whether it would run.
+static sbnn_status run_block_cm(const sbnn_mbv1* net, int block, const float* in, float* out, int N, void* stream, bool* done, bool ask = false) {
     const LayerShape &D = layer_table()[2 * block - 1], &P = layer_table()[2 * block];
     return dwconv3x3_conv1x1_tc_cm(net->pw[block - 1], net->dw_w[block - 1], net->dw_b[block - 1], in, round4((long long)N * D.hin * D.hin), out,
-                                   round4((long long)N * P.hout * P.hout), N, D.hin, D.stride, static_cast<cudaStream_t>(stream), done);
+                                   round4((long long)N * P.hout * P.hout), N, D.hin, D.stride, static_cast<cudaStream_t>(stream), done, ask);
 }
 
 extern "C" sbnn_status sbnn_debug_mobilenet_v1_launches(const sbnn_mbv1* net, int N, int last_layer, int* launches) {
@@ -242,8 +243,10 @@ extern "C" sbnn_status sbnn_debug_mobilenet_v1_launches(const sbnn_mbv1* net, in
     if (N <= 0 || N > net->max_batch) return fail(SBNN_ERR_SHAPE, "N=%d outside [1, max_batch=%d]", N, net->max_batch);
     *launches = last_layer + 1;
     for (int block = 1; 2 * block <= last_layer && block <= SBNN_MBV1_NUM_BLOCKS; ++block) {
-        const LayerShape& D = layer_table()[2 * block - 1];
-        *launches -= block_in_one_launch(net->pw[block - 1], N, D.hin, D.stride);
+        bool joined = false;
+        const sbnn_status r = run_block_cm(net, block, net->ws[0], net->ws[1], N, nullptr, &joined, true);
+        if (r != SBNN_OK) return r;
+        *launches -= joined;
     }
     return SBNN_OK;
 }

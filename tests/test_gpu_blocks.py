@@ -3,6 +3,7 @@
 Tolerance of a block: the pointwise layer's own (see test_gpu_routes.py) on the depthwise output, and what the depthwise output may be
 off by, ten roundings of 2^-24 of its magnitude and one more for storing the oracle's in fp32, taken through the weights' magnitudes.
 """
+import ctypes
 import functools
 
 import numpy as np
@@ -126,3 +127,29 @@ def test_the_blocks_that_are_joined():
         got = [b for b in range(1, 14) if big.debug_launches(n, 2 * b) == big.debug_launches(n, 2 * b - 2) + 1]
         assert got == blocks, n
     big.free()
+
+
+def launched(net, n, last):
+    """Kernel launches of the first layers, counted in a graph of them."""
+    x = torch.rand((n, 224, 224, 3), device="cuda")
+    _, _, side, cout = sbnn.mobilenet_v1_layer_shape(last)
+    out = torch.empty(max(cout * ((n * side * side + 3) // 4 * 4), 1024 * 4), device="cuda")
+    net.forward_prefix(x, out, n, last)
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph, stream=torch.cuda.Stream()):
+        net.forward_prefix(x, out, n, last)
+    count = ctypes.c_size_t()
+    nodes = ctypes.CDLL("libcudart.so.12").cudaGraphGetNodes
+    assert nodes(ctypes.c_void_p(graph.raw_cuda_graph()), None, ctypes.byref(count)) == 0
+    return count.value
+
+
+@pytest.mark.parametrize("limit", [None, 1000])
+def test_launches_are_those_of_the_forward_pass(limit):
+    """Also where a block could run in one launch, but its pointwise layer's images have no room on the device (limit)."""
+    net = make_net(6, limit)
+    for n in (1, 6):
+        for last in (1, 2, 4, 6, 28):
+            assert net.debug_launches(n, last) == launched(net, n, last), (n, last)
+    assert net.debug_launches(6, 2) == (2 if limit is None else 3)
+    net.free()
