@@ -231,6 +231,7 @@ sbnn_status dwconv3x3_conv1x1_tc_cm(const sbnn_packed* p, const float* dw_w, con
 // Builds the weight images that such calls of up to `max_batch` images use.
 sbnn_status prepare_block_tc(const sbnn_packed* p, int max_batch, int side, int stride);
 // While one is alive, the calls of its thread run on tensor-core tiles of this width, shared by that many CTAs (tests; tile 0: the FMA kernels).
+sbnn_status check_forced_choice(int tile, int split);   // tile 0, 64, 128 or 256; split 1, or up to 8 with tile 64
 struct ForcedChoiceScope {
     sbnn_packed::TcChoice choice;
     ForcedChoiceScope(int tile, int split);

@@ -1647,6 +1647,12 @@ sbnn_status prepare_block_tc(const sbnn_packed* p, int max_batch, int side, int 
     return SBNN_OK;
 }
 
+sbnn_status check_forced_choice(int tile, int split) {
+    if (tile != 0 && tile != 64 && tile != 128 && tile != 256) return fail(SBNN_ERR_UNSUPPORTED, "tile=%d is not 0, 64, 128 or 256", tile);
+    if (split < 1 || split > 8 || (split > 1 && tile != 64))
+        return fail(SBNN_ERR_UNSUPPORTED, "split=%d is not 1, or up to 8 with 64-channel tiles", split);
+    return SBNN_OK;
+}
 ForcedChoiceScope::ForcedChoiceScope(int tile, int split) : choice{tile, split, 0.0} { forced_choice = &choice; }
 ForcedChoiceScope::~ForcedChoiceScope() { forced_choice = nullptr; }
 
@@ -1679,14 +1685,12 @@ extern "C" sbnn_status sbnn_debug_conv_gs(const sbnn_packed* w, const float* x_d
                                           int tile, int split, void* cuda_stream) {
     clear_error();
     if (!w) return fail(SBNN_ERR_NULL, "packed weights must not be NULL");
-    if (tile != 0 && tile != 64 && tile != 128 && tile != 256) return fail(SBNN_ERR_UNSUPPORTED, "tile=%d is not 0, 64, 128 or 256", tile);
-    if (split < 1 || split > 8 || (split > 1 && tile != 64))
-        return fail(SBNN_ERR_UNSUPPORTED, "split=%d is not 1, or up to 8 with 64-channel tiles", split);
+    sbnn_status r = check_forced_choice(tile, split);
+    if (r != SBNN_OK) return r;
     const int runs = (w->Cin + 63) / 64 * w->KH * (ldx ? 1 : w->KW);   // (channel-major 3x3: the taps of a kernel row stay together)
     if (runs < split) return fail(SBNN_ERR_UNSUPPORTED, "the layer has %d steps to split, not %d", runs, split);
     const ForcedChoiceScope scope(tile, split);
     last_route = {0, 0, 0.0};
-    sbnn_status r;
     if (ldx == 0 && ldy == 0)
         r = w->KH == 3 ? sbnn_conv3x3_gs(w, x_dev, y_dev, N, H, W, flags, cuda_stream) : sbnn_conv1x1_gs(w, x_dev, y_dev, N, H, W, flags, cuda_stream);
     else if (w->KH == 3)

@@ -257,10 +257,11 @@ extern "C" sbnn_status sbnn_debug_mobilenet_v1_block(sbnn_mbv1* net, int block, 
     if (!net || !in || !outp) return fail(SBNN_ERR_NULL, "net, in_dev and out_dev must not be NULL");
     if (block < 1 || block > SBNN_MBV1_NUM_BLOCKS) return fail(SBNN_ERR_SHAPE, "block %d out of range", block);
     if (N < 0 || N > net->max_batch) return fail(SBNN_ERR_SHAPE, "N=%d outside [0, max_batch=%d]", N, net->max_batch);
+    sbnn_status r = check_forced_choice(tile, split);
+    if (r != SBNN_OK) return r;
     if (!aligned16(in) || !aligned16(outp)) return fail(SBNN_ERR_ALIGN, "in_dev and out_dev must be 16-byte aligned");
     if (N == 0) return SBNN_OK;
-    sbnn_status r = check_net_device(net);
-    if (r != SBNN_OK) return r;
+    if ((r = check_net_device(net)) != SBNN_OK) return r;
     bool done = false;
     const ForcedChoiceScope scope(tile, split);
     if ((r = run_block_cm(net, block, in, outp, N, stream, &done)) != SBNN_OK) return r;

@@ -153,3 +153,11 @@ def test_launches_are_those_of_the_forward_pass(limit):
             assert net.debug_launches(n, last) == launched(net, n, last), (n, last)
     assert net.debug_launches(6, 2) == (2 if limit is None else 3)
     net.free()
+
+
+@pytest.mark.parametrize("tile,split", [(128, 2), (256, 4), (64, 0), (64, -1), (64, 9), (96, 1), (0, 1), (64, 5)])
+def test_tiles_that_there_are_not(net, tile, split):
+    """Refused, and not run in some other way (block 5 has four steps to share)."""
+    x, ref, _ = block(5, 1)
+    with pytest.raises(sbnn.SbnnError):
+        net.debug_block(5, planes(x), torch.empty(ref.size, device="cuda"), 1, tile, split)
