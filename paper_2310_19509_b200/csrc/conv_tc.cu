@@ -103,17 +103,17 @@ struct DwArgs : TcArgs {
     CUtensorMap wmap;      // the depthwise weights [9][Cin]
     const float* dw_w;
     const float* dw_b;
-    long long M_in;        // pixels of the depthwise layer's input
 };
 
 // What a stage holds for the depthwise layer in front of a 1x1 layer (SRC_DW), for images of WI x WI input pixels, 112 to 28: of
 // SUB channels every input pixel that the 128 output pixels of a tile need, as BOXES tiled copies of PB consecutive pixels each
 // (box-major, then channel, then pixel), behind them the nine rows of weights and the bias of these channels.
 // Stride 1: the 128 pixels and a row and a pixel more on both sides are one run, except for 112 pixels a row, where a box
-// holds the run of one kernel row (408 pixels, where one run would take 360 and two boxes).
+// holds the run of one kernel row (three of 140 pixels; one run, in two boxes, would be 360).
 // Stride 2: the input rows of the output rows that the tile touches, BR rows to a box.
 // A box has LEAD pixels in front of the tile's, so that it starts at a multiple of 4 pixels and four pixels of a row at one; PB / 4
 // is odd, so that 16-byte loads of 8 channels fall into different banks.
+constexpr int kMaxDwChannels = 1024;
 template <int WI_, int S_>
 struct DwShape {
     static constexpr int WI = WI_, S = S_, WO = WI / S, SUB = S == 1 ? 16 : 8;
@@ -173,6 +173,9 @@ struct TC {
     // (shared by 7, the most for an exchange: 7 senders of up to 2 of a thread's 8 chunks)
     static_assert(!SPLIT || (BN == 64 && SB * B_BYTES + SA_MIN * A_BYTES >= 7 * 2 * 256 * 16), "the cluster's exchange");
     static_assert(IMAGES == 3 || (IMAGES == 1 && SRC == SRC_NHWC), "bf16 mode");
+    // Pixels that are summed again: the sums of 32 of them fit the staging tiles, or the stages hold all of their channels at once (see
+    // sum_kept_units).
+    static_assert(BN * 32 * 4 <= OUT_BYTES || (FUSED && SB * B_BYTES + SA_MIN * A_BYTES >= kMaxDwChannels * 32 * 4 + 6144), "sums of bad pixels");
 };
 
 __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
@@ -1469,7 +1472,7 @@ sbnn_status launch_tc(const sbnn_packed* p, const TcCall& c, int split, bool* do
     CUtensorMap amap, ymap;
     if constexpr (T::FUSED) {
         using D = typename T::DW;
-        a.dw_w = c.dw_w; a.dw_b = c.dw_b; a.M_in = c.M_in;
+        a.dw_w = c.dw_w; a.dw_b = c.dw_b;
         const unsigned long long dims[2] = {(unsigned long long)c.M_in, (unsigned long long)p->Cin}, wdims[2] = {(unsigned long long)p->Cin, 9};
         const unsigned long long strides[1] = {(unsigned long long)c.ldx * 4}, wstrides[1] = {(unsigned long long)p->Cin * 4};
         const unsigned box[2] = {(unsigned)D::PB, (unsigned)D::SUB}, wbox[2] = {(unsigned)D::SUB, 9u};
@@ -1615,7 +1618,7 @@ sbnn_status dwconv3x3_conv1x1_tc_cm(const sbnn_packed* p, const float* dw_w, con
     if (!ask) last_route = {0, 0, 0.0};
     const int out = side / stride;
     const long long M = (long long)N * out * out, M_in = (long long)N * side * side;
-    if ((p->Cin != 32 && p->Cin % 64) || p->Cout % 4 || M_in > kMaxPixels || !aligned16(x) || !aligned16(y) || !aligned16(dw_w) || !aligned16(dw_b)) return SBNN_OK;
+    if ((p->Cin != 32 && p->Cin % 64) || p->Cin > kMaxDwChannels || p->Cout % 4 || M_in > kMaxPixels || !aligned16(x) || !aligned16(y) || !aligned16(dw_w) || !aligned16(dw_b)) return SBNN_OK;
     TcChoice ch;
     if (forced_choice) ch = *forced_choice;
     else ch = decide_block(p, N, side, stride);
