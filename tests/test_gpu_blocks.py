@@ -161,3 +161,29 @@ def test_tiles_that_there_are_not(net, tile, split):
     x, ref, _ = block(5, 1)
     with pytest.raises(sbnn.SbnnError):
         net.debug_block(5, planes(x), torch.empty(ref.size, device="cuda"), 1, tile, split)
+
+
+@pytest.mark.parametrize("b,tile", [(1, 64), (2, 128), (3, 128), (4, 256), (5, 256)])
+def test_bad_depthwise_weights_as_in_two_launches(b, tile):
+    """Infinities and NaN in the depthwise weights and biases spoil the same outputs in one launch as in two: zeros outside the image are
+    multiplied by them, ReLU turns NaN into 0, and an infinity that is left reaches the outputs that keep its channel."""
+    x, _, tol = block(b, 1)
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()  # noqa: E731
+    of = lambda kind: [L for L in layers() if L["kind"] == kind]  # noqa: E731
+    pw, (fc,) = ([sbnn.pack_weights(L["w"], L["mask"], L["bias"], L["g"]) for L in of(kind)] for kind in ("pw", "fc"))
+    dw_w, dw_b = [L["w"].copy() for L in of("dw")], [L["bias"].copy() for L in of("dw")]
+    w, bias = dw_w[b - 1].reshape(3, 3, -1), dw_b[b - 1]
+    w[0, 0, 3], w[1, 1, 9], w[2, 1, 14], bias[20], bias[25] = np.inf, np.nan, -np.inf, np.inf, np.nan
+    bad = sbnn.MobileNetV1(pw, fc, [t(a) for a in dw_w], [t(a) for a in dw_b], t(layers()[0]["w"]), t(layers()[0]["bias"]), 1)
+    _, _, side, cout = sbnn.mobilenet_v1_layer_shape(2 * b)
+    mid, want = torch.empty((x.shape[-1], side * side), device="cuda"), torch.empty((cout, side * side), device="cuda")
+    bad.run_layer_cm(2 * b - 1, planes(x), mid, 1)
+    bad.run_layer_cm(2 * b, mid, want, 1)
+    want = want.cpu().numpy().T.reshape(1, side, side, cout)
+    got = run(bad, b, x, tile, 1)
+    assert np.isinf(want).any() and np.isfinite(want).any()
+    assert np.array_equal(np.isinf(got), np.isinf(want)) and np.array_equal(np.isnan(got), np.isnan(want))
+    finite = np.isfinite(want)
+    err = np.abs(got.astype(np.float64) - np.where(finite, want, 0))
+    assert np.all(err[finite] <= 2 * np.maximum(tol, 1e-5 * np.abs(want))[finite])
+    bad.free()

@@ -311,7 +311,7 @@ def spoil(x, how):
 @gpu
 @pytest.mark.parametrize("how", ["three", "one per pixel", "both signs", "all"])
 @pytest.mark.parametrize("k,layout,tile,split", [(1, "nhwc", 256, 1), (1, "cm-cm", 128, 1), (1, "cm", 64, 4), (3, "nhwc", 128, 1), (3, "cm-cm", 64, 1),
-                                                 (3, "nhwc", 64, 8)])
+                                                 (3, "nhwc", 64, 8), (1, "cm-cm", 64, 3), (3, "nhwc", 64, 7), (3, "cm", 64, 5)])
 def test_bad_activations_spoil_what_they_touch_and_little_time(k, layout, tile, split, how):
     """The same outputs are infinite or NaN as on the FMA kernels, the others keep their values, and the call does not take
     many times what it takes there (at most seven times, when every pixel has a bad channel; summed by a thread a pixel it was a hundred times)."""
@@ -367,7 +367,8 @@ def test_bad_activations_under_pruned_taps(layout, tile, split, taps):
 
 
 @gpu
-@pytest.mark.parametrize("layout,tile,split", [("nhwc", 64, 1), ("nhwc", 256, 1), ("cm-cm", 128, 1), ("nhwc", 64, 2)])
+@pytest.mark.parametrize("layout,tile,split", [("nhwc", 64, 1), ("nhwc", 256, 1), ("cm-cm", 128, 1), ("nhwc", 64, 2), ("nhwc", 64, 3),
+                                               ("cm-cm", 64, 6)])
 def test_sums_that_overflow_on_the_way(layout, tile, split):
     """fp32 sums depend on their order near the end of the range: where the tensor cores' order overflows in any channel, the
     order of the FMA kernels (products ascending, bias last) decides."""
