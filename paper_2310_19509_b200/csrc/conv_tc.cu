@@ -93,12 +93,14 @@ struct TcArgs {
     int relu;
     int split;             // CTAs of a cluster that share a tile's steps
     int sa, sb;            // stages of activations and of weights
-    int resident;          // every tile uses the same weights and all of them have a stage: they are loaded once
+    // Not shared: whether every tile uses the same weights and all of them have a stage, so that they are loaded once.  Shared: a CTA's part
+    // of a drain thread's chunks of outputs, in units of 2^-16 and rounded up (see store_shared_tile).  (One word for both: with eight
+    // bytes more of arguments a launch takes the host 0.4 us longer, 4.5 -> 4.9.)
+    int resident_or_share;
     int* status;
     ExactArgs ex;
-    int slots;             // the most of a drain thread's chunks of outputs that one CTA of the cluster stores
-    int share;             // chunks of a CTA in units of 2^-16, rounded up: the first of CTA r is r * share >> 16
 };
+static_assert(sizeof(TcArgs) == 160, "arguments of a launch");
 struct DwArgs : TcArgs {
     CUtensorMap wmap;      // the depthwise weights [9][Cin]
     const float* dw_w;
@@ -489,8 +491,8 @@ __device__ __forceinline__ void store_shared_tile(const typename T::Args& a, uin
     const uint32_t exchange = smem_u32(room);
     const unsigned char* const mine = room;
     const int m = m0 + (tid & 127), n00 = blockIdx.x / a.split % a.ntiles_n * T::BN, n0 = n00 + (tid >> 7) * T::COLS;
-    auto first_of = [&](int r) { return r * a.share >> 16; };
-    const int rank = (int)cluster_rank(), slots = a.slots;
+    const int share = a.resident_or_share, rank = (int)cluster_rank(), slots = (share + 65534) >> 16;
+    auto first_of = [&](int r) { return r * share >> 16; };
     const int first = first_of(rank), own = first_of(rank + 1) - first;
     __syncwarp();
     cluster_sync();
@@ -710,6 +712,7 @@ __global__ void __launch_bounds__(T::NT, 1)
 conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap ymap, const __grid_constant__ typename T::Args a) {
     constexpr int NUC = T::NUC, NU = T::NU, BN = T::BN;
     const int SA = a.sa, SB = a.sb;
+    const bool resident = !T::SPLIT && a.resident_or_share;
     extern __shared__ unsigned char raw[];
     const uint32_t raw_addr = smem_u32(raw);
     unsigned char* bst = raw + (((raw_addr + 1023u) & ~1023u) - raw_addr);    // weight stages, 1024-byte aligned
@@ -861,7 +864,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                         ring.next();
                         if (batch == 2) ring.next();
                     }
-                if (a.resident) break;
+                if (resident) break;
             }
             if (!ok) ring.settle(bfull, true);
         } else if (warp >= 18) {
@@ -919,14 +922,14 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                                                  idesc, i ? 1u : more);
                                 }
                             }
-                            if (!a.resident) umma_commit(bempty + s);
+                            if (!resident) umma_commit(bempty + s);
                             if (T::IMAGES == 3 || k0 == ke - 1) umma_commit(dfull + d);
                             umma_commit(aempty + as);
                         }
                         __syncwarp();
                     }
                 if (T::IMAGES == 1) unit += NU;
-                if (a.resident) ring = Ring(SB);            // the same stages again, still full from the first round
+                if (resident) ring = Ring(SB);            // the same stages again, still full from the first round
             }
         } else if (wg < 4) {
             // ---------------- split into bf16 images ----------------
@@ -1462,11 +1465,6 @@ sbnn_status launch_tc(const sbnn_packed* p, const TcCall& c, int split, bool* do
     a.wts = wts; a.bias = p->d_bias; a.y = c.y; a.ldy = c.ldy; a.M = (int)c.M; a.Cin = p->Cin; a.Cout = p->Cout;
     a.steps = (p->Cin + 63) / 64 * T::TAPS; a.ntiles_m = (int)((c.M + T::BM - 1) / T::BM); a.ntiles_n = (int)ntiles_n;
     a.W = c.W; a.H = c.H; a.relu = c.relu; a.split = T::SPLIT ? split : 1;
-    if (T::SPLIT) {
-        constexpr int CHUNKS = T::COLS / 4;
-        a.slots = (CHUNKS + split - 1) / split;
-        a.share = CHUNKS * 65536 / split + 1;   // (r * share / 65536 = r * CHUNKS / split for all r <= split <= 8)
-    }
     const bool cm = T::SRC == SRC_CM || T::SRC == SRC_CM3 || T::FUSED;
     a.ex = {c.x, cm ? 1 : p->Cin, cm ? c.ldx : 1, p->d_group_ptr, p->d_idx, p->d_val, use_tap_lists(p) ? p->d_taps : nullptr, p->G};
     CUtensorMap amap, ymap;
@@ -1500,8 +1498,9 @@ sbnn_status launch_tc(const sbnn_packed* p, const TcCall& c, int split, bool* do
     const unsigned grid = T::SPLIT ? (unsigned)(total * split) : (unsigned)std::min<long long>(total, device_sms());
     a.dm = T::SPLIT ? a.ntiles_m : (int)(grid / (unsigned)ntiles_n);
     a.dn = T::SPLIT ? 0 : (int)(grid % (unsigned)ntiles_n);
-    a.resident = !T::SPLIT && ntiles_n == 1 && a.steps * T::NU <= T::SB_MAX && a.steps * T::NU * T::B_BYTES + (T::FUSED ? T::SA_MIN : 3) * T::A_BYTES <= T::ROOM;
-    a.sb = a.resident ? a.steps * T::NU : T::SB;
+    const bool resident = !T::SPLIT && ntiles_n == 1 && a.steps * T::NU <= T::SB_MAX && a.steps * T::NU * T::B_BYTES + (T::FUSED ? T::SA_MIN : 3) * T::A_BYTES <= T::ROOM;
+    a.resident_or_share = T::SPLIT ? T::COLS / 4 * 65536 / split + 1 : resident;   // (r * share / 65536 = r * chunks / split for all r <= split <= 8)
+    a.sb = resident ? a.steps * T::NU : T::SB;
     a.sa = std::min(T::SA_MAX, (T::ROOM - a.sb * T::B_BYTES) / T::A_BYTES);
     if (T::FUSED) a.sa &= ~1;   // (see depthwise_split)
     const size_t smem = (size_t)a.sb * T::B_BYTES + (size_t)a.sa * T::A_BYTES + T::OUT_BYTES + T::CTRL + T::DW::OUTPUT + 1024;
