@@ -1284,7 +1284,15 @@ double tc_split_cost(const sbnn_packed* p, long long M, int split, int run, int 
     // Clusters of 5 to 7 start later: one 14 x 14 image, 512 -> 512, two steps a CTA in clusters of 4, 5, 6: 6.8, 7.3, 7.6 us; 2 x 28 x
     // 28, 128 -> 128 3x3, 18 steps in clusters of 4 and 5: 9.7 and 10.2.
     const double late = split > 4 && split < 8 ? 1500.0 : 0.0;
-    const double cost = (double)((runs + split - 1) / split * run) * (tc_step(64, images) + 50.0) + 9800.0 + late;
+    // Steps of a last 64 channels that are 32 or fewer take 0.6 of the others, and count for the CTAs that get them.  3x3 channel-major, 144 ->
+    // 32, nine kernel rows, the last three of 16 channels: shared by 4 11.0 us, by 5 11.6.
+    const long long half = (p->Cin - 1) % 64 < 32 ? runs - p->KH * p->KW / run : runs;
+    double most = 0.0;
+    for (int r = 0; r < split; ++r) {
+        const long long from = runs * r / split, to = runs * (r + 1) / split, whole = std::min(to, half) - std::min(from, half);
+        most = std::max(most, (double)whole + 0.6 * (double)(to - from - whole));
+    }
+    const double cost = most * run * (tc_step(64, images) + 50.0) + 9800.0 + late;
     if (cost >= limit) return 1e30;
     // Behind another launch the last clusters of 3 and of 5 of a full device find no place before others have ended.  In clusters of 3, of
     // which 45 run at a time: 9 x 5 tiles of 6 steps 10.3 us (unshared 7.5), 5 x 9 of 10 steps 11.9 (of 2: 9.6), 44 tiles of 4 steps 9.0, 43

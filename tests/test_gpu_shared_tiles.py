@@ -24,3 +24,16 @@ def test_tiles_shared_by_any_number_of_ctas(split, flags):
     err = np.abs(y.cpu().numpy().astype(np.float64) - ref.reshape(n, h, w, cout))
     assert np.all(err <= 1e-5 * s.reshape(err.shape))
     p.free()
+
+
+# 9 rows of kernels of which the last three are half as long: shared by 4 11.0, 10.4 and 10.8 us, by 5 11.6, 10.9 and 11.2; 6 equal rows:
+# 8.3 by 6, 10.2 by 4
+@pytest.mark.parametrize("n,hw,cin,cout,split", [(1, 56, 144, 32, 4), (10, 14, 148, 48, 4), (8, 13, 148, 80, 4), (5, 14, 128, 64, 6)])
+def test_the_last_steps_may_be_short(n, hw, cin, cout, split):
+    d = WL.single_conv_inputs(1, 1, 1, cin, cout, 3, 4, 30, 3, 0.05, 0.05)
+    p = sbnn.pack_weights(d["w"], d["mask"], d["bias"], 4)
+    m = n * hw * hw
+    ld = (m + 3) // 4 * 4
+    sbnn.conv3x3_gs_cm(p, torch.zeros((cin, ld), device="cuda"), ld, torch.empty((cout, ld), device="cuda"), ld, n, hw, hw, sbnn.SBNN_OUT_CM)
+    assert sbnn.debug_last_route() == (64, split)
+    p.free()
