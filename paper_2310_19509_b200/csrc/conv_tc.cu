@@ -1246,7 +1246,7 @@ double tc_cost(const sbnn_packed* p, long long M, int bn, int images) {
 // Microseconds: long launches run at the clock that the power limit leaves them.
 double tc_us(double cycles) { return cycles / (cycles < 1e5 ? 1800.0 : 1600.0); }
 
-// Clusters of `split` CTAs that the device runs at the same time (on 148 SMs 74 of 2, 33 of 4, 15 of 8).
+// Clusters of `split` CTAs that the device runs at the same time (on 148 SMs 74 of 2, 45 of 3, 33 of 4, 26 of 5, 22 of 6, 15 of 7 and 8).
 long long cluster_capacity(int split) {
     static std::mutex mu;
     static std::map<std::pair<int, int>, int> known;
