@@ -336,6 +336,8 @@ dwconv3x3_cm_col7_kernel(const float* __restrict__ w, const float* __restrict__ 
 // its neighbours by shuffle: 9 load requests for 14 outputs.  (With one scalar load per tap the kernel above
 // was limited by the number of load requests in flight, not by bytes.)  A warp holds 4 such strips in 28 lanes;
 // lanes 28-31 only take part in the shuffles.  A CTA of 4 warps covers 8 channels x 2 strips.
+// (48 registers; 40, for more CTAs, are up to 6 % faster when the layer alone is called again and again, 20 images of 512 channels 4.3 ->
+// 4.0 us, but cost 0.6 to 1.2 us a layer in the network, 33 images 437 -> 443 us.)
 template <int NI>
 __global__ void __launch_bounds__(128, 1)
 dwconv3x3_cm_w14_kernel(const float* __restrict__ w, const float* __restrict__ b, const float* __restrict__ x, int ldx,
